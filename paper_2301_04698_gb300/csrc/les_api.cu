@@ -131,6 +131,7 @@ struct les_handle {
   double* diag = nullptr;
   FusedBar* bar = nullptr;
   FusedCfg fused;
+  ChipPlan chip;
   les_unet* model = nullptr;
   int learned_fallbacks = 0;
   int cur = 0;           // scalar ping-pong: 0 -> A holds phi^k, 1 -> B
@@ -261,6 +262,7 @@ SolverArgs<T> solver_args(les_handle* h) {
   s.prof = &h->prof;
   s.bar = h->bar;
   s.fused = h->cfg.solver_path == 0 ? &h->fused : nullptr;
+  s.chip = &h->chip;
   s.e0 = (T*)h->fixed[B_E0];
   s.e1 = (T*)h->fixed[B_E1];
   return s;

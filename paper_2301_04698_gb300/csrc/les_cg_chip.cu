@@ -1,0 +1,783 @@
+// les_cg_chip.cu -- the on-chip conjugate-gradient Poisson solve (Sec. 2.4:
+// L_c psi = b, compact 7-point Laplacian, periodic in x and y, mirror or
+// periodic in z; mean of b removed, psi returned with zero mean) for any
+// grid whose vectors fit in the registers of one block per SM, FP32 or FP64.
+//
+// Each block of one persistent cooperative launch owns a brick of the grid
+// for the whole solve.  The brick extents along x, y and z differ by at most
+// one node between blocks, so no extent has to divide the grid.  A thread
+// owns one (x, y) column of the brick and a run of at most ZP planes of it,
+// and keeps p, r, q = L_c p and x of those nodes in registers.  Its z
+// neighbours are its own registers; the x and y neighbours, and the z
+// neighbours past either end of the run, come from a copy of p in shared
+// memory with a one-node ghost layer.  A brick that spans a periodic extent
+// reads its own far side, and a wall mirrors the node itself, so such sides
+// have no ghosts.  The ghost nodes are dealt to the threads: an iteration
+// loads the neighbours' published q faces and forms the ghost r and p from
+// them, so one exchange per iteration is enough.  Where a thread has few
+// planes and at most four ghosts (XS = false), x and the ghosts' r and p are
+// registers too; else x, the ghosts' r and their offsets lie in shared memory
+// (XS = true), which leaves room for 24 FP32 or 12 FP64 planes of p, r and q.
+//
+// The iteration is that of les_cg_resident.cu: one grid-wide sum of p.q,
+// r.r, r.q and q.q per iteration (alpha, and beta from |r - alpha q|^2
+// expanded in the four), posted and folded as in les_cg_regs.cu.
+//
+// What bounds it: the latency of the grid sum (two round trips through L2:
+// about 2.7 us of an iteration on the smallest grids) and, in FP64, the
+// arithmetic: a scheduler issues an FP64 warp instruction every 64 cycles, so
+// a five-step butterfly of four values in 16 warps alone costs 5000 cycles.
+// The four values are therefore reduced by a transposing butterfly (six
+// additions per warp instead of twenty), the plan weighs warps against planes
+// per thread, the FP64 stencil takes 7 operations, and x += alpha p is left
+// to the next sum's wait.
+//
+// Measured (GB300, us per iteration, 200-iteration solves; before: the
+// shared-memory kernel, or the one-pass streaming kernel where no whole
+// bricks fit):
+//   FP64  32^3 10.0 -> 5.5, 256 x 4 x 32 10.3 -> 5.6, 64 x 64 x 48 17.0 -> 10.8,
+//         50 x 47 x 33 28.9 -> 7.5, 77 x 130 x 50 66.4 -> 18.4, 96^3 77 -> 29
+//   FP32  32^3 4.3 -> 2.7, 64^3 5.1 -> 3.3, 96^3 7.5 -> 5.6, 160 x 160 x 48
+//         8.5 -> 6.5, 100 x 76 x 61 23.9 -> 4.3, 150 x 140 x 70 39.4 -> 9.1
+// FP32 grids 128 nodes wide keep les_cg_regs.cu, whose four-node lanes read
+// x neighbours by shuffles: 128 x 64 x 64 3.5 there, 4.6 here; 128 x 128 x 96
+// 5.3 and 8.9.
+#include <algorithm>
+#include <string>
+
+#include "les_gridsync.cuh"
+#include "les_internal.h"
+
+namespace les {
+namespace {
+
+constexpr int kChipThreads = 512;
+constexpr int kChipWarps = kChipThreads / 32;
+constexpr int kChipSpread = 8;      // arrival counters and copies of the partials per sum
+constexpr int kChipLine = 32;       // counters 128 bytes apart
+constexpr int kChipGhosts = 4;      // ghost nodes per thread in registers
+static_assert(kChipSpread * 4 == 32, "one lane of warp 0 per (copy, value) of the partials");
+
+template <typename T>
+struct ChipArgs {
+  int nx, ny, nz, walls;
+  T cx, cy, cz;        // 1/dx^2, 1/dy^2, 1/dz^2
+  int px, py, pz, zs;  // bricks along x, y, z; runs of planes per brick
+  int smem_p, smem_g;  // shared memory of P and (XS) of one ghost array, in elements (even)
+  long long n;
+  const T* b;
+  T* x;
+  T* rg;               // published faces of the first residual
+  T* qg0;              // published faces of q, even iterations
+  T* qg1;              // ... odd iterations
+  double* partials;    // two slots of kSumSlot words per block (the set-up and gauge sums)
+  unsigned* counters;  // kChipSpread arrival counters of the iterations' sums, kChipLine apart, zeroed
+  void* spread;        // [2 slots][kChipSpread copies][4 values][gridDim.x] partials of those sums
+  unsigned missing;    // test hook: arrivals on counter 0 that never come
+  FusedBar* bar;
+  SolverCtl* ctl;
+  double tol;
+  int maxit;
+  long long spin_cycles;
+  unsigned expected;
+  int guard;
+};
+
+// part i of n nodes in `parts` parts whose sizes differ by at most one
+__device__ __forceinline__ void chip_part(int n, int parts, int i, int& first, int& len) {
+  const int base = n / parts, rem = n - base * parts;
+  len = base + (i < rem ? 1 : 0);
+  first = i * base + min(i, rem);
+}
+__device__ __forceinline__ int chip_wrap(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
+__device__ __forceinline__ F2 acc_of(float v) { return F2{v, 0.f}; }
+__device__ __forceinline__ double acc_of(double v) { return v; }
+__device__ __forceinline__ F2 acc_xor(F2 a, int o) {
+  return F2{__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
+}
+__device__ __forceinline__ double acc_xor(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+__device__ __forceinline__ F2 acc_from_lane(F2 a, int l) {
+  return F2{__shfl_sync(0xffffffffu, a.hi, l), __shfl_sync(0xffffffffu, a.lo, l)};
+}
+__device__ __forceinline__ double acc_from_lane(double a, int l) { return __shfl_sync(0xffffffffu, a, l); }
+
+// alpha and beta from the totals; false on a zero or non-finite p.q or r.r.
+// An FP32 solve takes them in FP32 from the high parts of the totals.
+__device__ __forceinline__ bool chip_scalars(const F2 (&t)[4], float& ta, float& tb) {
+  const float pq = t[0].hi, r2 = t[1].hi, rq = t[2].hi, q2 = t[3].hi;
+  if (!(pq != 0.f) || !isfinite(pq) || !isfinite(r2)) return false;
+  const float alpha = r2 / pq;
+  ta = alpha;
+  tb = fmaf(alpha * alpha, q2, fmaf(-2.f * alpha, rq, r2)) / r2;  // |r - alpha q|^2 / r.r
+  return true;
+}
+__device__ __forceinline__ bool chip_scalars(const double (&t)[4], double& ta, double& tb) {
+  const double pq = t[0], r2 = t[1], rq = t[2], q2 = t[3];
+  if (!(pq != 0.0) || !isfinite(pq) || !isfinite(r2)) return false;
+  const double inv = 1.0 / (r2 * pq);  // one FP64 division for both
+  const double alpha = r2 * r2 * inv;
+  ta = alpha;
+  tb = fma(alpha * alpha, q2, fma(-2.0 * alpha, rq, r2)) * (pq * inv);
+  return true;
+}
+
+template <typename T, int ZP, bool XS>
+__global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
+  using Acc = decltype(Dot<T>().acc());  // FP32 pair (FP32 solve) or FP64
+  extern __shared__ __align__(16) unsigned char smraw[];
+  constexpr int NG = XS ? 1 : kChipGhosts;  // ghosts per thread held in registers
+  T* P = reinterpret_cast<T*>(smraw);  // p with its ghost layer
+  const int tid = threadIdx.x, nthr = blockDim.x;
+  const int lane = tid & 31, warp = tid >> 5, nwarp = nthr >> 5;
+  int i0, j0, k0, bx, by, bz;
+  chip_part(f.nx, f.px, blockIdx.x % f.px, i0, bx);
+  chip_part(f.ny, f.py, (blockIdx.x / f.px) % f.py, j0, by);
+  chip_part(f.nz, f.pz, blockIdx.x / (f.px * f.py), k0, bz);
+  const int SY = bx + 2, SZ = SY * (by + 2);
+  const int gpl = f.nx * f.ny;
+  const bool low = f.walls && k0 == 0, high = f.walls && k0 + bz == f.nz;  // the brick touches a wall
+  const T cx = f.cx, cy = f.cy, cz = f.cz;
+
+  // this thread's column and run of planes
+  const int ncol = bx * by;
+  const int run = tid / ncol;
+  const int col = tid - run * ncol;
+  const bool active = run < f.zs;
+  const int ly = col / bx, lx = col - ly * bx;
+  const int zq = bz / f.zs, zr = bz - zq * f.zs;
+  const int z0 = run * zq + min(run, zr);
+  const int nzp = active ? zq + (run < zr ? 1 : 0) : 0;
+  int pown = (z0 + 1) * SZ + (ly + 1) * SY + lx + 1;
+  int gown = (k0 + z0) * gpl + (j0 + ly) * f.nx + i0 + lx;
+  // offsets of the neighbours in P: a brick that spans a periodic extent
+  // wraps onto itself, a wall mirrors the node
+  const int oxm = f.px == 1 && lx == 0 ? bx - 1 : -1, oxp = f.px == 1 && lx == bx - 1 ? 1 - bx : 1;
+  const int oym = f.py == 1 && ly == 0 ? (by - 1) * SY : -SY, oyp = f.py == 1 && ly == by - 1 ? (1 - by) * SY : SY;
+  int ozm = -SZ, ozp = SZ;  // below the run's first plane, above its last
+  if (z0 == 0) {
+    if (low) ozm = 0;
+    else if (!f.walls && f.pz == 1) ozm = (bz - 1) * SZ;
+  }
+  if (z0 + nzp == bz) {
+    if (high) ozp = 0;
+    else if (!f.walls && f.pz == 1) ozp = (1 - bz) * SZ;
+  }
+  // nodes that a neighbouring brick reads
+  const bool fcol = (f.px > 1 && (lx == 0 || lx == bx - 1)) || (f.py > 1 && (ly == 0 || ly == by - 1));
+  const bool flow = f.pz > 1 && !low && z0 == 0, fhigh = f.pz > 1 && !high && z0 + nzp == bz;
+  auto is_face = [&](int j) { return fcol || (flow && j == 0) || (fhigh && j == nzp - 1); };
+
+  // the brick's ghost nodes: the z faces, then the y faces, then the x faces
+  const int nlo = f.pz > 1 && !low ? ncol : 0, nhi = f.pz > 1 && !high ? ncol : 0;
+  const int nyf = f.py > 1 ? bx * bz : 0, nxf = f.px > 1 ? by * bz : 0;  // nodes per y and x face
+  const int ngh = nlo + nhi + 2 * (nyf + nxf);
+  // offsets of ghost node id in P and in global memory.  A ghost beyond a
+  // wall does not occur: the sides that touch one have none.
+  auto ghost_at = [&](int id) -> int2 {
+    int gx = 0, gy = 0, gz = 0;
+    if (id < nlo + nhi) {
+      gz = id < nlo ? -1 : bz;
+      id -= id < nlo ? 0 : nlo;
+      gy = id / bx, gx = id - gy * bx;
+    } else if ((id -= nlo + nhi) < 2 * nyf) {
+      gy = id < nyf ? -1 : by;
+      id -= id < nyf ? 0 : nyf;
+      gz = id / bx, gx = id - gz * bx;
+    } else {
+      id -= 2 * nyf;
+      gx = id < nxf ? -1 : bx;
+      id -= id < nxf ? 0 : nxf;
+      gz = id / by, gy = id - gz * by;
+    }
+    return make_int2((gz + 1) * SZ + (gy + 1) * SY + gx + 1,
+                     chip_wrap(k0 + gz, f.nz) * gpl + chip_wrap(j0 + gy, f.ny) * f.nx + chip_wrap(i0 + gx, f.nx));
+  };
+  // XS: x by plane and thread, then r, q and the offsets of the ghost nodes
+  T* XM = P + f.smem_p;
+  T* GR = XM + ZP * nthr;
+  T* GQ = GR + f.smem_g;
+  int2* GT = reinterpret_cast<int2*>(GQ + f.smem_g);
+  int gsm[NG], ggl[NG];  // else: this thread's ghosts (-1: none)
+  if constexpr (XS) {
+    for (int id = tid; id < ngh; id += nthr) GT[id] = ghost_at(id);
+    gsm[0] = ggl[0] = 0;
+  } else {
+#pragma unroll
+    for (int g = 0; g < NG; ++g) {
+      const int id = tid + g * nthr;
+      gsm[g] = -1;
+      ggl[g] = 0;
+      if (id < ngh) {
+        const int2 o = ghost_at(id);
+        gsm[g] = o.x;
+        ggl[g] = o.y;
+      }
+    }
+  }
+
+  T p[ZP] = {}, r[ZP] = {}, q[ZP] = {};
+  T xr[XS ? 1 : ZP] = {};
+  auto get_x = [&](int j) -> T { return XS ? XM[j * nthr + tid] : xr[XS ? 0 : j]; };
+  auto set_x = [&](int j, T v) {
+    if constexpr (XS) XM[j * nthr + tid] = v;
+    else xr[j] = v;
+  };
+  // x += alpha p of an iteration is added during the next sum's wait, where
+  // registers for the old p are left (warp 0, which waits, adds it at once)
+  constexpr bool kDefer = !XS && ZP * sizeof(T) <= 32;
+  T po[kDefer ? ZP : 1] = {};
+  T rgh[NG] = {}, pgh[NG] = {};  // r and p at the ghost nodes
+  // L_c p at plane j of the run.  FP32: second differences formed before
+  // scaling, as in the other CG kernels.  FP64, where each operation counts:
+  // the six neighbours scaled, then the centre -- 7 operations instead of 9.
+  const T c0 = T(2) * (cx + cy + cz);
+  auto stencil = [&](int j) -> T {
+    const T* pj = P + pown + j * SZ;
+    const T d = j > 0 ? p[j > 0 ? j - 1 : 0] : pj[ozm];
+    const T u = (j + 1 < ZP && j + 1 < nzp) ? p[j + 1 < ZP ? j + 1 : ZP - 1] : pj[ozp];
+    if constexpr (sizeof(T) == 8) {
+      const T s = fma(cz, d + u, fma(cy, pj[oym] + pj[oyp], cx * (pj[oxm] + pj[oxp])));
+      return fma(-c0, p[j], s);
+    } else {
+      const T c2 = T(2) * p[j];
+      return (pj[oxm] + pj[oxp] - c2) * cx + (pj[oym] + pj[oyp] - c2) * cy + (d + u - c2) * cz;
+    }
+  };
+
+  // A at the ghost nodes into P (keep: as r and p there), outside the iterations
+  auto fill_ghosts = [&](const T* A, bool keep) {
+    if constexpr (XS) {
+      for (int id = tid; id < ngh; id += nthr) {
+        const int2 o = GT[id];
+        const T v = __ldcg(A + o.y);
+        P[o.x] = v;
+        if (keep) GR[id] = v;
+      }
+    } else {
+#pragma unroll
+      for (int g = 0; g < NG; ++g)
+        if (gsm[g] >= 0) {
+          const T v = __ldcg(A + ggl[g]);
+          P[gsm[g]] = v;
+          if (keep) rgh[g] = pgh[g] = v;
+        }
+    }
+  };
+
+  GridSync gs{f.bar, f.partials, f.spin_cycles, f.expected, 0u};
+  __shared__ struct {
+    T mean, ta, tb;
+    int status, restart;
+    double bb, rel;  // |b - mean|^2 and the relative residual of x0
+  } sc;
+  __shared__ T shv[4][kChipWarps];
+  __shared__ Acc tot[4];
+  __shared__ int s_fail;
+  double rr = 0.0, bb = 0.0, rel = 0.0;  // meaningful in thread 0
+  int status = 0;  // 0 running, 1 converged, 2 maxit, 3 breakdown, 4 zero rhs, 5 timeout
+  T rr_own = T(0);  // this thread's share of r.r for the next sum
+
+  // mean of b (b held in r)
+  {
+    Dot<T> a1[1];
+#pragma unroll
+    for (int j = 0; j < ZP; ++j)
+      if (j < nzp) {
+        r[j] = __ldcg(f.b + gown + j * gpl);
+        a1[0].add(r[j]);
+      }
+    double t[1];
+    const bool ok = grid_dot_t0<1>(a1, gs, t);
+    if (tid == 0) {
+      sc.status = ok ? 0 : 5;
+      sc.mean = (T)(t[0] / (double)f.n);
+    }
+    __syncthreads();
+    status = sc.status;
+  }
+  const T mean = sc.mean;
+  // x0 with its ghosts in p and the copy; r = (b - mean) - L_c x0, published
+  if (!status) {
+#pragma unroll
+    for (int j = 0; j < ZP; ++j)
+      if (j < nzp) {
+        p[j] = __ldcg(f.x + gown + j * gpl);
+        set_x(j, p[j]);
+        P[pown + j * SZ] = p[j];
+      }
+    fill_ghosts(f.x, false);
+    __syncthreads();
+    Dot<T> a2[2];
+#pragma unroll
+    for (int j = 0; j < ZP; ++j)
+      if (j < nzp) {
+        const T bm = r[j] - mean;
+        r[j] = bm - stencil(j);
+        if (is_face(j)) __stcg(f.rg + gown + j * gpl, r[j]);
+        a2[0].add(r[j] * r[j]);
+        a2[1].add(bm * bm);
+      }
+    rr_own = a2[0].s;
+    double s2[2];
+    const bool ok = grid_dot_t0<2>(a2, gs, s2);
+    if (tid == 0) {
+      // the plain solver judges a learned first guess: if it leaves a larger
+      // residual than x0 = 0, restart from zero (r = b - mean b, r.r = |b|^2)
+      sc.status = ok ? 0 : 5;
+      sc.restart = ok && f.guard && s2[0] > s2[1];
+      rr = sc.restart ? s2[1] : s2[0];
+      bb = s2[1];
+    }
+    __syncthreads();
+    status = sc.status;
+    if (!status && sc.restart) {
+      rr_own = T(0);
+#pragma unroll
+      for (int j = 0; j < ZP; ++j)
+        if (j < nzp) {
+          set_x(j, T(0));
+          r[j] = __ldcg(f.b + gown + j * gpl) - mean;
+          rr_own += r[j] * r[j];
+          if (is_face(j)) __stcg(f.rg + gown + j * gpl, r[j]);
+        }
+      Dot<T> none[1];
+      double t[1];
+      const bool ok2 = grid_dot_t0<1>(none, gs, t);  // a grid barrier: the new faces are visible
+      if (tid == 0) sc.status = ok2 ? 0 : 5;
+      __syncthreads();
+      status = sc.status;
+    }
+  }
+  if (tid == 0) {
+    if (!status) {
+      if (bb == 0.0) status = 4;
+      else {
+        rel = sqrt(rr / bb);
+        if (rel <= f.tol) status = 1;
+        else if (f.maxit <= 0) status = 2;
+      }
+    }
+    sc.status = status;
+    sc.bb = bb;
+    sc.rel = rel;
+  }
+  __syncthreads();
+  status = sc.status;
+  Acc rr_stop, rr_last;  // rr_last meaningful in thread 0
+  acc_from(f.tol * f.tol * sc.bb, rr_stop);
+  acc_from(rr, rr_last);
+  int iter = 0;
+  T ta = T(0), tb = T(0);
+  if (!status) {
+    // p_0 = r_0, with r_0 at the ghost nodes from the published faces
+#pragma unroll
+    for (int j = 0; j < ZP; ++j)
+      if (j < nzp) {
+        p[j] = r[j];
+        P[pown + j * SZ] = p[j];
+      }
+    fill_ghosts(f.rg, true);
+    __syncthreads();
+    const unsigned G = gridDim.x;
+    for (;;) {
+      // the offsets of the planes are formed anew in each iteration: hoisted out
+      // of the loop they would take the registers of the vectors
+      asm volatile("" : "+r"(pown), "+r"(gown));
+      T* qw = (iter & 1) ? f.qg1 : f.qg0;  // this iteration's q faces
+      T d0 = T(0), d2 = T(0), d3 = T(0);   // p.q, r.q, q.q
+#pragma unroll
+      for (int j = 0; j < ZP; ++j)
+        if (j < nzp) {
+          q[j] = stencil(j);
+          if (is_face(j)) __stcg(qw + gown + j * gpl, q[j]);
+          d0 += p[j] * q[j];
+          d2 += r[j] * q[j];
+          d3 += q[j] * q[j];
+        }
+      // each warp's four values by a transposing butterfly: after it lanes
+      // 8k .. 8k + 7 hold the warp's value k
+      {
+        const bool up = lane & 16, odd = lane & 8;
+        T a0 = up ? d2 : d0, a1 = up ? d3 : rr_own;                // kept
+        const T s0 = up ? d0 : d2, s1 = up ? rr_own : d3;          // given to lane ^ 16
+        a0 += __shfl_xor_sync(0xffffffffu, s0, 16);
+        a1 += __shfl_xor_sync(0xffffffffu, s1, 16);
+        T v = odd ? a1 : a0;
+        v += __shfl_xor_sync(0xffffffffu, odd ? a0 : a1, 8);
+        v += __shfl_xor_sync(0xffffffffu, v, 4);
+        v += __shfl_xor_sync(0xffffffffu, v, 2);
+        v += __shfl_xor_sync(0xffffffffu, v, 1);
+        if ((lane & 7) == 0) shv[lane >> 3][warp] = v;
+      }
+      // also orders every thread's q-face stores before warp 0's release
+      __syncthreads();
+      // this sum's partials: kChipSpread copies, this block reads copy b mod kChipSpread
+      Acc* slot = reinterpret_cast<Acc*>(f.spread) + (size_t)(iter & 1) * kChipSpread * 4 * G;
+      if (warp == 0) {
+        // lanes 8k .. 8k + 7: value k of the block
+        const int k = lane >> 3;
+        Acc a = acc_of(T(0));
+        for (int w = lane & 7; w < nwarp; w += 8) a = acc_add(a, acc_of(shv[k][w]));
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) a = acc_add(a, acc_xor(a, o));
+        // lane l writes value l mod 4 into copy l / 4
+        const Acc mine = acc_from_lane(a, 8 * (lane & 3));
+        acc_store(slot + ((size_t)(lane >> 2) * 4 + (lane & 3)) * G + blockIdx.x, mine);
+        __syncwarp();  // orders the lanes' stores before lane 0's release
+        if (lane == 0) red_release_add(f.counters + (blockIdx.x % kChipSpread) * kChipLine, 1u);
+        // posted: the other warps may start their deferred work
+        asm volatile("bar.arrive 2, %0;" ::"r"(nthr) : "memory");
+        // lanes 0 .. kChipSpread - 1 wait for one counter each (counter i
+        // takes blocks i, i + kChipSpread, ...; counter 0 also the test
+        // hook's missing arrivals)
+        bool done = lane >= kChipSpread;
+        const unsigned mine_n = lane < (int)G ? (G - lane + kChipSpread - 1) / kChipSpread : 0u;
+        const unsigned target = done ? 0u : ((unsigned)iter + 1u) * (mine_n + (lane == 0 ? f.missing : 0u));
+        const long long t0 = clock64();
+        int fail = 0;
+        for (unsigned spins = 1;; ++spins) {
+          if (!done) done = (int)(ld_acquire(f.counters + lane * kChipLine) - target) >= 0;
+          if (__all_sync(0xffffffffu, done)) break;
+          const bool quit = (spins & 63u) == 0u && (ld_volatile(&gs.bar->fail.v) != 0u || clock64() - t0 > gs.spin);
+          if (__any_sync(0xffffffffu, quit)) {
+            if (lane == 0) atomicExch(&gs.bar->fail.v, 1u);
+            fail = 1;
+            break;
+          }
+        }
+        __syncwarp();  // orders the lanes' acquires before the reads of every lane
+        if (lane == 0) s_fail = fail;
+        // every block has arrived (or the wait gave up)
+        asm volatile("bar.arrive 1, %0;" ::"r"(nthr) : "memory");
+      } else {
+        asm volatile("bar.sync 2, %0;" ::"r"(nthr) : "memory");
+        if constexpr (kDefer) {
+          if (iter > 0) {
+#pragma unroll
+            for (int j = 0; j < ZP; ++j) xr[XS ? 0 : j] += ta * po[kDefer ? j : 0];
+          }
+        }
+        asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory");
+      }
+      // warps 0 .. 3 fold one value each (in block order, so every block
+      // obtains the same totals); every thread loads the q of its ghosts
+      const Acc* mycopy = slot + (size_t)(blockIdx.x % kChipSpread) * 4 * G;
+      T gq[NG];
+      auto load_ghosts = [&] {
+        if constexpr (XS) {
+          for (int id = tid; id < ngh; id += nthr) cp_async(GQ + id, qw + GT[id].y);
+          cp_commit();
+        } else {
+#pragma unroll
+          for (int g = 0; g < NG; ++g) gq[g] = gsm[g] >= 0 ? __ldcg(qw + ggl[g]) : T(0);
+        }
+      };
+      if (warp < 4) {
+        for (int k = warp; k < 4; k += nwarp) {
+          Acc t = acc_of(T(0));
+          for (unsigned b0 = lane; b0 < G; b0 += 32 * 5) {
+            Acc w[5];
+#pragma unroll
+            for (int u = 0; u < 5; ++u)
+              w[u] = b0 + 32 * u < G ? acc_load(mycopy + (size_t)k * G + b0 + 32 * u) : acc_of(T(0));
+            if (k == warp && b0 == (unsigned)lane) load_ghosts();
+#pragma unroll
+            for (int u = 0; u < 5; ++u) t = acc_add(t, w[u]);
+          }
+          if (k == warp && (unsigned)lane >= G) load_ghosts();
+          t = acc_warp(t);
+          if (lane == 0) tot[k] = t;
+        }
+        // the folds are complete: thread 0 forms the status, alpha and beta
+        asm volatile("bar.sync 3, %0;" ::"r"(32 * min(nwarp, 4)) : "memory");
+        if (tid == 0) {
+          int st = 0;
+          if (s_fail) {
+            st = 5;
+          } else {
+            const Acc t4[4] = {tot[0], tot[1], tot[2], tot[3]};
+            rr_last = t4[1];
+            T al = T(0), be = T(0);
+            if (acc_le(t4[1], rr_stop)) st = 1;
+            else if (iter >= f.maxit) st = 2;
+            else if (!chip_scalars(t4, al, be)) st = 3;
+            sc.ta = al;
+            sc.tb = be;
+          }
+          sc.status = st;
+        }
+      } else {
+        load_ghosts();
+      }
+      if constexpr (XS) cp_wait<0>();
+      __syncthreads();
+      status = sc.status;
+      if (status) break;
+      ta = sc.ta;
+      tb = sc.tb;
+      rr_own = T(0);
+#pragma unroll
+      for (int j = 0; j < ZP; ++j)
+        if (j < nzp) {
+          if (!kDefer || warp == 0) set_x(j, get_x(j) + ta * p[j]);
+          else po[kDefer ? j : 0] = p[j];
+          r[j] -= ta * q[j];
+          rr_own += r[j] * r[j];
+          p[j] = r[j] + tb * p[j];
+          P[pown + j * SZ] = p[j];
+        }
+      if constexpr (XS) {
+        for (int id = tid; id < ngh; id += nthr) {
+          const int at = GT[id].x;
+          const T rv = GR[id] - ta * GQ[id];
+          GR[id] = rv;
+          P[at] = rv + tb * P[at];
+        }
+      } else {
+#pragma unroll
+        for (int g = 0; g < NG; ++g)
+          if (gsm[g] >= 0) {
+            rgh[g] -= ta * gq[g];
+            pgh[g] = rgh[g] + tb * pgh[g];
+            P[gsm[g]] = pgh[g];
+          }
+      }
+      iter += 1;
+      __syncthreads();
+    }
+  }
+  if (tid == 0) rel = (iter > 0 && sc.bb > 0.0) ? sqrt(acc_value(rr_last) / sc.bb) : sc.rel;
+
+  // zero-mean gauge (or zero for a zero right side), written back to x
+  if (status != 5) {
+    Dot<T> ax[1];
+#pragma unroll
+    for (int j = 0; j < ZP; ++j)
+      if (j < nzp) ax[0].add(get_x(j));
+    double t[1];
+    const bool ok = grid_dot_t0<1>(ax, gs, t);
+    if (tid == 0) {
+      if (!ok) status = 5;
+      sc.mean = (T)(t[0] / (double)f.n);
+      sc.status = status;
+    }
+    __syncthreads();
+    status = sc.status;
+    if (status != 5) {
+      const T mx = sc.mean;
+#pragma unroll
+      for (int j = 0; j < ZP; ++j)
+        if (j < nzp) __stcg(f.x + gown + j * gpl, status == 4 ? T(0) : get_x(j) - mx);
+    }
+  }
+  if (blockIdx.x == 0 && tid == 0) {
+    f.ctl->iter = iter;
+    f.ctl->rel = rel;
+    f.ctl->done = status;
+  }
+}
+
+// planes per thread with x and the ghosts in registers, and at most
+template <typename T>
+constexpr int kChipRegPlanes = sizeof(T) == 4 ? 8 : 4;
+template <typename T>
+constexpr int kChipMaxPlanes = sizeof(T) == 4 ? 24 : 12;
+
+// the instantiated plane counts that hold zp planes
+inline int chip_planes(int zp, bool xs, size_t es) {
+  static constexpr int r4[] = {1, 2, 4, 6, 8}, x4[] = {4, 8, 12, 16, 20, 24}, r8[] = {1, 2, 4}, x8[] = {4, 6, 8, 10, 12};
+  const int* t = es == 4 ? (xs ? x4 : r4) : (xs ? x8 : r8);
+  while (*t < zp) ++t;
+  return *t;
+}
+
+// Bricks of bx x by x bz nodes (rounded up), at most one per SM; for each
+// (px, py) as many bricks along z as the SMs hold, in runs that fit a block's
+// threads and a thread's planes.  Taken is the plan with the least time of
+// the busiest block in the model below (cycles; the latency of the grid sum
+// is common to all).  The model is a fit to some hundred timed plans: on 64^3
+// FP32 eight planes per thread in 16 warps take 4.1 us, four 3.3 us; on 32^3
+// FP64 two warps of four planes take 7.8 us, four of two 5.5, eight of one
+// 5.8; it picks within 0.1 us of the fastest timed plan on the grids above.
+template <typename T>
+bool make_chip_plan(const Grid<T>& g, int nsm, size_t smem_max, int max_blocks, ChipPlan& best) {
+  const int gmax = std::min(nsm, max_blocks);
+  double cost = 0;
+  bool found = false;
+  for (int px = 1; px <= std::min(g.nx, gmax); ++px) {
+    const int bx = (g.nx + px - 1) / px;
+    if (px > 1 && (g.nx + px - 2) / (px - 1) == bx) continue;  // as large, with more bricks
+    for (int py = 1; px * py <= gmax && py <= g.ny; ++py) {
+      const int by = (g.ny + py - 1) / py, ncol = bx * by;
+      if (ncol > kChipThreads || (py > 1 && (g.ny + py - 2) / (py - 1) == by)) continue;
+      int pz = std::min(g.nz, gmax / (px * py));
+      const int bz = (g.nz + pz - 1) / pz;
+      pz = (g.nz + bz - 1) / bz;
+      const size_t np = ((size_t)(bx + 2) * (by + 2) * (bz + 2) + 1) / 2 * 2;
+      const int yg = py > 1 ? 2 * bx * bz : 0, xg = px > 1 ? 2 * by * bz : 0, zg = pz > 1 ? 2 * ncol : 0;
+      for (int zs = 1; zs <= g.nz / pz && ncol * zs <= kChipThreads; ++zs) {
+        const int zp = (bz + zs - 1) / zs, nw = (ncol * zs + 31) / 32;
+        if (zp > kChipMaxPlanes<T>) continue;
+        const int gh = zg + yg + xg, ng = (gh + 1) / 2 * 2;
+        const bool xs = zp > kChipRegPlanes<T> || gh > kChipGhosts * 32 * nw;
+        const int zi = chip_planes(zp, xs, sizeof(T));
+        const size_t smem =
+            (np + (xs ? (size_t)zi * 32 * nw + 2 * (size_t)ng : 0)) * sizeof(T) + (xs ? ng * sizeof(int2) : 0);
+        if (smem > smem_max) continue;
+        // per scheduler: 60 cycles per warp and plane; per thread: the chain
+        // of its planes and ghosts; an x face is a strided access
+        const int wps = (nw + 3) / 4, gt = (gh + 32 * nw - 1) / (32 * nw);
+        double c = (xs ? 75.0 : 60.0) * wps * zp;
+        // FP64: a warp instruction every 64 cycles of a scheduler -- 14 per
+        // node, six of the reduction, two per ghost
+        if (sizeof(T) == 8) c = 86.0 * (wps * (14.0 * zp + 6.0) + 2.0 * gh / 128.0);
+        c += 200.0 * zp + 150.0 * gt + 3.0 * xg;
+        if (!found || c < cost) {
+          found = true;
+          cost = c;
+          best.px = px, best.py = py, best.pz = pz;
+          best.zs = zs, best.zp = zi, best.threads = 32 * nw;
+          best.xs = xs;
+          best.np = (int)np, best.ng = ng;
+          best.smem = smem;
+        }
+      }
+    }
+  }
+  return found;
+}
+
+template <typename T, bool XS, int... Z>
+const void* chip_kernel_of(int zp) {
+  const void* k = nullptr;
+  ((zp == Z ? (void)(k = (const void*)k_cg_chip<T, Z, XS>) : (void)0), ...);
+  return k;
+}
+template <typename T>
+const void* chip_kernel(int zp, bool xs) {
+  if constexpr (sizeof(T) == 4)
+    return xs ? chip_kernel_of<T, true, 4, 8, 12, 16, 20, 24>(zp) : chip_kernel_of<T, false, 1, 2, 4, 6, 8>(zp);
+  else
+    return xs ? chip_kernel_of<T, true, 4, 6, 8, 10, 12>(zp) : chip_kernel_of<T, false, 1, 2, 4>(zp);
+}
+
+}  // namespace
+
+template <typename T>
+int poisson_solve_chip(const SolverArgs<T>& a, const FusedCfg& fc, const T* b, T* x, double tol, int maxit,
+                       int* iters, double* rel, std::string* err, bool* used) {
+  *used = false;
+  if (!(a.op == LES_OP_COMPACT && a.solver == LES_SOLVER_CG && a.g.nz >= 2 && a.bar && a.r && a.p0 && a.p1) ||
+      (long long)a.g.nx * a.g.ny * a.g.nz > (long long)kChipThreads * kChipMaxPlanes<T> * a.nsm)
+    return LES_OK;
+  int dev = 0, nsm = 0, smem_optin = 0;
+  cudaError_t e;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+      (e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
+      (e = cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) {
+    if (err) *err = std::string("register-brick CG: ") + cudaGetErrorString(e);
+    return LES_ERR_CUDA;
+  }
+  // the plan depends on the grid, the device and the block cap alone: kept
+  // by the handle (a search takes tens of microseconds)
+  ChipPlan local, &pl = a.chip ? *a.chip : local;
+  if (pl.nsm != nsm || pl.max_blocks != fc.max_blocks) {
+    pl = ChipPlan{};
+    pl.nsm = nsm;
+    pl.max_blocks = fc.max_blocks;
+    // leave room for the reductions' static shared memory (about 2 KB)
+    pl.fits = make_chip_plan(a.g, nsm, (size_t)std::max(0, smem_optin - 4096), fc.max_blocks, pl);
+  }
+  if (!pl.fits) return LES_OK;
+  const void* kern = chip_kernel<T>(pl.zp, pl.xs);
+  const unsigned G = (unsigned)(pl.px * pl.py * pl.pz);
+  int per_sm = 0;
+  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem)) != cudaSuccess ||
+      (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, pl.threads, pl.smem)) != cudaSuccess) {
+    if (err) *err = std::string("register-brick CG occupancy: ") + cudaGetErrorString(e);
+    return LES_ERR_CUDA;
+  }
+  if (per_sm < 1 || (long long)G > (long long)per_sm * nsm) return LES_OK;  // not co-resident
+  ChipArgs<T> f;
+  f.nx = a.g.nx;
+  f.ny = a.g.ny;
+  f.nz = a.g.nz;
+  f.walls = a.g.walls;
+  f.cx = a.g.idx * a.g.idx;
+  f.cy = a.g.idy * a.g.idy;
+  f.cz = a.g.idz * a.g.idz;
+  f.px = pl.px;
+  f.py = pl.py;
+  f.pz = pl.pz;
+  f.zs = pl.zs;
+  f.smem_p = pl.np;
+  f.smem_g = pl.ng;
+  f.n = (long long)f.nx * f.ny * f.nz;
+  f.b = b;
+  f.x = x;
+  f.rg = a.r;
+  f.qg0 = a.p0;
+  f.qg1 = a.p1;
+  f.partials = a.partials;
+  // past the set-up sums' two slots: the counters, then the copies of the
+  // iterations' partials (2 x kChipSpread x 4 words per block)
+  f.counters = reinterpret_cast<unsigned*>(a.partials + 2 * (size_t)kSumSlot * G);
+  f.spread = a.partials + 2 * (size_t)kSumSlot * G + kChipSpread * kChipLine / 2;
+  f.missing = (unsigned)std::max(0, fc.missing);
+  f.bar = a.bar;
+  f.ctl = a.ctl;
+  f.tol = tol;
+  f.maxit = maxit;
+  f.spin_cycles = fc.spin_cycles;
+  // the test hook's missing arrivals apply to the iterations' sums (whose
+  // wait is this kernel's own); the set-up sums wait for the launched blocks
+  f.expected = G;
+  f.guard = a.guard;
+  *used = true;
+  if ((e = cudaMemsetAsync(a.bar, 0, sizeof(FusedBar), a.st)) != cudaSuccess ||
+      (e = cudaMemsetAsync(f.counters, 0, kChipSpread * kChipLine * sizeof(unsigned), a.st)) != cudaSuccess) {
+    if (err) *err = std::string("register-brick CG barrier reset: ") + cudaGetErrorString(e);
+    return LES_ERR_CUDA;
+  }
+  void* args[] = {&f};
+  {
+    ProfScope ps(a.prof, KI_CG_RESIDENT, a.st);
+    e = cudaLaunchCooperativeKernel(kern, dim3(G), dim3(pl.threads), args, pl.smem, a.st);
+  }
+  if (e != cudaSuccess) {
+    if (err) *err = std::string("register-brick CG launch: ") + cudaGetErrorString(e);
+    return LES_ERR_CUDA;
+  }
+  if ((e = cudaMemcpyAsync(a.ctl_host, a.ctl, sizeof(SolverCtl), cudaMemcpyDeviceToHost, a.st)) != cudaSuccess ||
+      (e = cudaStreamSynchronize(a.st)) != cudaSuccess) {
+    if (err) *err = std::string("register-brick CG: ") + cudaGetErrorString(e);
+    return LES_ERR_CUDA;
+  }
+  const SolverCtl& c = *a.ctl_host;
+  if (iters) *iters = c.iter;
+  if (rel) *rel = c.rel;
+  // algorithmic traffic of the solve, as for every CG kernel (its vectors
+  // stay on chip)
+  if (a.prof) a.prof->bytes[KI_CG_RESIDENT] += (kCgSetupFields + kCgIterFields * c.iter) * (double)f.n * sizeof(T);
+  switch (c.done) {
+    case 1:
+    case 4: return LES_OK;
+    case 2: return LES_ERR_NOT_CONVERGED;
+    case 3:
+      if (err) *err = "poisson: breakdown (zero or non-finite p.Ap / residual)";
+      return LES_ERR_NONFINITE;
+    case 5:
+      if (err) *err = "poisson: a grid barrier wait timed out";
+      return LES_ERR_TIMEOUT;
+    default:
+      if (err) *err = "poisson: register-brick CG returned no status";
+      return LES_ERR_CUDA;
+  }
+}
+
+template int poisson_solve_chip<float>(const SolverArgs<float>&, const FusedCfg&, const float*, float*, double, int,
+                                       int*, double*, std::string*, bool*);
+template int poisson_solve_chip<double>(const SolverArgs<double>&, const FusedCfg&, const double*, double*, double,
+                                        int, int*, double*, std::string*, bool*);
+
+}  // namespace les

@@ -598,12 +598,20 @@ int poisson_solve_resident(const SolverArgs<T>& a, const FusedCfg& fc, const T* 
   *used = false;
   if (!(a.op == LES_OP_COMPACT && a.solver == LES_SOLVER_CG && a.g.nz >= 2 && a.bar && a.r && a.p0 && a.p1))
     return LES_OK;
-  // FP32 grids 128 nodes wide: p, r and q in registers (les_cg_regs.cu)
+  // The vectors in registers: FP32 grids 128 nodes wide in les_cg_regs.cu
+  // (3.5 against 4.6 us per iteration on 128 x 64 x 64), every other grid in
+  // les_cg_chip.cu, up to 24 FP32 or 12 FP64 nodes per thread of one block per
+  // SM.  What is left for the kernel here are grids of whole bricks between
+  // that and the shared memory of all SMs, and cg_resident = 2.
   if constexpr (sizeof(T) == 4) {
     if (fc.resident == 0) {
       const int rc = poisson_solve_regs(a, fc, b, x, tol, maxit, iters, rel, err, used);
       if (*used || rc != LES_OK) return rc;
     }
+  }
+  if (fc.resident == 0) {
+    const int rc = poisson_solve_chip<T>(a, fc, b, x, tol, maxit, iters, rel, err, used);
+    if (*used || rc != LES_OK) return rc;
   }
   int dev = 0, nsm = 0, smem_optin = 0;
   cudaError_t e;

@@ -105,9 +105,8 @@ struct FusedCfg {
   int variant = 0;                      // 0 standard iterates (resident, else FP32 columns, else
                                         // two-phase streaming when tile-aligned, else one-pass),
                                         // 2 two-phase streaming, 3 one-pass one-reduction, 4 columns
-  int resident = 0;                     // 0 on-chip CG when the grid fits (p, r, q in registers where
-                                        // the grid allows), 1 never, 2 on chip with every vector in
-                                        // shared memory
+  int resident = 0;                     // 0 on-chip CG when the grid fits (vectors in registers), 1 never,
+                                        // 2 on chip with every vector in shared memory
 };
 
 struct LaunchCfg {
@@ -265,6 +264,19 @@ cudaError_t launch_cfl_max(const StageArgs<T>& a, const T* u, const T* v, const 
                            double* partials, SolverCtl* ctl);
 
 // ---- Poisson solver (les_solver.cu) ----------------------------------------
+// Brick plan of the register-brick CG (les_cg_chip.cu) for one grid; valid for
+// the SM count and block cap it was made for.
+struct ChipPlan {
+  int nsm = 0, max_blocks = 0;
+  bool fits = false;
+  int px = 0, py = 0, pz = 0;  // bricks along x, y, z
+  int zs = 0, zp = 0;          // runs of planes per brick, planes per thread (as instantiated)
+  bool xs = false;             // x and the ghosts in shared memory
+  int np = 0, ng = 0;          // elements of the copy of p, of a ghost array
+  int threads = 0;
+  size_t smem = 0;
+};
+
 template <typename T>
 struct SolverArgs {
   Grid<T> g;
@@ -288,6 +300,7 @@ struct SolverArgs {
   T* e0 = nullptr;                  // two spare vectors (the flexible CG's z and b)
   T* e1 = nullptr;
   const FusedCfg* fused = nullptr;  // enables the persistent CG when eligible
+  ChipPlan* chip = nullptr;         // the handle's brick plan (made on first use)
 };
 
 template <typename T>
@@ -318,6 +331,11 @@ int poisson_solve_wave(const SolverArgs<T>& a, const FusedCfg& fc, const T* b, T
 template <typename T>
 int poisson_solve_resident(const SolverArgs<T>& a, const FusedCfg& fc, const T* b, T* x, double tol, int maxit,
                            int* iters, double* rel, std::string* err, bool* used);
+// The same iterates with every vector of a brick in registers
+// (les_cg_chip.cu): any extents; *used as above.
+template <typename T>
+int poisson_solve_chip(const SolverArgs<T>& a, const FusedCfg& fc, const T* b, T* x, double tol, int maxit,
+                       int* iters, double* rel, std::string* err, bool* used);
 // The same iterates with p, r and q in registers (les_cg_regs.cu): FP32
 // grids with nx = 128; *used as above.
 int poisson_solve_regs(const SolverArgs<float>& a, const FusedCfg& fc, const float* b, float* x, double tol,
