@@ -12,14 +12,29 @@
 // [.,.] channel concatenation.  Weights travel as one flat FP32 vector, layer
 // by layer, W[cout][cin][kz][ky][kx] then bias[cout].
 //
-// Kernels: activations are channels-last BF16 ([batch][z][y][x][c], c
-// padded to a multiple of 16).  A convolution is an implicit GEMM on the
-// tensor cores -- rows are 16 voxels, K runs over (tap, 16-channel slab), N
-// over output channels -- issued as mma.sync m16n8k16 BF16 -> FP32 with the
-// bias and activation fused into the epilogue.  The input-gradient pass is
-// the same kernel on flipped, transposed weights; the weight gradient is a
-// second tensor-core GEMM over voxel chunks whose FP32 partials are summed in
-// chunk order (deterministic).  Adam keeps FP32 master weights.
+// Activations are channels-last BF16 ([batch][z][y][x][c], c padded to a
+// multiple of 16); weights [tap][cout][cin].  A convolution (k_conv) is an
+// implicit GEMM on the tensor cores, mma.sync m16n8k16 BF16 -> FP32: rows are
+// voxels, K runs over (tap, 16 channels), N over output channels.  A block
+// stages its tile's input with a halo of one voxel and the weights of its
+// output channels in shared memory once, and feeds the 27 taps from there
+// with ldmatrix; voxel and weight rows are an odd number of 16-byte units, so
+// the eight rows of a matrix fall on different banks.  Nearest doubling is
+// read through halved coordinates, concatenation from two arrays, and the
+// epilogue adds bias and activation (or, going back, multiplies by the
+// activation's slope), pools, and on the last layer applies the 1x1 head.
+// The input gradient is the same kernel on flipped, transposed weights.  The
+// weight gradient (k_wgrad) is a GEMM over voxels: a warp per (dz, dy) keeps
+// its three taps of every output channel and 16 input channels in registers
+// while the block walks its share of the tiles; the FP32 partials of the
+// shares are summed in order (deterministic).  Adam keeps FP32 master weights.
+//
+// What bounds it: at 32^3 and batch 1 the launches and the fill of 13 short
+// kernels (each loads its weights before it waits for its predecessor); at
+// batch 16 the shared-memory reads, 2 to 4 wavefronts per MMA.  mma.sync, not
+// tcgen05: N is 16 to 64 and a tile 64 or 256 voxels, and every product is
+// summed in the order of taps and channels, so the results do not depend on
+// the tile.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -50,286 +65,562 @@ enum { L_E1A, L_E1B, L_E2A, L_E2B, L_E3A, L_E3B, L_D2A, L_D2B, L_D1A, L_D1B, L_H
 __host__ __device__ inline int pad16(int c) { return (c + 15) / 16 * 16; }
 __host__ __device__ inline int pad8(int c) { return (c + 7) / 8 * 8; }
 
-// ---- tensor-core primitive ----------------------------------------------------
-__device__ __forceinline__ void mma_bf16(float (&d)[4], unsigned a0, unsigned a1, unsigned a2, unsigned a3,
-                                         unsigned b0, unsigned b1) {
+// ---- tensor-core primitives ---------------------------------------------------
+__device__ __forceinline__ void mma_bf16(float (&d)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
   asm volatile(
       "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
       "{%0,%1,%2,%3};\n"
       : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-__device__ __forceinline__ unsigned ld32(const bf16* p) { return *reinterpret_cast<const unsigned*>(p); }
-__device__ __forceinline__ unsigned pack2(bf16 lo, bf16 hi) {
-  return (unsigned)__bfloat16_as_ushort(lo) | ((unsigned)__bfloat16_as_ushort(hi) << 16);
+__device__ __forceinline__ void ldsm4(unsigned (&r)[4], unsigned addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
+               : "memory");
 }
-__device__ __forceinline__ int wrapn(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
+__device__ __forceinline__ void ldsm4t(unsigned (&r)[4], unsigned addr) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(addr)
+               : "memory");
+}
+// Programmatic dependent launch: a kernel starts while its predecessor in the
+// stream drains, and waits here before it touches what that one writes (every
+// kernel of a chain waits, so whatever ran before the predecessor is complete
+// too).  Only weights, which the chain does not write, are read before.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// voxel index of the tap neighbour of voxel v (cubic grid n, periodic)
-__device__ __forceinline__ int nbr(int v, int n, int dz, int dy, int dx) {
-  const int x = v % n, y = (v / n) % n, zb = v / (n * n);
-  const int z = zb % n, b = zb / n;
-  return ((b * n + wrapn(z + dz, n)) * n + wrapn(y + dy, n)) * n + wrapn(x + dx, n);
+__device__ __forceinline__ unsigned ld32(const bf16* p) { return *reinterpret_cast<const unsigned*>(p); }
+__device__ __forceinline__ unsigned pack2(float lo, float hi) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<const unsigned*>(&v);
 }
+// eight BF16 values of a 16-byte chunk
+struct Chunk {
+  float v[8];
+};
+__device__ __forceinline__ Chunk unpack8(uint4 u) {
+  Chunk c;
+  const unsigned w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    c.v[2 * q] = __uint_as_float(w[q] << 16);
+    c.v[2 * q + 1] = __uint_as_float(w[q] & 0xffff0000u);
+  }
+  return c;
+}
+__device__ __forceinline__ uint4 pack8(const Chunk& c) {
+  return make_uint4(pack2(c.v[0], c.v[1]), pack2(c.v[2], c.v[3]), pack2(c.v[4], c.v[5]), pack2(c.v[6], c.v[7]));
+}
+// leaky ReLU backward from the post-activation (same sign as the
+// pre-activation): g is BF16 already, the product is rounded to BF16
+__device__ __forceinline__ uint4 act_back(uint4 post, uint4 g) {
+  const Chunk p = unpack8(post);
+  Chunk c = unpack8(g);
+#pragma unroll
+  for (int q = 0; q < 8; ++q) c.v[q] = p.v[q] > 0.f ? c.v[q] : kLeak * c.v[q];
+  return pack8(c);
+}
+// periodic coordinate of a staged voxel: at most one before the grid, and any
+// number past it (ragged tiles)
+__device__ __forceinline__ int wrap_tile(int i, int n) { return i < 0 ? i + n : (i >= n ? i % n : i); }
 
 // ---- convolution as an implicit GEMM --------------------------------------------
+// Block tiles: 4 x 4 x 4 voxels by 4 warps, a z-plane each, where the grid is
+// small, and 4 x 8 x 8 by 8 warps of two row groups each (half the weight
+// loads per voxel, 1.5 times the MMAs per shared-memory read).
+template <int CFG>
+struct Tile;
+template <>
+struct Tile<0> {
+  static constexpr int Z = 4, Y = 4, X = 4, W = 4, MT = 1;
+};
+template <>
+struct Tile<1> {
+  static constexpr int Z = 4, Y = 8, X = 8, W = 8, MT = 2;
+};
+// staged input of KC x 16 channels, in 16-byte units: S per voxel (odd), P per
+// row (4 mod 8 where the rows of a matrix span two tile rows), PZ per plane
+template <int CFG, int KC>
+struct Staged {
+  using T = Tile<CFG>;
+  static constexpr int S = 2 * KC + 1;
+  static constexpr int U = (T::X + 2) * S;
+  static constexpr int P = T::X == 4 ? (U + 3) / 8 * 8 + 4 : U;
+  static constexpr int PZ = (T::Y + 2) * P;
+  static constexpr int IN = (T::Z + 2) * PZ;
+};
+template <int CFG, int KC, int NFB>
+constexpr size_t conv_smem() {
+  return 16 * ((size_t)Staged<CFG, KC>::IN + 27 * 8 * NFB * (2 * KC + 1));
+}
+
 struct ConvArgs {
   const bf16* in0;
-  int c0;  // channels of in0 (multiple of 16)
+  int c0, up0;  // channels of in0 (multiple of 16); 1: in0 lives on the halved grid
   const bf16* in1;
-  int c1;  // channels of in1 (0 if absent)
-  const bf16* w;  // [taps][cout][cin] with cin = c0 + c1
-  const float* bias;
-  void* out0;
+  int c1;          // channels of in1 (0 if absent)
+  const bf16* w;   // [27][cout][16 KC]
+  int cout;
+  const float* bias;  // forward: bias and leaky ReLU; NULL: neither
+  const bf16* post;   // backward: activations whose slope multiplies the result (oc0 channels)
+  bf16* out0;
   int oc0;
-  void* out1;
+  bf16* out1;
   int oc1;
-  int n, nvox, k;
-  int act;
+  bf16* pool;         // 2 x 2 x 2 means of the output (oc0 channels)
+  const bf16* hw;     // head: y = hw . output + hb, and the tile's FP64 sum of y
+  const float* hb;
+  float* y;
+  double* ysum;
+  int n, tx, ty, tz;  // grid, tiles along x, y, z
 };
 
-// 4 warps x 16 voxels per block; NF output-channel fragments of 8
-template <int NF, bool OUT_F32>
-__global__ void __launch_bounds__(128) k_conv(ConvArgs a) {
+// Halo tile of one sample into shared memory: channels [ch0, ch0 + 8 NC) of
+// [in0, in1] in NC 16-byte chunks per voxel.
+template <int CFG, int NC, int S, int P, int PZ, int NTHR>
+__device__ __forceinline__ void stage_halo(unsigned sm, const bf16* in0, int c0, int up0, const bf16* in1, int c1,
+                                           int ch0, int n, long long b, int z0, int y0, int x0) {
+  using T = Tile<CFG>;
+  constexpr int HX = T::X + 2, HY = T::Y + 2, NV = (T::Z + 2) * HY * HX;
+  const int m = n >> 1;
+  for (int e = threadIdx.x; e < NV * NC; e += NTHR) {
+    const int v = e / NC, c = e - v * NC;
+    const int x = v % HX, y = (v / HX) % HY, z = v / (HX * HY);
+    const int gz = wrap_tile(z0 - 1 + z, n), gy = wrap_tile(y0 - 1 + y, n), gx = wrap_tile(x0 - 1 + x, n);
+    const int ch = ch0 + 8 * c;
+    const bf16* src;
+    if (ch < c0)
+      src = in0 + (size_t)(up0 ? ((b * m + (gz >> 1)) * m + (gy >> 1)) * m + (gx >> 1) : ((b * n + gz) * n + gy) * n + gx) *
+                      c0 + ch;
+    else
+      src = in1 + (size_t)(((b * n + gz) * n + gy) * n + gx) * c1 + (ch - c0);
+    const unsigned d = sm + 16u * (unsigned)(z * PZ + y * P + x * S + c);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+  }
+}
+
+template <int CFG, int KC, int NFB>
+__global__ void __launch_bounds__(32 * Tile<CFG>::W) k_conv(ConvArgs a) {
+  using T = Tile<CFG>;
+  using G = Staged<CFG, KC>;
+  constexpr int NB = 8 * NFB, NTHR = 32 * T::W, WS = 2 * KC + 1, MT = T::MT;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ double shd[32];
+  const unsigned sin = (unsigned)__cvta_generic_to_shared(smraw), sw = sin + 16u * G::IN;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int gid = lane >> 2, tig = lane & 3;
-  const int v0 = (blockIdx.x * 4 + warp) * 16;
-  if (v0 >= a.nvox) return;
-  const int cin = a.c0 + a.c1;
-  const int r = a.k / 2;
-  const int rowA = v0 + gid, rowB = v0 + gid + 8;
-  const bool okA = rowA < a.nvox, okB = rowB < a.nvox;
-  float acc[NF][4];
+  const int co0 = blockIdx.y * NB;
+  // the weights first: they do not depend on the kernel before
+  for (int e = threadIdx.x; e < 27 * NB * 2 * KC; e += NTHR) {
+    const int row = e / (2 * KC), c = e - row * (2 * KC);
+    const int t = row / NB, r = row - t * NB;
+    const bf16* src = a.w + ((size_t)t * a.cout + co0 + r) * (16 * KC) + 8 * c;
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sw + 16u * (unsigned)(row * WS + c)), "l"(src)
+                 : "memory");
+  }
+  pdl_launch();
+  pdl_wait();
+  const int tps = a.tx * a.ty * a.tz;
+  const long long b = blockIdx.x / tps;
+  const int tile = blockIdx.x - (int)b * tps;
+  const int x0 = (tile % a.tx) * T::X, y0 = (tile / a.tx) % a.ty * T::Y, z0 = tile / (a.tx * a.ty) * T::Z;
+  stage_halo<CFG, 2 * KC, G::S, G::P, G::PZ, NTHR>(sin, a.in0, a.c0, a.up0, a.in1, a.c1, 0, a.n, b, z0, y0, x0);
+  cp_commit();
+  cp_wait<0>();
+  __syncthreads();
+
+  // the lane's row of each A matrix (voxel lane mod 16, channel half lane / 16)
+  // and of a B matrix pair
+  auto voxel = [&](int mt, int row, int& z, int& y, int& x) {
+    if (CFG == 0) {
+      z = warp, y = row >> 2, x = row & 3;
+    } else {
+      const int q = warp * MT + mt;
+      z = q >> 2, y = ((q & 3) << 1) + (row >> 3), x = row & 7;
+    }
+  };
+  unsigned pa[MT];
 #pragma unroll
-  for (int f = 0; f < NF; ++f) acc[f][0] = acc[f][1] = acc[f][2] = acc[f][3] = 0.f;
-  const int ntap = a.k * a.k * a.k;
-  for (int t = 0; t < ntap; ++t) {
-    const int dz = t / (a.k * a.k) - r, dy = (t / a.k) % a.k - r, dx = t % a.k - r;
-    const int na = nbr(okA ? rowA : v0, a.n, dz, dy, dx), nb = nbr(okB ? rowB : v0, a.n, dz, dy, dx);
-    const bf16* wt = a.w + (size_t)t * (NF * 8) * cin;
-    for (int kc = 0; kc < cin; kc += 16) {
-      const bf16* src;
-      int cs, cc;
-      if (kc < a.c0) {
-        src = a.in0;
-        cs = a.c0;
-        cc = kc;
-      } else {
-        src = a.in1;
-        cs = a.c1;
-        cc = kc - a.c0;
+  for (int mt = 0; mt < MT; ++mt) {
+    int z, y, x;
+    voxel(mt, lane & 15, z, y, x);
+    pa[mt] = sin + 16u * (unsigned)(z * G::PZ + y * G::P + x * G::S + (lane >> 4));
+  }
+  const unsigned pb = sw + 16u * (unsigned)(((lane & 7) + ((lane >> 4) & 1) * 8) * WS + ((lane >> 3) & 1));
+  float acc[MT][NFB][4];
+#pragma unroll
+  for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+    for (int f = 0; f < NFB; ++f) acc[mt][f][0] = acc[mt][f][1] = acc[mt][f][2] = acc[mt][f][3] = 0.f;
+#pragma unroll 1
+  for (int zy = 0; zy < 9; ++zy) {
+    const unsigned oa = 16u * (unsigned)((zy / 3) * G::PZ + (zy % 3) * G::P);
+    const unsigned ob = 16u * (unsigned)(zy * 3 * NB * WS);
+#pragma unroll
+    for (int tx = 0; tx < 3; ++tx)
+#pragma unroll
+      for (int kc = 0; kc < KC; ++kc) {
+        unsigned A[MT][4], B[NFB / 2][4];
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt) ldsm4(A[mt], pa[mt] + oa + 16u * (unsigned)(tx * G::S + 2 * kc));
+#pragma unroll
+        for (int h = 0; h < NFB / 2; ++h) ldsm4(B[h], pb + ob + 16u * (unsigned)((tx * NB + 16 * h) * WS + 2 * kc));
+#pragma unroll
+        for (int mt = 0; mt < MT; ++mt)
+#pragma unroll
+          for (int f = 0; f < NFB; ++f) mma_bf16(acc[mt][f], A[mt], B[f >> 1][2 * (f & 1)], B[f >> 1][2 * (f & 1) + 1]);
       }
-      const bf16* pa = src + (size_t)na * cs + cc + tig * 2;
-      const bf16* pb = src + (size_t)nb * cs + cc + tig * 2;
-      const unsigned a0 = okA ? ld32(pa) : 0u, a1 = okB ? ld32(pb) : 0u;
-      const unsigned a2 = okA ? ld32(pa + 8) : 0u, a3 = okB ? ld32(pb + 8) : 0u;
+  }
+  __syncthreads();  // the staged input is free: it takes the output tile
+
+  // epilogue: bias and activation, rounded to BF16 into [voxel][NB + 8]
+  bf16* so = reinterpret_cast<bf16*>(smraw);
+  constexpr int OS = NB + 8;
+  double ysum = 0.0;
 #pragma unroll
-      for (int f = 0; f < NF; ++f) {
-        const bf16* pw = wt + (size_t)(f * 8 + gid) * cin + kc + tig * 2;
-        mma_bf16(acc[f], a0, a1, a2, a3, ld32(pw), ld32(pw + 8));
+  for (int mt = 0; mt < MT; ++mt) {
+    unsigned packed[NFB][2];
+#pragma unroll
+    for (int f = 0; f < NFB; ++f) {
+      const int co = co0 + f * 8 + tig * 2;
+      float b0 = 0.f, b1 = 0.f;
+      if (a.bias) {
+        b0 = a.bias[co];
+        b1 = a.bias[co + 1];
+      }
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        float u0 = acc[mt][f][2 * h], u1 = acc[mt][f][2 * h + 1];
+        if (a.bias) {
+          u0 += b0;
+          u1 += b1;
+          u0 = u0 > 0.f ? u0 : kLeak * u0;
+          u1 = u1 > 0.f ? u1 : kLeak * u1;
+        }
+        packed[f][h] = pack2(u0, u1);
+        const int row = (warp * MT + mt) * 16 + gid + 8 * h;
+        *reinterpret_cast<unsigned*>(so + row * OS + f * 8 + tig * 2) = packed[f][h];
+      }
+    }
+    if (NFB == 2 && a.hw) {
+      // the output fragments are the A fragments of the 1x1 head
+      const unsigned A[4] = {packed[0][0], packed[0][1], packed[1][0], packed[1][1]};
+      float yv[4] = {0.f, 0.f, 0.f, 0.f};
+      mma_bf16(yv, A, ld32(a.hw + gid * 16 + tig * 2), ld32(a.hw + gid * 16 + tig * 2 + 8));
+      if (tig == 0) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          int z, y, x;
+          voxel(mt, gid + 8 * h, z, y, x);
+          if (z0 + z < a.n && y0 + y < a.n && x0 + x < a.n) {
+            const float v = yv[2 * h] + a.hb[0];
+            a.y[((b * a.n + z0 + z) * a.n + y0 + y) * a.n + x0 + x] = v;
+            ysum += (double)v;
+          }
+        }
       }
     }
   }
-  // epilogue: bias, activation, split store
+  __syncthreads();
+  // stored 16 bytes at a time; row q of the tile is voxel (q)
+  auto tile_voxel = [&](int q, int& z, int& y, int& x) {
+    if (CFG == 0) z = q >> 4, y = (q >> 2) & 3, x = q & 3;
+    else z = q >> 6, y = (q >> 3) & 7, x = q & 7;
+  };
+  for (int e = threadIdx.x; e < T::Z * T::Y * T::X * NFB; e += NTHR) {
+    const int q = e / NFB, c = e - q * NFB;
+    int z, y, x;
+    tile_voxel(q, z, y, x);
+    if (z0 + z >= a.n || y0 + y >= a.n || x0 + x >= a.n) continue;
+    const size_t v = (size_t)((b * a.n + z0 + z) * a.n + y0 + y) * a.n + x0 + x;
+    uint4 o = *reinterpret_cast<const uint4*>(so + q * OS + 8 * c);
+    const int co = co0 + 8 * c;
+    if (a.post) o = act_back(__ldg(reinterpret_cast<const uint4*>(a.post + v * a.oc0 + co)), o);
+    if (co < a.oc0) *reinterpret_cast<uint4*>(a.out0 + v * a.oc0 + co) = o;
+    else *reinterpret_cast<uint4*>(a.out1 + v * a.oc1 + (co - a.oc0)) = o;
+  }
+  if (a.pool) {
+    const int m = a.n >> 1;
+    for (int e = threadIdx.x; e < T::Z * T::Y * T::X / 8 * NFB; e += NTHR) {
+      const int q = e / NFB, c = e - q * NFB;
+      const int x = q % (T::X / 2), y = q / (T::X / 2) % (T::Y / 2), z = q / (T::X / 2 * (T::Y / 2));
+      if (z0 + 2 * z >= a.n || y0 + 2 * y >= a.n || x0 + 2 * x >= a.n) continue;
+      Chunk s = {};
 #pragma unroll
-  for (int f = 0; f < NF; ++f) {
-    const int co = f * 8 + tig * 2;
+      for (int k = 0; k < 8; ++k) {
+        const int r = ((2 * z + (k >> 2)) * T::Y + 2 * y + ((k >> 1) & 1)) * T::X + 2 * x + (k & 1);
+        const Chunk u = unpack8(*reinterpret_cast<const uint4*>(so + r * OS + 8 * c));
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int v = h ? rowB : rowA;
-      if (v >= a.nvox) continue;
-      float x0 = acc[f][2 * h], x1 = acc[f][2 * h + 1];
-      if (a.bias) {
-        x0 += a.bias[co];
-        x1 += a.bias[co + 1];
+        for (int i = 0; i < 8; ++i) s.v[i] += u.v[i];
       }
-      if (a.act) {
-        x0 = x0 > 0.f ? x0 : kLeak * x0;
-        x1 = x1 > 0.f ? x1 : kLeak * x1;
-      }
-      if (co < a.oc0) {
-        if (OUT_F32) {
-          float* o = reinterpret_cast<float*>(a.out0) + (size_t)v * a.oc0 + co;
-          *reinterpret_cast<float2*>(o) = make_float2(x0, x1);
-        } else {
-          bf16* o = reinterpret_cast<bf16*>(a.out0) + (size_t)v * a.oc0 + co;
-          *reinterpret_cast<__nv_bfloat162*>(o) = __floats2bfloat162_rn(x0, x1);
-        }
-      } else if (co - a.oc0 < a.oc1) {
-        bf16* o = reinterpret_cast<bf16*>(a.out1) + (size_t)v * a.oc1 + (co - a.oc0);
-        *reinterpret_cast<__nv_bfloat162*>(o) = __floats2bfloat162_rn(x0, x1);
-      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i) s.v[i] *= 0.125f;
+      *reinterpret_cast<uint4*>(a.pool + (size_t)(((b * m + z0 / 2 + z) * m + y0 / 2 + y) * m + x0 / 2 + x) * a.oc0 + co0 +
+                                8 * c) = pack8(s);
     }
+  }
+  if (a.hw) {
+    const double t = block_reduce<false>(ysum, shd);
+    if (threadIdx.x == 0) a.ysum[blockIdx.x] = t;
   }
 }
 
 // ---- weight gradient: gW[t][co][ci] = sum_v g[v][co] in[nbr(v, t)][ci] ----------
 struct WgradArgs {
-  const bf16* g;  // [nvox][gstride]
-  int gstride;
-  int cout;       // channels of g that take part (the rest read as 0)
+  const bf16* g;  // [voxels][16 CO]
   const bf16* in0;
-  int c0;
+  int c0, up0;
   const bf16* in1;
   int c1;
-  float* part;  // [nchunk][taps][cout16][cin]
-  int n, nvox, k, chunk;
+  float* part;   // [shares][27][16 CO][cin]
+  float* bpart;  // [shares][16 CO]
+  int cin, n, tx, ty, tz;
+  long long ntiles;
 };
+constexpr int kWgWarps = 9;  // one per (dz, dy)
 
-// one warp per (tap, 16 output channels, voxel chunk); NF = cin / 8 fragments
-template <int NF>
-__global__ void __launch_bounds__(32) k_wgrad(WgradArgs a) {
-  const int lane = threadIdx.x, gid = lane >> 2, tig = lane & 3;
-  const int t = blockIdx.x, cob = blockIdx.y, ch = blockIdx.z;
-  const int cin = a.c0 + a.c1;
-  const int r = a.k / 2;
-  const int dz = t / (a.k * a.k) - r, dy = (t / a.k) % a.k - r, dx = t % a.k - r;
-  const int co_a = cob * 16 + gid, co_b = co_a + 8;
-  const bool ok_a = co_a < a.cout, ok_b = co_b < a.cout;
-  const bf16 zero = __float2bfloat16(0.f);
-  float acc[NF][4];
-#pragma unroll
-  for (int f = 0; f < NF; ++f) acc[f][0] = acc[f][1] = acc[f][2] = acc[f][3] = 0.f;
-  const int vend = min(a.nvox, (ch + 1) * a.chunk);
-  for (int v0 = ch * a.chunk; v0 < vend; v0 += 16) {
-    const int va = v0 + tig * 2, vb = va + 8;  // K index (voxel) of this thread's fragment entries
-    // A (16 co x 16 voxels): A[m][k] = g[v0 + k][co0 + m]
-    auto gv = [&](int v, int co, bool ok) { return ok && v < vend ? a.g[(size_t)v * a.gstride + co] : zero; };
-    const unsigned a0 = pack2(gv(va, co_a, ok_a), gv(va + 1, co_a, ok_a));
-    const unsigned a1 = pack2(gv(va, co_b, ok_b), gv(va + 1, co_b, ok_b));
-    const unsigned a2 = pack2(gv(vb, co_a, ok_a), gv(vb + 1, co_a, ok_a));
-    const unsigned a3 = pack2(gv(vb, co_b, ok_b), gv(vb + 1, co_b, ok_b));
-    const bool k0 = va < vend, k1 = va + 1 < vend, k2 = vb < vend, k3 = vb + 1 < vend;
-    const int n0 = nbr(k0 ? va : v0, a.n, dz, dy, dx), n1 = nbr(k1 ? va + 1 : v0, a.n, dz, dy, dx);
-    const int n2 = nbr(k2 ? vb : v0, a.n, dz, dy, dx), n3 = nbr(k3 ? vb + 1 : v0, a.n, dz, dy, dx);
-#pragma unroll
-    for (int f = 0; f < NF; ++f) {
-      const int ci = f * 8 + gid;
-      const bf16* src;
-      int cs, cc;
-      if (ci < a.c0) {
-        src = a.in0;
-        cs = a.c0;
-        cc = ci;
-      } else {
-        src = a.in1;
-        cs = a.c1;
-        cc = ci - a.c0;
-      }
-      // B (16 voxels x 8 ci): B[k][n] = in[nbr(v0 + k)][ci0 + n]
-      const unsigned b0 = pack2(k0 ? src[(size_t)n0 * cs + cc] : zero, k1 ? src[(size_t)n1 * cs + cc] : zero);
-      const unsigned b1 = pack2(k2 ? src[(size_t)n2 * cs + cc] : zero, k3 ? src[(size_t)n3 * cs + cc] : zero);
-      mma_bf16(acc[f], a0, a1, a2, a3, b0, b1);
+template <int CO>
+constexpr size_t wgrad_smem() {
+  return 2 * 16 * ((size_t)Staged<1, 1>::IN + 256 * (2 * CO + 1));
+}
+
+// Block (ci slice, share): 16 input channels, every (share)-th tile.  A row of
+// voxel pairs is 16 K entries; both operands come transposed from rows of
+// voxels by ldmatrix.  The bias gradient is one more column, of ones, in the
+// blocks of the first slice.
+template <int CO>
+__global__ void __launch_bounds__(32 * kWgWarps) k_wgrad(WgradArgs a) {
+  using T = Tile<1>;
+  using G = Staged<1, 1>;
+  constexpr int NTHR = 32 * kWgWarps, GS = 2 * CO + 1, STAGE = G::IN + 256 * GS;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  const unsigned sm = (unsigned)__cvta_generic_to_shared(smraw);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int gid = lane >> 2, tig = lane & 3;
+  const int tps = a.tx * a.ty * a.tz;
+  pdl_launch();
+  pdl_wait();
+  auto stage = [&](long long tile, int buf) {
+    const unsigned s0 = sm + 16u * (unsigned)(buf * STAGE);
+    const long long b = tile / tps;
+    const int q0 = (int)(tile - b * tps);
+    const int x0 = (q0 % a.tx) * T::X, y0 = (q0 / a.tx) % a.ty * T::Y, z0 = q0 / (a.tx * a.ty) * T::Z;
+    stage_halo<1, 2, G::S, G::P, G::PZ, NTHR>(s0, a.in0, a.c0, a.up0, a.in1, a.c1, 16 * blockIdx.x, a.n, b, z0, y0, x0);
+    for (int e = threadIdx.x; e < 256 * 2 * CO; e += NTHR) {
+      const int q = e / (2 * CO), c = e - q * (2 * CO);
+      const int z = z0 + (q >> 6), y = y0 + ((q >> 3) & 7), x = x0 + (q & 7);
+      // voxels beyond the grid contribute nothing: zero bytes are copied
+      const bool in = z < a.n && y < a.n && x < a.n;
+      const bf16* src = in ? a.g + (size_t)(((b * a.n + z) * a.n + y) * a.n + x) * (16 * CO) + 8 * c : a.g;
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(s0 + 16u * (unsigned)(G::IN + q * GS + c)),
+                   "l"(src), "r"(in ? 16 : 0)
+                   : "memory");
     }
-  }
-  const int ntap = a.k * a.k * a.k;
-  const int co16 = (a.cout + 15) / 16 * 16;
-  float* base = a.part + (((size_t)ch * ntap + t) * co16) * cin;
+  };
+  float acc[3][CO][2][4], ab[CO][4];
 #pragma unroll
-  for (int f = 0; f < NF; ++f) {
-    const int ci = f * 8 + tig * 2;
-    base[(size_t)co_a * cin + ci] = acc[f][0];
-    base[(size_t)co_a * cin + ci + 1] = acc[f][1];
-    base[(size_t)co_b * cin + ci] = acc[f][2];
-    base[(size_t)co_b * cin + ci + 1] = acc[f][3];
+  for (int o = 0; o < CO; ++o) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) ab[o][k] = 0.f;
+#pragma unroll
+    for (int t = 0; t < 3; ++t)
+#pragma unroll
+      for (int f = 0; f < 2; ++f)
+#pragma unroll
+        for (int k = 0; k < 4; ++k) acc[t][o][f][k] = 0.f;
   }
+  const int dz = warp / 3, dy = warp % 3;
+  // lane addresses: A (voxel, channel half) of g, B of the input halo
+  const unsigned oa = 16u * (unsigned)(G::IN + ((lane & 7) + ((lane >> 4) & 1) * 8) * GS + ((lane >> 3) & 1));
+  const unsigned ob = 16u * (unsigned)(dz * G::PZ + (dy + ((lane >> 3) & 1)) * G::P + (lane & 7) * G::S + (lane >> 4));
+  const bool bias = blockIdx.x == 0 && warp == 4;
+  int buf = 0;
+  long long tile = blockIdx.y;
+  if (tile < a.ntiles) stage(tile, 0);
+  cp_commit();
+  for (; tile < a.ntiles; tile += gridDim.y, buf ^= 1) {
+    if (tile + gridDim.y < a.ntiles) stage(tile + gridDim.y, buf ^ 1);
+    cp_commit();
+    cp_wait<1>();
+    __syncthreads();
+    const unsigned s0 = sm + 16u * (unsigned)(buf * STAGE);
+#pragma unroll 2
+    for (int q = 0; q < 16; ++q) {  // two rows of eight voxels each
+      const int z = q >> 2, y = (q & 3) * 2;
+      unsigned A[CO][4];
+#pragma unroll
+      for (int o = 0; o < CO; ++o) ldsm4t(A[o], s0 + oa + 16u * (unsigned)(q * 16 * GS + 2 * o));
+#pragma unroll
+      for (int t = 0; t < 3; ++t) {
+        unsigned B[4];
+        ldsm4t(B, s0 + ob + 16u * (unsigned)(z * G::PZ + y * G::P + t * G::S));
+#pragma unroll
+        for (int o = 0; o < CO; ++o) {
+          mma_bf16(acc[t][o][0], A[o], B[0], B[1]);
+          mma_bf16(acc[t][o][1], A[o], B[2], B[3]);
+        }
+      }
+      if (bias)
+#pragma unroll
+        for (int o = 0; o < CO; ++o) mma_bf16(ab[o], A[o], 0x3F803F80u, 0x3F803F80u);
+    }
+    __syncthreads();  // the buffer is free for the tile after the next
+  }
+  const int cout = 16 * CO;
+  float* base = a.part + (size_t)blockIdx.y * 27 * cout * a.cin + 16 * blockIdx.x;
+#pragma unroll
+  for (int t = 0; t < 3; ++t)
+#pragma unroll
+    for (int o = 0; o < CO; ++o)
+#pragma unroll
+      for (int f = 0; f < 2; ++f)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          float* q = base + ((size_t)(warp * 3 + t) * cout + o * 16 + gid + 8 * h) * a.cin + f * 8 + tig * 2;
+          *reinterpret_cast<float2*>(q) = make_float2(acc[t][o][f][2 * h], acc[t][o][f][2 * h + 1]);
+        }
+  if (bias && tig == 0)
+#pragma unroll
+    for (int o = 0; o < CO; ++o) {
+      a.bpart[(size_t)blockIdx.y * cout + o * 16 + gid] = ab[o][0];
+      a.bpart[(size_t)blockIdx.y * cout + o * 16 + gid + 8] = ab[o][2];
+    }
 }
 
-// sum the chunk partials (chunk order) into the flat FP32 gradient
-// (layout W[co][ci][tap] of the real, unpadded channels)
-__global__ void k_wgrad_reduce(const float* part, int nchunk, int ntap, int co16, int cin_pad, int cout,
-                               int cin, float* gflat) {
-  const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-  const int total = cout * cin * ntap;
-  if (idx >= total) return;
-  const int t = idx % ntap, ci = (idx / ntap) % cin, co = idx / (ntap * cin);
+// The partials of every layer, summed over their shares in order, into the
+// flat FP32 gradient (W[co][ci][tap] of the real channels, then the biases).
+// A warp owns 32 consecutive values of a layer's [tap][co][ci] partials.
+struct ReduceLayer {
+  const float* part;
+  const float* bpart;
+  int shares, ntap, cout, coutp, cin, cinp;
+  long long off;  // of the layer in the flat gradient
+  int block0;     // first block of the layer
+};
+struct ReduceArgs {
+  ReduceLayer l[kNL];
+  float* grad;
+};
+constexpr int kRedWarps = 8;
+__global__ void __launch_bounds__(32 * kRedWarps) k_grad_reduce(ReduceArgs a) {
+  pdl_launch();
+  pdl_wait();
+  int li = 0;
+  while (li + 1 < kNL && (int)blockIdx.x >= a.l[li + 1].block0) ++li;
+  const ReduceLayer& L = a.l[li];
+  const int nw = L.ntap * L.coutp * L.cinp, total = nw + L.cout;
+  const int i = ((int)blockIdx.x - L.block0) * 32 + (threadIdx.x & 31), warp = threadIdx.x >> 5;
+  // each warp sums every kRedWarps-th share, then the warps in order
+  __shared__ float sh[kRedWarps][32];
   float s = 0.f;
-  for (int c = 0; c < nchunk; ++c) s += part[(((size_t)c * ntap + t) * co16 + co) * cin_pad + ci];
-  gflat[idx] = s;
-}
-
-// bias gradient: sum over voxels of g[v][co] (two passes, fixed order)
-__global__ void k_bias_partial(const bf16* g, int gstride, int cout_pad, int nvox, int chunk, float* part) {
-  const int co = threadIdx.x, ch = blockIdx.x;
-  if (co >= cout_pad) return;
-  float s = 0.f;
-  const int vend = min(nvox, (ch + 1) * chunk);
-  for (int v = ch * chunk; v < vend; ++v) s += __bfloat162float(g[(size_t)v * gstride + co]);
-  part[(size_t)ch * cout_pad + co] = s;
-}
-__global__ void k_bias_reduce(const float* part, int nchunk, int cout_pad, int cout, float* gb) {
-  const int co = threadIdx.x;
-  if (co >= cout) return;
-  float s = 0.f;
-  for (int c = 0; c < nchunk; ++c) s += part[(size_t)c * cout_pad + co];
-  gb[co] = s;
+  if (i < total) {
+    const float* p = i < nw ? L.part + i : L.bpart + (i - nw);
+    const size_t step = i < nw ? (size_t)nw : (size_t)L.coutp;
+#pragma unroll 4
+    for (int q = warp; q < L.shares; q += kRedWarps) s += p[q * step];
+  }
+  sh[warp][threadIdx.x & 31] = s;
+  __syncthreads();
+  if (warp != 0 || i >= total) return;
+  s = 0.f;
+#pragma unroll
+  for (int q = 0; q < kRedWarps; ++q) s += sh[q][threadIdx.x];
+  const int nreal = L.cout * L.cin * L.ntap;
+  if (i >= nw) {
+    a.grad[L.off + nreal + (i - nw)] = s;
+    return;
+  }
+  const int ci = i % L.cinp, co = i / L.cinp % L.coutp, t = i / (L.cinp * L.coutp);
+  if (ci < L.cin && co < L.cout) a.grad[L.off + ((size_t)co * L.cin + ci) * L.ntap + t] = s;
 }
 
 // ---- elementwise and resampling ---------------------------------------------------
-__global__ void k_pool(const bf16* in, int c, int n, int batch, bf16* out) {
-  const int m = n / 2;
-  const long long total = (long long)batch * m * m * m * c;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-    const int ch = (int)(i % c);
-    long long v = i / c;
-    const int x = (int)(v % m), y = (int)((v / m) % m), z = (int)((v / ((long long)m * m)) % m);
-    const int b = (int)(v / ((long long)m * m * m));
-    float s = 0.f;
+// Back through the 1x1 head: s = slope(post) * (gy w), gy the BF16 gradient of
+// y, and the head's own gradients sum gy post, sum gy (FP32 partials per block).
+// Thread pairs own the two 8-channel chunks of a voxel.
+__global__ void __launch_bounds__(256) k_head_back(const bf16* gy, const bf16* hw /* [8][16], row 0 */, const bf16* post,
+                                                   long long nvox, bf16* s, float* part, float* bpart) {
+  pdl_launch();
+  pdl_wait();
+  __shared__ float sh[8][2][9];
+  const int half = threadIdx.x & 1;
+  const Chunk w = unpack8(__ldg(reinterpret_cast<const uint4*>(hw + 8 * half)));
+  float acc[9] = {};
+  for (long long i = (blockIdx.x * 256LL + threadIdx.x) >> 1; i < nvox; i += gridDim.x * 128LL) {
+    const float g = __bfloat162float(gy[i]);
+    const uint4 pu = __ldg(reinterpret_cast<const uint4*>(post + i * 16 + 8 * half));
+    const Chunk p = unpack8(pu);
+    Chunk c;
+#pragma unroll
     for (int q = 0; q < 8; ++q) {
-      const int xx = 2 * x + (q & 1), yy = 2 * y + ((q >> 1) & 1), zz = 2 * z + (q >> 2);
-      s += __bfloat162float(in[((((size_t)b * n + zz) * n + yy) * n + xx) * c + ch]);
+      c.v[q] = g * w.v[q];
+      acc[q] += g * p.v[q];
     }
-    out[i] = __float2bfloat16(s * 0.125f);
+    acc[8] += g;
+    *reinterpret_cast<uint4*>(s + i * 16 + 8 * half) = act_back(pu, pack8(c));
+  }
+#pragma unroll
+  for (int q = 0; q < 9; ++q)
+#pragma unroll
+    for (int o = 16; o > 1; o >>= 1) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
+  if ((threadIdx.x & 31) < 2)
+#pragma unroll
+    for (int q = 0; q < 9; ++q) sh[threadIdx.x >> 5][half][q] = acc[q];
+  __syncthreads();
+  if (threadIdx.x < 18) {
+    const int h = threadIdx.x / 9, q = threadIdx.x - 9 * h;
+    float t = 0.f;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) t += sh[k][h][q];
+    if (q < 8) part[(size_t)blockIdx.x * 16 + 8 * h + q] = t;
+    else if (h == 0) bpart[blockIdx.x] = t;
   }
 }
-// gradient of pool: g_in[fine] (+)= g_out[coarse] / 8
-__global__ void k_pool_bwd(const bf16* gout, int c, int n, int batch, bf16* gin, int accumulate) {
-  const int m = n / 2;
-  const long long total = (long long)batch * n * n * n * c;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-    const int ch = (int)(i % c);
-    long long v = i / c;
-    const int x = (int)(v % n), y = (int)((v / n) % n), z = (int)((v / ((long long)n * n)) % n);
-    const int b = (int)(v / ((long long)n * n * n));
-    float g = __bfloat162float(gout[((((size_t)b * m + z / 2) * m + y / 2) * m + x / 2) * c + ch]) * 0.125f;
-    if (accumulate) g += __bfloat162float(gin[i]);
-    gin[i] = __float2bfloat16(g);
-  }
-}
-// nearest-neighbour doubling from an m-grid to n = 2m
-__global__ void k_up(const bf16* in, int c, int m, int batch, bf16* out) {
-  const int n = 2 * m;
-  const long long total = (long long)batch * n * n * n * c;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-    const int ch = (int)(i % c);
-    long long v = i / c;
-    const int x = (int)(v % n), y = (int)((v / n) % n), z = (int)((v / ((long long)n * n)) % n);
-    const int b = (int)(v / ((long long)n * n * n));
-    out[i] = in[((((size_t)b * m + z / 2) * m + y / 2) * m + x / 2) * c + ch];
-  }
-}
-// gradient of up: sum of the 8 fine children
-__global__ void k_up_bwd(const bf16* gout, int c, int m, int batch, bf16* gin) {
-  const int n = 2 * m;
-  const long long total = (long long)batch * m * m * m * c;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-    const int ch = (int)(i % c);
-    long long v = i / c;
-    const int x = (int)(v % m), y = (int)((v / m) % m), z = (int)((v / ((long long)m * m)) % m);
-    const int b = (int)(v / ((long long)m * m * m));
-    float s = 0.f;
+// Back through nearest doubling and the activation below it: the sum of the 8
+// fine children, rounded to BF16, times the slope at post.  c channels, coarse
+// grid m.
+__global__ void __launch_bounds__(256) k_up_back(const bf16* gout, int c, int m, long long total /* chunks */,
+                                                 const bf16* post, bf16* s) {
+  pdl_launch();
+  pdl_wait();
+  const int n = 2 * m, nc = c / 8;
+  for (long long i = blockIdx.x * 256LL + threadIdx.x; i < total; i += gridDim.x * 256LL) {
+    const int ch = (int)(i % nc);
+    const long long v = i / nc;
+    const int x = (int)(v % m), y = (int)(v / m % m), z = (int)(v / ((long long)m * m) % m);
+    const long long b = v / ((long long)m * m * m);
+    Chunk t = {};
+#pragma unroll
     for (int q = 0; q < 8; ++q) {
-      const int xx = 2 * x + (q & 1), yy = 2 * y + ((q >> 1) & 1), zz = 2 * z + (q >> 2);
-      s += __bfloat162float(gout[((((size_t)b * n + zz) * n + yy) * n + xx) * c + ch]);
+      const long long f = ((b * n + 2 * z + (q >> 2)) * n + 2 * y + ((q >> 1) & 1)) * n + 2 * x + (q & 1);
+      const Chunk u = unpack8(__ldg(reinterpret_cast<const uint4*>(gout + f * c + 8 * ch)));
+#pragma unroll
+      for (int k = 0; k < 8; ++k) t.v[k] += u.v[k];
     }
-    gin[i] = __float2bfloat16(s);
+    *reinterpret_cast<uint4*>(s + i * 8) = act_back(__ldg(reinterpret_cast<const uint4*>(post + i * 8)), pack8(t));
   }
 }
-// leaky ReLU backward from the post-activation (same sign as the pre-activation)
-__global__ void k_act_bwd(const bf16* post, const bf16* g, long long total, bf16* out) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-    const float gv = __bfloat162float(g[i]);
-    out[i] = __float2bfloat16(__bfloat162float(post[i]) > 0.f ? gv : kLeak * gv);
+// Back through the 2 x 2 x 2 mean, added to the gradient that reached the same
+// activations over the skip connection, times the slope at post.  Fine grid n.
+__global__ void __launch_bounds__(256) k_pool_back(const bf16* gout, int c, int n, long long total /* chunks */,
+                                                   const bf16* gskip, const bf16* post, bf16* s) {
+  pdl_launch();
+  pdl_wait();
+  const int m = n / 2, nc = c / 8;
+  for (long long i = blockIdx.x * 256LL + threadIdx.x; i < total; i += gridDim.x * 256LL) {
+    const int ch = (int)(i % nc);
+    const long long v = i / nc;
+    const int x = (int)(v % n), y = (int)(v / n % n), z = (int)(v / ((long long)n * n) % n);
+    const long long b = v / ((long long)n * n * n);
+    const long long q = ((b * m + z / 2) * m + y / 2) * m + x / 2;
+    const Chunk g = unpack8(__ldg(reinterpret_cast<const uint4*>(gout + q * c + 8 * ch)));
+    Chunk t = unpack8(__ldg(reinterpret_cast<const uint4*>(gskip + i * 8)));
+#pragma unroll
+    for (int k = 0; k < 8; ++k) t.v[k] = g.v[k] * 0.125f + t.v[k];
+    *reinterpret_cast<uint4*>(s + i * 8) = act_back(__ldg(reinterpret_cast<const uint4*>(post + i * 8)), pack8(t));
   }
 }
 
@@ -346,55 +637,62 @@ __global__ void k_sumsq(const T* b, long long n3, double* out) {
   const double r = block_reduce<false>(acc, sh);
   if (threadIdx.x == 0) out[(size_t)s * gridDim.x + blockIdx.x] = r;
 }
-// s = sqrt(mean b^2) per sample from the block partials
-__global__ void k_scale(const double* part, int nblk, long long n3, int batch, double* scale) {
-  const int s = threadIdx.x;
-  if (s >= batch) return;
-  double acc = 0.0;
-  for (int q = 0; q < nblk; ++q) acc += part[(size_t)s * nblk + q];
-  scale[s] = sqrt(acc / (double)n3);
+constexpr int kSumBlocks = 64;  // partials of sum b^2 per sample
+// The scale s = sqrt(mean b^2) of sample `q` from its partials (one warp, the
+// result in every lane)
+__device__ __forceinline__ double sample_scale(const double* part, long long q, long long n3) {
+  const int lane = threadIdx.x & 31;
+  const double* p = part + q * kSumBlocks;
+  return sqrt(warp_sum(p[lane] + p[lane + 32]) / (double)n3);
 }
-// x0[v][0] = b / s, other 15 channels 0; optional normalised target t = psi / s
+// x0[v][0] = b / s, other 15 channels 0; optional normalised target t = psi / s.
+// A grid row of blocks per sample; its first block keeps s.
 template <typename T>
-__global__ void k_pack(const T* b, const T* psi, long long n3, int batch, const double* scale, double out_scale,
-                       bf16* x0, float* tgt) {
-  const long long total = (long long)batch * n3;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-    const int s = (int)(i / n3);
-    const double sc = scale[s];
-    const double inv = sc > 0.0 ? 1.0 / sc : 0.0;
-    __nv_bfloat162 lo = __floats2bfloat162_rn((float)((double)b[i] * inv), 0.f);
-    __nv_bfloat162 z = __floats2bfloat162_rn(0.f, 0.f);
-    __nv_bfloat162* o = reinterpret_cast<__nv_bfloat162*>(x0 + (size_t)i * 16);
-    o[0] = lo;
-#pragma unroll
-    for (int q = 1; q < 8; ++q) o[q] = z;
+__global__ void __launch_bounds__(256) k_pack(const T* b, const T* psi, long long n3, const double* part, double* scale,
+                                              double out_scale, bf16* x0, float* tgt) {
+  __shared__ double sh;
+  pdl_launch();
+  pdl_wait();
+  const long long s = blockIdx.y;
+  if (threadIdx.x < 32) {
+    const double sc = sample_scale(part, s, n3);
+    if (threadIdx.x == 0) {
+      sh = sc;
+      if (blockIdx.x == 0) scale[s] = sc;
+    }
+  }
+  __syncthreads();
+  const double inv = sh > 0.0 ? 1.0 / sh : 0.0;
+  for (long long v = blockIdx.x * 256LL + threadIdx.x; v < n3; v += gridDim.x * 256LL) {
+    const long long i = s * n3 + v;
+    uint4* o = reinterpret_cast<uint4*>(x0 + i * 16);
+    o[0] = make_uint4(pack2((float)((double)b[i] * inv), 0.f), 0u, 0u, 0u);
+    o[1] = make_uint4(0u, 0u, 0u, 0u);
     if (tgt) tgt[i] = (float)((double)psi[i] * inv / out_scale);
   }
 }
-// MSE over batch x n3 of y (channel 0 of [.][8] FP32) vs t; gy = 2 (y - t) / count
-// in channel 0 of a 16-channel BF16 gradient
+// MSE over batch x n3 of y vs t; gy = 2 (y - t) / count in BF16
 __global__ void k_loss(const float* y, const float* t, long long total, bf16* gy, double* part) {
   __shared__ double sh[32];
+  pdl_launch();
+  pdl_wait();
   double acc = 0.0;
   const float inv = 2.f / (float)total;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-    const float d = y[(size_t)i * 8] - t[i];
+    const float d = y[i] - t[i];
     acc += (double)d * d;
-    __nv_bfloat162* o = reinterpret_cast<__nv_bfloat162*>(gy + (size_t)i * 16);
-    o[0] = __floats2bfloat162_rn(d * inv, 0.f);
-    const __nv_bfloat162 z = __floats2bfloat162_rn(0.f, 0.f);
-#pragma unroll
-    for (int q = 1; q < 8; ++q) o[q] = z;
+    gy[i] = __float2bfloat16(d * inv);
   }
   const double r = block_reduce<false>(acc, sh);
   if (threadIdx.x == 0) part[blockIdx.x] = r;
 }
 // Energy norm of the error on the periodic n^3 grid (unit spacing) over
 // batch samples: loss = sum d (6 d - sum of the six neighbours) / count,
-// d = y - t; gy = 2 (6 d - sum of the six neighbours) / count in channel 0.
+// d = y - t; gy = 2 (6 d - sum of the six neighbours) / count.
 __global__ void k_loss_energy(const float* y, const float* t, int n, long long total, bf16* gy, double* part) {
   __shared__ double sh[32];
+  pdl_launch();
+  pdl_wait();
   double acc = 0.0;
   const float inv = 2.f / (float)total;
   const long long n3 = (long long)n * n * n;
@@ -404,7 +702,7 @@ __global__ void k_loss_energy(const float* y, const float* t, int n, long long t
     const int x = v % n, yy = (v / n) % n, z = v / (n * n);
     auto d = [&](int xx, int yv, int zz) {
       const long long q = s0 + ((long long)zz * n + yv) * n + xx;
-      return y[(size_t)q * 8] - t[q];
+      return y[q] - t[q];
     };
     const float d0 = d(x, yy, z);
     const int xm = x == 0 ? n - 1 : x - 1, xp = x == n - 1 ? 0 : x + 1;
@@ -413,58 +711,68 @@ __global__ void k_loss_energy(const float* y, const float* t, int n, long long t
     const float ld = 6.f * d0 - (d(xm, yy, z) + d(xp, yy, z)) - (d(x, ym, z) + d(x, yp, z)) -
                      (d(x, yy, zm) + d(x, yy, zp));
     acc += (double)d0 * ld;
-    __nv_bfloat162* o = reinterpret_cast<__nv_bfloat162*>(gy + (size_t)i * 16);
-    o[0] = __floats2bfloat162_rn(ld * inv, 0.f);
-    const __nv_bfloat162 zr = __floats2bfloat162_rn(0.f, 0.f);
-#pragma unroll
-    for (int q = 1; q < 8; ++q) o[q] = zr;
+    gy[i] = __float2bfloat16(ld * inv);
   }
   const double r = block_reduce<false>(acc, sh);
   if (threadIdx.x == 0) part[blockIdx.x] = r;
 }
 __global__ void k_sum_part(const double* part, int n, double* out) {
   __shared__ double sh[32];
+  pdl_launch();
+  pdl_wait();
   double acc = 0.0;
   for (int i = threadIdx.x; i < n; i += blockDim.x) acc += part[i];
   const double r = block_reduce<false>(acc, sh);
   if (threadIdx.x == 0) *out = r;
 }
-// per-sample mean of y (channel 0)
-__global__ void k_ymean(const float* y, long long n3, double* out) {
-  __shared__ double sh[32];
-  const int s = blockIdx.x;
-  double acc = 0.0;
-  for (long long i = threadIdx.x; i < n3; i += blockDim.x) acc += (double)y[((size_t)s * n3 + i) * 8];
-  const double r = block_reduce<false>(acc, sh);
-  if (threadIdx.x == 0) out[s] = r / (double)n3;
-}
-// psi_0 = s (y - mean y)
+// psi_0 = s (y - mean y), the mean from the head's tile sums.  A grid row of
+// blocks per sample.
 template <typename T>
-__global__ void k_unpack(const float* y, long long n3, int batch, const double* scale, double out_scale,
-                         const double* ymean, T* psi) {
-  const long long total = (long long)batch * n3;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
-    const int s = (int)(i / n3);
-    psi[i] = (T)(scale[s] * out_scale * ((double)y[(size_t)i * 8] - ymean[s]));
-  }
+__global__ void __launch_bounds__(256) k_unpack(const float* y, long long n3, const double* scale, double out_scale,
+                                                const double* ysum, int tiles, T* psi) {
+  __shared__ double sh[32];
+  __shared__ double mean;
+  pdl_launch();
+  pdl_wait();
+  const long long s = blockIdx.y;
+  double t = 0.0;
+  for (int q = threadIdx.x; q < tiles; q += 256) t += ysum[s * tiles + q];
+  t = block_reduce<false>(t, sh);
+  if (threadIdx.x == 0) mean = t / (double)n3;
+  __syncthreads();
+  const double m = mean, sc = scale[s] * out_scale;
+  for (long long v = blockIdx.x * 256LL + threadIdx.x; v < n3; v += gridDim.x * 256LL)
+    psi[s * n3 + v] = (T)(sc * ((double)y[s * n3 + v] - m));
 }
 
 // master FP32 (flat) -> forward BF16 [tap][co_pad8][ci_pad16] and backward
-// BF16 [flipped tap][ci_pad16][co_pad8 -> padded to 16] weights, FP32 bias
-__global__ void k_weights(const float* flat, int cin, int cout, int k, int cinp, int coutp, int coutp16,
-                          bf16* wf, bf16* wb, float* bias) {
-  const int ntap = k * k * k;
+// BF16 [flipped tap][ci_pad16][co_pad8 -> padded to 16] weights, FP32 bias;
+// a grid row of blocks per layer
+struct WeightLayer {
+  bf16 *wf, *wb;
+  float* bias;
+  long long off;
+  int cin, cout, ntap;
+};
+struct WeightArgs {
+  WeightLayer l[kNL];
+  const float* flat;
+};
+__global__ void k_weights(WeightArgs a) {
+  const WeightLayer& L = a.l[blockIdx.y];
+  const float* flat = a.flat + L.off;
+  const int cinp = pad16(L.cin), coutp = pad8(L.cout), coutp16 = pad16(L.cout), ntap = L.ntap;
   const int total = ntap * coutp16 * cinp;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
     const int ci = i % cinp, co = (i / cinp) % coutp16, t = i / (cinp * coutp16);
-    const float w = (co < cout && ci < cin) ? flat[((size_t)co * cin + ci) * ntap + t] : 0.f;
-    if (co < coutp) wf[((size_t)t * coutp + co) * cinp + ci] = __float2bfloat16(w);
+    const float w = (co < L.cout && ci < L.cin) ? flat[((size_t)co * L.cin + ci) * ntap + t] : 0.f;
+    if (co < coutp) L.wf[((size_t)t * coutp + co) * cinp + ci] = __float2bfloat16(w);
     // backward data: out channel = ci, in channel = co, tap flipped
-    wb[((size_t)(ntap - 1 - t) * cinp + ci) * coutp16 + co] = __float2bfloat16(w);
+    L.wb[((size_t)(ntap - 1 - t) * cinp + ci) * coutp16 + co] = __float2bfloat16(w);
   }
   if (blockIdx.x == 0)
     for (int co = threadIdx.x; co < coutp; co += blockDim.x)
-      bias[co] = co < cout ? flat[(size_t)cout * cin * ntap + co] : 0.f;
+      L.bias[co] = co < L.cout ? flat[(size_t)L.cout * L.cin * ntap + co] : 0.f;
 }
 
 __global__ void k_adam(float* w, const float* g, float* m, float* v, long long n, float lr, float b1, float b2,
@@ -492,7 +800,7 @@ struct les_unet {
   cudaStream_t st = nullptr;
   char* ws = nullptr;
   size_t ws_bytes = 0;
-  int nsm = 148;
+  int nsm = 152;
   size_t nparams = 0;
   size_t woff[kNL] = {};  // flat offsets of each layer's W (bias follows)
   // device buffers
@@ -500,12 +808,11 @@ struct les_unet {
   bf16* wf[kNL] = {};
   bf16* wb[kNL] = {};
   float* bias[kNL] = {};
-  bf16 *x0, *a1a, *e1, *p1, *a2a, *e2, *p2, *a3a, *e3, *u3, *a4a, *g2, *u2, *a5a, *g1;
+  bf16 *x0, *a1a, *e1, *p1, *a2a, *e2, *p2, *a3a, *e3, *a4a, *g2, *a5a, *g1, *gy;
   float *y, *tgt;
-  bf16 *G0, *G1, *G2, *G3, *G4;  // gradient scratch (largest level, 48 channels)
-  float* wpart = nullptr;
-  size_t wpart_floats = 0;
-  double *scale, *ymean, *dpart, *loss;
+  bf16 *G0, *G1, *G2, *G3, *G4;  // gradient scratch
+  float *wpart[kNL] = {}, *bpart[kNL] = {};  // weight and bias gradient partials of the layers' shares
+  double *scale, *ysum, *dpart, *loss;
   int step = 0;
   int loss_kind = 0;       // 0 mean squared error, 1 energy norm of the error
   double out_scale = 1.0;  // psi_0 = s * out_scale * (y - mean y)
@@ -528,6 +835,24 @@ struct Carve {
   }
 };
 
+int level_of(int l) { return (l <= L_E1B || l >= L_D1A) ? 0 : ((l <= L_E2B || l >= L_D2A) ? 1 : 2); }
+long long tiles_of(int cfg, int n, long long batch) {
+  const int zy = cfg ? 8 : 4;
+  const long long t = (n + zy - 1) / zy;
+  return batch * ((n + 3) / 4) * t * t;
+}
+// Shares of the voxel tiles in a weight gradient: a wave of blocks per slice of
+// 16 input channels, but no more partials than 2 M floats (8 MB).
+int wgrad_shares(const les_unet* u, int l, long long batch) {
+  const LayerDef& L = kLayers[l];
+  if (l == L_HEAD) return 2 * u->nsm;
+  const int cinp = pad16(L.cin);
+  const long long tiles = tiles_of(1, u->n >> level_of(l), batch);
+  const long long cap = std::max<long long>(1, (2LL << 20) / (27LL * L.cout * cinp));
+  const long long wave = std::max<long long>(1, 2LL * u->nsm / (cinp / 16));
+  return (int)std::max<long long>(1, std::min(tiles, std::min(cap, wave)));
+}
+
 size_t layout(les_unet* u, char* base, bool dry) {
   Carve c{base, 0, dry};
   const size_t n3 = (size_t)u->n * u->n * u->n, B = (size_t)u->batch;
@@ -542,16 +867,15 @@ size_t layout(les_unet* u, char* base, bool dry) {
   u->grad = c.take<float>(np * 4);
   u->m1 = c.take<float>(np * 4);
   u->m2 = c.take<float>(np * 4);
-  size_t maxpart = 0;
   for (int l = 0; l < kNL; ++l) {
     const LayerDef& L = kLayers[l];
     const int nt = L.k * L.k * L.k, cinp = pad16(L.cin), cop = pad8(L.cout), cop16 = pad16(L.cout);
     u->wf[l] = c.take<bf16>((size_t)nt * cop * cinp * 2);
     u->wb[l] = c.take<bf16>((size_t)nt * cinp * cop16 * 2);
     u->bias[l] = c.take<float>((size_t)cop * 4);
-    const size_t nv = (l <= L_E1B || l >= L_D1A) ? v1 : ((l <= L_E2B || l >= L_D2A) ? v2 : v3);
-    const size_t nch = (nv + 4095) / 4096;
-    maxpart = std::max(maxpart, nch * nt * (size_t)cop16 * cinp);
+    const size_t sh = (size_t)wgrad_shares(u, l, u->batch);
+    u->wpart[l] = c.take<float>(sh * (l == L_HEAD ? 16 : (size_t)nt * L.cout * cinp) * 4);
+    u->bpart[l] = c.take<float>(sh * (size_t)L.cout * 4);
   }
   u->x0 = c.take<bf16>(v1 * 16 * 2);
   u->a1a = c.take<bf16>(v1 * 16 * 2);
@@ -562,20 +886,21 @@ size_t layout(les_unet* u, char* base, bool dry) {
   u->p2 = c.take<bf16>(v3 * 32 * 2);
   u->a3a = c.take<bf16>(v3 * 64 * 2);
   u->e3 = c.take<bf16>(v3 * 64 * 2);
-  u->u3 = c.take<bf16>(v2 * 64 * 2);
   u->a4a = c.take<bf16>(v2 * 32 * 2);
   u->g2 = c.take<bf16>(v2 * 32 * 2);
-  u->u2 = c.take<bf16>(v1 * 32 * 2);
   u->a5a = c.take<bf16>(v1 * 16 * 2);
   u->g1 = c.take<bf16>(v1 * 16 * 2);
-  u->y = c.take<float>(v1 * 8 * 4);
+  u->gy = c.take<bf16>(v1 * 2);
+  u->y = c.take<float>(v1 * 4);
   u->tgt = c.take<float>(v1 * 4);
-  for (bf16** g : {&u->G0, &u->G1, &u->G2, &u->G3, &u->G4}) *g = c.take<bf16>(v1 * 48 * 2);
-  u->wpart_floats = maxpart;
-  u->wpart = c.take<float>(maxpart * 4);
+  u->G0 = c.take<bf16>(v1 * 16 * 2);  // gradient at e1 over the skip connection
+  u->G1 = c.take<bf16>(v2 * 32 * 2);  // ... at e2
+  u->G2 = c.take<bf16>(v1 * 32 * 2);  // gradient on its way between levels
+  u->G3 = c.take<bf16>(v1 * 16 * 2);  // gradients before the activations of a block's second
+  u->G4 = c.take<bf16>(v1 * 16 * 2);  // ... and first convolution
   u->scale = c.take<double>(B * 8);
-  u->ymean = c.take<double>(B * 8);
-  u->dpart = c.take<double>(8192 * 8);
+  u->ysum = c.take<double>((size_t)tiles_of(0, u->n, u->batch) * 8);
+  u->dpart = c.take<double>((4096 + B * kSumBlocks) * 8);
   u->loss = c.take<double>(8);
   return c.off + 256;
 }
@@ -587,159 +912,227 @@ int unet_fail(les_unet* u, cudaError_t e, const char* where) {
 
 unsigned eblocks(long long total) { return (unsigned)std::min<long long>((total + 255) / 256, 8192); }
 
-template <int NF>
-void launch_conv_nf(const ConvArgs& a, bool f32, cudaStream_t st) {
-  const unsigned blocks = (unsigned)((a.nvox / 16 + 3) / 4);
-  if (f32) k_conv<NF, true><<<blocks, 128, 0, st>>>(a);
-  else k_conv<NF, false><<<blocks, 128, 0, st>>>(a);
+// launch that may start while the kernel before it in the stream drains (the
+// kernel waits with pdl_wait)
+template <typename... K, typename... A>
+cudaError_t launch_pdl(void (*k)(K...), dim3 grid, int threads, size_t smem, cudaStream_t st, A... args) {
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = dim3((unsigned)threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  return cudaLaunchKernelEx(&c, k, K(args)...);
 }
 
-// conv over nvox voxels: in = [in0 (c0), in1 (c1)] -> out = [out0 (oc0), out1 (oc1)]
-cudaError_t conv(les_unet* u, int level_n, int nvox, const bf16* in0, int c0, const bf16* in1, int c1, const bf16* w,
-                 const float* bias, int k, void* out0, int oc0, void* out1, int oc1, bool act, bool f32) {
-  ConvArgs a{in0, c0, in1, c1, w, bias, out0, oc0, out1, oc1, level_n, nvox, k, act ? 1 : 0};
-  const int nf = (oc0 + oc1) / 8;
+using ConvKernel = void (*)(ConvArgs);
+struct ConvChoice {
+  ConvKernel k = nullptr;
+  size_t smem = 0;
+};
+template <int CFG, int KC, int NFB>
+ConvChoice choice() {
+  return {k_conv<CFG, KC, NFB>, conv_smem<CFG, KC, NFB>()};
+}
+template <int KC>
+ConvChoice choice_kc(int cfg, int nfb) {
+  if (cfg) return nfb == 4 ? choice<1, KC, 4>() : choice<1, KC, 2>();
+  return nfb == 4 ? choice<0, KC, 4>() : choice<0, KC, 2>();
+}
+ConvChoice conv_kernel(int kc, int cfg, int nfb) {
+  switch (kc) {
+    case 1: return choice_kc<1>(cfg, nfb);
+    case 2: return choice_kc<2>(cfg, nfb);
+    case 3: return choice_kc<3>(cfg, nfb);
+    case 4: return choice_kc<4>(cfg, nfb);
+    case 6: return choice_kc<6>(cfg, nfb);
+    default: return {};
+  }
+}
+constexpr size_t kConvSmemMax = 227 * 1024;
+
+// shared-memory limits of the kernels, once per network
+cudaError_t kernel_limits() {
+  for (int kc : {1, 2, 3, 4, 6})
+    for (int cfg : {0, 1})
+      for (int nfb : {2, 4}) {
+        const ConvChoice c = conv_kernel(kc, cfg, nfb);
+        if (c.smem > kConvSmemMax) continue;
+        const cudaError_t e = cudaFuncSetAttribute(c.k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)c.smem);
+        if (e != cudaSuccess) return e;
+      }
+  cudaError_t e = cudaFuncSetAttribute(k_wgrad<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wgrad_smem<1>());
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_wgrad<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wgrad_smem<2>());
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_wgrad<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)wgrad_smem<4>());
+  return e;
+}
+
+// The widest tile and output slice that still give every SM a block: large
+// tiles halve the weight and halo loads per voxel, small ones fill the chip on
+// the coarse levels.
+cudaError_t conv(les_unet* u, int n, int batch, ConvArgs a) {
+  const int kc = (a.c0 + a.c1) / 16;
+  a.cout = a.oc0 + a.oc1;
+  a.n = n;
+  static constexpr int order[4][2] = {{1, 4}, {1, 2}, {0, 4}, {0, 2}};
+  int cfg = 0, nfb = 2;
+  for (const auto& o : order) {
+    const size_t smem = conv_kernel(kc, o[0], o[1]).smem;
+    if (a.cout % (8 * o[1]) || smem > kConvSmemMax) continue;
+    if (tiles_of(o[0], n, batch) * (a.cout / (8 * o[1])) < u->nsm - u->nsm / 4) continue;
+    cfg = o[0], nfb = o[1];
+    break;
+  }
+  const ConvChoice c = conv_kernel(kc, cfg, nfb);
+  if (!c.k) return cudaErrorInvalidValue;
+  a.tz = (n + 3) / 4;
+  a.ty = a.tx = cfg ? (n + 7) / 8 : (n + 3) / 4;
   ProfScope ps(u->prof, KI_UNET_CONV, u->st);
-  switch (nf) {
-    case 1: launch_conv_nf<1>(a, f32, u->st); break;
-    case 2: launch_conv_nf<2>(a, f32, u->st); break;
-    case 4: launch_conv_nf<4>(a, f32, u->st); break;
-    case 6: launch_conv_nf<6>(a, f32, u->st); break;
-    case 8: launch_conv_nf<8>(a, f32, u->st); break;
-    case 12: launch_conv_nf<12>(a, f32, u->st); break;
+  return launch_pdl(c.k, dim3((unsigned)tiles_of(cfg, n, batch), (unsigned)(a.cout / (8 * nfb))), cfg ? 256 : 128, c.smem,
+                    u->st, a);
+}
+// tiles per sample of the last convolution (whose tiles sum y)
+int head_tiles(const les_unet* u, int batch) {
+  const long long t1 = tiles_of(1, u->n, batch);
+  const bool big = t1 >= u->nsm - u->nsm / 4;
+  return (int)(tiles_of(big ? 1 : 0, u->n, 1));
+}
+
+// forward convolution of layer l
+cudaError_t conv_fwd(les_unet* u, int l, int n, int batch, const bf16* in0, int c0, int up0, const bf16* in1, int c1,
+                     bf16* out, bf16* pool) {
+  ConvArgs a{};
+  a.in0 = in0, a.c0 = c0, a.up0 = up0, a.in1 = in1, a.c1 = c1;
+  a.w = u->wf[l];
+  a.bias = u->bias[l];
+  a.out0 = out, a.oc0 = kLayers[l].cout;
+  a.pool = pool;
+  if (l == L_D1B) a.hw = u->wf[L_HEAD], a.hb = u->bias[L_HEAD], a.y = u->y, a.ysum = u->ysum;
+  return conv(u, n, batch, a);
+}
+// input gradient of layer l from g (its pre-activation gradient), times the
+// slope of the activations post where given
+cudaError_t conv_back(les_unet* u, int l, int n, int batch, const bf16* g, const bf16* post, bf16* out0, int oc0,
+                      bf16* out1, int oc1) {
+  ConvArgs a{};
+  a.in0 = g, a.c0 = kLayers[l].cout;
+  a.w = u->wb[l];
+  a.post = post;
+  a.out0 = out0, a.oc0 = oc0, a.out1 = out1, a.oc1 = oc1;
+  return conv(u, n, batch, a);
+}
+
+// weight and bias gradient partials of layer l given g (gradient at its pre-activation)
+cudaError_t wgrad(les_unet* u, int l, int n, int batch, const bf16* g, const bf16* in0, int c0, int up0, const bf16* in1,
+                  int c1) {
+  const LayerDef& L = kLayers[l];
+  WgradArgs a{g, in0, c0, up0, in1, c1, u->wpart[l], u->bpart[l], c0 + c1, n, (n + 7) / 8, (n + 7) / 8, (n + 3) / 4, 0};
+  a.ntiles = tiles_of(1, n, batch);
+  const dim3 grid((unsigned)((c0 + c1) / 16), (unsigned)wgrad_shares(u, l, batch));
+  ProfScope ps(u->prof, KI_UNET_WGRAD, u->st);
+  switch (L.cout / 16) {
+    case 1: return launch_pdl(k_wgrad<1>, grid, 32 * kWgWarps, wgrad_smem<1>(), u->st, a);
+    case 2: return launch_pdl(k_wgrad<2>, grid, 32 * kWgWarps, wgrad_smem<2>(), u->st, a);
+    case 4: return launch_pdl(k_wgrad<4>, grid, 32 * kWgWarps, wgrad_smem<4>(), u->st, a);
     default: return cudaErrorInvalidValue;
   }
-  return cudaGetLastError();
-}
-
-template <int NF>
-void launch_wgrad_nf(const WgradArgs& a, dim3 grid, cudaStream_t st) {
-  k_wgrad<NF><<<grid, 32, 0, st>>>(a);
-}
-
-// weight + bias gradient of layer l given g (gradient at its pre-activation)
-cudaError_t wgrad(les_unet* u, int l, int level_n, int nvox, const bf16* g, int gstride, const bf16* in0, int c0,
-                  const bf16* in1, int c1) {
-  const LayerDef& L = kLayers[l];
-  const int nt = L.k * L.k * L.k, cop = pad8(L.cout), cop16 = pad16(L.cout), cin = c0 + c1;
-  const int chunk = 4096;
-  const int nch = (nvox + chunk - 1) / chunk;
-  WgradArgs a{g, gstride, cop, in0, c0, in1, c1, u->wpart, level_n, nvox, L.k, chunk};
-  dim3 grid(nt, cop16 / 16, nch);
-  {
-    ProfScope ps(u->prof, KI_UNET_WGRAD, u->st);
-    switch (cin / 8) {
-      case 2: launch_wgrad_nf<2>(a, grid, u->st); break;
-      case 4: launch_wgrad_nf<4>(a, grid, u->st); break;
-      case 6: launch_wgrad_nf<6>(a, grid, u->st); break;
-      case 8: launch_wgrad_nf<8>(a, grid, u->st); break;
-      case 12: launch_wgrad_nf<12>(a, grid, u->st); break;
-      default: return cudaErrorInvalidValue;
-    }
-  }
-  const int total = L.cout * L.cin * nt;
-  k_wgrad_reduce<<<(total + 255) / 256, 256, 0, u->st>>>(u->wpart, nch, nt, cop16, cin, L.cout, L.cin,
-                                                         u->grad + u->woff[l]);
-  const int bchunk = 2048, nb = (nvox + bchunk - 1) / bchunk;
-  float* bpart = u->wpart;  // free again after the reduce (stream order)
-  k_bias_partial<<<nb, std::max(32, cop), 0, u->st>>>(g, gstride, cop, nvox, bchunk, bpart);
-  k_bias_reduce<<<1, std::max(32, cop), 0, u->st>>>(bpart, nb, cop, L.cout,
-                                                    u->grad + u->woff[l] + (size_t)L.cout * L.cin * nt);
-  return cudaGetLastError();
 }
 
 cudaError_t refresh_weights(les_unet* u) {
+  WeightArgs a;
+  a.flat = u->master;
+  int most = 0;
   for (int l = 0; l < kNL; ++l) {
     const LayerDef& L = kLayers[l];
-    const int nt = L.k * L.k * L.k;
-    const int total = nt * pad16(L.cout) * pad16(L.cin);
-    k_weights<<<(total + 255) / 256, 256, 0, u->st>>>(u->master + u->woff[l], L.cin, L.cout, L.k, pad16(L.cin),
-                                                      pad8(L.cout), pad16(L.cout), u->wf[l], u->wb[l], u->bias[l]);
+    a.l[l] = {u->wf[l], u->wb[l], u->bias[l], (long long)u->woff[l], L.cin, L.cout, L.k * L.k * L.k};
+    most = std::max(most, L.k * L.k * L.k * pad16(L.cout) * pad16(L.cin));
   }
+  k_weights<<<dim3((unsigned)((most + 1023) / 1024), kNL), 256, 0, u->st>>>(a);
   return cudaGetLastError();
 }
 
+#define CK(x)                             \
+  if ((e = (x)) != cudaSuccess) return e;
 // forward pass on the packed input x0 (batch b); y receives the head output
 cudaError_t forward(les_unet* u, int b) {
   const int n1 = u->n, n2 = n1 / 2, n3 = n2 / 2;
-  const int v1 = b * n1 * n1 * n1, v2 = v1 / 8, v3 = v2 / 8;
   cudaError_t e;
-#define CK(x)                               \
-  if ((e = (x)) != cudaSuccess) return e;
-  CK(conv(u, n1, v1, u->x0, 16, nullptr, 0, u->wf[L_E1A], u->bias[L_E1A], 3, u->a1a, 16, nullptr, 0, true, false));
-  CK(conv(u, n1, v1, u->a1a, 16, nullptr, 0, u->wf[L_E1B], u->bias[L_E1B], 3, u->e1, 16, nullptr, 0, true, false));
-  k_pool<<<eblocks((long long)v2 * 16), 256, 0, u->st>>>(u->e1, 16, n1, b, u->p1);
-  CK(conv(u, n2, v2, u->p1, 16, nullptr, 0, u->wf[L_E2A], u->bias[L_E2A], 3, u->a2a, 32, nullptr, 0, true, false));
-  CK(conv(u, n2, v2, u->a2a, 32, nullptr, 0, u->wf[L_E2B], u->bias[L_E2B], 3, u->e2, 32, nullptr, 0, true, false));
-  k_pool<<<eblocks((long long)v3 * 32), 256, 0, u->st>>>(u->e2, 32, n2, b, u->p2);
-  CK(conv(u, n3, v3, u->p2, 32, nullptr, 0, u->wf[L_E3A], u->bias[L_E3A], 3, u->a3a, 64, nullptr, 0, true, false));
-  CK(conv(u, n3, v3, u->a3a, 64, nullptr, 0, u->wf[L_E3B], u->bias[L_E3B], 3, u->e3, 64, nullptr, 0, true, false));
-  k_up<<<eblocks((long long)v2 * 64), 256, 0, u->st>>>(u->e3, 64, n3, b, u->u3);
-  CK(conv(u, n2, v2, u->u3, 64, u->e2, 32, u->wf[L_D2A], u->bias[L_D2A], 3, u->a4a, 32, nullptr, 0, true, false));
-  CK(conv(u, n2, v2, u->a4a, 32, nullptr, 0, u->wf[L_D2B], u->bias[L_D2B], 3, u->g2, 32, nullptr, 0, true, false));
-  k_up<<<eblocks((long long)v1 * 32), 256, 0, u->st>>>(u->g2, 32, n2, b, u->u2);
-  CK(conv(u, n1, v1, u->u2, 32, u->e1, 16, u->wf[L_D1A], u->bias[L_D1A], 3, u->a5a, 16, nullptr, 0, true, false));
-  CK(conv(u, n1, v1, u->a5a, 16, nullptr, 0, u->wf[L_D1B], u->bias[L_D1B], 3, u->g1, 16, nullptr, 0, true, false));
-  CK(conv(u, n1, v1, u->g1, 16, nullptr, 0, u->wf[L_HEAD], u->bias[L_HEAD], 1, u->y, 8, nullptr, 0, false, true));
-  return cudaGetLastError();
+  CK(conv_fwd(u, L_E1A, n1, b, u->x0, 16, 0, nullptr, 0, u->a1a, nullptr));
+  CK(conv_fwd(u, L_E1B, n1, b, u->a1a, 16, 0, nullptr, 0, u->e1, u->p1));
+  CK(conv_fwd(u, L_E2A, n2, b, u->p1, 16, 0, nullptr, 0, u->a2a, nullptr));
+  CK(conv_fwd(u, L_E2B, n2, b, u->a2a, 32, 0, nullptr, 0, u->e2, u->p2));
+  CK(conv_fwd(u, L_E3A, n3, b, u->p2, 32, 0, nullptr, 0, u->a3a, nullptr));
+  CK(conv_fwd(u, L_E3B, n3, b, u->a3a, 64, 0, nullptr, 0, u->e3, nullptr));
+  CK(conv_fwd(u, L_D2A, n2, b, u->e3, 64, 1, u->e2, 32, u->a4a, nullptr));
+  CK(conv_fwd(u, L_D2B, n2, b, u->a4a, 32, 0, nullptr, 0, u->g2, nullptr));
+  CK(conv_fwd(u, L_D1A, n1, b, u->g2, 32, 1, u->e1, 16, u->a5a, nullptr));
+  CK(conv_fwd(u, L_D1B, n1, b, u->a5a, 16, 0, nullptr, 0, u->g1, nullptr));
+  return cudaSuccess;
 }
 
-// backward through one block B(.; a->c) with input [in0, in1], first conv la,
-// second lb, outputs post_a (first activation) and post_b; gout is the
-// gradient at post_b.  Writes the input gradient to gin0 / gin1 (if given).
-cudaError_t block_back(les_unet* u, int la, int lb, int ln, int nvox, const bf16* in0, int c0, const bf16* in1, int c1,
-                       const bf16* post_a, const bf16* post_b, const bf16* gout, bf16* gin0, bf16* gin1, bf16* s1,
-                       bf16* s2) {
-  const int ca = pad8(kLayers[la].cout), cb = pad8(kLayers[lb].cout);
-  cudaError_t e;
-  k_act_bwd<<<eblocks((long long)nvox * cb), 256, 0, u->st>>>(post_b, gout, (long long)nvox * cb, s1);
-  CK(wgrad(u, lb, ln, nvox, s1, cb, post_a, ca, nullptr, 0));
-  CK(conv(u, ln, nvox, s1, cb, nullptr, 0, u->wb[lb], nullptr, 3, s2, ca, nullptr, 0, false, false));
-  k_act_bwd<<<eblocks((long long)nvox * ca), 256, 0, u->st>>>(post_a, s2, (long long)nvox * ca, s1);
-  CK(wgrad(u, la, ln, nvox, s1, ca, in0, c0, in1, c1));
-  if (gin0) CK(conv(u, ln, nvox, s1, ca, nullptr, 0, u->wb[la], nullptr, 3, gin0, c0, gin1, c1, false, false));
-  return cudaGetLastError();
-}
-
-// full backward from gy (in G0, [v1][16], channel 0 real); fills u->grad
+// full backward from gy; fills u->grad.  Per block B(.; a -> c): G3 holds the
+// gradient before the second activation, G4 before the first.
 cudaError_t backward(les_unet* u, int b) {
   const int n1 = u->n, n2 = n1 / 2, n3 = n2 / 2;
-  const int v1 = b * n1 * n1 * n1, v2 = v1 / 8, v3 = v2 / 8;
+  const long long v1 = (long long)b * n1 * n1 * n1, v2 = v1 / 8, v3 = v2 / 8;
   cudaError_t e;
-  bf16 *gy = u->G0, *gA = u->G1, *gB = u->G2, *s1 = u->G3, *s2 = u->G4;
-  // head (1x1, no activation): weight grad and gradient at g1
-  CK(wgrad(u, L_HEAD, n1, v1, gy, 16, u->g1, 16, nullptr, 0));
-  CK(conv(u, n1, v1, gy, 16, nullptr, 0, u->wb[L_HEAD], nullptr, 1, gA, 16, nullptr, 0, false, false));
-  // D1: input [u2 (32), e1 (16)] -> grads g_u2 (gB, 32 ch) and g_e1 (gy reused, 16 ch)
-  bf16* g_e1 = gy;
-  CK(block_back(u, L_D1A, L_D1B, n1, v1, u->u2, 32, u->e1, 16, u->a5a, u->g1, gA, gB, g_e1, s1, s2));
-  // up backward: g_g2 (v2 x 32) into gA
-  k_up_bwd<<<eblocks((long long)v2 * 32), 256, 0, u->st>>>(gB, 32, n2, b, gA);
-  // D2: input [u3 (64), e2 (32)] -> g_u3 (gB, v2 x 64), g_e2 (s2... keep in a dedicated slot)
-  bf16* g_e2 = u->G4 + (size_t)v1 * 32;  // tail of the last scratch buffer
-  CK(block_back(u, L_D2A, L_D2B, n2, v2, u->u3, 64, u->e2, 32, u->a4a, u->g2, gA, gB, g_e2, s1, s2));
-  k_up_bwd<<<eblocks((long long)v3 * 64), 256, 0, u->st>>>(gB, 64, n3, b, gA);  // g_e3
-  // L3: input p2 (32) -> g_p2 (gB, v3 x 32)
-  CK(block_back(u, L_E3A, L_E3B, n3, v3, u->p2, 32, nullptr, 0, u->a3a, u->e3, gA, gB, nullptr, s1, s2));
-  k_pool_bwd<<<eblocks((long long)v2 * 32), 256, 0, u->st>>>(gB, 32, n2, b, g_e2, 1);
-  // L2: input p1 (16) -> g_p1 (gB, v2 x 16)
-  CK(block_back(u, L_E2A, L_E2B, n2, v2, u->p1, 16, nullptr, 0, u->a2a, u->e2, g_e2, gB, nullptr, s1, s2));
-  k_pool_bwd<<<eblocks((long long)v1 * 16), 256, 0, u->st>>>(gB, 16, n1, b, g_e1, 1);
-  // L1: input x0 (16, channel 0 real); its gradient is not needed
-  CK(block_back(u, L_E1A, L_E1B, n1, v1, u->x0, 16, nullptr, 0, u->a1a, u->e1, g_e1, nullptr, nullptr, s1, s2));
-  return cudaGetLastError();
-#undef CK
+  auto blocks = [&](long long total) { return dim3((unsigned)std::min<long long>((total + 255) / 256, 16LL * u->nsm)); };
+  const int hsh = wgrad_shares(u, L_HEAD, b);
+  CK(launch_pdl(k_head_back, dim3((unsigned)hsh), 256, 0, u->st, u->gy, u->wf[L_HEAD], u->g1, v1, u->G3, u->wpart[L_HEAD],
+                u->bpart[L_HEAD]));
+  CK(wgrad(u, L_D1B, n1, b, u->G3, u->a5a, 16, 0, nullptr, 0));
+  CK(conv_back(u, L_D1B, n1, b, u->G3, u->a5a, u->G4, 16, nullptr, 0));
+  CK(wgrad(u, L_D1A, n1, b, u->G4, u->g2, 32, 1, u->e1, 16));
+  CK(conv_back(u, L_D1A, n1, b, u->G4, nullptr, u->G2, 32, u->G0, 16));
+  CK(launch_pdl(k_up_back, blocks(v2 * 4), 256, 0, u->st, u->G2, 32, n2, v2 * 4, u->g2, u->G3));
+  CK(wgrad(u, L_D2B, n2, b, u->G3, u->a4a, 32, 0, nullptr, 0));
+  CK(conv_back(u, L_D2B, n2, b, u->G3, u->a4a, u->G4, 32, nullptr, 0));
+  CK(wgrad(u, L_D2A, n2, b, u->G4, u->e3, 64, 1, u->e2, 32));
+  CK(conv_back(u, L_D2A, n2, b, u->G4, nullptr, u->G2, 64, u->G1, 32));
+  CK(launch_pdl(k_up_back, blocks(v3 * 8), 256, 0, u->st, u->G2, 64, n3, v3 * 8, u->e3, u->G3));
+  CK(wgrad(u, L_E3B, n3, b, u->G3, u->a3a, 64, 0, nullptr, 0));
+  CK(conv_back(u, L_E3B, n3, b, u->G3, u->a3a, u->G4, 64, nullptr, 0));
+  CK(wgrad(u, L_E3A, n3, b, u->G4, u->p2, 32, 0, nullptr, 0));
+  CK(conv_back(u, L_E3A, n3, b, u->G4, nullptr, u->G2, 32, nullptr, 0));
+  CK(launch_pdl(k_pool_back, blocks(v2 * 4), 256, 0, u->st, u->G2, 32, n2, v2 * 4, u->G1, u->e2, u->G3));
+  CK(wgrad(u, L_E2B, n2, b, u->G3, u->a2a, 32, 0, nullptr, 0));
+  CK(conv_back(u, L_E2B, n2, b, u->G3, u->a2a, u->G4, 32, nullptr, 0));
+  CK(wgrad(u, L_E2A, n2, b, u->G4, u->p1, 16, 0, nullptr, 0));
+  CK(conv_back(u, L_E2A, n2, b, u->G4, nullptr, u->G2, 16, nullptr, 0));
+  CK(launch_pdl(k_pool_back, blocks(v1 * 2), 256, 0, u->st, u->G2, 16, n1, v1 * 2, u->G0, u->e1, u->G3));
+  CK(wgrad(u, L_E1B, n1, b, u->G3, u->a1a, 16, 0, nullptr, 0));
+  CK(conv_back(u, L_E1B, n1, b, u->G3, u->a1a, u->G4, 16, nullptr, 0));
+  CK(wgrad(u, L_E1A, n1, b, u->G4, u->x0, 16, 0, nullptr, 0));
+  ReduceArgs r;
+  r.grad = u->grad;
+  int blk = 0;
+  for (int l = 0; l < kNL; ++l) {
+    const LayerDef& L = kLayers[l];
+    const int nt = L.k * L.k * L.k, cinp = pad16(L.cin);
+    r.l[l] = {u->wpart[l], u->bpart[l], wgrad_shares(u, l, b), nt, L.cout, L.cout, L.cin, cinp, (long long)u->woff[l], blk};
+    blk += (nt * L.cout * cinp + L.cout + 31) / 32;
+  }
+  return launch_pdl(k_grad_reduce, dim3((unsigned)blk), 32 * kRedWarps, 0, u->st, r);
 }
+#undef CK
 
 template <typename T>
 cudaError_t pack_inputs(les_unet* u, const T* b, const T* psi, int batch) {
   const long long n3 = (long long)u->n * u->n * u->n;
-  const int nblk = 64;
-  k_sumsq<T><<<dim3(nblk, batch), 256, 0, u->st>>>(b, n3, u->dpart);
-  k_scale<<<1, 64, 0, u->st>>>(u->dpart, nblk, n3, batch, u->scale);
-  k_pack<T><<<eblocks(batch * n3), 256, 0, u->st>>>(b, psi, n3, batch, u->scale, u->out_scale, u->x0,
-                                                     psi ? u->tgt : nullptr);
-  return cudaGetLastError();
+  // an ordinary launch: whatever wrote the weights is complete before the
+  // chain of overlapping launches begins
+  k_sumsq<T><<<dim3(kSumBlocks, batch), 256, 0, u->st>>>(b, n3, u->dpart + 4096);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  const unsigned bx = (unsigned)std::min<long long>((n3 + 255) / 256, std::max(1, 16 * u->nsm / batch));
+  return launch_pdl(k_pack<T>, dim3(bx, (unsigned)batch), 256, 0, u->st, b, psi, n3, u->dpart + 4096, u->scale,
+                    u->out_scale, u->x0, psi ? u->tgt : (float*)nullptr);
 }
 
 template <typename T>
@@ -748,9 +1141,9 @@ int run_forward(les_unet* u, const T* b, int batch, T* psi0) {
   if ((e = pack_inputs<T>(u, b, (const T*)nullptr, batch)) != cudaSuccess) return unet_fail(u, e, "pack");
   if ((e = forward(u, batch)) != cudaSuccess) return unet_fail(u, e, "forward");
   const long long n3 = (long long)u->n * u->n * u->n;
-  k_ymean<<<batch, 256, 0, u->st>>>(u->y, n3, u->ymean);
-  k_unpack<T><<<eblocks(batch * n3), 256, 0, u->st>>>(u->y, n3, batch, u->scale, u->out_scale, u->ymean, psi0);
-  e = cudaGetLastError();
+  const unsigned bx = (unsigned)std::min<long long>((n3 + 255) / 256, std::max(1, 16 * u->nsm / batch));
+  e = launch_pdl(k_unpack<T>, dim3(bx, (unsigned)batch), 256, 0, u->st, u->y, n3, u->scale, u->out_scale, u->ysum,
+                 head_tiles(u, batch), psi0);
   return e == cudaSuccess ? LES_OK : unet_fail(u, e, "unpack");
 }
 
@@ -761,10 +1154,12 @@ int run_loss_grad(les_unet* u, const T* b, const T* psi, int batch, double* loss
   if ((e = forward(u, batch)) != cudaSuccess) return unet_fail(u, e, "forward");
   const long long total = (long long)batch * u->n * u->n * u->n;
   const int nb = (int)std::min<long long>((total + 255) / 256, 4096);
-  if (u->loss_kind == 1) k_loss_energy<<<nb, 256, 0, u->st>>>(u->y, u->tgt, u->n, total, u->G0, u->dpart);
-  else k_loss<<<nb, 256, 0, u->st>>>(u->y, u->tgt, total, u->G0, u->dpart);
-  k_sum_part<<<1, 256, 0, u->st>>>(u->dpart, nb, u->loss);
-  if ((e = backward(u, batch)) != cudaSuccess) return unet_fail(u, e, "backward");
+  if (u->loss_kind == 1)
+    e = launch_pdl(k_loss_energy, dim3((unsigned)nb), 256, 0, u->st, u->y, u->tgt, u->n, total, u->gy, u->dpart);
+  else e = launch_pdl(k_loss, dim3((unsigned)nb), 256, 0, u->st, u->y, u->tgt, total, u->gy, u->dpart);
+  if (e == cudaSuccess) e = launch_pdl(k_sum_part, dim3(1), 256, 0, u->st, u->dpart, nb, u->loss);
+  if (e == cudaSuccess) e = backward(u, batch);
+  if (e != cudaSuccess) return unet_fail(u, e, "backward");
   if (loss) {
     double h = 0;
     if ((e = cudaMemcpyAsync(&h, u->loss, 8, cudaMemcpyDeviceToHost, u->st)) != cudaSuccess ||
@@ -824,7 +1219,8 @@ int les_unet_create(int32_t n, int32_t batch, void* workspace, size_t bytes, voi
   u->ws = (char*)workspace;
   u->ws_bytes = bytes;
   layout(u, u->ws, false);
-  cudaError_t e = cudaMemsetAsync(u->ws, 0, need, u->st);
+  cudaError_t e = kernel_limits();
+  if (e == cudaSuccess) e = cudaMemsetAsync(u->ws, 0, need, u->st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(u->st);
   if (e != cudaSuccess) {
     delete u;
