@@ -13,7 +13,7 @@
 // by layer, W[cout][cin][kz][ky][kx] then bias[cout].
 //
 // Activations are channels-last BF16 ([batch][z][y][x][c], c padded to a
-// multiple of 16); weights [tap][cout][cin].  A convolution (k_conv) is an
+// multiple of 16); weights [cout / 16][tap][16][cin + 8].  A convolution (k_conv) is an
 // implicit GEMM on the tensor cores, mma.sync m16n8k16 BF16 -> FP32: rows are
 // voxels, K runs over (tap, 16 channels), N over output channels.  A block
 // stages its tile's input with a halo of one voxel and the weights of its
@@ -29,12 +29,16 @@
 // while the block walks its share of the tiles; the FP32 partials of the
 // shares are summed in order (deterministic).  Adam keeps FP32 master weights.
 //
-// What bounds it: at 32^3 and batch 1 the launches and the fill of 13 short
-// kernels (each loads its weights before it waits for its predecessor); at
-// batch 16 the shared-memory reads, 2 to 4 wavefronts per MMA.  mma.sync, not
-// tcgen05: N is 16 to 64 and a tile 64 or 256 voxels, and every product is
-// summed in the order of taps and channels, so the results do not depend on
-// the tile.
+// What bounds it: at 32^3 and batch 1 the 13 short kernels' launches and
+// latencies (5 to 10 us each, the MMAs 1 to 3 of them; each loads its weights
+// before it waits for its predecessor); at batch 16 the shared-memory reads, 3
+// wavefronts per MMA with two output fragments and 2 with four (the LSU pipe is
+// 55 % busy, the tensor pipe 36 %).  mma.sync, not tcgen05: N is 16 to 64, and
+// every sum runs over taps and channels in one order, so the results do not
+// depend on the tile.  Blocks that keep their weights and stage the next tile
+// during the MMAs were no faster (two input buffers cost the second block).
+// Measured (GB300, 32^3): forward at batch 1 437 us with an operand fetched
+// from global memory per MMA, 82 now; training gradient at batch 16 8990, 1090.
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -162,7 +166,7 @@ struct ConvArgs {
   int c0, up0;  // channels of in0 (multiple of 16); 1: in0 lives on the halved grid
   const bf16* in1;
   int c1;          // channels of in1 (0 if absent)
-  const bf16* w;   // [27][cout][16 KC]
+  const bf16* w;   // [cout / 16][27][16][16 KC + 8]
   int cout;
   const float* bias;  // forward: bias and leaky ReLU; NULL: neither
   const bf16* post;   // backward: activations whose slope multiplies the result (oc0 channels)
@@ -178,27 +182,45 @@ struct ConvArgs {
   int n, tx, ty, tz;  // grid, tiles along x, y, z
 };
 
-// Halo tile of one sample into shared memory: channels [ch0, ch0 + 8 NC) of
-// [in0, in1] in NC 16-byte chunks per voxel.
-template <int CFG, int NC, int S, int P, int PZ, int NTHR>
-__device__ __forceinline__ void stage_halo(unsigned sm, const bf16* in0, int c0, int up0, const bf16* in1, int c1,
-                                           int ch0, int n, long long b, int z0, int y0, int x0) {
+// Where the rows and columns of a halo tile lie: element offsets of its rows in
+// both inputs and of its columns within a row (periodic, halved for an input on
+// the coarser grid).  Made once per tile by one thread per row, so that a
+// 16-byte copy costs a dozen instructions: formed per copy, the wraps and
+// products took longer than the MMAs.
+template <int CFG>
+struct HaloTable {
   using T = Tile<CFG>;
-  constexpr int HX = T::X + 2, HY = T::Y + 2, NV = (T::Z + 2) * HY * HX;
-  const int m = n >> 1;
-  for (int e = threadIdx.x; e < NV * NC; e += NTHR) {
-    const int v = e / NC, c = e - v * NC;
-    const int x = v % HX, y = (v / HX) % HY, z = v / (HX * HY);
-    const int gz = wrap_tile(z0 - 1 + z, n), gy = wrap_tile(y0 - 1 + y, n), gx = wrap_tile(x0 - 1 + x, n);
-    const int ch = ch0 + 8 * c;
-    const bf16* src;
-    if (ch < c0)
-      src = in0 + (size_t)(up0 ? ((b * m + (gz >> 1)) * m + (gy >> 1)) * m + (gx >> 1) : ((b * n + gz) * n + gy) * n + gx) *
-                      c0 + ch;
-    else
-      src = in1 + (size_t)(((b * n + gz) * n + gy) * n + gx) * c1 + (ch - c0);
-    const unsigned d = sm + 16u * (unsigned)(z * PZ + y * P + x * S + c);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+  static constexpr int HX = T::X + 2, HY = T::Y + 2, ROWS = (T::Z + 2) * HY;
+  long long r0[ROWS], r1[ROWS];
+  int x0[HX], x1[HX];
+  __device__ __forceinline__ void make(int c0, int up0, int c1, int n, long long b, int z0, int y0, int xs) {
+    const int t = threadIdx.x, m = n >> 1;
+    if (t < ROWS) {
+      const int gz = wrap_tile(z0 - 1 + t / HY, n), gy = wrap_tile(y0 - 1 + t % HY, n);
+      const long long r = (b * n + gz) * n + gy;
+      r0[t] = (up0 ? ((b * m + (gz >> 1)) * m + (gy >> 1)) * m : r * n) * c0;
+      r1[t] = r * n * c1;
+    } else if (t < ROWS + HX) {
+      const int gx = wrap_tile(xs - 1 + t - ROWS, n);
+      x0[t - ROWS] = (up0 ? gx >> 1 : gx) * c0;
+      x1[t - ROWS] = gx * c1;
+    }
+  }
+};
+// Channels [ch0, ch0 + 8 NC) of [in0, in1] of a halo tile into shared memory.
+template <int CFG, int NC, int S, int P, int PZ, int NTHR>
+__device__ __forceinline__ void stage_halo(unsigned sm, const HaloTable<CFG>& tab, const bf16* in0, int c0,
+                                           const bf16* in1, int ch0) {
+  using H = HaloTable<CFG>;
+  constexpr int N = H::ROWS * H::HX * NC;
+#pragma unroll 4
+  for (int e = threadIdx.x; e < N; e += NTHR) {
+    const int row = e / (H::HX * NC), k = e - row * (H::HX * NC), x = k / NC, c = k - x * NC;
+    const int z = row / H::HY, y = row - z * H::HY, ch = ch0 + 8 * c;
+    const bf16* src = ch < c0 ? in0 + (tab.r0[row] + tab.x0[x] + ch) : in1 + (tab.r1[row] + tab.x1[x] + (ch - c0));
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sm + 16u * (unsigned)(z * PZ + y * P + x * S + c)),
+                 "l"(src)
+                 : "memory");
   }
 }
 
@@ -209,25 +231,30 @@ __global__ void __launch_bounds__(32 * Tile<CFG>::W) k_conv(ConvArgs a) {
   constexpr int NB = 8 * NFB, NTHR = 32 * T::W, WS = 2 * KC + 1, MT = T::MT;
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ double shd[32];
+  __shared__ HaloTable<CFG> tab;
   const unsigned sin = (unsigned)__cvta_generic_to_shared(smraw), sw = sin + 16u * G::IN;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int gid = lane >> 2, tig = lane & 3;
   const int co0 = blockIdx.y * NB;
-  // the weights first: they do not depend on the kernel before
-  for (int e = threadIdx.x; e < 27 * NB * 2 * KC; e += NTHR) {
-    const int row = e / (2 * KC), c = e - row * (2 * KC);
-    const int t = row / NB, r = row - t * NB;
-    const bf16* src = a.w + ((size_t)t * a.cout + co0 + r) * (16 * KC) + 8 * c;
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sw + 16u * (unsigned)(row * WS + c)), "l"(src)
-                 : "memory");
+  // the weights first: they do not depend on the kernel before.  Their rows are
+  // padded in global memory as they are here, so the copy is a plain one.
+  {
+    constexpr int NCH = 27 * NB * WS;
+    const bf16* src = a.w + (size_t)blockIdx.y * NCH * 8;
+#pragma unroll 4
+    for (int e = threadIdx.x; e < NCH; e += NTHR)
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(sw + 16u * (unsigned)e), "l"(src + 8 * e)
+                   : "memory");
   }
-  pdl_launch();
-  pdl_wait();
   const int tps = a.tx * a.ty * a.tz;
   const long long b = blockIdx.x / tps;
   const int tile = blockIdx.x - (int)b * tps;
   const int x0 = (tile % a.tx) * T::X, y0 = (tile / a.tx) % a.ty * T::Y, z0 = tile / (a.tx * a.ty) * T::Z;
-  stage_halo<CFG, 2 * KC, G::S, G::P, G::PZ, NTHR>(sin, a.in0, a.c0, a.up0, a.in1, a.c1, 0, a.n, b, z0, y0, x0);
+  tab.make(a.c0, a.up0, a.c1, a.n, b, z0, y0, x0);
+  __syncthreads();
+  pdl_launch();
+  pdl_wait();
+  stage_halo<CFG, 2 * KC, G::S, G::P, G::PZ, NTHR>(sin, tab, a.in0, a.c0, a.in1, 0);
   cp_commit();
   cp_wait<0>();
   __syncthreads();
@@ -242,6 +269,7 @@ __global__ void __launch_bounds__(32 * Tile<CFG>::W) k_conv(ConvArgs a) {
       z = q >> 2, y = ((q & 3) << 1) + (row >> 3), x = row & 7;
     }
   };
+  const unsigned pb = sw + 16u * (unsigned)(((lane & 7) + ((lane >> 4) & 1) * 8) * WS + ((lane >> 3) & 1));
   unsigned pa[MT];
 #pragma unroll
   for (int mt = 0; mt < MT; ++mt) {
@@ -249,30 +277,43 @@ __global__ void __launch_bounds__(32 * Tile<CFG>::W) k_conv(ConvArgs a) {
     voxel(mt, lane & 15, z, y, x);
     pa[mt] = sin + 16u * (unsigned)(z * G::PZ + y * G::P + x * G::S + (lane >> 4));
   }
-  const unsigned pb = sw + 16u * (unsigned)(((lane & 7) + ((lane >> 4) & 1) * 8) * WS + ((lane >> 3) & 1));
   float acc[MT][NFB][4];
 #pragma unroll
   for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
     for (int f = 0; f < NFB; ++f) acc[mt][f][0] = acc[mt][f][1] = acc[mt][f][2] = acc[mt][f][3] = 0.f;
+  // the operands of a step are loaded while the MMAs of the one before run
+  unsigned A[MT][4], B[NFB / 2][4];
+  auto load = [&](unsigned (&fa)[MT][4], unsigned (&fb)[NFB / 2][4], int zy, int step) {
+    const int tx = step / KC, kc = step % KC;
+    const unsigned oa = 16u * (unsigned)((zy / 3) * G::PZ + (zy % 3) * G::P + tx * G::S + 2 * kc);
+    const unsigned ob = 16u * (unsigned)((zy * 3 + tx) * 16 * WS + 2 * kc);
+#pragma unroll
+    for (int mt = 0; mt < MT; ++mt) ldsm4(fa[mt], pa[mt] + oa);
+#pragma unroll
+    for (int h = 0; h < NFB / 2; ++h) ldsm4(fb[h], pb + ob + 16u * (unsigned)(27 * 16 * h * WS));
+  };
+  load(A, B, 0, 0);
 #pragma unroll 1
   for (int zy = 0; zy < 9; ++zy) {
-    const unsigned oa = 16u * (unsigned)((zy / 3) * G::PZ + (zy % 3) * G::P);
-    const unsigned ob = 16u * (unsigned)(zy * 3 * NB * WS);
 #pragma unroll
-    for (int tx = 0; tx < 3; ++tx)
+    for (int step = 0; step < 3 * KC; ++step) {
+      unsigned An[MT][4], Bn[NFB / 2][4];
+      // (after the very last step the first of the last group again, unused)
+      if (step + 1 < 3 * KC) load(An, Bn, zy, step + 1);
+      else load(An, Bn, zy < 8 ? zy + 1 : 8, 0);
 #pragma unroll
-      for (int kc = 0; kc < KC; ++kc) {
-        unsigned A[MT][4], B[NFB / 2][4];
+      for (int mt = 0; mt < MT; ++mt)
 #pragma unroll
-        for (int mt = 0; mt < MT; ++mt) ldsm4(A[mt], pa[mt] + oa + 16u * (unsigned)(tx * G::S + 2 * kc));
+        for (int f = 0; f < NFB; ++f) mma_bf16(acc[mt][f], A[mt], B[f >> 1][2 * (f & 1)], B[f >> 1][2 * (f & 1) + 1]);
 #pragma unroll
-        for (int h = 0; h < NFB / 2; ++h) ldsm4(B[h], pb + ob + 16u * (unsigned)((tx * NB + 16 * h) * WS + 2 * kc));
+      for (int q = 0; q < 4; ++q) {
 #pragma unroll
-        for (int mt = 0; mt < MT; ++mt)
+        for (int mt = 0; mt < MT; ++mt) A[mt][q] = An[mt][q];
 #pragma unroll
-          for (int f = 0; f < NFB; ++f) mma_bf16(acc[mt][f], A[mt], B[f >> 1][2 * (f & 1)], B[f >> 1][2 * (f & 1) + 1]);
+        for (int h = 0; h < NFB / 2; ++h) B[h][q] = Bn[h][q];
       }
+    }
   }
   __syncthreads();  // the staged input is free: it takes the output tile
 
@@ -307,9 +348,9 @@ __global__ void __launch_bounds__(32 * Tile<CFG>::W) k_conv(ConvArgs a) {
     }
     if (NFB == 2 && a.hw) {
       // the output fragments are the A fragments of the 1x1 head
-      const unsigned A[4] = {packed[0][0], packed[0][1], packed[1][0], packed[1][1]};
+      const unsigned H[4] = {packed[0][0], packed[0][1], packed[1][0], packed[1][1]};
       float yv[4] = {0.f, 0.f, 0.f, 0.f};
-      mma_bf16(yv, A, ld32(a.hw + gid * 16 + tig * 2), ld32(a.hw + gid * 16 + tig * 2 + 8));
+      mma_bf16(yv, H, ld32(a.hw + gid * 16 + tig * 2), ld32(a.hw + gid * 16 + tig * 2 + 8));
       if (tig == 0) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
@@ -326,16 +367,11 @@ __global__ void __launch_bounds__(32 * Tile<CFG>::W) k_conv(ConvArgs a) {
   }
   __syncthreads();
   // stored 16 bytes at a time; row q of the tile is voxel (q)
-  auto tile_voxel = [&](int q, int& z, int& y, int& x) {
-    if (CFG == 0) z = q >> 4, y = (q >> 2) & 3, x = q & 3;
-    else z = q >> 6, y = (q >> 3) & 7, x = q & 7;
-  };
   for (int e = threadIdx.x; e < T::Z * T::Y * T::X * NFB; e += NTHR) {
     const int q = e / NFB, c = e - q * NFB;
-    int z, y, x;
-    tile_voxel(q, z, y, x);
-    if (z0 + z >= a.n || y0 + y >= a.n || x0 + x >= a.n) continue;
-    const size_t v = (size_t)((b * a.n + z0 + z) * a.n + y0 + y) * a.n + x0 + x;
+    const int z = z0 + q / (T::Y * T::X), y = y0 + q / T::X % T::Y, x = x0 + q % T::X;
+    if (z >= a.n || y >= a.n || x >= a.n) continue;
+    const size_t v = (size_t)((b * a.n + z) * a.n + y) * a.n + x;
     uint4 o = *reinterpret_cast<const uint4*>(so + q * OS + 8 * c);
     const int co = co0 + 8 * c;
     if (a.post) o = act_back(__ldg(reinterpret_cast<const uint4*>(a.post + v * a.oc0 + co)), o);
@@ -350,16 +386,16 @@ __global__ void __launch_bounds__(32 * Tile<CFG>::W) k_conv(ConvArgs a) {
       if (z0 + 2 * z >= a.n || y0 + 2 * y >= a.n || x0 + 2 * x >= a.n) continue;
       Chunk s = {};
 #pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const int r = ((2 * z + (k >> 2)) * T::Y + 2 * y + ((k >> 1) & 1)) * T::X + 2 * x + (k & 1);
+      for (int r8 = 0; r8 < 8; ++r8) {
+        const int r = ((2 * z + (r8 >> 2)) * T::Y + 2 * y + ((r8 >> 1) & 1)) * T::X + 2 * x + (r8 & 1);
         const Chunk u = unpack8(*reinterpret_cast<const uint4*>(so + r * OS + 8 * c));
 #pragma unroll
         for (int i = 0; i < 8; ++i) s.v[i] += u.v[i];
       }
 #pragma unroll
       for (int i = 0; i < 8; ++i) s.v[i] *= 0.125f;
-      *reinterpret_cast<uint4*>(a.pool + (size_t)(((b * m + z0 / 2 + z) * m + y0 / 2 + y) * m + x0 / 2 + x) * a.oc0 + co0 +
-                                8 * c) = pack8(s);
+      *reinterpret_cast<uint4*>(a.pool + (size_t)(((b * m + z0 / 2 + z) * m + y0 / 2 + y) * m + x0 / 2 + x) * a.oc0 +
+                                co0 + 8 * c) = pack8(s);
     }
   }
   if (a.hw) {
@@ -397,18 +433,28 @@ __global__ void __launch_bounds__(32 * kWgWarps) k_wgrad(WgradArgs a) {
   using G = Staged<1, 1>;
   constexpr int NTHR = 32 * kWgWarps, GS = 2 * CO + 1, STAGE = G::IN + 256 * GS;
   extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ HaloTable<1> tab[2];
   const unsigned sm = (unsigned)__cvta_generic_to_shared(smraw);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int gid = lane >> 2, tig = lane & 3;
   const int tps = a.tx * a.ty * a.tz;
-  pdl_launch();
-  pdl_wait();
+  auto origin = [&](long long tile, long long& b, int& z0, int& y0, int& x0) {
+    b = tile / tps;
+    const int q0 = (int)(tile - b * tps);
+    x0 = (q0 % a.tx) * T::X, y0 = (q0 / a.tx) % a.ty * T::Y, z0 = q0 / (a.tx * a.ty) * T::Z;
+  };
+  auto table = [&](long long tile, int buf) {
+    long long b;
+    int z0, y0, x0;
+    origin(tile, b, z0, y0, x0);
+    tab[buf].make(a.c0, a.up0, a.c1, a.n, b, z0, y0, x0);
+  };
   auto stage = [&](long long tile, int buf) {
     const unsigned s0 = sm + 16u * (unsigned)(buf * STAGE);
-    const long long b = tile / tps;
-    const int q0 = (int)(tile - b * tps);
-    const int x0 = (q0 % a.tx) * T::X, y0 = (q0 / a.tx) % a.ty * T::Y, z0 = q0 / (a.tx * a.ty) * T::Z;
-    stage_halo<1, 2, G::S, G::P, G::PZ, NTHR>(s0, a.in0, a.c0, a.up0, a.in1, a.c1, 16 * blockIdx.x, a.n, b, z0, y0, x0);
+    long long b;
+    int z0, y0, x0;
+    origin(tile, b, z0, y0, x0);
+    stage_halo<1, 2, G::S, G::P, G::PZ, NTHR>(s0, tab[buf], a.in0, a.c0, a.in1, 16 * blockIdx.x);
     for (int e = threadIdx.x; e < 256 * 2 * CO; e += NTHR) {
       const int q = e / (2 * CO), c = e - q * (2 * CO);
       const int z = z0 + (q >> 6), y = y0 + ((q >> 3) & 7), x = x0 + (q & 7);
@@ -439,13 +485,20 @@ __global__ void __launch_bounds__(32 * kWgWarps) k_wgrad(WgradArgs a) {
   const bool bias = blockIdx.x == 0 && warp == 4;
   int buf = 0;
   long long tile = blockIdx.y;
-  if (tile < a.ntiles) stage(tile, 0);
+  table(tile, 0);
+  if (tile + gridDim.y < a.ntiles) table(tile + gridDim.y, 1);
+  __syncthreads();
+  pdl_launch();
+  pdl_wait();
+  stage(tile, 0);
   cp_commit();
   for (; tile < a.ntiles; tile += gridDim.y, buf ^= 1) {
     if (tile + gridDim.y < a.ntiles) stage(tile + gridDim.y, buf ^ 1);
     cp_commit();
     cp_wait<1>();
     __syncthreads();
+    // the table of the tile after the next (this buffer's was read above)
+    if (tile + 2 * (long long)gridDim.y < a.ntiles) table(tile + 2 * (long long)gridDim.y, buf);
     const unsigned s0 = sm + 16u * (unsigned)(buf * STAGE);
 #pragma unroll 2
     for (int q = 0; q < 16; ++q) {  // two rows of eight voxels each
@@ -519,7 +572,7 @@ __global__ void __launch_bounds__(32 * kRedWarps) k_grad_reduce(ReduceArgs a) {
   if (i < total) {
     const float* p = i < nw ? L.part + i : L.bpart + (i - nw);
     const size_t step = i < nw ? (size_t)nw : (size_t)L.coutp;
-#pragma unroll 4
+#pragma unroll 8
     for (int q = warp; q < L.shares; q += kRedWarps) s += p[q * step];
   }
   sh[warp][threadIdx.x & 31] = s;
@@ -650,25 +703,26 @@ __device__ __forceinline__ double sample_scale(const double* part, long long q, 
 template <typename T>
 __global__ void __launch_bounds__(256) k_pack(const T* b, const T* psi, long long n3, const double* part, double* scale,
                                               double out_scale, bf16* x0, float* tgt) {
-  __shared__ double sh;
+  __shared__ double sh[2];  // 1 / s, 1 / (s out_scale): one thread's divisions
   pdl_launch();
   pdl_wait();
   const long long s = blockIdx.y;
   if (threadIdx.x < 32) {
     const double sc = sample_scale(part, s, n3);
     if (threadIdx.x == 0) {
-      sh = sc;
+      sh[0] = sc > 0.0 ? 1.0 / sc : 0.0;
+      sh[1] = sh[0] / out_scale;
       if (blockIdx.x == 0) scale[s] = sc;
     }
   }
   __syncthreads();
-  const double inv = sh > 0.0 ? 1.0 / sh : 0.0;
+  const double inv = sh[0], invt = sh[1];
   for (long long v = blockIdx.x * 256LL + threadIdx.x; v < n3; v += gridDim.x * 256LL) {
     const long long i = s * n3 + v;
     uint4* o = reinterpret_cast<uint4*>(x0 + i * 16);
     o[0] = make_uint4(pack2((float)((double)b[i] * inv), 0.f), 0u, 0u, 0u);
     o[1] = make_uint4(0u, 0u, 0u, 0u);
-    if (tgt) tgt[i] = (float)((double)psi[i] * inv / out_scale);
+    if (tgt) tgt[i] = (float)((double)psi[i] * invt);
   }
 }
 // MSE over batch x n3 of y vs t; gy = 2 (y - t) / count in BF16
@@ -745,9 +799,10 @@ __global__ void __launch_bounds__(256) k_unpack(const float* y, long long n3, co
     psi[s * n3 + v] = (T)(sc * ((double)y[s * n3 + v] - m));
 }
 
-// master FP32 (flat) -> forward BF16 [tap][co_pad8][ci_pad16] and backward
-// BF16 [flipped tap][ci_pad16][co_pad8 -> padded to 16] weights, FP32 bias;
-// a grid row of blocks per layer
+// master FP32 (flat) -> forward BF16 [co / 16][tap][16][ci_pad16 + 8] and
+// backward BF16 [ci / 16][flipped tap][16][co_pad16 + 8] weights (the padding
+// stays zero), FP32 bias; the 1x1 head forward only, as [co_pad8][ci_pad16].
+// A grid row of blocks per layer.
 struct WeightLayer {
   bf16 *wf, *wb;
   float* bias;
@@ -766,9 +821,13 @@ __global__ void k_weights(WeightArgs a) {
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
     const int ci = i % cinp, co = (i / cinp) % coutp16, t = i / (cinp * coutp16);
     const float w = (co < L.cout && ci < L.cin) ? flat[((size_t)co * L.cin + ci) * ntap + t] : 0.f;
-    if (co < coutp) L.wf[((size_t)t * coutp + co) * cinp + ci] = __float2bfloat16(w);
+    if (ntap == 1) {
+      if (co < coutp) L.wf[(size_t)co * cinp + ci] = __float2bfloat16(w);
+      continue;
+    }
+    L.wf[(((size_t)(co >> 4) * ntap + t) * 16 + (co & 15)) * (cinp + 8) + ci] = __float2bfloat16(w);
     // backward data: out channel = ci, in channel = co, tap flipped
-    L.wb[((size_t)(ntap - 1 - t) * cinp + ci) * coutp16 + co] = __float2bfloat16(w);
+    L.wb[(((size_t)(ci >> 4) * ntap + ntap - 1 - t) * 16 + (ci & 15)) * (coutp16 + 8) + co] = __float2bfloat16(w);
   }
   if (blockIdx.x == 0)
     for (int co = threadIdx.x; co < coutp; co += blockDim.x)
@@ -870,8 +929,8 @@ size_t layout(les_unet* u, char* base, bool dry) {
   for (int l = 0; l < kNL; ++l) {
     const LayerDef& L = kLayers[l];
     const int nt = L.k * L.k * L.k, cinp = pad16(L.cin), cop = pad8(L.cout), cop16 = pad16(L.cout);
-    u->wf[l] = c.take<bf16>((size_t)nt * cop * cinp * 2);
-    u->wb[l] = c.take<bf16>((size_t)nt * cinp * cop16 * 2);
+    u->wf[l] = c.take<bf16>((size_t)nt * cop16 * (cinp + 8) * 2);
+    u->wb[l] = c.take<bf16>((size_t)nt * cinp * (cop16 + 8) * 2);
     u->bias[l] = c.take<float>((size_t)cop * 4);
     const size_t sh = (size_t)wgrad_shares(u, l, u->batch);
     u->wpart[l] = c.take<float>(sh * (l == L_HEAD ? 16 : (size_t)nt * L.cout * cinp) * 4);
@@ -953,7 +1012,7 @@ ConvChoice conv_kernel(int kc, int cfg, int nfb) {
     default: return {};
   }
 }
-constexpr size_t kConvSmemMax = 227 * 1024;
+constexpr size_t kConvSmemMax = 227 * 1024 - 4096;  // beside the tables
 
 // shared-memory limits of the kernels, once per network
 cudaError_t kernel_limits() {
@@ -977,15 +1036,13 @@ cudaError_t kernel_limits() {
 // tiles halve the weight and halo loads per voxel, small ones fill the chip on
 // the coarse levels.
 cudaError_t conv(les_unet* u, int n, int batch, ConvArgs a) {
-  const int kc = (a.c0 + a.c1) / 16;
-  a.cout = a.oc0 + a.oc1;
+  const int kc = (a.c0 + a.c1) / 16, cout = a.oc0 + a.oc1;
   a.n = n;
   static constexpr int order[4][2] = {{1, 4}, {1, 2}, {0, 4}, {0, 2}};
   int cfg = 0, nfb = 2;
   for (const auto& o : order) {
-    const size_t smem = conv_kernel(kc, o[0], o[1]).smem;
-    if (a.cout % (8 * o[1]) || smem > kConvSmemMax) continue;
-    if (tiles_of(o[0], n, batch) * (a.cout / (8 * o[1])) < u->nsm - u->nsm / 4) continue;
+    if (cout % (8 * o[1]) || conv_kernel(kc, o[0], o[1]).smem > kConvSmemMax) continue;
+    if (tiles_of(o[0], n, batch) * (cout / (8 * o[1])) < u->nsm - u->nsm / 4) continue;
     cfg = o[0], nfb = o[1];
     break;
   }
@@ -994,7 +1051,7 @@ cudaError_t conv(les_unet* u, int n, int batch, ConvArgs a) {
   a.tz = (n + 3) / 4;
   a.ty = a.tx = cfg ? (n + 7) / 8 : (n + 3) / 4;
   ProfScope ps(u->prof, KI_UNET_CONV, u->st);
-  return launch_pdl(c.k, dim3((unsigned)tiles_of(cfg, n, batch), (unsigned)(a.cout / (8 * nfb))), cfg ? 256 : 128, c.smem,
+  return launch_pdl(c.k, dim3((unsigned)tiles_of(cfg, n, batch), (unsigned)(cout / (8 * nfb))), cfg ? 256 : 128, c.smem,
                     u->st, a);
 }
 // tiles per sample of the last convolution (whose tiles sum y)
