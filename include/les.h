@@ -143,9 +143,8 @@ typedef struct les_config {
   double   sat_tol;          /* secant stop |theta_l* - theta_l| (K)        */
   int32_t  sat_maxit;
   int32_t  solver_path;      /* 0: one persistent cooperative launch per CG
-                                solve when eligible (compact operator, nx a
-                                multiple of 128 floats / 64 doubles, ny a
-                                multiple of the tile rows), else 1;
+                                solve when eligible (compact operator),
+                                else 1;
                                 1: one launch per CG phase               */
   int32_t  advection;        /* LES_ADV_QUICK (paper's default) |
                                 LES_ADV_WENO3 (its alternative, Sec. 2.4)  */
@@ -488,9 +487,9 @@ typedef struct les_tuning {
                                       memory when the grid fits there (see
                                       cg_resident), else variant 4 for
                                       FP32 grids of whole columns,
-                                      else variant 2 on tile-aligned grids,
-                                      else variant 3; 1 is not accepted;
-                                      2 the
+                                      else two streaming phases per
+                                      iteration on any grid; 1 is not
+                                      accepted; 2 the
                                       two-phase streaming CG (two barriers
                                       per iteration); 3 one pass over memory
                                       and one grid reduction per iteration,

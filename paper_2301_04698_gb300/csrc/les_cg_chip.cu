@@ -29,7 +29,7 @@
 // a five-step butterfly of four values in 16 warps alone costs 5000 cycles.
 // The four values are therefore reduced by a transposing butterfly (six
 // additions per warp instead of twenty), the plan weighs warps against planes
-// per thread, the FP64 stencil takes 7 operations, and x += alpha p is left
+// per thread, the FP64 stencil takes six operations, and x += alpha p is left
 // to the next sum's wait.
 //
 // Measured (GB300, us per iteration, 200-iteration solves; before: the
@@ -229,15 +229,18 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
   T rgh[NG] = {}, pgh[NG] = {};  // r and p at the ghost nodes
   // L_c p at plane j of the run.  FP32: second differences formed before
   // scaling, as in the other CG kernels.  FP64, where each operation counts:
-  // the six neighbours scaled, then the centre -- 7 operations instead of 9.
+  // q' with L_c p = -c0 q', c0 the centre coefficient -- six operations instead
+  // of nine.  The recurrences of r and p do not see the factor; the update of x
+  // takes it up (its alpha is -1 / c0 times theirs).
+  constexpr bool kScaled = sizeof(T) == 8;
   const T c0 = T(2) * (cx + cy + cz);
+  const T ax = cx / c0, ay = cy / c0, az = cz / c0, mc0 = T(-1) / c0;
   auto stencil = [&](int j) -> T {
     const T* pj = P + pown + j * SZ;
     const T d = j > 0 ? p[j > 0 ? j - 1 : 0] : pj[ozm];
     const T u = (j + 1 < ZP && j + 1 < nzp) ? p[j + 1 < ZP ? j + 1 : ZP - 1] : pj[ozp];
-    if constexpr (sizeof(T) == 8) {
-      const T s = fma(cz, d + u, fma(cy, pj[oym] + pj[oyp], cx * (pj[oxm] + pj[oxp])));
-      return fma(-c0, p[j], s);
+    if constexpr (kScaled) {
+      return fma(-az, d + u, fma(-ay, pj[oym] + pj[oyp], fma(-ax, pj[oxm] + pj[oxp], p[j])));
     } else {
       const T c2 = T(2) * p[j];
       return (pj[oxm] + pj[oxp] - c2) * cx + (pj[oym] + pj[oyp] - c2) * cy + (d + u - c2) * cz;
@@ -266,7 +269,7 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
 
   GridSync gs{f.bar, f.partials, f.spin_cycles, f.expected, 0u};
   __shared__ struct {
-    T mean, ta, tb;
+    T mean, ta, tb, tx;  // alpha and beta of r and p, alpha of x
     int status, restart;
     double bb, rel;  // |b - mean|^2 and the relative residual of x0
   } sc;
@@ -312,7 +315,7 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
     for (int j = 0; j < ZP; ++j)
       if (j < nzp) {
         const T bm = r[j] - mean;
-        r[j] = bm - stencil(j);
+        r[j] = kScaled ? fma(c0, stencil(j), bm) : bm - stencil(j);
         if (is_face(j)) __stcg(f.rg + gown + j * gpl, r[j]);
         a2[0].add(r[j] * r[j]);
         a2[1].add(bm * bm);
@@ -367,7 +370,7 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
   acc_from(f.tol * f.tol * sc.bb, rr_stop);
   acc_from(rr, rr_last);
   int iter = 0;
-  T ta = T(0), tb = T(0);
+  T ta = T(0), tb = T(0), tx = T(0);
   if (!status) {
     // p_0 = r_0, with r_0 at the ghost nodes from the published faces
 #pragma unroll
@@ -454,7 +457,7 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
         if constexpr (kDefer) {
           if (iter > 0) {
 #pragma unroll
-            for (int j = 0; j < ZP; ++j) xr[XS ? 0 : j] += ta * po[kDefer ? j : 0];
+            for (int j = 0; j < ZP; ++j) xr[XS ? 0 : j] += tx * po[kDefer ? j : 0];
           }
         }
         asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory");
@@ -503,6 +506,7 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
             else if (!chip_scalars(t4, al, be)) st = 3;
             sc.ta = al;
             sc.tb = be;
+            sc.tx = kScaled ? al * mc0 : al;
           }
           sc.status = st;
         }
@@ -515,11 +519,12 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
       if (status) break;
       ta = sc.ta;
       tb = sc.tb;
+      tx = sc.tx;
       rr_own = T(0);
 #pragma unroll
       for (int j = 0; j < ZP; ++j)
         if (j < nzp) {
-          if (!kDefer || warp == 0) set_x(j, get_x(j) + ta * p[j]);
+          if (!kDefer || warp == 0) set_x(j, get_x(j) + tx * p[j]);
           else po[kDefer ? j : 0] = p[j];
           r[j] -= ta * q[j];
           rr_own += r[j] * r[j];
@@ -628,9 +633,9 @@ bool make_chip_plan(const Grid<T>& g, int nsm, size_t smem_max, int max_blocks, 
         // of its planes and ghosts; an x face is a strided access
         const int wps = (nw + 3) / 4, gt = (gh + 32 * nw - 1) / (32 * nw);
         double c = (xs ? 75.0 : 60.0) * wps * zp;
-        // FP64: a warp instruction every 64 cycles of a scheduler -- 14 per
+        // FP64: a warp instruction every 64 cycles of a scheduler -- 13 per
         // node, six of the reduction, two per ghost
-        if (sizeof(T) == 8) c = 86.0 * (wps * (14.0 * zp + 6.0) + 2.0 * gh / 128.0);
+        if (sizeof(T) == 8) c = 86.0 * (wps * (13.0 * zp + 6.0) + 2.0 * gh / 128.0);
         c += 200.0 * zp + 150.0 * gt + 3.0 * xg;
         if (!found || c < cost) {
           found = true;

@@ -103,8 +103,8 @@ struct FusedCfg {
   int missing = 0;                      // test hook: arrivals that never come
   int stencil_path = 0;                 // 0 column marches where eligible (else rolling), 1 rolling z-march
   int variant = 0;                      // 0 standard iterates (resident, else FP32 columns, else
-                                        // two-phase streaming when tile-aligned, else one-pass),
-                                        // 2 two-phase streaming, 3 one-pass one-reduction, 4 columns
+                                        // two-phase streaming on any grid), 2 two-phase streaming
+                                        // in tuned tiles, 3 one-pass one-reduction, 4 columns
   int resident = 0;                     // 0 on-chip CG when the grid fits (vectors in registers), 1 never,
                                         // 2 on chip with every vector in shared memory
 };
@@ -314,6 +314,11 @@ bool fused_cg_eligible(const Grid<T>& g, int op, int solver, int ty);
 template <typename T>
 int poisson_solve_fused(const SolverArgs<T>& a, const FusedCfg& fc, const T* b, T* x, double tol, int maxit,
                         int* iters, double* rel, std::string* err);
+// Persistent two-phase streaming CG (les_cg_stream.cu): any grid, compact
+// operator.
+template <typename T>
+int poisson_solve_stream(const SolverArgs<T>& a, const FusedCfg& fc, const T* b, T* x, double tol, int maxit,
+                         int* iters, double* rel, std::string* err);
 // Persistent one-reduction CG, one pass per iteration (les_cg_roll.cu): any
 // grid, compact operator.
 template <typename T>

@@ -345,16 +345,13 @@ class SmHold {
 template <typename T>
 int poisson_solve(const SolverArgs<T>& a, const T* b, T* x, double tol, int maxit, int* iters, double* rel,
                   std::string* err) {
-  // persistent CG: on chip when the grid fits there (p, r and q in
-  // registers on FP32 grids 128 nodes wide, else every vector in shared
-  // memory); else the
-  // one-pass kernel with 64 x 16 columns (variant 4, and variant 0 for FP32
-  // grids of whole columns), the two-phase streaming kernel on tile-aligned
-  // grids (variant 0 or 2) or the one-pass kernel (variant 0 on other grids,
-  // or variant 3).  Persistent solves of
-  // different handles (ensemble members stepped from several host threads)
-  // share the SMs through the budget above: capped ones run together, an
-  // uncapped one alone.
+  // persistent CG: on chip when the grid fits there; else, for FP32 grids of
+  // whole 64 x 16 or 32 x 32 columns, the one-pass kernel with register windows
+  // (variant 4); else the two-phase streaming kernel for any grid.  Variant 2 is
+  // the two-phase kernel with tuned tiles on tile-aligned grids, 3 the one-pass
+  // kernel for any grid.  Persistent solves of different handles (ensemble
+  // members stepped from several host threads) share the SMs through the budget
+  // above: capped ones run together, an uncapped one alone.
   const bool cg_c = a.op == LES_OP_COMPACT && a.solver == LES_SOLVER_CG;
   std::unique_ptr<SmHold> hold;
   if (a.bar && a.fused) {
@@ -370,14 +367,18 @@ int poisson_solve(const SolverArgs<T>& a, const T* b, T* x, double tol, int maxi
     const int rc = poisson_solve_resident<T>(a, *a.fused, b, x, tol, maxit, iters, rel, err, &used);
     if (used || rc != LES_OK) return rc;
   }
-  // FP32 grids of whole 64 x 16 columns: the one-pass kernel with register
-  // windows is the default (1.5x the two-phase kernel on 1536^2 x 256)
+  // FP32 grids of whole columns: the one-pass kernel streams 6 fields per
+  // iteration against 9 (512 x 512 x 64: 117 us against 175)
   if (a.bar && cg_c && (var == 4 || (var == 0 && sizeof(T) == 4)) && wave_cg_eligible(a.g.nx, a.g.ny, a.g.nz))
     return poisson_solve_wave<T>(a, *a.fused, b, x, tol, maxit, iters, rel, err);
-  if (a.bar && cg_c && (var == 3 || var == 4 || (var == 0 && !tiled)))
-    return poisson_solve_roll<T>(a, *a.fused, b, x, tol, maxit, iters, rel, err);
-  if (a.bar && tiled && (var == 0 || var == 2))
-    return poisson_solve_fused<T>(a, *a.fused, b, x, tol, maxit, iters, rel, err);
+  if (a.bar && cg_c && (var == 3 || var == 4)) return poisson_solve_roll<T>(a, *a.fused, b, x, tol, maxit, iters, rel, err);
+  // every other grid: two phases, in FP64 because arithmetic bounds it (256 x
+  // 256 x 128: 198 us per iteration, 333 with the tile-aligned two-phase kernel,
+  // 612 and 629 with the one-pass kernels), in FP32 because tiles of any width
+  // keep its lanes full (1000 x 1000 x 100: 804 us against 1505 one-pass, 640 x
+  // 500 x 100: 281 against 403 tile-aligned)
+  if (a.bar && cg_c && var == 0) return poisson_solve_stream<T>(a, *a.fused, b, x, tol, maxit, iters, rel, err);
+  if (a.bar && tiled && var == 2) return poisson_solve_fused<T>(a, *a.fused, b, x, tol, maxit, iters, rel, err);
   auto fail = [&](cudaError_t e, const char* where) {
     if (err) *err = std::string(where) + ": " + cudaGetErrorString(e);
     return LES_ERR_CUDA;

@@ -71,8 +71,8 @@ def test_chip_cg_matches_oracle(les_mod, precision, shape, max_blocks, walls):
         x = x0.clone()
         rc, it, res = sim.poisson_solve(bt, x, tol, 20000)
         assert rc == 0 and res <= tol
-        fits = stream == 0 and shape != (33, 31, 29)
-        assert launches(sim) == {"cg_resident" if fits else "cg_roll": 1}
+        chip = "cg_fused" if shape == (33, 31, 29) else "cg_resident"
+        assert launches(sim) == {"cg_roll" if stream else chip: 1}
         xn = x.cpu().double().numpy()
         assert abs(xn.mean()) < (1e-14 if precision == 64 else 1e-6) * np.abs(xn).max()
         assert rel(xn, xr) < (1e-8 if precision == 64 else 5e-4), stream
