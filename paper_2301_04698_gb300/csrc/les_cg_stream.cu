@@ -447,14 +447,18 @@ using Tile64 = StreamTile<64, 16>;
 using Tile32 = StreamTile<32, 32>;
 using Tile32s = StreamTile<32, 16>;
 
-// work of a tile plan in node slots: the padded tiles, their rings (a ring
-// node forms p again: a tenth of a node's work) and, per run of planes, one
-// more plane of p and its loads
 struct StreamPlan {
   int shape = 0, ntx = 0, nty = 0, nchunk = 1;
   long long units = 0;
 };
-StreamPlan make_stream_plan(int nx, int ny, int nz, long long G) {
+// The tile shape and the runs of planes per tile with the least work of the
+// busiest block, in node slots (every lane counts, with a node or without).  A
+// run costs planes beyond its own -- one more of p and the fill of its loads --
+// and a plane costs slots beyond its nodes: its ring and, where arithmetic does
+// not hide them (FP32), the barrier and the loop.  Fitted to timed plans: FP64
+// 200 x 180 x 90 prefers 32 x 16 tiles (100 us per iteration against 108 with
+// 64 x 16), FP32 470 x 239 x 58 64 x 16 ones (56 us against 70).
+StreamPlan make_stream_plan(int nx, int ny, int nz, long long G, bool fp64) {
   static constexpr int shapes[3][2] = {{64, 16}, {32, 32}, {32, 16}};
   StreamPlan best;
   double cost = 0;
@@ -468,9 +472,8 @@ StreamPlan make_stream_plan(int nx, int ny, int nz, long long G) {
       const long long nchunk = std::max<long long>(1, std::min<long long>(nz, G * turns / tiles));
       const long long units = tiles * nchunk, per = (units + G - 1) / G;
       const double zrun = (double)((nz + nchunk - 1) / nchunk);
-      // FP64 slots of a unit's plane: warps x nodes per thread, whether or not
-      // every lane has a node
-      const double c = (double)per * (zrun + 0.7) * (wx * wy + 0.25 * 2 * (wx + wy) + 24.0);
+      const double c = fp64 ? (double)per * (zrun + 0.7) * (wx * wy + 0.5 * (wx + wy) + 24.0)
+                            : (double)per * (zrun + 2.0) * (wx * wy + (wx + wy) + (wx == 64 ? 200.0 : 240.0));
       if (best.units == 0 || c < cost) {
         cost = c;
         best = {q, ntx, nty, (int)nchunk, units};
@@ -503,7 +506,8 @@ int poisson_solve_stream(const SolverArgs<T>& a, const FusedCfg& fc, const T* b,
   StreamPlan pl;
   const void* kern = nullptr;
   for (int pass = 0; pass < 2; ++pass) {  // the plan depends on the resident blocks, they on the shape
-    pl = make_stream_plan(a.g.nx, a.g.ny, a.g.nz, std::min<long long>((long long)per_sm * nsm, fc.max_blocks));
+    pl = make_stream_plan(a.g.nx, a.g.ny, a.g.nz, std::min<long long>((long long)per_sm * nsm, fc.max_blocks),
+                          sizeof(T) == 8);
     kern = stream_kernel<T>(pl.shape);
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kStreamThreads, 0)) != cudaSuccess) {
       if (err) *err = std::string("streaming CG occupancy: ") + cudaGetErrorString(e);
