@@ -27,22 +27,11 @@
 #include <algorithm>
 #include <string>
 
-#include "les_gridsync.cuh"
 #include "les_internal.h"
+#include "les_stream.cuh"
 
 namespace les {
 namespace {
-
-constexpr int kStreamThreads = 256;
-
-// tile shapes: WX x WY columns, NO per thread (x = lane + 32 (m mod NWX),
-// y = warp + 8 (m / NWX)), planes of (WY + 2) rows of SP elements
-template <int WX_, int WY_>
-struct StreamTile {
-  static constexpr int WX = WX_, WY = WY_, NWX = WX / 32, NO = WX * WY / kStreamThreads;
-  static constexpr int SP = WX + 2, SN = SP * (WY + 2);
-  static_assert(2 * (WX + WY) <= kStreamThreads && 8 * (NO / NWX) == WY, "one ring node per thread");
-};
 
 template <typename T>
 struct StreamArgs {
@@ -64,73 +53,6 @@ struct StreamArgs {
   unsigned expected;
   int guard;
 };
-
-__device__ __forceinline__ void stream_part(int n, int parts, int i, int& first, int& len) {
-  const int base = n / parts, rem = n - base * parts;
-  len = base + (i < rem ? 1 : 0);
-  first = i * base + min(i, rem);
-}
-__device__ __forceinline__ int stream_wrap(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
-__device__ __forceinline__ int stream_z(int k, int nz, int walls) {
-  if (walls) return k < 0 ? -1 - k : (k >= nz ? 2 * nz - 1 - k : k);
-  return k < 0 ? k + nz : (k >= nz ? k - nz : k);
-}
-
-// Long per-thread sums: FP32 within a run of 16 additions, compensated across
-template <typename T>
-struct StreamSum;
-template <>
-struct StreamSum<float> {
-  F2 s{0.f, 0.f};
-  float run = 0.f;
-  int cnt = 0;
-  __device__ __forceinline__ void add(float v) { run += v; }
-  __device__ __forceinline__ void tick() {
-    if ((++cnt & 3) == 0) flush();
-  }
-  __device__ __forceinline__ void flush() {
-    f2_acc(s, run);
-    run = 0.f;
-  }
-  __device__ __forceinline__ F2 acc() {
-    flush();
-    return s;
-  }
-};
-template <>
-struct StreamSum<double> {
-  double s = 0.0;
-  __device__ __forceinline__ void add(double v) { s += v; }
-  __device__ __forceinline__ void tick() {}
-  __device__ __forceinline__ double acc() { return s; }
-};
-template <int NV, typename T>
-__device__ __forceinline__ bool stream_sum(StreamSum<T> (&d)[NV], GridSync& gs, double (&tot)[NV]) {
-  decltype(d[0].acc()) v[NV];
-#pragma unroll
-  for (int q = 0; q < NV; ++q) v[q] = d[q].acc();
-  return grid_sum_t0<NV>(v, gs, tot);
-}
-
-// nodes handled together in the streaming sweeps: 16 bytes
-template <typename T>
-struct StreamVec {
-  static constexpr int N = 16 / (int)sizeof(T);
-  T v[N];
-};
-template <typename T>
-__device__ __forceinline__ StreamVec<T> svld(const T* p) {
-  const uint4 u = __ldcg(reinterpret_cast<const uint4*>(p));
-  StreamVec<T> r;
-  memcpy(&r, &u, 16);
-  return r;
-}
-template <typename T>
-__device__ __forceinline__ void svst(T* p, const StreamVec<T>& r) {
-  uint4 u;
-  memcpy(&u, &r, 16);
-  __stcg(reinterpret_cast<uint4*>(p), u);
-}
 
 template <typename T, typename S>
 __global__ void __launch_bounds__(kStreamThreads, 2) k_cg_stream(StreamArgs<T> f) {
@@ -258,18 +180,8 @@ __global__ void __launch_bounds__(kStreamThreads, 2) k_cg_stream(StreamArgs<T> f
         go[m] = ex < w && ey < h ? (y0 + ey) * f.nx + x0 + ex : -1;
       }
       const int eo = (warp + 1) * SP + lane + 1;  // of node 0 in sm; node m: + 8 (m / NWX) SP + 32 (m mod NWX)
-      int gr = -1, er = 0;
-      {
-        int ex = 0, ey = 0;
-        bool ok = true;
-        if (tid < 2 * w) ex = tid < w ? tid : tid - w, ey = tid < w ? -1 : h;
-        else if (tid < 2 * (w + h)) ex = tid - 2 * w < h ? -1 : w, ey = (tid - 2 * w) - (tid - 2 * w < h ? 0 : h);
-        else ok = false;
-        if (ok) {
-          gr = stream_wrap(y0 + ey, f.ny) * f.nx + stream_wrap(x0 + ex, f.nx);
-          er = (ey + 1) * SP + ex + 1;
-        }
-      }
+      int gr, er;
+      stream_ring<S>(tid, x0, y0, w, h, f.nx, f.ny, gr, er);
       T rv[NO], ov[NO], xv[NO], rh = T(0), oh = T(0);  // r, p_{i-1}, x of the plane in flight; its ring
       auto load = [&](int kk, bool inside) {
         const size_t base = (size_t)stream_z(kk, f.nz, f.walls) * plane;
@@ -441,46 +353,6 @@ __global__ void __launch_bounds__(kStreamThreads, 2) k_cg_stream(StreamArgs<T> f
     f.ctl->rel = rel;
     f.ctl->done = status;
   }
-}
-
-using Tile64 = StreamTile<64, 16>;
-using Tile32 = StreamTile<32, 32>;
-using Tile32s = StreamTile<32, 16>;
-
-struct StreamPlan {
-  int shape = 0, ntx = 0, nty = 0, nchunk = 1;
-  long long units = 0;
-};
-// The tile shape and the runs of planes per tile with the least work of the
-// busiest block, in node slots (every lane counts, with a node or without).  A
-// run costs planes beyond its own -- one more of p and the fill of its loads --
-// and a plane costs slots beyond its nodes: its ring and, where arithmetic does
-// not hide them (FP32), the barrier and the loop.  Fitted to timed plans: FP64
-// 200 x 180 x 90 prefers 32 x 16 tiles (100 us per iteration against 108 with
-// 64 x 16), FP32 470 x 239 x 58 64 x 16 ones (56 us against 70).
-StreamPlan make_stream_plan(int nx, int ny, int nz, long long G, bool fp64) {
-  static constexpr int shapes[3][2] = {{64, 16}, {32, 32}, {32, 16}};
-  StreamPlan best;
-  double cost = 0;
-  for (int q = 0; q < 3; ++q) {
-    const int wx = shapes[q][0], wy = shapes[q][1];
-    const int ntx = (nx + wx - 1) / wx, nty = (ny + wy - 1) / wy;
-    const long long tiles = (long long)ntx * nty;
-    // the units are dealt to the blocks in turns: for each number of turns as
-    // many runs of planes per tile as fill them
-    for (int turns = 1; turns <= 8; ++turns) {
-      const long long nchunk = std::max<long long>(1, std::min<long long>(nz, G * turns / tiles));
-      const long long units = tiles * nchunk, per = (units + G - 1) / G;
-      const double zrun = (double)((nz + nchunk - 1) / nchunk);
-      const double c = fp64 ? (double)per * (zrun + 0.7) * (wx * wy + 0.5 * (wx + wy) + 24.0)
-                            : (double)per * (zrun + 2.0) * (wx * wy + (wx + wy) + (wx == 64 ? 200.0 : 240.0));
-      if (best.units == 0 || c < cost) {
-        cost = c;
-        best = {q, ntx, nty, (int)nchunk, units};
-      }
-    }
-  }
-  return best;
 }
 
 template <typename T>

@@ -319,6 +319,11 @@ int poisson_solve_fused(const SolverArgs<T>& a, const FusedCfg& fc, const T* b, 
 template <typename T>
 int poisson_solve_stream(const SolverArgs<T>& a, const FusedCfg& fc, const T* b, T* x, double tol, int maxit,
                          int* iters, double* rel, std::string* err);
+// Weighted Jacobi in one persistent launch (les_jacobi.cu): any grid, compact
+// operator.
+template <typename T>
+int poisson_solve_jacobi(const SolverArgs<T>& a, const FusedCfg& fc, const T* b, T* x, double tol, int maxit,
+                         int* iters, double* rel, std::string* err);
 // Persistent one-reduction CG, one pass per iteration (les_cg_roll.cu): any
 // grid, compact operator.
 template <typename T>

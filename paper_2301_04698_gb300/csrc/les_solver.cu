@@ -9,6 +9,8 @@
 // beta, the residual and the stop decision stay on the device, so iterations
 // are launched back to back and the host only polls the control block between
 // batches.  Weighted Jacobi (the paper's solver) uses one kernel per sweep.
+// These launches per phase serve solver_path 1, the consistent (wide) operator
+// and the allocation-free solve; otherwise a solve is one persistent launch.
 #include <algorithm>
 #include <memory>
 #include <string>
@@ -379,6 +381,8 @@ int poisson_solve(const SolverArgs<T>& a, const T* b, T* x, double tol, int maxi
   // 500 x 100: 281 against 403 tile-aligned)
   if (a.bar && cg_c && var == 0) return poisson_solve_stream<T>(a, *a.fused, b, x, tol, maxit, iters, rel, err);
   if (a.bar && tiled && var == 2) return poisson_solve_fused<T>(a, *a.fused, b, x, tol, maxit, iters, rel, err);
+  if (a.bar && a.fused && a.solver == LES_SOLVER_JACOBI)
+    return poisson_solve_jacobi<T>(a, *a.fused, b, x, tol, maxit, iters, rel, err);
   auto fail = [&](cudaError_t e, const char* where) {
     if (err) *err = std::string(where) + ": " + cudaGetErrorString(e);
     return LES_ERR_CUDA;
