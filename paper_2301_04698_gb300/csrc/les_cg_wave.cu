@@ -26,15 +26,18 @@
 // ring slot, for a column at a periodic edge (whose wrap is not a box) as
 // per-thread cp.async copies of 16-byte chunks and node pairs.  Per plane
 // step, after one block barrier:
-//   A  p(f) = r(f) + beta p_old(f) at every position
+//   A  p(f) = r(f) + beta p_old(f) at every position; every other pass, x +=
+//      alpha_{i-1} p_old + alpha_i p at the owned ones
 //   B  q(f-1) = L_c p, r'(f-1) = r(f-1) - alpha q(f-1) within the halo of one
 //   C  w(f-2) = L_c r' at the owned positions
-//   D  x += alpha p, and p, r' of plane f-2 stored
+//   D  p, r' of plane f-2 stored
 // r and p are double-buffered by iteration parity (the pass reads the
 // neighbours' r_i while writing r_{i+1}); the grid sum is the barrier
-// between passes.  Per iteration each node is read three times (r_i,
-// p_{i-1}, x) and written three times (p_i, r_{i+1}, x); the halo re-reads a
-// third of r_i and p_{i-1}, mostly from L2.
+// between passes.  Per iteration each node's r_i and p_{i-1} are read and p_i and
+// r_{i+1} written, and x is read and written every other one (an update of x
+// needs nothing of q: both take place where p_{i-1} and p_i are at hand, in one
+// pass out of two, which saves 4 of 24 bytes); the halo re-reads a third of r_i
+// and p_{i-1}, mostly from L2.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -53,8 +56,7 @@ namespace {
 
 constexpr int WH = 2;   // halo of the staged planes
 constexpr int NT = 256;  // threads per block
-constexpr int D = 4;     // r_i / p_{i-1} ring: planes f .. f+3
-constexpr int DX = 6;    // x ring: planes f-2 .. f+3
+constexpr int D = 4;     // r_i / p_{i-1} / x rings: planes f .. f+3
 
 // A column shape: WX x WY owned nodes (64 x 16 or 32 x 32).  Staged planes
 // keep rows of SP elements with the owned columns from element 4 on (16-byte
@@ -88,7 +90,7 @@ struct Copies {
 
 template <typename T, typename C>
 size_t wave_smem() {
-  return ((size_t)(2 * D + 4) * C::SN + (size_t)DX * C::WX * C::WY) * sizeof(T);
+  return ((size_t)(2 * D + 4) * C::SN + (size_t)D * C::WX * C::WY) * sizeof(T);
 }
 
 template <typename T>
@@ -202,7 +204,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_cg_wave(const __
   T* RINGP = RINGR + D * SN;               // [D][SN] p_{i-1} as copied
   T* PP = RINGP + D * SN;                  // [2][SN] p of a plane, by plane parity
   T* RP = PP + 2 * SN;                     // [2][SN] r' of a plane, by plane parity
-  T* RINGX = RP + 2 * SN;                  // [DX][WY][WX] x of the owned nodes
+  T* RINGX = RP + 2 * SN;                  // [D][WY][WX] x of the owned nodes
   // one barrier per ring slot: the TMA copies of a plane (r_i, p_{i-1}, x)
   // complete on it; bit s of phase is the parity this thread waits for next
   __shared__ __align__(8) uint64_t bars[D];
@@ -391,9 +393,14 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_cg_wave(const __
 
   // ---- iterations ----------------------------------------------------------------
   int iter = 0;
+  T ta = T(0);  // alpha of the last pass
   while (!status) {
-    const T ta = sc.ta, tb = sc.tb;
+    const T tp = ta;  // alpha_{i-1}
+    ta = sc.ta;
+    const T tb = sc.tb;
     const bool first = iter == 0;
+    // x takes two updates every other pass: p_{i-1} is read anyway
+    const bool upd = iter & 1;
     const T* ri = f.r[iter & 1];
     T* ro = f.r[(iter + 1) & 1];
     const T* pold = f.p[(iter + 1) & 1];  // p_{i-1}
@@ -486,8 +493,8 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_cg_wave(const __
         const int slot = (kk + 2 * D) % D;
         T* rr_ = RINGR + slot * SN;
         T* pp_ = RINGP + slot * SN;
-        T* xx_ = RINGX + ((kk + 2 * DX) % DX) * (WX * WY);
-        const bool xrun = kk >= k0 && kk < k1;
+        T* xx_ = RINGX + slot * (WX * WY);
+        const bool xrun = upd && kk >= k0 && kk < k1;
         if (tma) {
           if (tid == 0) {
             const unsigned bytes = (unsigned)((first ? 1 : 2) * SN * sizeof(T) + (xrun ? WX * WY * sizeof(T) : 0));
@@ -548,6 +555,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_cg_wave(const __
         fetch(fp + D - 1);
         const T* rr_ = RINGR + ((fp + 2 * D) % D) * SN;
         const T* pp_ = RINGP + ((fp + 2 * D) % D) * SN;
+        const T* xx_ = RINGX + ((fp + 2 * D) % D) * (WX * WY);
         T* pnew = PP + (fp & 1) * SN;
         // A: p(fp) = r(fp) + beta p_old(fp)
 #pragma unroll
@@ -559,6 +567,9 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_cg_wave(const __
           pw2[m] = pv;
           ra1[m] = rv;
           pnew[e] = pv;
+          if (m < NO && upd && fp >= k0 && fp < k1)
+            __stcg(f.x + (size_t)fp * plane + go0 + (NWARP * (m / NWX)) * f.nx + 32 * (m % NWX),
+                   xx_[((tid >> 5) + NWARP * (m / NWX)) * WX + (tid & 31) + 32 * (m % NWX)] + tp * pp_[e] + ta * pv);
         }
         // B: q(fp-1), r'(fp-1) within the halo of one (needs p(fp-2))
         if (fp >= k0) {
@@ -585,7 +596,6 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_cg_wave(const __
         if (fp >= k0 + 2) {
           const int k = fp - 2;
           const T* rc = RP + (k & 1) * SN;
-          const T* xx_ = RINGX + ((k + 2 * DX) % DX) * (WX * WY);
           const size_t base = (size_t)k * plane;
 #pragma unroll
           for (int m = 0; m < NO; ++m) {
@@ -596,7 +606,6 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_cg_wave(const __
             s[0].add(rw1[m] * rw1[m]);
             s[1].add(rw1[m] * w);
             const size_t g = base + go0 + (NWARP * (m / NWX)) * f.nx + 32 * (m % NWX);
-            __stcg(f.x + g, xx_[((tid >> 5) + NWARP * (m / NWX)) * WX + (tid & 31) + 32 * (m % NWX)] + ta * pw0[m]);
             __stcg(pw + g, pw0[m]);
             __stcg(ro + g, rw1[m]);
           }
@@ -651,10 +660,18 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_cg_wave(const __
 
   // ---- zero-mean gauge (or zero for a zero right side) ------------------------
   if (status != 5) {
+    const bool pend = iter & 1;  // the last pass left alpha p to the next
+    const T* pl = f.p[(iter + 1) & 1];
     WaveSum<T> s[1];
     int cnt = 0;
     for (long long c = gtid; c < nch; c += gstride) {
-      const Ch xq = ldch(f.x + (size_t)c * VC);
+      Ch xq = ldch(f.x + (size_t)c * VC);
+      if (pend) {
+        const Ch pq2 = ldch(pl + (size_t)c * VC);
+#pragma unroll
+        for (int q = 0; q < VC; ++q) xq.e[q] += ta * pq2.e[q];
+        stch(f.x + (size_t)c * VC, xq);
+      }
 #pragma unroll
       for (int q = 0; q < VC; ++q) s[0].add(xq.e[q]);
       if ((++cnt & 3) == 0) s[0].flush();
@@ -824,8 +841,9 @@ int solve_wave(const SolverArgs<T>& a, const FusedCfg& fc, const T* b, T* x, dou
   if (iters) *iters = c.iter;
   if (rel) *rel = c.rel;
   // algorithmic traffic of the solve (kCgIterFields per iteration; this
-  // kernel streams 6 per iteration plus a third of r_i and p_{i-1} again for
-  // the halo, and one set-up sweep for alpha_0)
+  // kernel streams 5 per iteration, x being read and written every other one,
+  // plus a third of r_i and p_{i-1} again for the halo, and one set-up sweep
+  // for alpha_0)
   if (a.prof) a.prof->bytes[KI_CG_WAVE] += (kCgSetupFields + 1.0 + kCgIterFields * c.iter) * (double)f.n * sizeof(T);
   switch (c.done) {
     case 1:
