@@ -467,7 +467,9 @@ int les_ensemble_step(les_handle *const *hs, int32_t m, int32_t nsteps, les_step
  * cg_resident = 0 or 2 the standard CG solve first tries a decomposition of
  * the grid into one brick per thread block, at most one block per SM: with
  * cg_resident = 0 bricks of any extents with p, r and q in registers (up to
- * 24 FP32 or 12 FP64 nodes per thread), then, and with cg_resident = 2 alone,
+ * 24 FP32 or 12 FP64 nodes per thread), or in FP32 of up to 32 x 16 x 64
+ * nodes with p in shared memory and r in registers, then, and with
+ * cg_resident = 2 alone,
  * bricks whose x extent (32, 64 or 128) divides nx and whose y extent divides
  * ny, with x, r, p and q in the per-block shared memory; the blocks then
  * exchange only brick faces through global memory, and cg_tile_rows and

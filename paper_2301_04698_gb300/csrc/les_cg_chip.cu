@@ -45,81 +45,10 @@
 #include <algorithm>
 #include <string>
 
-#include "les_gridsync.cuh"
-#include "les_internal.h"
+#include "les_chip.cuh"
 
 namespace les {
 namespace {
-
-constexpr int kChipThreads = 512;
-constexpr int kChipWarps = kChipThreads / 32;
-constexpr int kChipSpread = 8;      // arrival counters and copies of the partials per sum
-constexpr int kChipLine = 32;       // counters 128 bytes apart
-constexpr int kChipGhosts = 4;      // ghost nodes per thread in registers
-static_assert(kChipSpread * 4 == 32, "one lane of warp 0 per (copy, value) of the partials");
-
-template <typename T>
-struct ChipArgs {
-  int nx, ny, nz, walls;
-  T cx, cy, cz;        // 1/dx^2, 1/dy^2, 1/dz^2
-  int px, py, pz, zs;  // bricks along x, y, z; runs of planes per brick
-  int smem_p, smem_g;  // shared memory of P and (XS) of one ghost array, in elements (even)
-  long long n;
-  const T* b;
-  T* x;
-  T* rg;               // published faces of the first residual
-  T* qg0;              // published faces of q, even iterations
-  T* qg1;              // ... odd iterations
-  double* partials;    // two slots of kSumSlot words per block (the set-up and gauge sums)
-  unsigned* counters;  // kChipSpread arrival counters of the iterations' sums, kChipLine apart, zeroed
-  void* spread;        // [2 slots][kChipSpread copies][4 values][gridDim.x] partials of those sums
-  unsigned missing;    // test hook: arrivals on counter 0 that never come
-  FusedBar* bar;
-  SolverCtl* ctl;
-  double tol;
-  int maxit;
-  long long spin_cycles;
-  unsigned expected;
-  int guard;
-};
-
-// part i of n nodes in `parts` parts whose sizes differ by at most one
-__device__ __forceinline__ void chip_part(int n, int parts, int i, int& first, int& len) {
-  const int base = n / parts, rem = n - base * parts;
-  len = base + (i < rem ? 1 : 0);
-  first = i * base + min(i, rem);
-}
-__device__ __forceinline__ int chip_wrap(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
-__device__ __forceinline__ F2 acc_of(float v) { return F2{v, 0.f}; }
-__device__ __forceinline__ double acc_of(double v) { return v; }
-__device__ __forceinline__ F2 acc_xor(F2 a, int o) {
-  return F2{__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
-}
-__device__ __forceinline__ double acc_xor(double a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
-__device__ __forceinline__ F2 acc_from_lane(F2 a, int l) {
-  return F2{__shfl_sync(0xffffffffu, a.hi, l), __shfl_sync(0xffffffffu, a.lo, l)};
-}
-__device__ __forceinline__ double acc_from_lane(double a, int l) { return __shfl_sync(0xffffffffu, a, l); }
-
-// alpha and beta from the totals; false on a zero or non-finite p.q or r.r.
-// An FP32 solve takes them in FP32 from the high parts of the totals.
-__device__ __forceinline__ bool chip_scalars(const F2 (&t)[4], float& ta, float& tb) {
-  const float pq = t[0].hi, r2 = t[1].hi, rq = t[2].hi, q2 = t[3].hi;
-  if (!(pq != 0.f) || !isfinite(pq) || !isfinite(r2)) return false;
-  const float alpha = r2 / pq;
-  ta = alpha;
-  tb = fmaf(alpha * alpha, q2, fmaf(-2.f * alpha, rq, r2)) / r2;  // |r - alpha q|^2 / r.r
-  return true;
-}
-__device__ __forceinline__ bool chip_scalars(const double (&t)[4], double& ta, double& tb) {
-  const double pq = t[0], r2 = t[1], rq = t[2], q2 = t[3];
-  if (!(pq != 0.0) || !isfinite(pq) || !isfinite(r2)) return false;
-  const double inv = 1.0 / (r2 * pq);  // one FP64 division for both
-  const double alpha = r2 * r2 * inv;
-  ta = alpha;
-  tb = fma(alpha * alpha, q2, fma(-2.0 * alpha, rq, r2)) * (pq * inv);
-  return true;
-}
 
 template <typename T, int ZP, bool XS>
 __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
@@ -128,7 +57,7 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
   constexpr int NG = XS ? 1 : kChipGhosts;  // ghosts per thread held in registers
   T* P = reinterpret_cast<T*>(smraw);  // p with its ghost layer
   const int tid = threadIdx.x, nthr = blockDim.x;
-  const int lane = tid & 31, warp = tid >> 5, nwarp = nthr >> 5;
+  const int warp = tid >> 5;
   int i0, j0, k0, bx, by, bz;
   chip_part(f.nx, f.px, blockIdx.x % f.px, i0, bx);
   chip_part(f.ny, f.py, (blockIdx.x / f.px) % f.py, j0, by);
@@ -381,7 +310,6 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
       }
     fill_ghosts(f.rg, true);
     __syncthreads();
-    const unsigned G = gridDim.x;
     for (;;) {
       // the offsets of the planes are formed anew in each iteration: hoisted out
       // of the loop they would take the registers of the vectors
@@ -397,121 +325,42 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
           d2 += r[j] * q[j];
           d3 += q[j] * q[j];
         }
-      // each warp's four values by a transposing butterfly: after it lanes
-      // 8k .. 8k + 7 hold the warp's value k
-      {
-        const bool up = lane & 16, odd = lane & 8;
-        T a0 = up ? d2 : d0, a1 = up ? d3 : rr_own;                // kept
-        const T s0 = up ? d0 : d2, s1 = up ? rr_own : d3;          // given to lane ^ 16
-        a0 += __shfl_xor_sync(0xffffffffu, s0, 16);
-        a1 += __shfl_xor_sync(0xffffffffu, s1, 16);
-        T v = odd ? a1 : a0;
-        v += __shfl_xor_sync(0xffffffffu, odd ? a0 : a1, 8);
-        v += __shfl_xor_sync(0xffffffffu, v, 4);
-        v += __shfl_xor_sync(0xffffffffu, v, 2);
-        v += __shfl_xor_sync(0xffffffffu, v, 1);
-        if ((lane & 7) == 0) shv[lane >> 3][warp] = v;
-      }
-      // also orders every thread's q-face stores before warp 0's release
-      __syncthreads();
-      // this sum's partials: kChipSpread copies, this block reads copy b mod kChipSpread
-      Acc* slot = reinterpret_cast<Acc*>(f.spread) + (size_t)(iter & 1) * kChipSpread * 4 * G;
-      if (warp == 0) {
-        // lanes 8k .. 8k + 7: value k of the block
-        const int k = lane >> 3;
-        Acc a = acc_of(T(0));
-        for (int w = lane & 7; w < nwarp; w += 8) a = acc_add(a, acc_of(shv[k][w]));
-#pragma unroll
-        for (int o = 4; o > 0; o >>= 1) a = acc_add(a, acc_xor(a, o));
-        // lane l writes value l mod 4 into copy l / 4
-        const Acc mine = acc_from_lane(a, 8 * (lane & 3));
-        acc_store(slot + ((size_t)(lane >> 2) * 4 + (lane & 3)) * G + blockIdx.x, mine);
-        __syncwarp();  // orders the lanes' stores before lane 0's release
-        if (lane == 0) red_release_add(f.counters + (blockIdx.x % kChipSpread) * kChipLine, 1u);
-        // posted: the other warps may start their deferred work
-        asm volatile("bar.arrive 2, %0;" ::"r"(nthr) : "memory");
-        // lanes 0 .. kChipSpread - 1 wait for one counter each (counter i
-        // takes blocks i, i + kChipSpread, ...; counter 0 also the test
-        // hook's missing arrivals)
-        bool done = lane >= kChipSpread;
-        const unsigned mine_n = lane < (int)G ? (G - lane + kChipSpread - 1) / kChipSpread : 0u;
-        const unsigned target = done ? 0u : ((unsigned)iter + 1u) * (mine_n + (lane == 0 ? f.missing : 0u));
-        const long long t0 = clock64();
-        int fail = 0;
-        for (unsigned spins = 1;; ++spins) {
-          if (!done) done = (int)(ld_acquire(f.counters + lane * kChipLine) - target) >= 0;
-          if (__all_sync(0xffffffffu, done)) break;
-          const bool quit = (spins & 63u) == 0u && (ld_volatile(&gs.bar->fail.v) != 0u || clock64() - t0 > gs.spin);
-          if (__any_sync(0xffffffffu, quit)) {
-            if (lane == 0) atomicExch(&gs.bar->fail.v, 1u);
-            fail = 1;
-            break;
-          }
-        }
-        __syncwarp();  // orders the lanes' acquires before the reads of every lane
-        if (lane == 0) s_fail = fail;
-        // every block has arrived (or the wait gave up)
-        asm volatile("bar.arrive 1, %0;" ::"r"(nthr) : "memory");
-      } else {
-        asm volatile("bar.sync 2, %0;" ::"r"(nthr) : "memory");
-        if constexpr (kDefer) {
-          if (iter > 0) {
-#pragma unroll
-            for (int j = 0; j < ZP; ++j) xr[XS ? 0 : j] += tx * po[kDefer ? j : 0];
-          }
-        }
-        asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory");
-      }
-      // warps 0 .. 3 fold one value each (in block order, so every block
-      // obtains the same totals); every thread loads the q of its ghosts
-      const Acc* mycopy = slot + (size_t)(blockIdx.x % kChipSpread) * 4 * G;
       T gq[NG];
-      auto load_ghosts = [&] {
-        if constexpr (XS) {
-          for (int id = tid; id < ngh; id += nthr) cp_async(GQ + id, qw + GT[id].y);
-          cp_commit();
+      chip_sum<false>(
+          f, iter, d0, rr_own, d2, d3, shv, tot, s_fail,
+          [&] {
+            if constexpr (kDefer) {
+              if (iter > 0) {
+#pragma unroll
+                for (int j = 0; j < ZP; ++j) xr[XS ? 0 : j] += tx * po[kDefer ? j : 0];
+              }
+            }
+          },
+          [&] {  // the q of the ghosts
+            if constexpr (XS) {
+              for (int id = tid; id < ngh; id += nthr) cp_async(GQ + id, qw + GT[id].y);
+              cp_commit();
+            } else {
+#pragma unroll
+              for (int g = 0; g < NG; ++g) gq[g] = gsm[g] >= 0 ? __ldcg(qw + ggl[g]) : T(0);
+            }
+          });
+      if (tid == 0) {  // the status, alpha and beta
+        int st = 0;
+        if (s_fail) {
+          st = 5;
         } else {
-#pragma unroll
-          for (int g = 0; g < NG; ++g) gq[g] = gsm[g] >= 0 ? __ldcg(qw + ggl[g]) : T(0);
+          const Acc t4[4] = {tot[0], tot[1], tot[2], tot[3]};
+          rr_last = t4[1];
+          T al = T(0), be = T(0);
+          if (acc_le(t4[1], rr_stop)) st = 1;
+          else if (iter >= f.maxit) st = 2;
+          else if (!chip_scalars(t4, al, be)) st = 3;
+          sc.ta = al;
+          sc.tb = be;
+          sc.tx = kScaled ? al * mc0 : al;
         }
-      };
-      if (warp < 4) {
-        for (int k = warp; k < 4; k += nwarp) {
-          Acc t = acc_of(T(0));
-          for (unsigned b0 = lane; b0 < G; b0 += 32 * 5) {
-            Acc w[5];
-#pragma unroll
-            for (int u = 0; u < 5; ++u)
-              w[u] = b0 + 32 * u < G ? acc_load(mycopy + (size_t)k * G + b0 + 32 * u) : acc_of(T(0));
-            if (k == warp && b0 == (unsigned)lane) load_ghosts();
-#pragma unroll
-            for (int u = 0; u < 5; ++u) t = acc_add(t, w[u]);
-          }
-          if (k == warp && (unsigned)lane >= G) load_ghosts();
-          t = acc_warp(t);
-          if (lane == 0) tot[k] = t;
-        }
-        // the folds are complete: thread 0 forms the status, alpha and beta
-        asm volatile("bar.sync 3, %0;" ::"r"(32 * min(nwarp, 4)) : "memory");
-        if (tid == 0) {
-          int st = 0;
-          if (s_fail) {
-            st = 5;
-          } else {
-            const Acc t4[4] = {tot[0], tot[1], tot[2], tot[3]};
-            rr_last = t4[1];
-            T al = T(0), be = T(0);
-            if (acc_le(t4[1], rr_stop)) st = 1;
-            else if (iter >= f.maxit) st = 2;
-            else if (!chip_scalars(t4, al, be)) st = 3;
-            sc.ta = al;
-            sc.tb = be;
-            sc.tx = kScaled ? al * mc0 : al;
-          }
-          sc.status = st;
-        }
-      } else {
-        load_ghosts();
+        sc.status = st;
       }
       if constexpr (XS) cp_wait<0>();
       __syncthreads();
@@ -649,7 +498,22 @@ bool make_chip_plan(const Grid<T>& g, int nsm, size_t smem_max, int max_blocks, 
       }
     }
   }
-  return found;
+  if (found || sizeof(T) != 4) return found;
+  // larger FP32 grids: p in shared memory, r in registers (les_cg_brick.cu)
+  const int px = (g.nx + kBrickX - 1) / kBrickX, py = (g.ny + kBrickY - 1) / kBrickY;
+  if (px < 2 || py < 2 || px * py > gmax) return false;
+  int pz = std::min(g.nz, gmax / (px * py));
+  const int bz = (g.nz + pz - 1) / pz;
+  pz = (g.nz + bz - 1) / bz;
+  const int zp = (bz + 7) / 8 * 8;
+  int np = 0, ng = 0;
+  if (zp > kBrickPlanes || zp < 24 || brick_smem(zp, &np, &ng) > smem_max) return false;
+  best.px = px, best.py = py, best.pz = pz;
+  best.zs = 1, best.zp = zp, best.threads = kBrickX * kBrickY;
+  best.brick = true;
+  best.np = np, best.ng = ng;
+  best.smem = brick_smem(zp, &np, &ng);
+  return true;
 }
 
 template <typename T, bool XS, int... Z>
@@ -673,7 +537,7 @@ int poisson_solve_chip(const SolverArgs<T>& a, const FusedCfg& fc, const T* b, T
                        int* iters, double* rel, std::string* err, bool* used) {
   *used = false;
   if (!(a.op == LES_OP_COMPACT && a.solver == LES_SOLVER_CG && a.g.nz >= 2 && a.bar && a.r && a.p0 && a.p1) ||
-      (long long)a.g.nx * a.g.ny * a.g.nz > (long long)kChipThreads * kChipMaxPlanes<T> * a.nsm)
+      (long long)a.g.nx * a.g.ny * a.g.nz > (long long)kChipThreads * (sizeof(T) == 4 ? kBrickPlanes : kChipMaxPlanes<T>) * a.nsm)
     return LES_OK;
   int dev = 0, nsm = 0, smem_optin = 0;
   cudaError_t e;
@@ -694,7 +558,7 @@ int poisson_solve_chip(const SolverArgs<T>& a, const FusedCfg& fc, const T* b, T
     pl.fits = make_chip_plan(a.g, nsm, (size_t)std::max(0, smem_optin - 4096), fc.max_blocks, pl);
   }
   if (!pl.fits) return LES_OK;
-  const void* kern = chip_kernel<T>(pl.zp, pl.xs);
+  const void* kern = pl.brick ? brick_kernel(pl.zp) : chip_kernel<T>(pl.zp, pl.xs);
   const unsigned G = (unsigned)(pl.px * pl.py * pl.pz);
   int per_sm = 0;
   if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.smem)) != cudaSuccess ||

@@ -601,8 +601,9 @@ int poisson_solve_resident(const SolverArgs<T>& a, const FusedCfg& fc, const T* 
   // The vectors in registers: FP32 grids 128 nodes wide in les_cg_regs.cu
   // (3.5 against 4.6 us per iteration on 128 x 64 x 64), every other grid in
   // les_cg_chip.cu, up to 24 FP32 or 12 FP64 nodes per thread of one block per
-  // SM.  What is left for the kernel here are grids of whole bricks between
-  // that and the shared memory of all SMs, and cg_resident = 2.
+  // SM, and above that, in FP32 up to 64 planes of 32 x 16 columns per SM, in
+  // les_cg_brick.cu.  What is left for the kernel here are FP64 grids of whole
+  // bricks between that and the shared memory of all SMs, and cg_resident = 2.
   if constexpr (sizeof(T) == 4) {
     if (fc.resident == 0) {
       const int rc = poisson_solve_regs(a, fc, b, x, tol, maxit, iters, rel, err, used);

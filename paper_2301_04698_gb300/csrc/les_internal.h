@@ -272,6 +272,7 @@ struct ChipPlan {
   int px = 0, py = 0, pz = 0;  // bricks along x, y, z
   int zs = 0, zp = 0;          // runs of planes per brick, planes per thread (as instantiated)
   bool xs = false;             // x and the ghosts in shared memory
+  bool brick = false;          // p in shared memory and r in registers only (les_cg_brick.cu)
   int np = 0, ng = 0;          // elements of the copy of p, of a ghost array
   int threads = 0;
   size_t smem = 0;
@@ -341,8 +342,8 @@ int poisson_solve_wave(const SolverArgs<T>& a, const FusedCfg& fc, const T* b, T
 template <typename T>
 int poisson_solve_resident(const SolverArgs<T>& a, const FusedCfg& fc, const T* b, T* x, double tol, int maxit,
                            int* iters, double* rel, std::string* err, bool* used);
-// The same iterates with every vector of a brick in registers
-// (les_cg_chip.cu): any extents; *used as above.
+// The same iterates with every vector of a brick on chip (les_cg_chip.cu), or
+// all but x (les_cg_brick.cu): any extents; *used as above.
 template <typename T>
 int poisson_solve_chip(const SolverArgs<T>& a, const FusedCfg& fc, const T* b, T* x, double tol, int maxit,
                        int* iters, double* rel, std::string* err, bool* used);

@@ -4,7 +4,8 @@ direction, sides that wrap onto themselves, walls, one block, few and many
 planes per thread, ghosts in registers and in shared memory."""
 import numpy as np
 import pytest
-import torch
+
+torch = pytest.importorskip("torch")
 
 from paper_2301_04698_gb300 import inputs
 
@@ -48,7 +49,14 @@ def launches(sim):
     (64, (22, 23, 12), 1),      # 12 planes per thread in FP64
     (64, (30, 30, 11), 2),      # runs of unequal length
     (32, (500, 3, 3), 0),       # long rows, several bricks along x
-    (64, (17, 130, 5), 20)])    # more ghosts than registers take
+    (64, (17, 130, 5), 20),     # more ghosts than registers take
+    # p in shared memory, r in registers, q formed twice:
+    (32, (64, 32, 64), 4),      # whole bricks of 64 planes, walls or their own z neighbour
+    (32, (60, 31, 57), 5),      # partial rows and columns, 57 of 64 planes
+    (32, (64, 32, 90), 8),      # two bricks along z
+    (32, (96, 48, 28), 9),      # 28 of 32 planes
+    (32, (50, 30, 80), 6),      # 80 planes of a brick: not on chip
+    (32, (50, 31, 80), 8)])     # 40 of 40 planes
 def test_chip_cg_matches_oracle(les_mod, precision, shape, max_blocks, walls):
     """Against the FP64 oracle (its CG to 1e-12) and the one-pass streaming CG,
     which follows the same iterates; tolerances as for the other CG kernels:
@@ -71,7 +79,7 @@ def test_chip_cg_matches_oracle(les_mod, precision, shape, max_blocks, walls):
         x = x0.clone()
         rc, it, res = sim.poisson_solve(bt, x, tol, 20000)
         assert rc == 0 and res <= tol
-        chip = "cg_fused" if shape == (33, 31, 29) else "cg_resident"
+        chip = "cg_fused" if shape in ((33, 31, 29), (50, 30, 80)) else "cg_resident"
         assert launches(sim) == {"cg_roll" if stream else chip: 1}
         xn = x.cpu().double().numpy()
         assert abs(xn.mean()) < (1e-14 if precision == 64 else 1e-6) * np.abs(xn).max()
