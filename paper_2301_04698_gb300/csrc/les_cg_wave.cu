@@ -13,31 +13,38 @@
 // beta_{i+1} = r'.r' / r_i.r_i (p_{i+1}.L_c p_{i+1} expanded with L_c
 // symmetric), every vector formed from its definition.
 //
-// A block of 256 threads owns a 64 x 16 (or 32 x 32) column and marches a
-// run of planes.  Each thread holds fixed positions of the column's plane
-// with its halo of two (four owned nodes and two of the halo ring per
-// thread) for the whole run, so the z neighbours of both stencils are
-// registers: per position p on the planes f-2 .. f, r' on f-3 .. f-1 and r_i
-// on f-1 .. f, where f is the plane that enters the march.  Only in-plane
-// neighbours pass through shared memory (one plane of p and one of r', each
-// double-buffered by plane parity).  The planes of r_i and p_{i-1} (halo
-// two) and of x (owned nodes) arrive through rings filled three planes
-// ahead: for an interior column as TMA boxes completing on one mbarrier per
-// ring slot, for a column at a periodic edge (whose wrap is not a box) as
-// per-thread cp.async copies of 16-byte chunks and node pairs.  Per plane
+// A block owns a column of 128 x 16, 64 x 16 or 32 x 32 nodes and marches a run of
+// planes.  A thread holds a pair of nodes along x in two adjacent rows, and some
+// threads one pair of the column's halo of two, for the whole run, so the z
+// neighbours of both stencils are registers: per pair p on the planes f-2 .. f, r'
+// on f-3 .. f-1 and r_i on f-1 .. f, where f is the plane that enters the march.
+// The other row is a register too; the remaining in-plane neighbours pass through
+// shared memory (one plane of p and one of r', each double-buffered).  The planes
+// of r_i and p_{i-1} (halo two) arrive by TMA through rings filled five planes
+// ahead, one mbarrier per ring slot, and x a plane ahead in registers.  Per plane
 // step, after one block barrier:
-//   A  p(f) = r(f) + beta p_old(f) at every position; every other pass, x +=
-//      alpha_{i-1} p_old + alpha_i p at the owned ones
-//   B  q(f-1) = L_c p, r'(f-1) = r(f-1) - alpha q(f-1) within the halo of one
-//   C  w(f-2) = L_c r' at the owned positions
-//   D  p, r' of plane f-2 stored
+//   A  p(f) = r(f) + beta p_old(f), stored; every other pass, x += alpha_{i-1}
+//      p_old + alpha_i p
+//   B  q(f-1) = L_c p, r'(f-1) = r(f-1) - alpha q(f-1) within the halo of one,
+//      stored
+//   C  w(f-2) = L_c r' at the owned nodes
 // r and p are double-buffered by iteration parity (the pass reads the
 // neighbours' r_i while writing r_{i+1}); the grid sum is the barrier
 // between passes.  Per iteration each node's r_i and p_{i-1} are read and p_i and
 // r_{i+1} written, and x is read and written every other one (an update of x
 // needs nothing of q: both take place where p_{i-1} and p_i are at hand, in one
-// pass out of two, which saves 4 of 24 bytes); the halo re-reads a third of r_i
-// and p_{i-1}, mostly from L2.
+// pass out of two, which saves 4 of 24 bytes).  Every other pass takes the columns
+// and their planes in reverse and so begins with what the last one left in L2.
+//
+// What bounds it: memory.  768 x 768 x 128 in FP32 takes 322 us an iteration, where
+// its 20 bytes a node would take 222 us at the rate of a plain copy; without the
+// arithmetic of B and C it takes 309 us, without the copies 232.  With one node per
+// lane and position, windows that were moved each step and half the columns' planes
+// fetched by every thread it was bound by instruction issue (132 a node, 393 us).
+// What took it from there, in that order: pairs in packed FP32 arithmetic with a
+// march unrolled by six (windows, ring slots and buffers known at compile time),
+// the copies left to two threads, rows of 288 bytes instead of strips, byte
+// pointers that follow the march (351 -> 325 us), the reverse passes (341 -> 322).
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -54,58 +61,84 @@
 namespace les {
 namespace {
 
-constexpr int WH = 2;   // halo of the staged planes
-constexpr int NT = 256;  // threads per block
-constexpr int D = 4;     // r_i / p_{i-1} / x rings: planes f .. f+3
+constexpr int WH = 2;  // halo of the staged planes
+constexpr int D = 6;   // r_i / p_{i-1} rings: planes f .. f+5
 
-// A column shape: WX x WY owned nodes (64 x 16 or 32 x 32).  Staged planes
-// keep rows of SP elements with the owned columns from element 4 on (16-byte
-// aligned rows, so whole 16-byte chunks are copied).  Positions per thread:
-// four owned nodes (x = lane + 32 (m mod NWX), y = warp + 8 (m / NWX)) and
-// two of the halo ring (two rows below and above, two columns left and
-// right).
+// A column shape: WX x WY owned nodes in pairs along x.
+// A thread owns a pair in two adjacent rows, and one of its threads each pair
+// of the halo ring, those within the halo of one first (the rows and pairs next
+// to the owned ones), then the two outer rows.
 template <int WX_, int WY_>
 struct Col {
-  static constexpr int WX = WX_, WY = WY_;
-  static constexpr int SX = WX + 2 * WH, SY = WY + 2 * WH;
-  static constexpr int SP = WX + 8, SN = SP * SY;
-  static constexpr int NWX = WX / 32, NWARP = NT / 32;
-  static constexpr int NO = WX * WY / NT, NR = 2 * SX * WH + 2 * WH * WY, NS = NO + (NR + NT - 1) / NT;
-  static_assert(NO == 4 && NS == 6 && NWARP * (NO / NWX) == WY, "column shape and thread count");
+  static constexpr int WX = WX_, WY = WY_, PX = WX / 2;
+  static constexpr int NT = PX * WY / 2;                // threads
+  static constexpr int NH1 = 2 * (PX + 2) + 2 * WY;     // pairs of the halo of one
+  static constexpr int NH = NH1 + 2 * (PX + 2);         // and with the outer rows
+  static constexpr int SP = WX + 4, SN = SP * (WY + 2 * WH);  // a plane of p or r' with its halo
+  static_assert(NT % 256 == 0 && NH <= NT - 64 && WY % 8 == 0, "column shape and thread count");
 };
+using Col128 = Col<128, 16>;
 using Col64 = Col<64, 16>;
 using Col32 = Col<32, 32>;
 
-// the staging copies of a plane: owned rows in 16-byte chunks; each halo row
-// in chunks with a pair of nodes at either end; a pair at either end of each
-// owned row
+// A staged plane of r_i or p_{i-1}.  A column inside the grid takes boxes of
+// rows with 16 bytes of halo at either end; one at an x edge, whose halo wraps,
+// takes the owned nodes and, as a strip of 16-byte rows each, the two ends (a
+// strip costs the copy engine as many requests as the owned rows: with strips
+// in every column.
+// All rows come in one box; in a column at a y edge the two rows below, the WY
+// owned and the two above come in three, each on a 128-byte boundary.
 template <typename T, typename C>
-struct Copies {
-  static constexpr int V = 16 / (int)sizeof(T);        // nodes per 16-byte chunk
-  static constexpr int OC = C::WX * C::WY / V / NT;     // owned chunks per thread
-  static constexpr int RC = C::WX / V + 2;              // copies per halo row
-  static constexpr int NH = 2 * WH * RC + 2 * C::WY;    // halo copies per plane
-  static_assert(OC * V * NT == C::WX * C::WY && NH <= NT, "copy plan");
+struct Staged {
+  static constexpr int SZ = (int)sizeof(T), SW = 16 / SZ;  // nodes of a strip's row
+  static constexpr int ROWS = C::WY + 2 * WH;
+  static constexpr int RW = C::WX + 2 * SW;                               // a row with its ends
+  static constexpr int O1 = (WH * RW * SZ + 127) / 128 * 128;             // bytes: the owned rows of a y edge
+  static constexpr int CB = C::WX * ROWS * SZ, SB = C::WY * 16 + 256;     // bytes: owned columns, a strip
+  static constexpr int RB = CB + 2 * SB;                                  // bytes: the whole
+  static constexpr unsigned TX = (unsigned)(RW * ROWS * SZ);              // bytes that arrive
+  static_assert(CB % 128 == 0 && RB % 128 == 0 && WH * C::WX * SZ % 128 == 0 && C::WY * RW * SZ % 128 == 0 &&
+                    C::WY * 16 % 128 == 0 && 16 * ROWS <= SB && O1 + (C::WY + WH) * RW * SZ <= RB,
+                "box alignment");
 };
 
 template <typename T, typename C>
-size_t wave_smem() {
-  return ((size_t)(2 * D + 4) * C::SN + (size_t)D * C::WX * C::WY) * sizeof(T);
+constexpr size_t wave_smem() {
+  return (size_t)D * 2 * Staged<T, C>::RB + (size_t)4 * C::SN * sizeof(T);
+}
+
+// pairs of nodes: packed FP32 arithmetic (two results per instruction, each
+// rounded as by the scalar one)
+template <typename T>
+struct Vec2;
+template <>
+struct Vec2<float> {
+  using V = float2;
+};
+template <>
+struct Vec2<double> {
+  using V = double2;
+};
+__device__ __forceinline__ float2 vadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 vmul(float2 a, float2 b) { return __fmul2_rn(a, b); }
+__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
+__device__ __forceinline__ double2 vadd(double2 a, double2 b) { return double2{a.x + b.x, a.y + b.y}; }
+__device__ __forceinline__ double2 vmul(double2 a, double2 b) { return double2{a.x * b.x, a.y * b.y}; }
+__device__ __forceinline__ double2 vfma(double2 a, double2 b, double2 c) {
+  return double2{fma(a.x, b.x, c.x), fma(a.y, b.y, c.y)};
 }
 
 template <typename T>
 struct WaveArgs {
-  // TMA descriptors of r[0], r[1], p[0], p[1] (boxes of a staged plane, SP x
-  // SY x 1) and x (boxes of the owned nodes, WX x WY x 1); use_tma = 0 when
-  // they could not be encoded
-  CUtensorMap tm_r[2], tm_p[2], tm_x;
-  int use_tma;
+  // TMA descriptors of r[0], r[1], p[0], p[1]: boxes of rows with their ends, of
+  // the owned columns, of a strip, each WY + 4, WY and 2 rows high
+  CUtensorMap tm[4][3][3];
   int nx, ny, nz, walls;
   T cx, cy, cz;  // 1/dx^2, 1/dy^2, 1/dz^2
   int ntx, nty, zrun, nchunk;
   // runs of a block: units (column, z-run of zrun planes) u = blockIdx.x,
-  // + gridDim.x, ... below nunits; then, with more columns than blocks, an
-  // equal share (tail_per planes) of the tail_planes of the columns left
+  // + gridDim.x, ... below nunits; then an equal share (tail_per planes) of the
+  // tail_planes of the columns left
   int nunits, tail_planes, tail_per;
   long long n;
   const T* b;
@@ -145,6 +178,10 @@ struct WaveSum<float> {
   F2 s{0.f, 0.f};
   float run = 0.f;
   __device__ __forceinline__ void add(float v) { run += v; }
+  __device__ __forceinline__ void add(float2 v) {
+    f2_acc(s, v.x);
+    f2_acc(s, v.y);
+  }
   __device__ __forceinline__ void flush() {
     f2_acc(s, run);
     run = 0.f;
@@ -155,6 +192,7 @@ template <>
 struct WaveSum<double> {
   double s = 0.0;
   __device__ __forceinline__ void add(double v) { s += v; }
+  __device__ __forceinline__ void add(double2 v) { s += v.x + v.y; }
   __device__ __forceinline__ void flush() {}
   __device__ __forceinline__ double acc() const { return s; }
 };
@@ -196,18 +234,19 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, i
 }
 
 template <typename T, typename C>
-__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_cg_wave(const __grid_constant__ WaveArgs<T> f) {
-  constexpr int WX = C::WX, WY = C::WY, SX = C::SX, SP = C::SP, SN = C::SN;
-  constexpr int NO = C::NO, NR = C::NR, NS = C::NS, NWX = C::NWX, NWARP = C::NWARP;
+__global__ void __launch_bounds__(C::NT, sizeof(T) == 4 ? 512 / C::NT : 1) k_cg_wave(const __grid_constant__ WaveArgs<T> f) {
+  constexpr int WX = C::WX, WY = C::WY, PX = C::PX, NT = C::NT, SP = C::SP, SN = C::SN;
+  using G = Staged<T, C>;
+  using V = typename Vec2<T>::V;
   extern __shared__ __align__(128) unsigned char smraw[];
-  T* RINGR = reinterpret_cast<T*>(smraw);  // [D][SN] r_i as copied
-  T* RINGP = RINGR + D * SN;               // [D][SN] p_{i-1} as copied
-  T* PP = RINGP + D * SN;                  // [2][SN] p of a plane, by plane parity
-  T* RP = PP + 2 * SN;                     // [2][SN] r' of a plane, by plane parity
-  T* RINGX = RP + 2 * SN;                  // [D][WY][WX] x of the owned nodes
-  // one barrier per ring slot: the TMA copies of a plane (r_i, p_{i-1}, x)
+  unsigned char* const RINGR = smraw;                        // [D][RB] r_i as copied
+  unsigned char* const RINGP = RINGR + D * G::RB;            // [D][RB] p_{i-1} as copied
+  T* const PP = reinterpret_cast<T*>(RINGP + D * G::RB);     // [2][SN] p of a plane, alternating
+  T* const RP = PP + 2 * SN;                                 // [2][SN] r' of a plane, alternating
+  // one barrier per ring slot: the TMA copies of a plane (r_i, p_{i-1})
   // complete on it; bit s of phase is the parity this thread waits for next
   __shared__ __align__(8) uint64_t bars[D];
+  __shared__ decltype(WaveSum<T>().acc()) sums[4][NT];
   unsigned phase = 0;
   if (threadIdx.x == 0) {
     for (int q = 0; q < D; ++q) mbar_init(&bars[q], 1);
@@ -253,13 +292,21 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_cg_wave(const __
     }
     __stcg(reinterpret_cast<VQ*>(ptr), q);
   };
-  const int cpr = f.nx / VC;  // chunks per row
   const long long nch = f.n / VC;
+  const int cpr = f.nx / VC;  // chunks per row
+  // a chunk's place (i / VC, j, k) and the grid's stride as one
+  const int pi0 = (int)(gtid % cpr), si = (int)(gstride % cpr);
+  const int pj0 = (int)(gtid / cpr % f.ny), sj = (int)(gstride / cpr % f.ny);
+  const int pk0 = (int)(gtid / cpr / f.ny), sk = (int)(gstride / cpr / f.ny);
   auto each_chunk = [&](auto&& body) {
+    int pi = pi0, pj = pj0, pk = pk0;
     for (long long c = gtid; c < nch; c += gstride) {
-      const long long rw = c / cpr;
-      const int i0 = (int)(c - rw * cpr) * VC;
-      body((size_t)c * VC, i0, (int)(rw % f.ny), (int)(rw / f.ny));
+      body((size_t)c * VC, pi * VC, pj, pk);
+      pi += si;
+      pj += sj;
+      pk += sk;
+      if (pi >= cpr) pi -= cpr, ++pj;
+      if (pj >= f.ny) pj -= f.ny, ++pk;
     }
   };
   // the 7-point operator at a chunk's nodes straight from global memory
@@ -392,243 +439,287 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 2 : 1) k_cg_wave(const __
   }
 
   // ---- iterations ----------------------------------------------------------------
+  const V vcx{cx, cx}, vcy{cy, cy}, vcz{cz, cz}, m2{T(-2), T(-2)};
+  // L_c at the pair c with its left and right nodes and its neighbours in y and z
+  auto lap = [&](T l, V c, T r, V ym, V yp, V zm, V zp) -> V {
+    const V sx = vfma(c, m2, V{l + c.y, c.x + r}), sy = vfma(c, m2, vadd(ym, yp)), sz = vfma(c, m2, vadd(zm, zp));
+    return vfma(sz, vcz, vfma(sy, vcy, vmul(sx, vcx)));
+  };
+  auto ld2 = [](const T* q) -> V { return *reinterpret_cast<const V*>(q); };
+  auto st2 = [](T* q, V v) { *reinterpret_cast<V*>(q) = v; };
+  auto st2g = [](T* q, V v) { __stcg(reinterpret_cast<V*>(q), v); };
   int iter = 0;
   T ta = T(0);  // alpha of the last pass
   while (!status) {
     const T tp = ta;  // alpha_{i-1}
     ta = sc.ta;
     const T tb = sc.tb;
-    const bool first = iter == 0;
+    const V vtp{tp, tp}, vta{ta, ta}, vna{-ta, -ta}, vtb{tb, tb};
     // x takes two updates every other pass: p_{i-1} is read anyway
     const bool upd = iter & 1;
-    const T* ri = f.r[iter & 1];
+    // every other pass takes the units and their planes in reverse: it begins
+    // with what the last one left in L2
+    const bool rev = upd;
     T* ro = f.r[(iter + 1) & 1];
-    const T* pold = f.p[(iter + 1) & 1];  // p_{i-1}
     T* pw = f.p[iter & 1];
-    WaveSum<T> s[4];  // r'.r', r'.w, r'.q, p.q
-    int u = blockIdx.x;
-    int ts = (int)blockIdx.x * f.tail_per, te = min(ts + f.tail_per, f.tail_planes);
+    // r'.r', r'.w, r'.q, p.q: of a run of planes, and in shared memory of the pass
+    V run[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      run[q] = V{T(0), T(0)};
+      sums[q][tid] = decltype(WaveSum<T>().acc()){};
+    }
+    auto flush = [&]() {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        WaveSum<T> a{sums[q][tid]};
+        a.add(run[q]);
+        sums[q][tid] = a.acc();
+        run[q] = V{T(0), T(0)};
+      }
+    };
+    // r and p of the last pass, written by plain stores, are read by TMA
+    asm volatile("fence.proxy.async;" ::: "memory");
+    const int nfull = f.nunits > (int)blockIdx.x ? (f.nunits - 1 - (int)blockIdx.x) / (int)gridDim.x + 1 : 0;
+    const int ts = min((int)blockIdx.x * f.tail_per, f.tail_planes), te = min(ts + f.tail_per, f.tail_planes);
+    int ui = 0, tt = ts;  // units done, next plane of the tail
     for (;;) {
       int col, k0, k1;
-      if (u < f.nunits) {
+      if (ui < nfull && (!rev || tt >= te)) {
+        const int u = (int)blockIdx.x + (rev ? nfull - 1 - ui : ui) * (int)gridDim.x;
         col = u % (int)ncol;
         k0 = (u / (int)ncol) * f.zrun;
         k1 = min(k0 + f.zrun, f.nz);
-        u += gridDim.x;
-      } else if (ts < te) {  // the units are whole columns here
-        col = f.nunits + ts / f.nz;
-        k0 = ts % f.nz;
-        k1 = min(f.nz, k0 + (te - ts));
-        ts += k1 - k0;
+        ++ui;
+      } else if (tt < te) {  // the units, if any, are whole columns here
+        col = f.nunits + tt / f.nz;
+        k0 = tt % f.nz;
+        k1 = min(f.nz, k0 + (te - tt));
+        tt += k1 - k0;
       } else {
         break;
       }
+      if (rev) {  // planes counted from the top
+        const int k = k0;
+        k0 = f.nz - k1;
+        k1 = f.nz - k;
+      }
+      auto stored = [&](int k) { return rev ? f.nz - 1 - k : k; };
       const int x0 = (col % f.ntx) * WX, y0 = (col / f.ntx) * WY;
-      // this thread's positions: index in a staged plane, in-plane global
-      // offset; the halo slots' classes (valid, within the halo of one)
-      // (owned slots: a base plus constants, x = lane + 32 (m mod NWX),
-      // y = warp + 8 (m / NWX))
-      int esr[NS - NO] = {};  // halo slots
-      unsigned valid = (1u << NO) - 1u, in1 = (1u << NO) - 1u;
-      const int go0 = (y0 + (tid >> 5)) * f.nx + x0 + (tid & 31);  // global offset of owned slot 0
-      const int eo0 = ((tid >> 5) + WH) * SP + (tid & 31) + 4;      // staged index of owned slot 0
-      auto es = [&](int m) { return m < NO ? eo0 + NWARP * (m / NWX) * SP + 32 * (m % NWX) : esr[m - NO]; };
-#pragma unroll
-      for (int m = NO; m < NS; ++m) {
-        int ex, ey;
-        {
-          const int j = tid + (m - NO) * NT;
-          if (j < 2 * SX * WH) {  // the two rows below and the two above
-            const int top = j >= SX * WH;
-            const int jj = j - top * SX * WH;
-            ey = (top ? WY : -WH) + jj / SX;
-            ex = jj % SX - WH;
-          } else {  // two columns left and right of the owned rows
-            const int jj = min(j - 2 * SX * WH, 4 * WY - 1);
-            const int c = jj & 3;
-            ey = jj >> 2;
-            ex = c < 2 ? c - WH : WX - 2 + c;
-          }
-          if (j < NR) {
-            valid |= 1u << m;
-            if (ex >= -1 && ex <= WX && ey >= -1 && ey <= WY) in1 |= 1u << m;
-          }
-        }
-        esr[m - NO] = (ey + WH) * SP + (ex + 4);
+      // this thread's pairs: owned rows py and py + 1, and one of the halo (formed
+      // again for each unit: held across them they cost spills)
+      int t = tid;
+      asm volatile("" : "+r"(t));
+      const int px = 2 * (t % PX), py = 2 * (t / PX);
+      const int eo = (py + WH) * SP + px + 2;  // in a plane of p or r'; the halo pair's: eh
+      int hrow, hpair;
+      if (t < 2 * (PX + 2)) {
+        hrow = t < PX + 2 ? -1 : WY;
+        hpair = t % (PX + 2) - 1;
+      } else if (t < C::NH1) {
+        hrow = (t - 2 * (PX + 2)) >> 1;
+        hpair = (t & 1) ? PX : -1;
+      } else {
+        const int j = min(t - C::NH1, 2 * (PX + 2) - 1);
+        hrow = j < PX + 2 ? -2 : WY + 1;
+        hpair = j % (PX + 2) - 1;
       }
-      // interior columns take TMA boxes (the periodic wrap of an edge column
-      // is not a box); the others take per-thread copies
-      const bool tma = f.use_tma && x0 >= 4 && x0 + WX + 4 <= f.nx && y0 >= WH && y0 + WY + WH <= f.ny;
-      // this thread's staging copies (shared and in-plane global offsets)
-      using CP = Copies<T, C>;
-      int od[CP::OC], os[CP::OC];
-#pragma unroll
-      for (int j = 0; j < CP::OC; ++j) {
-        const int c = tid + j * NT, ey = c / (WX / CP::V), ex = (c % (WX / CP::V)) * CP::V;
-        od[j] = (ey + WH) * SP + ex + 4;  // in a staged plane; x rows are dense: ey WX + ex
-        os[j] = (y0 + ey) * f.nx + x0 + ex;
-      }
-      int hd = 0, hs = 0, hk = 0;  // halo copy: kind 0 none, 1 a pair of nodes, 2 a chunk
-      if (tid < CP::NH) {
-        int ey, ex;
-        if (tid < 2 * WH * CP::RC) {
-          const int r = tid / CP::RC, j = tid % CP::RC;
-          ey = r < WH ? r - WH : WY + r - WH;
-          ex = j == 0 ? -WH : (j == CP::RC - 1 ? WX : (j - 1) * CP::V);
-          hk = (j == 0 || j == CP::RC - 1) ? 1 : 2;
-        } else {
-          const int c = tid - 2 * WH * CP::RC;
-          ey = c >> 1;
-          ex = (c & 1) ? WX : -WH;
-          hk = 1;
-        }
-        hd = (ey + WH) * SP + ex + 4;
-        hs = wrapw(y0 + ey, f.ny) * f.nx + wrapw(x0 + ex, f.nx);
-      }
-      // plane kk of r_i, p_{i-1} (every position) and of x (owned positions,
-      // planes of the run) into their ring slots; one commit group per plane
-      auto fetch = [&](int kk) {
-        const int zs = zmapw(kk, f.nz, f.walls);
-        const size_t base = (size_t)zs * plane;
-        const int slot = (kk + 2 * D) % D;
-        T* rr_ = RINGR + slot * SN;
-        T* pp_ = RINGP + slot * SN;
-        T* xx_ = RINGX + slot * (WX * WY);
-        const bool xrun = upd && kk >= k0 && kk < k1;
-        if (tma) {
-          if (tid == 0) {
-            const unsigned bytes = (unsigned)((first ? 1 : 2) * SN * sizeof(T) + (xrun ? WX * WY * sizeof(T) : 0));
-            mbar_expect_tx(&bars[slot], bytes);
-            tma_load_3d(rr_, &f.tm_r[iter & 1], x0 - 4, y0 - WH, zs, &bars[slot]);
-            if (!first) tma_load_3d(pp_, &f.tm_p[(iter + 1) & 1], x0 - 4, y0 - WH, zs, &bars[slot]);
-            if (xrun) tma_load_3d(xx_, &f.tm_x, x0, y0, kk, &bars[slot]);
-          }
-          return;
-        }
-        const T* rs = ri + base;
-        const T* ps = pold + base;
-        const T* xs = f.x + base;
-#pragma unroll
-        for (int j = 0; j < CP::OC; ++j) {
-          const int c = tid + j * NT;
-          cp_async_bytes<16>(rr_ + od[j], rs + os[j]);
-          if (!first) cp_async_bytes<16>(pp_ + od[j], ps + os[j]);
-          if (xrun) cp_async_bytes<16>(xx_ + (c / (WX / CP::V)) * WX + (c % (WX / CP::V)) * CP::V, xs + os[j]);
-        }
-        if (hk == 2) {
-          cp_async_bytes<16>(rr_ + hd, rs + hs);
-          if (!first) cp_async_bytes<16>(pp_ + hd, ps + hs);
-        } else if (hk == 1) {
-          cp_async_bytes<2 * sizeof(T)>(rr_ + hd, rs + hs);
-          if (!first) cp_async_bytes<2 * sizeof(T)>(pp_ + hd, ps + hs);
-        }
-        cp_commit();
+      const bool halo2 = t < C::NH, halo1 = t < C::NH1;
+      const int eh = (hrow + WH) * SP + 2 * hpair + 2;
+      const int go = (y0 + py) * f.nx + x0 + px;  // in-plane global offset of the lower pair
+      // an interior column's rows are one box, those of a y edge three
+      const bool yin = y0 >= WH && y0 + WY + WH <= f.ny;
+      const bool xin = x0 > 0 && x0 + WX < f.nx;
+      // the pairs in a staged plane
+      const int pitch = xin ? G::RW : WX;
+      auto row_at = [&](int row, int p, int o1) {  // o1: bytes, of the owned rows of a y edge
+        return yin ? (row + WH) * p : (row < 0 ? (row + WH) * p : o1 / G::SZ + row * p);
       };
-      // register windows per position: p on f-2 .. f, r' on f-3 .. f-1, r_i
-      // on f-1 .. f
-      T pw0[NS], pw1[NS], pw2[NS], rw0[NS], rw1[NS], rw2[NS], ra0[NS], ra1[NS];
-#pragma unroll
-      for (int m = 0; m < NS; ++m) pw0[m] = pw1[m] = pw2[m] = rw0[m] = rw1[m] = rw2[m] = ra0[m] = ra1[m] = T(0);
-      __syncthreads();  // the previous column's readers are done with every buffer
-      for (int kk = k0 - 2; kk < k0 - 2 + D - 1; ++kk) fetch(kk);
-      int cnt = 0;
-      // wait (bounded) for the TMA copies of plane kk; a wait that runs out
-      // raises the grid's fail flag, so every grid sum of the launch fails
-      auto wait_plane = [&](int kk) {
-        const int slot = (kk + 2 * D) % D;
-        const long long t0 = clock64();
-        unsigned spins = 0;
-        while (!mbar_try_wait(&bars[slot], (phase >> slot) & 1u)) {
-          if ((++spins & 63u) == 0u && (ld_volatile(&f.bar->fail.v) != 0u || clock64() - t0 > f.spin_cycles)) {
-            atomicExch(&f.bar->fail.v, 1u);
-            break;
+      int so[2], ho;
+      if (xin) {
+        so[0] = row_at(py, G::RW, G::O1) + G::SW + px;
+        ho = row_at(hrow, G::RW, G::O1) + G::SW + 2 * hpair;
+      } else {
+        so[0] = (py + WH) * WX + px;
+        if (hpair >= 0 && hpair < PX) ho = (hrow + WH) * WX + 2 * hpair;
+        else if (hpair < 0) ho = G::CB / G::SZ + row_at(hrow, G::SW, 128) + G::SW - 2;
+        else ho = (G::CB + G::SB) / G::SZ + row_at(hrow, G::SW, 128);
+      }
+      so[1] = so[0] + pitch;
+      const int xl = x0 == 0 ? f.nx - G::SW : x0 - G::SW, xr = x0 + WX == f.nx ? 0 : x0 + WX;
+      // plane kk of r_i or (isp) p_{i-1} into ring slot sl, issued by one thread
+      auto copy = [&](bool isp, int sl, int kk) {
+        if (kk > k1 + 1) return;
+        const int zs = stored(zmapw(kk, f.nz, f.walls));
+        if (!isp) mbar_expect_tx(&bars[sl], 2 * G::TX);
+        const CUtensorMap(*tm)[3] = f.tm[isp && iter ? 2 + ((iter + 1) & 1) : iter & 1];  // beta_0 = 0: r for p_{-1}
+        unsigned char* at = (isp ? RINGP : RINGR) + sl * G::RB;
+        // all rows at once; of a y edge the owned, those below, those above
+#pragma unroll 1
+        for (int seg = yin ? 0 : 1; seg < (yin ? 1 : 4); ++seg) {
+          const int y = seg == 0 ? y0 - WH
+                                 : (seg == 1 ? y0
+                                             : (seg == 2 ? (y0 == 0 ? f.ny : y0) - WH : (y0 + WY == f.ny ? 0 : y0 + WY)));
+          const int h = seg > 2 ? 2 : seg;
+          // bytes down to these rows, where a row has rb bytes and the owned begin at o1
+          auto down = [&](int rb, int o1) { return seg == 1 ? o1 : (seg == 3 ? o1 + WY * rb : 0); };
+          if (xin) {
+            tma_load_3d(at + down(G::RW * G::SZ, G::O1), &tm[0][h], x0 - G::SW, y, zs, &bars[sl]);
+          } else {
+            tma_load_3d(at + down(WX * G::SZ, WH * WX * G::SZ), &tm[1][h], x0, y, zs, &bars[sl]);
+            at += G::CB + down(16, 128);
+            tma_load_3d(at, &tm[2][h], xl, y, zs, &bars[sl]);
+            tma_load_3d(at + G::SB, &tm[2][h], xr, y, zs, &bars[sl]);
+            at -= G::CB + down(16, 128);
           }
         }
-        phase ^= 1u << slot;
       };
-      for (int fp = k0 - 2; fp <= k1 + 1; ++fp) {
-        // plane fp has landed: the later copies may still fly
-        if (tma) wait_plane(fp);
-        else cp_wait<D - 2>();
-        __syncthreads();
-        // the slot of plane fp - 1 is free (its r_i is held in registers)
-        fetch(fp + D - 1);
-        const T* rr_ = RINGR + ((fp + 2 * D) % D) * SN;
-        const T* pp_ = RINGP + ((fp + 2 * D) % D) * SN;
-        const T* xx_ = RINGX + ((fp + 2 * D) % D) * (WX * WY);
-        T* pnew = PP + (fp & 1) * SN;
-        // A: p(fp) = r(fp) + beta p_old(fp)
-#pragma unroll
-        for (int m = 0; m < NS; ++m) {
-          if (m >= NO && !(valid >> m & 1u)) continue;
-          const int e = es(m);
-          const T rv = rr_[e];
-          const T pv = first ? rv : rv + tb * pp_[e];
-          pw2[m] = pv;
-          ra1[m] = rv;
-          pnew[e] = pv;
-          if (m < NO && upd && fp >= k0 && fp < k1)
-            __stcg(f.x + (size_t)fp * plane + go0 + (NWARP * (m / NWX)) * f.nx + 32 * (m % NWX),
-                   xx_[((tid >> 5) + NWARP * (m / NWX)) * WX + (tid & 31) + 32 * (m % NWX)] + tp * pp_[e] + ta * pv);
-        }
-        // B: q(fp-1), r'(fp-1) within the halo of one (needs p(fp-2))
-        if (fp >= k0) {
-          const T* pc = PP + ((fp - 1) & 1) * SN;
-          T* rnew = RP + ((fp - 1) & 1) * SN;
-          const bool count = fp - 1 >= k0 && fp - 1 < k1;
-#pragma unroll
-          for (int m = 0; m < NS; ++m) {
-            if (m >= NO && !(in1 >> m & 1u)) continue;
-            const int e = es(m);
-            const T c2 = T(2) * pw1[m];
-            const T qv = (pc[e - 1] + pc[e + 1] - c2) * cx + (pc[e - SP] + pc[e + SP] - c2) * cy +
-                         (pw0[m] + pw2[m] - c2) * cz;
-            const T r1 = ra0[m] - ta * qv;
-            rw2[m] = r1;
-            rnew[e] = r1;
-            if (m < NO && count) {
-              s[2].add(r1 * qv);
-              s[3].add(pw1[m] * qv);
+      // in the march by a thread each of the last two warps, which have no halo pairs
+      auto fetch = [&](int sl, int kk) {
+        if (tid == NT - 64 || tid == NT - 32) copy(tid == NT - 32, sl, kk);
+      };
+      // wait (bounded) for the copies in a ring slot; a wait that runs out raises
+      // the grid's fail flag, so every grid sum of the launch fails
+      auto landed = [&](int sl) {
+        if (!mbar_try_wait(&bars[sl], (phase >> sl) & 1u)) {
+          const long long t0 = clock64();
+          while (!mbar_try_wait(&bars[sl], (phase >> sl) & 1u)) {
+            if (clock64() - t0 > f.spin_cycles) {
+              atomicExch(&f.bar->fail.v, 1u);
+              break;
             }
           }
         }
-        // C, D: w(fp-2) and the outputs of plane fp-2 (needs r'(fp-3))
-        if (fp >= k0 + 2) {
-          const int k = fp - 2;
-          const T* rc = RP + (k & 1) * SN;
-          const size_t base = (size_t)k * plane;
+        phase ^= 1u << sl;
+      };
+      // register windows per pair, by plane mod 3: p on f-2 .. f, r' on
+      // f-3 .. f-1, r_i on f-1 .. f; slot 2 is the halo pair
+      V pv[3][3], rv[3][2], ra[3][3], xv[2];
 #pragma unroll
-          for (int m = 0; m < NO; ++m) {
-            const int e = es(m);
-            const T c2 = T(2) * rw1[m];
-            const T w = (rc[e - 1] + rc[e + 1] - c2) * cx + (rc[e - SP] + rc[e + SP] - c2) * cy +
-                        (rw0[m] + rw2[m] - c2) * cz;
-            s[0].add(rw1[m] * rw1[m]);
-            s[1].add(rw1[m] * w);
-            const size_t g = base + go0 + (NWARP * (m / NWX)) * f.nx + 32 * (m % NWX);
-            __stcg(pw + g, pw0[m]);
-            __stcg(ro + g, rw1[m]);
+      for (int q = 0; q < 3; ++q)
+#pragma unroll
+        for (int m = 0; m < 3; ++m) {
+          pv[q][m] = ra[q][m] = V{T(0), T(0)};
+          if (m < 2) rv[q][m] = xv[m] = V{T(0), T(0)};
+        }
+      __syncthreads();  // the previous unit's readers are done with every buffer
+      if ((tid & 31) == 0)
+#pragma unroll 1
+        for (int q = tid >> 6; q < D - 1; q += NT / 64) copy((tid >> 5) & 1, q, k0 - 2 + q);
+      int cnt = 0;
+      // the owned pairs in global memory, as byte pointers that follow the march
+      // (offsets formed from the plane each time cost 30 integer instructions a
+      // step): p of plane fp, r' of fp - 1, x of fp
+      const long long dg = (rev ? -(long long)plane : (long long)plane) * (long long)sizeof(T);
+      const long long g0 = ((long long)stored(k0 - 2) * (long long)plane + go) * (long long)sizeof(T);
+      const unsigned nxb = (unsigned)(f.nx * sizeof(T));
+      char *gp = reinterpret_cast<char*>(pw) + g0, *gr = reinterpret_cast<char*>(ro) + (g0 - dg),
+           *gx = reinterpret_cast<char*>(f.x) + g0;
+      auto at2 = [&](char* q, int m) { return reinterpret_cast<T*>(m ? q + nxb : q); };
+      // plane fp enters the march; PH = (fp - k0 + 2) mod 6, so that every ring
+      // slot, buffer and window is known at compile time
+      // FULL: planes fp .. fp - 2 are all of the run, so that a step is one block of
+      // code but for the halo pairs and x
+      auto step = [&](auto ph, auto full, int fp) {
+        constexpr int PH = decltype(ph)::value;
+        constexpr bool FULL = decltype(full)::value;
+        constexpr int P0 = PH % 3, P1 = (PH + 2) % 3, P2 = (PH + 1) % 3;  // planes fp, fp-1, fp-2
+        T* const pn = PP + (PH & 1) * SN;        // p of planes fp, fp-1
+        T* const pc = PP + ((PH + 1) & 1) * SN;
+        T* const rn = RP + ((PH + 1) & 1) * SN;  // r' of planes fp-1, fp-2
+        T* const rc = RP + (PH & 1) * SN;
+        landed(PH);
+        __syncthreads();
+        fetch((PH + D - 1) % D, fp + D - 1);  // into the slot of plane fp - 1, which A has read
+        const T* sr = reinterpret_cast<const T*>(RINGR + PH * G::RB);
+        const T* sp = reinterpret_cast<const T*>(RINGP + PH * G::RB);
+        // A: p(fp) = r(fp) + beta p_old(fp)
+        const V a0 = ld2(sr + so[0]), a1 = ld2(sr + so[1]), o0 = ld2(sp + so[0]), o1 = ld2(sp + so[1]);
+        const V p0 = vfma(vtb, o0, a0), p1 = vfma(vtb, o1, a1);
+        // neighbours of p(fp - 1), read before anything is written
+        const V pym = ld2(pc + eo - SP), pyp = ld2(pc + eo + 2 * SP);
+        const T pl0 = pc[eo - 1], pr0 = pc[eo + 2], pl1 = pc[eo + SP - 1], pr1 = pc[eo + SP + 2];
+        ra[P0][0] = a0;
+        ra[P0][1] = a1;
+        pv[P0][0] = p0;
+        pv[P0][1] = p1;
+        xv[0] = vfma(vtp, o0, xv[0]);
+        xv[1] = vfma(vtp, o1, xv[1]);
+        st2(pn + eo, p0);
+        st2(pn + eo + SP, p1);
+        if (FULL || (fp >= k0 && fp < k1)) {
+          st2g(at2(gp, 0), p0);
+          st2g(at2(gp, 1), p1);
+        }
+        // B: q(fp-1), r'(fp-1) within the halo of one
+        if (FULL || fp >= k0) {
+          const V q0 = lap(pl0, pv[P1][0], pr0, pym, pv[P1][1], pv[P2][0], p0);
+          const V q1 = lap(pl1, pv[P1][1], pr1, pv[P1][0], pyp, pv[P2][1], p1);
+          const V r0 = vfma(vna, q0, ra[P1][0]), r1 = vfma(vna, q1, ra[P1][1]);
+          rv[P1][0] = r0;
+          rv[P1][1] = r1;
+          st2(rn + eo, r0);
+          st2(rn + eo + SP, r1);
+          if (FULL || (fp > k0 && fp <= k1)) {
+            run[2] = vfma(r1, q1, vfma(r0, q0, run[2]));
+            run[3] = vfma(pv[P1][1], q1, vfma(pv[P1][0], q0, run[3]));
+            st2g(at2(gr, 0), r0);
+            st2g(at2(gr, 1), r1);
           }
-          if ((++cnt & 15) == 0)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) s[q].flush();
         }
-        // roll the windows
-#pragma unroll
-        for (int m = 0; m < NS; ++m) {
-          pw0[m] = pw1[m];
-          pw1[m] = pw2[m];
-          rw0[m] = rw1[m];
-          rw1[m] = rw2[m];
-          ra0[m] = ra1[m];
+        // C: w(fp-2) at the owned nodes
+        if (FULL || fp >= k0 + 2) {
+          const V ylo = ld2(rc + eo - SP), yhi = ld2(rc + eo + 2 * SP);
+          const V c0 = rv[P2][0], c1 = rv[P2][1];
+          const V w0 = lap(rc[eo - 1], c0, rc[eo + 2], ylo, c1, rv[P0][0], rv[P1][0]);
+          const V w1 = lap(rc[eo + SP - 1], c1, rc[eo + SP + 2], c0, yhi, rv[P0][1], rv[P1][1]);
+          run[0] = vfma(c1, c1, vfma(c0, c0, run[0]));
+          run[1] = vfma(c1, w1, vfma(c0, w0, run[1]));
         }
+        // the halo pair
+        if (halo2) {
+          const V r = ld2(sr + ho), p = vfma(vtb, ld2(sp + ho), r);
+          pv[P0][2] = p;
+          ra[P0][2] = r;
+          st2(pn + eh, p);
+          if (halo1 && (FULL || fp >= k0)) {
+            const V q = lap(pc[eh - 1], pv[P1][2], pc[eh + 2], ld2(pc + eh - SP), ld2(pc + eh + SP), pv[P2][2], p);
+            st2(rn + eh, vfma(vna, q, ra[P1][2]));
+          }
+        }
+        if (upd) {
+          if (FULL || (fp >= k0 && fp < k1)) {
+            st2g(at2(gx, 0), vfma(vta, p0, xv[0]));
+            st2g(at2(gx, 1), vfma(vta, p1, xv[1]));
+          }
+          if (FULL ? fp + 1 < k1 : (fp + 1 >= k0 && fp + 1 < k1)) {
+            xv[0] = __ldcg(reinterpret_cast<const V*>(at2(gx + dg, 0)));
+            xv[1] = __ldcg(reinterpret_cast<const V*>(at2(gx + dg, 1)));
+          }
+        }
+        if ((++cnt & 15) == 0) flush();
+        gp += dg;
+        gr += dg;
+        gx += dg;
+      };
+      auto march = [&](auto ph, int fp) {
+        if (fp >= k0 + 2 && fp < k1) step(ph, std::true_type{}, fp);
+        else step(ph, std::false_type{}, fp);
+        return fp <= k1;
+      };
+      for (int fp = k0 - 2;; fp += 6) {
+        if (!march(std::integral_constant<int, 0>{}, fp)) break;
+        if (!march(std::integral_constant<int, 1>{}, fp + 1)) break;
+        if (!march(std::integral_constant<int, 2>{}, fp + 2)) break;
+        if (!march(std::integral_constant<int, 3>{}, fp + 3)) break;
+        if (!march(std::integral_constant<int, 4>{}, fp + 4)) break;
+        if (!march(std::integral_constant<int, 5>{}, fp + 5)) break;
       }
-      // the copies issued beyond the run (planes k1 + 2 .. k1 + D) land
-      // before the buffers are used again
-      if (tma)
-        for (int kk = k1 + 2; kk <= k1 + D; ++kk) wait_plane(kk);
-      cp_wait<0>();
     }
+    flush();
+    WaveSum<T> s[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) s[q] = WaveSum<T>{sums[q][tid]};
     double t[4];
     const bool ok = wave_sum_t0<4>(s, gs, t);
     iter += 1;
@@ -769,13 +860,15 @@ int solve_wave(const SolverArgs<T>& a, const FusedCfg& fc, const T* b, T* x, dou
   f.maxit = maxit;
   f.spin_cycles = fc.spin_cycles;
   f.guard = a.guard;
-  // TMA boxes for the interior columns: a staged plane of r and p_{i-1}
-  // (SP x SY, from x0 - 4), the owned nodes of x (WX x WY)
-  f.use_tma = encode_map<T>(&f.tm_r[0], a.r, f.nx, f.ny, f.nz, C::SP, C::SY) &&
-              encode_map<T>(&f.tm_r[1], a.q, f.nx, f.ny, f.nz, C::SP, C::SY) &&
-              encode_map<T>(&f.tm_p[0], a.p0, f.nx, f.ny, f.nz, C::SP, C::SY) &&
-              encode_map<T>(&f.tm_p[1], a.p1, f.nx, f.ny, f.nz, C::SP, C::SY) &&
-              encode_map<T>(&f.tm_x, x, f.nx, f.ny, f.nz, C::WX, C::WY);
+  const T* vec[4] = {a.r, a.q, a.p0, a.p1};
+  bool maps = true;
+  for (int v = 0; v < 4; ++v)
+    for (int w = 0; w < 3; ++w)
+      for (int h = 0; h < 3; ++h)
+        maps = maps && encode_map<T>(&f.tm[v][w][h], vec[v], f.nx, f.ny, f.nz,
+                                     w == 2 ? Staged<T, C>::SW : (w == 1 || f.nx < Staged<T, C>::RW ? C::WX : Staged<T, C>::RW),
+                                     h == 2 ? WH : (h == 1 || f.ny < Staged<T, C>::ROWS ? C::WY : Staged<T, C>::ROWS));
+  if (!maps) return poisson_solve_roll<T>(a, fc, b, x, tol, maxit, iters, rel, err);
   int per_sm = 0, dev = 0, nsm = 0;
   cudaError_t e;
   const void* kern = (const void*)k_cg_wave<T, C>;
@@ -783,7 +876,7 @@ int solve_wave(const SolverArgs<T>& a, const FusedCfg& fc, const T* b, T* x, dou
   if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
       (e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
       (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess ||
-      (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, smem)) != cudaSuccess) {
+      (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, C::NT, smem)) != cudaSuccess) {
     if (err) *err = std::string("wave CG occupancy: ") + cudaGetErrorString(e);
     return LES_ERR_CUDA;
   }
@@ -816,7 +909,16 @@ int solve_wave(const SolverArgs<T>& a, const FusedCfg& fc, const T* b, T* x, dou
     f.nunits = (int)(ncol * f.nchunk);
     f.tail_planes = 0;
     f.tail_per = 0;
-    G = std::max<long long>(1, std::min<long long>(G, f.nunits));
+    // or all planes in equal shares, when the second run of a block whose share
+    // spans two columns (four planes more and a start, as long as another two)
+    // costs less than the blocks that whole runs leave idle
+    const long long per = (ncol * f.nz + G - 1) / G;
+    if (per + 10 < f.zrun + 4) {
+      f.nunits = 0;
+      f.tail_planes = (int)(ncol * f.nz);
+      f.tail_per = (int)per;
+    }
+    G = std::max<long long>(1, std::min<long long>(G, f.nunits ? f.nunits : (f.tail_planes + per - 1) / per));
   }
   f.expected = (unsigned)G + (unsigned)std::max(0, fc.missing);
   if ((e = cudaMemsetAsync(a.bar, 0, sizeof(FusedBar), a.st)) != cudaSuccess) {
@@ -826,7 +928,7 @@ int solve_wave(const SolverArgs<T>& a, const FusedCfg& fc, const T* b, T* x, dou
   void* args[] = {&f};
   {
     ProfScope ps(a.prof, KI_CG_WAVE, a.st);
-    e = cudaLaunchCooperativeKernel(kern, dim3((unsigned)G), dim3(NT), args, smem, a.st);
+    e = cudaLaunchCooperativeKernel(kern, dim3((unsigned)G), dim3(C::NT), args, smem, a.st);
   }
   if (e != cudaSuccess) {
     if (err) *err = std::string("wave CG launch: ") + cudaGetErrorString(e);
@@ -865,7 +967,7 @@ int solve_wave(const SolverArgs<T>& a, const FusedCfg& fc, const T* b, T* x, dou
 
 bool wave_cg_eligible(int nx, int ny, int nz) {
   return (col_fits(nx, ny, Col64::WX, Col64::WY) || col_fits(nx, ny, Col32::WX, Col32::WY)) && nz >= 2 &&
-         (long long)nx * ny < (1LL << 31);
+         (long long)nx * ny < (1LL << 29);  // 32-bit byte offsets in a plane
 }
 
 template <typename T>
@@ -878,6 +980,11 @@ int poisson_solve_wave(const SolverArgs<T>& a, const FusedCfg& fc, const T* b, T
   if (!wave_cg_eligible(a.g.nx, a.g.ny, a.g.nz) ||
       !(aligned(b) && aligned(x) && aligned(a.r) && aligned(a.q) && aligned(a.p0) && aligned(a.p1)))
     return poisson_solve_roll<T>(a, fc, b, x, tol, maxit, iters, rel, err);
+  // the wider the column, the fewer lines its ends take: 105 -> 98 us an iteration
+  // on 256 x 256 x 256, 61 -> 56 on 256 x 256 x 128, the same on 768 x 768 x 128
+  if constexpr (sizeof(T) == 4)
+    if (col_fits(a.g.nx, a.g.ny, Col128::WX, Col128::WY))
+      return solve_wave<T, Col128>(a, fc, b, x, tol, maxit, iters, rel, err);
   if (col_fits(a.g.nx, a.g.ny, Col64::WX, Col64::WY))
     return solve_wave<T, Col64>(a, fc, b, x, tol, maxit, iters, rel, err);
   return solve_wave<T, Col32>(a, fc, b, x, tol, maxit, iters, rel, err);
