@@ -12,9 +12,9 @@
 // What bounds it: instruction issue (about 75 per node and iteration) and shared
 // memory, 12 accesses per node and iteration (five neighbours twice, p read and
 // written).  Measured (GB300, us per iteration; before: the streaming kernels,
-// which take 27 to 36 bytes per node through L2): 192 x 192 x 128 38.2 -> 19.9,
-// 160 x 160 x 128 30.6 -> 14.8, 256 x 256 x 64 39.0 -> 18.5, 150 x 130 x 110 23.3 ->
-// 13.7.  Bricks of any extents, with their strides and column offsets in registers,
+// which take 27 to 36 bytes per node through L2): 192 x 192 x 128 38.2 -> 18.5,
+// 160 x 160 x 128 30.6 -> 14.7, 256 x 256 x 64 39.0 -> 18.4, 150 x 130 x 110 23.3 ->
+// 13.1.  Bricks of any extents, with their strides and column offsets in registers,
 // spilled r and took 53 us on the first of these.
 #include <algorithm>
 #include <string>
@@ -142,7 +142,8 @@ __global__ void __launch_bounds__(BX* BY, 1) k_cg_brick(ChipArgs<float> f) {
     double bb, rel;  // |b - mean|^2 and the relative residual of x0
   } sc;
   __shared__ float shv[4][kChipWarps];
-  __shared__ F2 tot[4];
+  __shared__ F2 part[32];
+  F2 tot[4];  // in warp 0
   __shared__ int s_fail;
   double rr = 0.0, bb = 0.0, rel = 0.0;  // meaningful in thread 0
   int status = 0;  // 0 running, 1 converged, 2 maxit, 3 breakdown, 4 zero rhs, 5 timeout
@@ -255,7 +256,7 @@ __global__ void __launch_bounds__(BX* BY, 1) k_cg_brick(ChipArgs<float> f) {
         d2.add(j, r[j] * q);
         d3.add(j, q * q);
       });
-      chip_sum<true>(f, iter, d0.total(own), rr_own, d2.total(own), d3.total(own), shv, tot, s_fail, ChipNothing{}, [&] {
+      chip_sum<true>(f, iter, d0.total(own), rr_own, d2.total(own), d3.total(own), shv, part, tot, s_fail, ChipNothing{}, [&] {
         each_ghost([&](int id, float*, int g) { cp_async(GQ + id, qw + g); });
         cp_commit();
       });
@@ -264,12 +265,11 @@ __global__ void __launch_bounds__(BX* BY, 1) k_cg_brick(ChipArgs<float> f) {
         if (s_fail) {
           st = 5;
         } else {
-          const F2 t4[4] = {tot[0], tot[1], tot[2], tot[3]};
-          rr_last = t4[1];
+          rr_last = tot[1];
           float al = 0.f, be = 0.f;
-          if (acc_le(t4[1], rr_stop)) st = 1;
+          if (acc_le(tot[1], rr_stop)) st = 1;
           else if (iter >= f.maxit) st = 2;
-          else if (!chip_scalars(t4, al, be)) st = 3;
+          else if (!chip_scalars(tot, al, be)) st = 3;
           sc.ta = al;
           sc.tb = be;
         }

@@ -21,10 +21,12 @@
 //
 // The iteration is that of les_cg_resident.cu: one grid-wide sum of p.q,
 // r.r, r.q and q.q per iteration (alpha, and beta from |r - alpha q|^2
-// expanded in the four), posted and folded as in les_cg_regs.cu.
+// expanded in the four).  With XS = false the sum's partials and the faces' q are
+// tagged words (les_chip.cuh); with more faces these cost more than they save (150 x
+// 140 x 70 FP32: 13 us per iteration instead of 8.7), and the counters order them.
 //
-// What bounds it: the latency of the grid sum (two round trips through L2:
-// about 2.7 us of an iteration on the smallest grids) and, in FP64, the
+// What bounds it: the latency of the grid sum (2.2 us of an iteration on the
+// smallest grids; 2.6 with counters) and, in FP64, the
 // arithmetic: a scheduler issues an FP64 warp instruction every 64 cycles, so
 // a five-step butterfly of four values in 16 warps alone costs 5000 cycles.
 // The four values are therefore reduced by a transposing butterfly (six
@@ -32,13 +34,13 @@
 // per thread, the FP64 stencil takes six operations, and x += alpha p is left
 // to the next sum's wait.
 //
-// Measured (GB300, us per iteration, 200-iteration solves; before: the
+// Measured (GB300, us per iteration; before: the
 // shared-memory kernel, or the one-pass streaming kernel where no whole
 // bricks fit):
-//   FP64  32^3 10.0 -> 5.5, 256 x 4 x 32 10.3 -> 5.6, 64 x 64 x 48 17.0 -> 10.8,
-//         50 x 47 x 33 28.9 -> 7.5, 77 x 130 x 50 66.4 -> 18.4, 96^3 77 -> 29
-//   FP32  32^3 4.3 -> 2.7, 64^3 5.1 -> 3.3, 96^3 7.5 -> 5.6, 160 x 160 x 48
-//         8.5 -> 6.5, 100 x 76 x 61 23.9 -> 4.3, 150 x 140 x 70 39.4 -> 9.1
+//   FP64  32^3 9.9 -> 4.6, 256 x 4 x 32 10.1 -> 4.7, 64 x 64 x 48 16.9 -> 9.3,
+//         50 x 47 x 33 28.3 -> 7.2, 77 x 130 x 50 66.8 -> 16.7, 96^3 77 -> 26
+//   FP32  32^3 4.2 -> 2.2, 64^3 5.0 -> 3.0, 96^3 7.3 -> 5.5, 160 x 160 x 48
+//         8.4 -> 6.2, 100 x 76 x 61 23.6 -> 4.0, 150 x 140 x 70 36.7 -> 8.7
 // FP32 grids 128 nodes wide keep les_cg_regs.cu, whose four-node lanes read
 // x neighbours by shuffles: 128 x 64 x 64 3.5 there, 4.6 here; 128 x 128 x 96
 // 5.3 and 8.9.
@@ -203,11 +205,26 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
     double bb, rel;  // |b - mean|^2 and the relative residual of x0
   } sc;
   __shared__ T shv[4][kChipWarps];
-  __shared__ Acc tot[4];
+  __shared__ Acc part[32];
   __shared__ int s_fail;
   double rr = 0.0, bb = 0.0, rel = 0.0;  // meaningful in thread 0
   int status = 0;  // 0 running, 1 converged, 2 maxit, 3 breakdown, 4 zero rhs, 5 timeout
   T rr_own = T(0);  // this thread's share of r.r for the next sum
+
+  // XS = false: a node's tagged word among the published faces of q
+  constexpr int W = 2 * (int)sizeof(T);
+  const int half = (int)(f.n / 2);
+  auto word = [&](int s, int g) { return (g < half ? f.qt[0][s] : f.qt[1][s] - (size_t)half * W) + (size_t)g * W; };
+  if constexpr (!XS) {  // no tag of an earlier solve: cleared here, for everyone after the first sum
+    chip_sum_clear(f.spread);
+#pragma unroll
+    for (int j = 0; j < ZP; ++j)
+      if (j < nzp && is_face(j)) {
+        tagged_store(word(0, gown + j * gpl), T(0), 0u);
+        tagged_store(word(1, gown + j * gpl), T(0), 0u);
+      }
+  }
+  if (tid == 0) s_fail = 0;
 
   // mean of b (b held in r)
   {
@@ -320,42 +337,57 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
       for (int j = 0; j < ZP; ++j)
         if (j < nzp) {
           q[j] = stencil(j);
-          if (is_face(j)) __stcg(qw + gown + j * gpl, q[j]);
+          if (is_face(j)) {
+            if constexpr (XS) __stcg(qw + gown + j * gpl, q[j]);
+            else tagged_store(word(iter & 1, gown + j * gpl), q[j], chip_tag(iter));
+          }
           d0 += p[j] * q[j];
           d2 += r[j] * q[j];
           d3 += q[j] * q[j];
         }
-      T gq[NG];
-      chip_sum<false>(
-          f, iter, d0, rr_own, d2, d3, shv, tot, s_fail,
-          [&] {
-            if constexpr (kDefer) {
-              if (iter > 0) {
+      Tagged<T> gq[NG];  // the q of the ghosts
+      Acc tot[4];        // the totals, in warp 0
+      auto deferred = [&] {
+        if constexpr (kDefer) {
+          if (iter > 0) {
 #pragma unroll
-                for (int j = 0; j < ZP; ++j) xr[XS ? 0 : j] += tx * po[kDefer ? j : 0];
-              }
-            }
-          },
-          [&] {  // the q of the ghosts
-            if constexpr (XS) {
-              for (int id = tid; id < ngh; id += nthr) cp_async(GQ + id, qw + GT[id].y);
-              cp_commit();
-            } else {
+            for (int j = 0; j < ZP; ++j) xr[XS ? 0 : j] += tx * po[kDefer ? j : 0];
+          }
+        }
+      };
+      if constexpr (XS) {
+        chip_sum<false>(f, iter, d0, rr_own, d2, d3, shv, part, tot, s_fail, deferred, [&] {
+          for (int id = tid; id < ngh; id += nthr) cp_async(GQ + id, qw + GT[id].y);
+          cp_commit();
+        });
+      } else {
+        unsigned miss = 0;
 #pragma unroll
-              for (int g = 0; g < NG; ++g) gq[g] = gsm[g] >= 0 ? __ldcg(qw + ggl[g]) : T(0);
-            }
-          });
+        for (int g = 0; g < NG; ++g) miss |= gsm[g] >= 0 ? 1u << g : 0u;
+        chip_sum_tagged(
+            f, iter, d0, rr_own, d2, d3, shv, part, tot, s_fail, deferred,
+            [&] {
+#pragma unroll
+              for (int g = 0; g < NG; ++g)
+                if (miss >> g & 1u) tagged_load(gq[g], word(iter & 1, ggl[g]));
+            },
+            [&] {
+#pragma unroll
+              for (int g = 0; g < NG; ++g)
+                if ((miss >> g & 1u) && tagged_ok(gq[g], chip_tag(iter))) miss &= ~(1u << g);
+              return miss == 0u;
+            });
+      }
       if (tid == 0) {  // the status, alpha and beta
         int st = 0;
         if (s_fail) {
           st = 5;
         } else {
-          const Acc t4[4] = {tot[0], tot[1], tot[2], tot[3]};
-          rr_last = t4[1];
+          rr_last = tot[1];
           T al = T(0), be = T(0);
-          if (acc_le(t4[1], rr_stop)) st = 1;
+          if (acc_le(tot[1], rr_stop)) st = 1;
           else if (iter >= f.maxit) st = 2;
-          else if (!chip_scalars(t4, al, be)) st = 3;
+          else if (!chip_scalars(tot, al, be)) st = 3;
           sc.ta = al;
           sc.tb = be;
           sc.tx = kScaled ? al * mc0 : al;
@@ -391,7 +423,7 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
 #pragma unroll
         for (int g = 0; g < NG; ++g)
           if (gsm[g] >= 0) {
-            rgh[g] -= ta * gq[g];
+            rgh[g] -= ta * tagged_value(gq[g]);
             pgh[g] = rgh[g] + tb * pgh[g];
             P[gsm[g]] = pgh[g];
           }
@@ -536,7 +568,7 @@ template <typename T>
 int poisson_solve_chip(const SolverArgs<T>& a, const FusedCfg& fc, const T* b, T* x, double tol, int maxit,
                        int* iters, double* rel, std::string* err, bool* used) {
   *used = false;
-  if (!(a.op == LES_OP_COMPACT && a.solver == LES_SOLVER_CG && a.g.nz >= 2 && a.bar && a.r && a.p0 && a.p1) ||
+  if (!(a.op == LES_OP_COMPACT && a.solver == LES_SOLVER_CG && a.g.nz >= 2 && a.bar && a.r && a.q && a.p0 && a.p1) ||
       (long long)a.g.nx * a.g.ny * a.g.nz > (long long)kChipThreads * (sizeof(T) == 4 ? kBrickPlanes : kChipMaxPlanes<T>) * a.nsm)
     return LES_OK;
   int dev = 0, nsm = 0, smem_optin = 0;
@@ -587,6 +619,10 @@ int poisson_solve_chip(const SolverArgs<T>& a, const FusedCfg& fc, const T* b, T
   f.rg = a.r;
   f.qg0 = a.p0;
   f.qg1 = a.p1;
+  f.qt[0][0] = reinterpret_cast<char*>(a.p0);
+  f.qt[1][0] = reinterpret_cast<char*>(a.p1);
+  f.qt[0][1] = reinterpret_cast<char*>(a.q);
+  f.qt[1][1] = reinterpret_cast<char*>(a.r);
   f.partials = a.partials;
   // past the set-up sums' two slots: the counters, then the copies of the
   // iterations' partials (2 x kChipSpread x 4 words per block)

@@ -27,9 +27,12 @@ struct ChipArgs {
   T* rg;               // published faces of the first residual
   T* qg0;              // published faces of q, even iterations
   T* qg1;              // ... odd iterations
+  // the same as tagged words, one per node of the grid: those of the first half of the
+  // nodes at qt[0][parity], the others at qt[1][parity]
+  char* qt[2][2];
   double* partials;    // two slots of kSumSlot words per block (the set-up and gauge sums)
   unsigned* counters;  // kChipSpread arrival counters of the iterations' sums, kChipLine apart, zeroed
-  void* spread;        // [2 slots][kChipSpread copies][4 values][gridDim.x] partials of those sums
+  void* spread;        // [2 slots][kChipSpread copies][gridDim.x][4 values] partials of those sums, or tagged words
   unsigned missing;    // test hook: arrivals on counter 0 that never come
   FusedBar* bar;
   SolverCtl* ctl;
@@ -78,37 +81,76 @@ __device__ __forceinline__ bool chip_scalars(const double (&t)[4], double& ta, d
   return true;
 }
 
+// a warp's four values by a transposing butterfly (six additions instead of twenty)
+template <typename T>
+__device__ __forceinline__ void chip_butterfly(T d0, T d1, T d2, T d3, T (&shv)[4][kChipWarps]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // after the butterfly lanes 8k .. 8k + 7 hold the warp's value k
+  const bool up = lane & 16, odd = lane & 8;
+  T a0 = up ? d2 : d0, a1 = up ? d3 : d1;        // kept
+  const T s0 = up ? d0 : d2, s1 = up ? d1 : d3;  // given to lane ^ 16
+  a0 += __shfl_xor_sync(0xffffffffu, s0, 16);
+  a1 += __shfl_xor_sync(0xffffffffu, s1, 16);
+  T v = odd ? a1 : a0;
+  v += __shfl_xor_sync(0xffffffffu, odd ? a0 : a1, 8);
+  v += __shfl_xor_sync(0xffffffffu, v, 4);
+  v += __shfl_xor_sync(0xffffffffu, v, 2);
+  v += __shfl_xor_sync(0xffffffffu, v, 1);
+  if ((lane & 7) == 0) shv[lane >> 3][warp] = v;
+}
+
+// warps that fold and the words of a lane in flight (160 or 192 blocks in one turn): an
+// FP64 addition takes a scheduler 64 cycles, so fewer warps with more of their own
+template <typename Acc>
+constexpr int kFoldWarps = 8;
+template <>
+constexpr int kFoldWarps<double> = 4;
+template <typename Acc>
+constexpr int kFoldWords = kFoldWarps<Acc> == 4 ? 5 : 3;
+
+// the fold's end: lane l holds the sum of value l mod 4 over some of the blocks of
+// part id; the four totals, the same in every block, in the lanes of warp 0
+template <typename Acc>
+__device__ __forceinline__ void chip_fold_warp(Acc t, Acc (&part)[32], int id) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 16; o >= 4; o >>= 1) t = acc_add(t, acc_xor(t, o));
+  if (lane < 4) part[id * 4 + lane] = t;
+}
+template <typename Acc>
+__device__ __forceinline__ void chip_fold(Acc (&part)[32], Acc (&tot)[4]) {
+  constexpr int FW = kFoldWarps<Acc>;
+  asm volatile("bar.sync 3, %0;" ::"r"(min((int)blockDim.x, 32 * FW)) : "memory");
+  if (threadIdx.x < 32) {
+    Acc t = part[threadIdx.x % (4 * FW)];
+#pragma unroll
+    for (int o = 2 * FW; o >= 4; o >>= 1) t = acc_add(t, acc_xor(t, o));
+#pragma unroll
+    for (int k = 0; k < 4; ++k) tot[k] = acc_from_lane(t, k);
+  }
+}
+
 // The grid-wide sum of p.q, r.r, r.q and q.q at iteration `iter`: each warp's four
 // values by a transposing butterfly; warp 0 combines the warps' (FP32 ones as
 // compensated pairs), writes them into kChipSpread copies, arrives on one of
-// kChipSpread counters and waits for all of them; warps 0 .. 3 fold one value each
-// from the block's copy, in block order, so every block obtains the same totals in
-// tot.  meanwhile() runs in the other warps while warp 0 waits and must not depend
-// on the sum; load() runs in every thread once all blocks have arrived and may read
-// what they published before; in warps 0 .. 3 its loads follow the fold's own, or with
-// LoadFirst precede them, which takes fewer registers.  At the return tot and fail are valid in warps 0 .. 3.
+// kChipSpread counters and waits for all of them; the first kFoldWarps warps fold a
+// part of the blocks each from the block's copy, in a fixed order, so every block
+// obtains the same totals in tot (in warp 0).  A block's four values lie together: a line that eight
+// blocks read has four writers, not sixteen.  meanwhile() runs in the other warps
+// while warp 0 waits and must not depend on the sum; load() runs in every thread once
+// all blocks have arrived and may read what they published before; in the folding warps
+// its loads follow the fold's own, or with LoadFirst precede them, which takes fewer
+// registers.  At the return tot and fail are valid in warp 0.
 struct ChipNothing {
   __device__ __forceinline__ void operator()() const {}
 };
 template <bool LoadFirst, typename T, typename Acc, typename Meanwhile, typename Load>
 __device__ __forceinline__ void chip_sum(const ChipArgs<T>& f, int iter, T d0, T d1, T d2, T d3, T (&shv)[4][kChipWarps],
-                                         Acc (&tot)[4], int& fail, Meanwhile&& meanwhile, Load&& load) {
+                                         Acc (&part)[32], Acc (&tot)[4], int& fail, Meanwhile&& meanwhile,
+                                         Load&& load) {
   const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarp = nthr >> 5;
   const unsigned G = gridDim.x;
-  // after the butterfly lanes 8k .. 8k + 7 hold the warp's value k
-  {
-    const bool up = lane & 16, odd = lane & 8;
-    T a0 = up ? d2 : d0, a1 = up ? d3 : d1;        // kept
-    const T s0 = up ? d0 : d2, s1 = up ? d1 : d3;  // given to lane ^ 16
-    a0 += __shfl_xor_sync(0xffffffffu, s0, 16);
-    a1 += __shfl_xor_sync(0xffffffffu, s1, 16);
-    T v = odd ? a1 : a0;
-    v += __shfl_xor_sync(0xffffffffu, odd ? a0 : a1, 8);
-    v += __shfl_xor_sync(0xffffffffu, v, 4);
-    v += __shfl_xor_sync(0xffffffffu, v, 2);
-    v += __shfl_xor_sync(0xffffffffu, v, 1);
-    if ((lane & 7) == 0) shv[lane >> 3][warp] = v;
-  }
+  chip_butterfly(d0, d1, d2, d3, shv);
   // also orders every thread's q-face stores before warp 0's release
   __syncthreads();
   // this sum's partials: kChipSpread copies, this block reads copy b mod kChipSpread
@@ -122,7 +164,7 @@ __device__ __forceinline__ void chip_sum(const ChipArgs<T>& f, int iter, T d0, T
     for (int o = 4; o > 0; o >>= 1) a = acc_add(a, acc_xor(a, o));
     // lane l writes value l mod 4 into copy l / 4
     const Acc mine = acc_from_lane(a, 8 * (lane & 3));
-    acc_store(slot + ((size_t)(lane >> 2) * 4 + (lane & 3)) * G + blockIdx.x, mine);
+    acc_store(slot + ((size_t)(lane >> 2) * G + blockIdx.x) * 4 + (lane & 3), mine);
     __syncwarp();  // orders the lanes' stores before lane 0's release
     if (lane == 0) red_release_add(f.counters + (blockIdx.x % kChipSpread) * kChipLine, 1u);
     // posted: the other warps may start their own work
@@ -155,24 +197,170 @@ __device__ __forceinline__ void chip_sum(const ChipArgs<T>& f, int iter, T d0, T
     asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory");
   }
   const Acc* mycopy = slot + (size_t)(blockIdx.x % kChipSpread) * 4 * G;
-  if (LoadFirst || warp >= 4) load();
-  if (warp < 4) {
-    for (int k = warp; k < 4; k += nwarp) {
+  constexpr int FW = kFoldWarps<Acc>, U = kFoldWords<Acc>;
+  if (LoadFirst || warp >= FW) load();
+  if (warp < FW) {
+    for (int id = warp; id < FW; id += nwarp) {  // eight blocks at a time, a lane per value
       Acc t = acc_of(T(0));
-      for (unsigned b0 = lane; b0 < G; b0 += 32 * 5) {
-        Acc w[5];
+      for (unsigned b0 = (unsigned)id * 8 + (lane >> 2); b0 - (lane >> 2) < G; b0 += 8 * FW * U) {
+        Acc w[U];
 #pragma unroll
-        for (int u = 0; u < 5; ++u)
-          w[u] = b0 + 32 * u < G ? acc_load(mycopy + (size_t)k * G + b0 + 32 * u) : acc_of(T(0));
-        if (!LoadFirst && k == warp && b0 == (unsigned)lane) load();
+        for (int u = 0; u < U; ++u)
+          w[u] = b0 + 8 * FW * u < G ? acc_load(mycopy + (size_t)(b0 + 8 * FW * u) * 4 + (lane & 3)) : acc_of(T(0));
+        if (!LoadFirst && id == warp && b0 == (unsigned)id * 8 + (lane >> 2)) load();
 #pragma unroll
-        for (int u = 0; u < 5; ++u) t = acc_add(t, w[u]);
+        for (int u = 0; u < U; ++u) t = acc_add(t, w[u]);
       }
-      if (!LoadFirst && k == warp && (unsigned)lane >= G) load();
-      t = acc_warp(t);
-      if (lane == 0) tot[k] = t;
+      if (!LoadFirst && id == warp && (unsigned)id * 8 >= G) load();
+      chip_fold_warp(t, part, id);
     }
-    asm volatile("bar.sync 3, %0;" ::"r"(32 * min(nwarp, 4)) : "memory");
+    chip_fold(part, tot);
+  }
+}
+
+// ---- tagged words ------------------------------------------------------------
+// A value that other blocks wait for travels with the number of its iteration: every
+// 8 bytes hold 32 bits of it and a 32-bit tag, written and read whole, so a reader
+// that finds the tag has the value, and neither side orders it against anything
+// else.  A writer that released a flag would wait for its stores to reach L2, and a
+// reader that had seen it would read the value by another trip.  The tags are NaN
+// patterns, which no finite value left in the same memory can look like.
+__device__ __forceinline__ unsigned chip_tag(int iter) { return 0xff800001u + ((unsigned)iter & 0x3fffffu); }
+template <typename V>
+struct Tagged {  // F2 or double: 16 bytes
+  unsigned long long w[2];
+};
+template <>
+struct Tagged<float> {
+  unsigned long long w[1];
+};
+__device__ __forceinline__ void tagged_load(Tagged<float>& t, const char* at) {
+  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(t.w[0]) : "l"(at));
+}
+template <typename V>
+__device__ __forceinline__ void tagged_load(Tagged<V>& t, const char* at) {
+  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(t.w[0]), "=l"(t.w[1]) : "l"(at));
+}
+__device__ __forceinline__ bool tagged_ok(const Tagged<float>& t, unsigned tag) { return (unsigned)(t.w[0] >> 32) == tag; }
+template <typename V>
+__device__ __forceinline__ bool tagged_ok(const Tagged<V>& t, unsigned tag) {
+  return (unsigned)(t.w[0] >> 32) == tag && (unsigned)(t.w[1] >> 32) == tag;
+}
+__device__ __forceinline__ float tagged_value(const Tagged<float>& t) { return __uint_as_float((unsigned)t.w[0]); }
+__device__ __forceinline__ F2 tagged_value(const Tagged<F2>& t) {
+  return F2{__uint_as_float((unsigned)t.w[0]), __uint_as_float((unsigned)t.w[1])};
+}
+__device__ __forceinline__ double tagged_value(const Tagged<double>& t) {
+  return __hiloint2double((int)(unsigned)t.w[1], (int)(unsigned)t.w[0]);
+}
+__device__ __forceinline__ void tagged_store16(char* at, unsigned a, unsigned b, unsigned tag) {
+  const unsigned long long hi = (unsigned long long)tag << 32;
+  asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(at), "l"(hi | a), "l"(hi | b) : "memory");
+}
+__device__ __forceinline__ void tagged_store(char* at, float v, unsigned tag) {
+  const unsigned long long w = (unsigned long long)tag << 32 | __float_as_uint(v);
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(at), "l"(w) : "memory");
+}
+__device__ __forceinline__ void tagged_store(char* at, F2 v, unsigned tag) {
+  tagged_store16(at, __float_as_uint(v.hi), __float_as_uint(v.lo), tag);
+}
+__device__ __forceinline__ void tagged_store(char* at, double v, unsigned tag) {
+  tagged_store16(at, (unsigned)__double2loint(v), (unsigned)__double2hiint(v), tag);
+}
+
+// The words of a sum's partials: [2 slots][gridDim.x][4 values] of 16 bytes.  A
+// block's four lie together, so that a line has two writers: with a value's words of
+// all blocks together, and eight writers to a line that is being read, an iteration on
+// 32^3 in FP32 took 3.1 us instead of 2.2.  Several copies do not help.  A block may
+// write a slot again two sums later: it gets there only after every block has posted
+// the sum between, and so has read this one.  Cleared by each block for itself before
+// the set-up sums, which order that for everyone.
+__device__ __forceinline__ void chip_sum_clear(void* spread) {
+  const int slot = threadIdx.x >> 2, k = threadIdx.x & 3;
+  if (slot < 2)
+    tagged_store16(static_cast<char*>(spread) + (((size_t)slot * gridDim.x + blockIdx.x) * 4 + k) * 16, 0u, 0u, 0u);
+}
+
+// The same sum by tagged words: warp 0 posts the block's four values; the first
+// kFoldWarps warps read the words of a part of the blocks each, until all have come,
+// and fold them in a fixed order, so every block obtains the same totals in tot (in
+// warp 0).  meanwhile() runs in the other warps before they wait.  When the sum has
+// come, issue() starts the loads of what this thread awaits of the neighbours; check()
+// takes what has come and tells whether that was all, and both are called again until
+// it is (begun earlier, they disturb the lines that are being written: 100 x 76 x 61
+// FP32 takes 4.2 us, not 4.05).  fail (0 before the first sum) is set when a wait runs
+// out, in other warps perhaps too late for this sum but in time for the next.
+template <typename T, typename Acc, typename Meanwhile, typename Issue, typename Check>
+__device__ __forceinline__ void chip_sum_tagged(const ChipArgs<T>& f, int iter, T d0, T d1, T d2, T d3, T (&shv)[4][kChipWarps],
+                                         Acc (&part)[32], Acc (&tot)[4], volatile int& fail, Meanwhile&& meanwhile, Issue&& issue,
+                                         Check&& check) {
+  const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarp = nthr >> 5;
+  constexpr int FW = kFoldWarps<Acc>, U = kFoldWords<Acc>;
+  const unsigned G = gridDim.x, tag = chip_tag(iter);
+  chip_butterfly(d0, d1, d2, d3, shv);
+  __syncthreads();
+  char* slot = static_cast<char*>(f.spread) + (size_t)(iter & 1) * 4 * G * 16;
+  if (warp == 0) {
+    // lanes 8k .. 8k + 7: value k of the block
+    const int k = lane >> 3, c = lane & 7;
+    Acc a = acc_of(T(0));
+    for (int w = c; w < nwarp; w += 8) a = acc_add(a, acc_of(shv[k][w]));
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) a = acc_add(a, acc_xor(a, o));
+    if (c == 0) tagged_store(slot + ((size_t)blockIdx.x * 4 + k) * 16, a, tag);
+    // posted: the other warps may start their own work
+    asm volatile("bar.arrive 2, %0;" ::"r"(nthr) : "memory");
+  } else {
+    asm volatile("bar.sync 2, %0;" ::"r"(nthr) : "memory");
+    meanwhile();
+  }
+  const long long t0 = clock64();
+  // every 64th turn: has another block given up, or has the time run out?
+  auto over = [&](unsigned spins) {
+    const bool quit = (spins & 63u) == 0u && (ld_volatile(&f.bar->fail.v) != 0u || clock64() - t0 > f.spin_cycles);
+    if (!__any_sync(0xffffffffu, quit)) return false;
+    if (lane == 0) {
+      atomicExch(&f.bar->fail.v, 1u);
+      fail = 1;
+    }
+    return true;
+  };
+  if (warp < FW) {
+    for (int id = warp; id < FW; id += nwarp) {  // eight blocks at a time, a lane per value
+      Acc t = acc_of(T(0));
+      for (unsigned base = (unsigned)id * 8 + (lane >> 2); base - (lane >> 2) < G; base += 8 * FW * U) {
+        const char* at = slot + ((size_t)base * 4 + (lane & 3)) * 16;
+        Tagged<Acc> w[U];
+        unsigned miss = 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) miss |= base + 8 * FW * u < G ? 1u << u : 0u;
+        const unsigned have = miss;
+        for (unsigned spins = 1;; ++spins) {
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (miss >> u & 1u) tagged_load(w[u], at + 512 * FW * u);
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if ((miss >> u & 1u) && tagged_ok(w[u], tag)) miss &= ~(1u << u);
+          if (__all_sync(0xffffffffu, miss == 0u && f.missing == 0u) || over(spins)) break;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) t = acc_add(t, have >> u & 1u ? tagged_value(w[u]) : acc_of(T(0)));
+      }
+      if (id + nwarp >= FW) {
+        if (nwarp > FW) asm volatile("bar.arrive 1, %0;" ::"r"(nthr) : "memory");
+        issue();
+      }
+      chip_fold_warp(t, part, id);
+    }
+    chip_fold(part, tot);
+  } else {
+    asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory");
+    issue();
+  }
+  for (unsigned spins = 1;; ++spins) {
+    if (__all_sync(0xffffffffu, check()) || over(spins)) break;
+    issue();
   }
 }
 

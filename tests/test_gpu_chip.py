@@ -123,3 +123,25 @@ def test_chip_cg_nonfinite_right_side_is_a_breakdown(les_mod, value):
         sim.poisson_solve(b, torch.zeros_like(b), 1e-6, 100)
     assert e.value.status == les_mod.LES_ERR_NONFINITE
     sim.close()
+
+
+@pytest.mark.parametrize("precision,shape", [(32, (40, 40, 40)), (64, (24, 24, 24)), (32, (100, 76, 61))])
+def test_chip_cg_repeats_bit_for_bit(les_mod, precision, shape):
+    """The sums and the neighbours' faces carry the number of their iteration: a
+    solve must not take what an earlier one of the same handle left, and the sums
+    are folded in a fixed order, so solves in turn repeat those of a new handle."""
+    nx, ny, nz = shape
+    case = inputs.Case(name="chiprep", nx=nx, ny=ny, nz=nz, dx=35.0, dy=30.0, dz=10.0, walls=True,
+                       precision=precision, init="zero", physics=())
+    dt = torch.float64 if precision == 64 else torch.float32
+    bs = [torch.from_numpy(inputs.uniform(70 + s, 0, case.n, -1, 1).reshape(case.shape)).to("cuda", dt) for s in range(2)]
+
+    def solve(sim, b, n):
+        x = torch.zeros_like(b)
+        sim.poisson_solve(b, x, 1e-30, n, allow_not_converged=True)
+        return x.cpu()
+
+    fresh = {(s, n): solve(les_mod.Simulation(case), bs[s], n) for s in range(2) for n in (7, 30)}
+    sim = les_mod.Simulation(case)
+    for s, n in [(0, 30), (1, 30), (1, 7), (0, 30), (0, 7), (1, 30)]:
+        assert torch.equal(solve(sim, bs[s], n), fresh[s, n]), (s, n)
