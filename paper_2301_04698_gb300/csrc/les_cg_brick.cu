@@ -12,12 +12,13 @@
 // What bounds it: instruction issue (about 75 per node and iteration) and shared
 // memory, 12 accesses per node and iteration (five neighbours twice, p read and
 // written).  Measured (GB300, us per iteration; before: the streaming kernels,
-// which take 27 to 36 bytes per node through L2): 192 x 192 x 128 38.2 -> 18.5,
-// 160 x 160 x 128 30.6 -> 14.7, 256 x 256 x 64 39.0 -> 18.4, 150 x 130 x 110 23.3 ->
-// 13.1.  Bricks of any extents, with their strides and column offsets in registers,
+// which take 27 to 36 bytes per node through L2): 192 x 192 x 128 38.2 -> 18.2,
+// 160 x 160 x 128 30.6 -> 12.7, 256 x 256 x 64 39.0 -> 17.5, 150 x 130 x 110 23.3 ->
+// 12.1.  Bricks of any extents, with their strides and column offsets in registers,
 // spilled r and took 53 us on the first of these.
 #include <algorithm>
 #include <string>
+#include <type_traits>
 
 #include "les_chip.cuh"
 
@@ -60,20 +61,29 @@ __global__ void __launch_bounds__(BX* BY, 1) k_cg_brick(ChipArgs<float> f) {
   const bool flow = own && f.pz > 1 && !low, fhigh = own && f.pz > 1 && !high;
   auto is_face = [&](int j) { return fcol || (flow && j == 0) || (fhigh && j == bz - 1); };
 
-  // body(id, place in P, offset in global memory) for the brick's ghost nodes: the
-  // z faces by column, the y faces a warp per row, the x faces a half warp per plane
-  auto each_ghost = [&](auto&& body) {
-    if (own && f.pz > 1) {
-      if (!low) body(tid, C - SZ, chip_wrap(k0 - 1, f.nz) * gpl + (j0 + warp) * f.nx + i0 + lane);
-      if (!high) body(BX * BY + tid, C + SZ * bz, chip_wrap(k0 + bz, f.nz) * gpl + (j0 + warp) * f.nx + i0 + lane);
-    }
+  // body(id, place in P, offset in global memory) for the brick's ghost nodes, by the
+  // warps from W0 on: the z faces a warp per row, the y faces a warp per row, the x faces
+  // a half warp per plane
+  auto each_ghost = [&](auto first, auto&& body) {
+    constexpr int W0 = decltype(first)::value, NW = BY - W0;
+    if (warp < W0) return;
+    if (f.pz > 1)
+#pragma unroll
+      for (int y = warp - W0; y < BY; y += NW) {
+        float* at = P + (y + 1) * SY + lane + 1;
+        const int g = (j0 + y) * f.nx + i0 + lane;
+        if (lane < bx && y < by) {
+          if (!low) body(y * BX + lane, at, chip_wrap(k0 - 1, f.nz) * gpl + g);
+          if (!high) body((BY + y) * BX + lane, at + SZ * (bz + 1), chip_wrap(k0 + bz, f.nz) * gpl + g);
+        }
+      }
     int id0 = 2 * BX * BY;
 #pragma unroll
     for (int side = 0; side < 2; ++side) {
       const int g = k0 * gpl + chip_wrap(side ? j0 + by : j0 - 1, f.ny) * f.nx + i0 + lane;
       float* at = P + SZ + (side ? (by + 1) * SY : 0) + lane + 1;
       if (lane < bx)
-        for (int z = warp; z < bz; z += BY) body(id0 + z * BX + lane, at + z * SZ, g + z * gpl);
+        for (int z = warp - W0; z < bz; z += NW) body(id0 + z * BX + lane, at + z * SZ, g + z * gpl);
       id0 += ZP * BX;
     }
     const int y = lane & 15;
@@ -82,10 +92,13 @@ __global__ void __launch_bounds__(BX* BY, 1) k_cg_brick(ChipArgs<float> f) {
       const int g = k0 * gpl + (j0 + y) * f.nx + chip_wrap(side ? i0 + bx : i0 - 1, f.nx);
       float* at = P + SZ + (y + 1) * SY + (side ? bx + 1 : 0);
       if (y < by)
-        for (int z = 2 * warp + (lane >> 4); z < bz; z += 2 * BY) body(id0 + z * BY + y, at + z * SZ, g + z * gpl);
+        for (int z = 2 * (warp - W0) + (lane >> 4); z < bz; z += 2 * NW)
+          body(id0 + z * BY + y, at + z * SZ, g + z * gpl);
       id0 += ZP * BY;
     }
   };
+  using AllWarps = std::integral_constant<int, 0>;
+  using GhostWarps = std::integral_constant<int, kFoldWarps<F2>>;
   static_assert(BX == 32 && BY == 16, "the ghost loops' mapping");
 
   float r[ZP] = {};
@@ -119,7 +132,7 @@ __global__ void __launch_bounds__(BX* BY, 1) k_cg_brick(ChipArgs<float> f) {
   };
   // A at the ghost nodes into P (keep: as r there too), outside the iterations
   auto fill_ghosts = [&](const float* A, bool keep) {
-    each_ghost([&](int id, float* at, int g) {
+    each_ghost(AllWarps{}, [&](int id, float* at, int g) {
       const float v = __ldcg(A + g);
       *at = v;
       if (keep) GR[id] = v;
@@ -148,6 +161,9 @@ __global__ void __launch_bounds__(BX* BY, 1) k_cg_brick(ChipArgs<float> f) {
   double rr = 0.0, bb = 0.0, rel = 0.0;  // meaningful in thread 0
   int status = 0;  // 0 running, 1 converged, 2 maxit, 3 breakdown, 4 zero rhs, 5 timeout
   float rr_own = 0.f;  // this thread's share of r.r for the next sum
+
+  chip_sum_clear<F2>(f.spread);  // no tag of an earlier solve: cleared here, for everyone after the first sum
+  if (tid == 0) s_fail = 0;
 
   // mean of b (b held in r)
   {
@@ -256,10 +272,13 @@ __global__ void __launch_bounds__(BX* BY, 1) k_cg_brick(ChipArgs<float> f) {
         d2.add(j, r[j] * q);
         d3.add(j, q * q);
       });
-      chip_sum<true>(f, iter, d0.total(own), rr_own, d2.total(own), d3.total(own), shv, part, tot, s_fail, ChipNothing{}, [&] {
-        each_ghost([&](int id, float*, int g) { cp_async(GQ + id, qw + g); });
-        cp_commit();
-      });
+      chip_sum<GhostWarps::value, 3>(
+          f, iter, d0.total(own), rr_own, d2.total(own), d3.total(own), shv, part, tot, s_fail, ChipNothing{},
+          [&] {
+            each_ghost(GhostWarps{}, [&](int id, float*, int g) { cp_async(GQ + id, qw + g); });
+            cp_commit();
+          },
+          ChipNothing{});
       if (tid == 0) {  // the status, alpha and beta
         int st = 0;
         if (s_fail) {
@@ -311,7 +330,7 @@ __global__ void __launch_bounds__(BX* BY, 1) k_cg_brick(ChipArgs<float> f) {
           g += 8 * gpl;
         }
       }
-      each_ghost([&](int id, float* at, int) {
+      each_ghost(AllWarps{}, [&](int id, float* at, int) {
         const float rv = GR[id] - ta * GQ[id];
         GR[id] = rv;
         *at = rv + tb * *at;

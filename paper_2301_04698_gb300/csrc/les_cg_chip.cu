@@ -21,12 +21,12 @@
 //
 // The iteration is that of les_cg_resident.cu: one grid-wide sum of p.q,
 // r.r, r.q and q.q per iteration (alpha, and beta from |r - alpha q|^2
-// expanded in the four).  With XS = false the sum's partials and the faces' q are
-// tagged words (les_chip.cuh); with more faces these cost more than they save (150 x
-// 140 x 70 FP32: 13 us per iteration instead of 8.7), and the counters order them.
+// expanded in the four; les_chip.cuh).  With XS = false the faces' q are tagged words;
+// with more faces these cost more than they save (150 x 140 x 70 FP32: 13 us per
+// iteration instead of 9.3), and counters order them.
 //
-// What bounds it: the latency of the grid sum (2.2 us of an iteration on the
-// smallest grids; 2.6 with counters) and, in FP64, the
+// What bounds it: the latency of the grid sum (2.1 us of an iteration on the
+// smallest grids) and, in FP64, the
 // arithmetic: a scheduler issues an FP64 warp instruction every 64 cycles, so
 // a five-step butterfly of four values in 16 warps alone costs 5000 cycles.
 // The four values are therefore reduced by a transposing butterfly (six
@@ -37,13 +37,13 @@
 // Measured (GB300, us per iteration; before: the
 // shared-memory kernel, or the one-pass streaming kernel where no whole
 // bricks fit):
-//   FP64  32^3 9.9 -> 4.6, 256 x 4 x 32 10.1 -> 4.7, 64 x 64 x 48 16.9 -> 9.3,
-//         50 x 47 x 33 28.3 -> 7.2, 77 x 130 x 50 66.8 -> 16.7, 96^3 77 -> 26
-//   FP32  32^3 4.2 -> 2.2, 64^3 5.0 -> 3.0, 96^3 7.3 -> 5.5, 160 x 160 x 48
-//         8.4 -> 6.2, 100 x 76 x 61 23.6 -> 4.0, 150 x 140 x 70 36.7 -> 8.7
+//   FP64  32^3 9.9 -> 4.7, 256 x 4 x 32 10.1 -> 4.7, 64 x 64 x 48 16.9 -> 9.3,
+//         50 x 47 x 33 28.3 -> 6.8, 77 x 130 x 50 66.8 -> 16.4, 96^3 77 -> 26.5
+//   FP32  32^3 4.2 -> 2.1, 64^3 5.0 -> 2.9, 96^3 7.3 -> 5.0, 160 x 160 x 48
+//         8.4 -> 6.0, 100 x 76 x 61 23.6 -> 3.85, 150 x 140 x 70 36.7 -> 9.3
 // FP32 grids 128 nodes wide keep les_cg_regs.cu, whose four-node lanes read
-// x neighbours by shuffles: 128 x 64 x 64 3.5 there, 4.6 here; 128 x 128 x 96
-// 5.3 and 8.9.
+// x neighbours by shuffles: 128 x 64 x 64 2.8 there, 4.1 here; 128 x 128 x 96
+// 5.0 and 8.4.
 #include <algorithm>
 #include <string>
 
@@ -212,16 +212,16 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
   T rr_own = T(0);  // this thread's share of r.r for the next sum
 
   // XS = false: a node's tagged word among the published faces of q
-  constexpr int W = 2 * (int)sizeof(T);
+  constexpr int W = Tagged<T>::BYTES;
   const int half = (int)(f.n / 2);
   auto word = [&](int s, int g) { return (g < half ? f.qt[0][s] : f.qt[1][s] - (size_t)half * W) + (size_t)g * W; };
-  if constexpr (!XS) {  // no tag of an earlier solve: cleared here, for everyone after the first sum
-    chip_sum_clear(f.spread);
+  chip_sum_clear<Acc>(f.spread);  // no tag of an earlier solve: cleared here, for everyone after the first sum
+  if constexpr (!XS) {
 #pragma unroll
     for (int j = 0; j < ZP; ++j)
       if (j < nzp && is_face(j)) {
-        tagged_store(word(0, gown + j * gpl), T(0), 0u);
-        tagged_store(word(1, gown + j * gpl), T(0), 0u);
+        tagged_clear<T>(word(0, gown + j * gpl));
+        tagged_clear<T>(word(1, gown + j * gpl));
       }
   }
   if (tid == 0) s_fail = 0;
@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
           q[j] = stencil(j);
           if (is_face(j)) {
             if constexpr (XS) __stcg(qw + gown + j * gpl, q[j]);
-            else tagged_store(word(iter & 1, gown + j * gpl), q[j], chip_tag(iter));
+            else tagged_store(word(iter & 1, gown + j * gpl), q[j], iter);
           }
           d0 += p[j] * q[j];
           d2 += r[j] * q[j];
@@ -347,6 +347,7 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
         }
       Tagged<T> gq[NG];  // the q of the ghosts
       Acc tot[4];        // the totals, in warp 0
+      constexpr int WORDS = sizeof(T) == 8 && ZP < 10 ? 5 : 3;
       auto deferred = [&] {
         if constexpr (kDefer) {
           if (iter > 0) {
@@ -356,15 +357,19 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
         }
       };
       if constexpr (XS) {
-        chip_sum<false>(f, iter, d0, rr_own, d2, d3, shv, part, tot, s_fail, deferred, [&] {
-          for (int id = tid; id < ngh; id += nthr) cp_async(GQ + id, qw + GT[id].y);
-          cp_commit();
-        });
+        chip_sum<1, WORDS>(
+            f, iter, d0, rr_own, d2, d3, shv, part, tot, s_fail, deferred,
+            [&] {
+              const int t0 = 32 * chip_ghost_warp<1>();
+              for (int id = tid - t0; id < ngh; id += nthr - t0) cp_async(GQ + id, qw + GT[id].y);
+              cp_commit();
+            },
+            ChipNothing{});
       } else {
         unsigned miss = 0;
 #pragma unroll
         for (int g = 0; g < NG; ++g) miss |= gsm[g] >= 0 ? 1u << g : 0u;
-        chip_sum_tagged(
+        chip_sum<-1, WORDS>(
             f, iter, d0, rr_own, d2, d3, shv, part, tot, s_fail, deferred,
             [&] {
 #pragma unroll
@@ -374,7 +379,7 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
             [&] {
 #pragma unroll
               for (int g = 0; g < NG; ++g)
-                if ((miss >> g & 1u) && tagged_ok(gq[g], chip_tag(iter))) miss &= ~(1u << g);
+                if ((miss >> g & 1u) && tagged_ok(gq[g], iter)) miss &= ~(1u << g);
               return miss == 0u;
             });
       }
@@ -624,8 +629,7 @@ int poisson_solve_chip(const SolverArgs<T>& a, const FusedCfg& fc, const T* b, T
   f.qt[0][1] = reinterpret_cast<char*>(a.q);
   f.qt[1][1] = reinterpret_cast<char*>(a.r);
   f.partials = a.partials;
-  // past the set-up sums' two slots: the counters, then the copies of the
-  // iterations' partials (2 x kChipSpread x 4 words per block)
+  // past the set-up sums' two slots: the counters, then the iterations' partials
   f.counters = reinterpret_cast<unsigned*>(a.partials + 2 * (size_t)kSumSlot * G);
   f.spread = a.partials + 2 * (size_t)kSumSlot * G + kChipSpread * kChipLine / 2;
   f.missing = (unsigned)std::max(0, fc.missing);

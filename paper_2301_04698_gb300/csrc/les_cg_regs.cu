@@ -25,35 +25,28 @@
 // solver in les_cg_resident.cu):
 //   matvec   q = L_c p; the q faces a neighbour reads are published;
 //            p.q, r.q and q.q (r.r was formed with r, in the update)
-//   sum      each warp reduces its four values in FP32 (a transposing
-//            butterfly: six shuffles for all four); warp 0 combines the
-//            warps' values as compensated FP32 pairs, writes them into
-//            kSpread copies and arrives on one of kSpread counters (block b
-//            on counter b mod kSpread), and its lanes 0 .. kSpread - 1 wait
-//            for one counter each (the grid sum of les_gridsync.cuh, with
-//            its arrivals and reads spread over as many L2 lines); then
-//            warps 0 .. 3 fold one value each from the block's copy, in
-//            block order, while the other warps copy the neighbours' q
-//            faces into shared memory asynchronously; thread 0 forms
-//            alpha and beta = |r - alpha q|^2 / r.r from the totals
+//   sum      that of les_chip.cuh (chip_sum); once it has come the neighbours'
+//            q faces are copied into shared memory asynchronously; thread 0
+//            forms alpha and beta = |r - alpha q|^2 / r.r from the totals
 //   update   r -= alpha q, p = r + beta p (registers and the shared copy of
 //            p); at the ghost nodes r -= alpha q_ghost and p = r + beta p;
 //            x += alpha p in warp 0, while the other warps keep p and add
 //            alpha p to x during the next sum's wait, when they are idle
+// The arithmetic takes two nodes per instruction (packed FP32).
+//
+// What bounds it: the grid sum (2.1 us of an iteration) and shared memory.  Measured
+// (GB300, us per iteration): 128 x 64 x 32 2.4, 128 x 64 x 64 2.8, 128 x 128 x 96 5.0;
+// with a sum whose partials were released and then read 3.0, 3.35, 5.1.
 #include <algorithm>
 #include <string>
 
-#include "les_gridsync.cuh"
-#include "les_internal.h"
+#include "les_chip.cuh"
 
 namespace les {
 namespace {
 
 constexpr int kRegNx = 128;       // grid width: 32 lanes x 4 nodes
-constexpr int kRegMaxWarps = 16;  // 512 threads of at most 128 registers
-constexpr int kSpread = 8;        // arrival counters and copies of the partials per sum
-constexpr int kLineWords = 32;    // counters 128 bytes apart
-static_assert(kSpread * 4 == 32, "one lane of warp 0 per (copy, value) of the partials");
+constexpr int kRegMaxWarps = kChipWarps;  // 512 threads of at most 128 registers
 
 struct RegArgs {
   int ny, nz, walls;
@@ -67,8 +60,8 @@ struct RegArgs {
   float* qg0;        // published faces of q, even iterations
   float* qg1;        // ... odd iterations
   double* partials;  // two slots of kSumSlot words per block (the set-up and gauge sums)
-  unsigned* counters;  // kSpread arrival counters of the iterations' sums, kLineWords apart, zeroed
-  F2* spread;          // [2 slots][kSpread copies][4 values][gridDim.x] partials of those sums
+  unsigned* counters;  // as in ChipArgs
+  void* spread;
   unsigned missing;    // test hook: arrivals on counter 0 that never come
   FusedBar* bar;
   SolverCtl* ctl;
@@ -113,18 +106,19 @@ __global__ void __launch_bounds__(kRegMaxWarps * 32, 1) k_cg_regs(RegArgs f) {
   const float cx = f.cx, cy = f.cy, cz = f.cz;
   // this thread's own rows: plane j of its run lies at pown + j SZ in P,
   // xown + j xpl in X and gown + j gpl in global memory (never wrapped)
-  const int pown = (z0 + 1) * SZ + (ly + 1) * kRegNx + x4;
-  const int xpl = by * kRegNx, xown = (z0 * by + ly) * kRegNx + x4;
-  const size_t gpl = (size_t)f.ny * kRegNx;
-  const size_t gown = ((size_t)(k0 + z0) * f.ny + j0 + ly) * kRegNx + x4;
+  int pown = (z0 + 1) * SZ + (ly + 1) * kRegNx + x4;
+  const int xpl = by * kRegNx;
+  int xown = (z0 * by + ly) * kRegNx + x4;
+  const int gpl = f.ny * kRegNx;
+  int gown = ((k0 + z0) * f.ny + j0 + ly) * kRegNx + x4;
   const bool frow = ly == 0 || ly == by - 1;  // a y face: every plane is read by a neighbour
 
   auto prow = [&](int y, int z) { return (z + 1) * SZ + (y + 1) * kRegNx; };
   // global start of brick row (y, z), at most one node outside the brick
-  auto grow = [&](int y, int z) -> size_t {
+  auto grow = [&](int y, int z) -> int {
     int j = j0 + y;
     j = j < 0 ? j + f.ny : (j >= f.ny ? j - f.ny : j);
-    return ((size_t)reg_zghost(k0 + z, f.nz, f.walls) * f.ny + j) * kRegNx;
+    return (reg_zghost(k0 + z, f.nz, f.walls) * f.ny + j) * kRegNx;
   };
   auto ghost_row = [&](int row, int& y, int& z) {
     if (row < 2 * by) {
@@ -159,12 +153,14 @@ __global__ void __launch_bounds__(kRegMaxWarps * 32, 1) k_cg_regs(RegArgs f) {
     const float4 nn = lds4(pj + kRegNx);
     const float4 d = j > 0 ? p[j > 0 ? j - 1 : 0] : lds4(pj - SZ);
     const float4 u = (j + 1 < ZP && j + 1 < nzp) ? p[j + 1 < ZP ? j + 1 : ZP - 1] : lds4(pj + SZ);
-    auto node = [&](float pc, float pw, float pe, float ps, float pn, float pd, float pu) {
-      const float c2 = 2.f * pc;
-      return (pw + pe - c2) * cx + (ps + pn - c2) * cy + (pd + pu - c2) * cz;
+    // a pair of nodes from the sums of its neighbours along x, and those in y and z
+    auto pair = [&](float2 pc, float2 sx, float2 ps, float2 pn, float2 pd, float2 pu) {
+      const float2 tx = __ffma2_rn(pc, f32x2(-2.f), sx), ty = __ffma2_rn(pc, f32x2(-2.f), __fadd2_rn(ps, pn)),
+                   tz = __ffma2_rn(pc, f32x2(-2.f), __fadd2_rn(pd, pu));
+      return __ffma2_rn(tz, f32x2(cz), __ffma2_rn(ty, f32x2(cy), __fmul2_rn(tx, f32x2(cx))));
     };
-    return make_float4(node(c.x, w0, c.y, s.x, nn.x, d.x, u.x), node(c.y, c.x, c.z, s.y, nn.y, d.y, u.y),
-                       node(c.z, c.y, c.w, s.z, nn.z, d.z, u.z), node(c.w, c.z, e3, s.w, nn.w, d.w, u.w));
+    return join2(pair(lo2(c), float2{w0 + c.y, c.x + c.z}, lo2(s), lo2(nn), lo2(d), lo2(u)),
+                 pair(hi2(c), float2{c.y + c.w, c.z + e3}, hi2(s), hi2(nn), hi2(d), hi2(u)));
   };
 
   GridSync gs{f.bar, f.partials, f.spin_cycles, f.expected, 0u};
@@ -173,14 +169,18 @@ __global__ void __launch_bounds__(kRegMaxWarps * 32, 1) k_cg_regs(RegArgs f) {
     float mean, ta, tb;
     int status;
   } sc;
-  __shared__ float shv[4][kRegMaxWarps];
-  __shared__ F2 tot[4];
+  __shared__ float shv[4][kChipWarps];
+  __shared__ F2 part[32];
+  F2 tot[4];  // in warp 0
   __shared__ int s_fail;
   double rr = 0.0, bb = 0.0, rel = 0.0;  // meaningful in thread 0
   int status = 0;  // 0 running, 1 converged, 2 maxit, 3 breakdown, 4 zero rhs, 5 timeout
   // this thread's share of r.r for the next sum, formed where r is (the
   // initial residual, then each update), in the order the sums expect
   float rr_own = 0.f;
+
+  chip_sum_clear<F2>(f.spread);  // no tag of an earlier solve: cleared here, for everyone after the first sum
+  if (tid == 0) s_fail = 0;
 
   // mean of b (b held in r)
   {
@@ -273,7 +273,6 @@ __global__ void __launch_bounds__(kRegMaxWarps * 32, 1) k_cg_regs(RegArgs f) {
   acc_from(rr, rr_last);
   int iter = 0;
   float ta = 0.f, tb = 0.f;
-  unsigned it_sum = 0;  // sums of the iterations completed
   if (!status) {
     // p_0 = r_0, with r_0 at the ghost nodes from the published faces
     __syncthreads();  // the initial residual's stencil reads of the copy are done
@@ -286,224 +285,81 @@ __global__ void __launch_bounds__(kRegMaxWarps * 32, 1) k_cg_regs(RegArgs f) {
     fill_ghosts(f.rg, true);
     __syncthreads();
     for (;;) {
+      // the places of the planes are formed anew in each iteration: hoisted out of the
+      // loop they would take the registers of the vectors
+      asm volatile("" : "+r"(pown), "+r"(xown), "+r"(gown));
       float* qw = (iter & 1) ? f.qg1 : f.qg0;  // this iteration's q faces
-      Dot<float> d[4];                         // p.q, r.r, r.q, q.q
+      float2 d0{0.f, 0.f}, d2{0.f, 0.f}, d3{0.f, 0.f};  // p.q, r.q, q.q
 #pragma unroll
       for (int j = 0; j < ZP; ++j)
         if (j < nzp) {
           q[j] = stencil(j);
           if (is_face(j)) stg4(qw + gown + j * gpl, q[j]);
-          d[0].add(p[j].x * q[j].x);
-          d[0].add(p[j].y * q[j].y);
-          d[0].add(p[j].z * q[j].z);
-          d[0].add(p[j].w * q[j].w);
-          d[2].add(r[j].x * q[j].x);
-          d[2].add(r[j].y * q[j].y);
-          d[2].add(r[j].z * q[j].z);
-          d[2].add(r[j].w * q[j].w);
-          d[3].add(q[j].x * q[j].x);
-          d[3].add(q[j].y * q[j].y);
-          d[3].add(q[j].z * q[j].z);
-          d[3].add(q[j].w * q[j].w);
+          dot4(d0, p[j], q[j]);
+          dot4(d2, r[j], q[j]);
+          dot4(d3, q[j], q[j]);
         }
-      d[1].s = rr_own;
-      // the grid sum.  Each warp's four values in FP32 by a transposing
-      // butterfly: after it lanes 8k .. 8k + 7 hold the warp's value k.
-      {
-        const bool up = lane & 16, odd = lane & 8;
-        float a0 = up ? d[2].s : d[0].s, a1 = up ? d[3].s : d[1].s;        // kept
-        const float s0 = up ? d[0].s : d[2].s, s1 = up ? d[1].s : d[3].s;  // given to lane ^ 16
-        a0 += __shfl_xor_sync(0xffffffffu, s0, 16);
-        a1 += __shfl_xor_sync(0xffffffffu, s1, 16);
-        float v = odd ? a1 : a0;
-        v += __shfl_xor_sync(0xffffffffu, odd ? a0 : a1, 8);
-        v += __shfl_xor_sync(0xffffffffu, v, 4);
-        v += __shfl_xor_sync(0xffffffffu, v, 2);
-        v += __shfl_xor_sync(0xffffffffu, v, 1);
-        if ((lane & 7) == 0) shv[lane >> 3][warp] = v;
-      }
-      // also orders every thread's q-face stores before warp 0's release
-      __syncthreads();
-      const unsigned G = gridDim.x;
-      // this sum's partials: kSpread copies, so that the blocks' reads of
-      // them spread over as many L2 lines; this block reads copy b mod kSpread
-      F2* slot = f.spread + (size_t)(it_sum & 1u) * kSpread * 4 * G;
-      if (warp == 0) {
-        // lanes 8k .. 8k + 7: value k of the block as a compensated pair
-        const int k = lane >> 3;
-        F2 a = F2{0.f, 0.f};
-        for (int w = lane & 7; w < nwarp; w += 8) a = f2_add(a, F2{shv[k][w], 0.f});
+      chip_sum<kFoldWarps<F2>, 3>(
+          f, iter, d0.x + d0.y, rr_own, d2.x + d2.y, d3.x + d3.y, shv, part, tot, s_fail,
+          [&] {  // the last iteration's x += alpha p of this warp's rows, deferred from its update
+            if (iter > 0) {
 #pragma unroll
-        for (int o = 4; o > 0; o >>= 1)
-          a = f2_add(a, F2{__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)});
-        // lane l writes value l mod 4 into copy l / 4
-        const int src = 8 * (lane & 3);
-        const F2 mine = F2{__shfl_sync(0xffffffffu, a.hi, src), __shfl_sync(0xffffffffu, a.lo, src)};
-        acc_store(slot + ((size_t)(lane >> 2) * 4 + (lane & 3)) * G + blockIdx.x, mine);
-        // orders the lanes' stores before lane 0's release
-        __syncwarp();
-        if (lane == 0) red_release_add(f.counters + (blockIdx.x % kSpread) * kLineWords, 1u);
-        // posted: the other warps may start on shared memory
-        asm volatile("bar.arrive 2, %0;" ::"r"(nthr) : "memory");
-        // lanes 0 .. kSpread - 1 wait for the arrivals on one counter each
-        // (counter i takes blocks i, i + kSpread, ...; counter 0 also the
-        // test hook's missing ones)
-        bool done = lane >= kSpread;
-        const unsigned mine_n = lane < (int)G ? (G - lane + kSpread - 1) / kSpread : 0u;
-        const unsigned target = done ? 0u : (it_sum + 1u) * (mine_n + (lane == 0 ? f.missing : 0u));
-        const long long t0 = clock64();
-        int fail = 0;
-        for (unsigned spins = 1;; ++spins) {
-          if (!done) done = (int)(ld_acquire(f.counters + lane * kLineWords) - target) >= 0;
-          if (__all_sync(0xffffffffu, done)) break;
-          const bool quit = (spins & 63u) == 0u && (ld_volatile(&gs.bar->fail.v) != 0u || clock64() - t0 > gs.spin);
-          if (__any_sync(0xffffffffu, quit)) {
-            if (lane == 0) atomicExch(&gs.bar->fail.v, 1u);
-            fail = 1;
-            break;
-          }
-        }
-        // orders the lanes' acquires before the reads of every lane
-        __syncwarp();
-        if (lane == 0) s_fail = fail;
-        // every block has arrived (or the wait gave up): the other warps may
-        // read the partials and the q faces published before the arrivals
-        asm volatile("bar.arrive 1, %0;" ::"r"(nthr) : "memory");
-      } else {
-        // while warp 0 waits: the last iteration's x += alpha p of this
-        // warp's rows (deferred from its update), once warp 0 has posted
-        asm volatile("bar.sync 2, %0;" ::"r"(nthr) : "memory");
-        if (iter > 0) {
-#pragma unroll
-          for (int j = 0; j < ZP; ++j)
-            if (j < nzp) {
-              float4 xv = lds4(X + xown + j * xpl);
-              const float4 pv = lds4(PO + xown + j * xpl);
-              xv.x += ta * pv.x;
-              xv.y += ta * pv.y;
-              xv.z += ta * pv.z;
-              xv.w += ta * pv.w;
-              sts4(X + xown + j * xpl, xv);
+              for (int j = 0; j < ZP; ++j)
+                if (j < nzp)
+                  sts4(X + xown + j * xpl, fma4(ta, lds4(PO + xown + j * xpl), lds4(X + xown + j * xpl)));
             }
-        }
-        asm volatile("bar.sync 1, %0;" ::"r"(nthr) : "memory");
-      }
-      const F2* mycopy = slot + (size_t)(blockIdx.x % kSpread) * 4 * G;
-      // warps 0 .. 3 fold one value each (in block order, so every block
-      // obtains the same totals) while the others copy the ghost rows of q
-      // into GQ (every warp, after its folds, in a block of four warps or
-      // fewer)
-      const int l0 = nwarp > 4 ? 4 : 0;
-      if (warp >= l0) {
-        for (int row = warp - l0; row < nr; row += nwarp - l0) {
-          int y, z;
-          ghost_row(row, y, z);
-          cp_async_bytes<16>(GQ + row * kRegNx + x4, qw + grow(y, z) + x4);
-        }
-        cp_commit();
-      }
-      if (warp < 4) {
-        for (int k = warp; k < 4; k += nwarp) {
-          F2 t = F2{0.f, 0.f};
-          for (unsigned b0 = lane; b0 < G; b0 += 32 * 5) {
-            F2 w[5];
-#pragma unroll
-            for (int u = 0; u < 5; ++u)
-              w[u] = b0 + 32 * u < G ? acc_load(mycopy + (size_t)k * G + b0 + 32 * u) : F2{0.f, 0.f};
-#pragma unroll
-            for (int u = 0; u < 5; ++u) t = f2_add(t, w[u]);
-          }
-          t = warp_sum_f2(t);
-          if (lane == 0) tot[k] = t;
-        }
-        // the folds are complete: thread 0 forms the status, alpha and beta
-        asm volatile("bar.sync 3, %0;" ::"r"(32 * min(nwarp, 4)) : "memory");
-        if (tid == 0) {
-          int st = 0;
-          if (s_fail) {
-            st = 5;
-          } else {
-            const F2 t1 = tot[1];
-            rr_last = t1;
-            if (acc_le(t1, rr_stop)) st = 1;
-            else if (iter >= f.maxit) st = 2;
-            else {
-              const float pq = tot[0].hi, r2 = t1.hi, rq = tot[2].hi, q2 = tot[3].hi;
-              if (!(pq != 0.f) || !isfinite(pq) || !isfinite(r2)) {
-                st = 3;
-              } else {
-                const float alpha = r2 / pq;
-                const float rn = fmaf(alpha * alpha, q2, fmaf(-2.f * alpha, rq, r2));  // |r - alpha q|^2
-                sc.ta = alpha;
-                sc.tb = rn / r2;
-              }
+          },
+          [&] {  // the neighbours' q at the ghost rows
+            const int l0 = chip_ghost_warp<kFoldWarps<F2>>();
+            for (int row = warp - l0; row < nr; row += nwarp - l0) {
+              int y, z;
+              ghost_row(row, y, z);
+              cp_async_bytes<16>(GQ + row * kRegNx + x4, qw + grow(y, z) + x4);
             }
-          }
-          sc.status = st;
+            cp_commit();
+          },
+          ChipNothing{});
+      if (tid == 0) {  // the status, alpha and beta
+        int st = 0;
+        float al = 0.f, be = 0.f;
+        if (s_fail) {
+          st = 5;
+        } else {
+          rr_last = tot[1];
+          if (acc_le(tot[1], rr_stop)) st = 1;
+          else if (iter >= f.maxit) st = 2;
+          else if (!chip_scalars(tot, al, be)) st = 3;
         }
-      }
-      if (!l0) {
-        for (int row = warp; row < nr; row += nwarp) {
-          int y, z;
-          ghost_row(row, y, z);
-          cp_async_bytes<16>(GQ + row * kRegNx + x4, qw + grow(y, z) + x4);
-        }
-        cp_commit();
+        sc.ta = al;
+        sc.tb = be;
+        sc.status = st;
       }
       cp_wait<0>();
-      it_sum += 1u;
       __syncthreads();
       status = sc.status;
       if (status) break;
       ta = sc.ta;
       tb = sc.tb;
-      float rr_new = 0.f;
+      float2 rr_new{0.f, 0.f};
 #pragma unroll
       for (int j = 0; j < ZP; ++j)
         if (j < nzp) {
-          if (warp == 0) {
-            float4 xv = lds4(X + xown + j * xpl);
-            xv.x += ta * p[j].x;
-            xv.y += ta * p[j].y;
-            xv.z += ta * p[j].z;
-            xv.w += ta * p[j].w;
-            sts4(X + xown + j * xpl, xv);
-          } else {
-            sts4(PO + xown + j * xpl, p[j]);
-          }
-          r[j].x -= ta * q[j].x;
-          r[j].y -= ta * q[j].y;
-          r[j].z -= ta * q[j].z;
-          r[j].w -= ta * q[j].w;
-          rr_new += r[j].x * r[j].x;
-          rr_new += r[j].y * r[j].y;
-          rr_new += r[j].z * r[j].z;
-          rr_new += r[j].w * r[j].w;
-          p[j].x = r[j].x + tb * p[j].x;
-          p[j].y = r[j].y + tb * p[j].y;
-          p[j].z = r[j].z + tb * p[j].z;
-          p[j].w = r[j].w + tb * p[j].w;
+          if (warp == 0) sts4(X + xown + j * xpl, fma4(ta, p[j], lds4(X + xown + j * xpl)));
+          else sts4(PO + xown + j * xpl, p[j]);
+          r[j] = fma4(-ta, q[j], r[j]);
+          dot4(rr_new, r[j], r[j]);
+          p[j] = fma4(tb, p[j], r[j]);
           sts4(P + pown + j * SZ, p[j]);
         }
       for (int row = warp; row < nr; row += nwarp) {
         int y, z;
         ghost_row(row, y, z);
-        const float4 gq = lds4(GQ + row * kRegNx + x4);
-        float4 rv = lds4(RG + row * kRegNx + x4);
-        rv.x -= ta * gq.x;
-        rv.y -= ta * gq.y;
-        rv.z -= ta * gq.z;
-        rv.w -= ta * gq.w;
+        const float4 rv = fma4(-ta, lds4(GQ + row * kRegNx + x4), lds4(RG + row * kRegNx + x4));
         sts4(RG + row * kRegNx + x4, rv);
         float* pg = P + prow(y, z) + x4;
-        float4 pv = lds4(pg);
-        pv.x = rv.x + tb * pv.x;
-        pv.y = rv.y + tb * pv.y;
-        pv.z = rv.z + tb * pv.z;
-        pv.w = rv.w + tb * pv.w;
-        sts4(pg, pv);
+        sts4(pg, fma4(tb, lds4(pg), rv));
       }
-      rr_own = rr_new;
+      rr_own = rr_new.x + rr_new.y;
       iter += 1;
       __syncthreads();
     }
@@ -657,10 +513,9 @@ int poisson_solve_regs(const SolverArgs<float>& a, const FusedCfg& fc, const flo
   f.qg0 = a.p0;
   f.qg1 = a.p1;
   f.partials = a.partials;
-  // past the set-up sums' two slots: the counters, then the copies of the
-  // iterations' partials (2 x kSpread x 4 words per block)
+  // past the set-up sums' two slots: the counters, then the iterations' partials
   f.counters = reinterpret_cast<unsigned*>(a.partials + 2 * (size_t)kSumSlot * pl.G);
-  f.spread = reinterpret_cast<F2*>(a.partials + 2 * (size_t)kSumSlot * pl.G + kSpread * kLineWords / 2);
+  f.spread = a.partials + 2 * (size_t)kSumSlot * pl.G + kChipSpread * kChipLine / 2;
   f.missing = (unsigned)std::max(0, fc.missing);
   f.bar = a.bar;
   f.ctl = a.ctl;
@@ -672,7 +527,7 @@ int poisson_solve_regs(const SolverArgs<float>& a, const FusedCfg& fc, const flo
   f.expected = (unsigned)pl.G;
   *used = true;
   if ((e = cudaMemsetAsync(a.bar, 0, sizeof(FusedBar), a.st)) != cudaSuccess ||
-      (e = cudaMemsetAsync(f.counters, 0, kSpread * kLineWords * sizeof(unsigned), a.st)) != cudaSuccess) {
+      (e = cudaMemsetAsync(f.counters, 0, kChipSpread * kChipLine * sizeof(unsigned), a.st)) != cudaSuccess) {
     if (err) *err = std::string("register CG barrier reset: ") + cudaGetErrorString(e);
     return LES_ERR_CUDA;
   }
