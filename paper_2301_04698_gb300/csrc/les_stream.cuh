@@ -103,17 +103,53 @@ using Tile64 = StreamTile<64, 16>;
 using Tile32 = StreamTile<32, 32>;
 using Tile32s = StreamTile<32, 16>;
 
+// The work of a launch: units (a tile's run of planes) dealt to the blocks in turns,
+// nchunk runs per tile; or (nchunk = 0) the planes of all tiles one after the other in
+// equal shares, a share being the end of one tile's planes and the beginning of
+// another's.
 struct StreamPlan {
   int shape = 0, ntx = 0, nty = 0, nchunk = 1;
-  long long units = 0;
+  long long units = 0;  // units, or planes
 };
-// The tile shape and the runs of planes per tile with the least work of the
-// busiest block, in node slots (every lane counts, with a node or without).  A
-// run costs planes beyond its own -- one more of p and the fill of its loads --
-// and a plane costs slots beyond its nodes: its ring and, where arithmetic does
-// not hide them (FP32), the barrier and the loop.  Fitted to timed plans: FP64
-// 200 x 180 x 90 prefers 32 x 16 tiles (100 us per iteration against 108 with
-// 64 x 16), FP32 470 x 239 x 58 64 x 16 ones (56 us against 70).
+template <bool Shares>
+struct StreamTurns {
+  int u, end;  // a tile has 512 nodes or more: the planes of all tiles are an int
+  __device__ __forceinline__ explicit StreamTurns(int units) {
+    u = blockIdx.x;
+    end = units;
+    if (Shares) {
+      int len;
+      stream_part(units, gridDim.x, blockIdx.x, u, len);
+      end = u + len;
+    }
+  }
+  // the block's next tile and its planes k0 .. k0 + kn - 1
+  __device__ __forceinline__ bool next(int nchunk, int nz, int& tile, int& k0, int& kn) {
+    if (u >= end) return false;
+    if (Shares) {
+      tile = u / nz;
+      k0 = u - tile * nz;
+      kn = min(nz - k0, end - u);
+      u += kn;
+    } else {
+      tile = u / nchunk;
+      stream_part(nz, nchunk, u - tile * nchunk, k0, kn);
+      u += gridDim.x;
+    }
+    return true;
+  }
+};
+// The tile shape and the division of the planes with the least work of the busiest
+// block, in node slots (every lane counts, with a node or without).  A run costs
+// planes beyond its own -- one more of p and the fill of its loads -- and a plane
+// costs slots beyond its nodes: its ring and, where arithmetic does not hide them
+// (FP32), the barrier and the loop.  Fitted to timed plans: FP64 200 x 180 x 90
+// prefers 32 x 16 tiles (100 us per iteration against 108 with 64 x 16), FP32 470 x
+// 239 x 58 64 x 16 ones (56 us against 70).  Equal shares, for FP64 alone: 256 x 256 x
+// 128 192 -> 187 us, 512 x 512 x 128 719 -> 678, 512 x 256 x 64 202 -> 188; their
+// neighbours in the grid are at other planes at the time, and where memory bounds the
+// march (FP32) their rings are then read twice: 470 x 239 x 58 54 us in runs, 59 in
+// shares.
 inline StreamPlan make_stream_plan(int nx, int ny, int nz, long long G, bool fp64) {
   static constexpr int shapes[3][2] = {{64, 16}, {32, 32}, {32, 16}};
   StreamPlan best;
@@ -122,19 +158,23 @@ inline StreamPlan make_stream_plan(int nx, int ny, int nz, long long G, bool fp6
     const int wx = shapes[q][0], wy = shapes[q][1];
     const int ntx = (nx + wx - 1) / wx, nty = (ny + wy - 1) / wy;
     const long long tiles = (long long)ntx * nty;
-    // the units are dealt to the blocks in turns: for each number of turns as
-    // many runs of planes per tile as fill them
+    const double plane = fp64 ? wx * wy + 0.5 * (wx + wy) + 24.0 : wx * wy + (wx + wy) + (wx == 64 ? 200.0 : 240.0);
+    const double fill = fp64 ? 0.7 : 2.0;
+    auto offer = [&](double planes, int nchunk, long long units) {
+      if (best.units == 0 || planes * plane < cost) {
+        cost = planes * plane;
+        best = {q, ntx, nty, nchunk, units};
+      }
+    };
+    // for each number of turns as many runs of planes per tile as fill them
     for (int turns = 1; turns <= 8; ++turns) {
       const long long nchunk = std::max<long long>(1, std::min<long long>(nz, G * turns / tiles));
       const long long units = tiles * nchunk, per = (units + G - 1) / G;
-      const double zrun = (double)((nz + nchunk - 1) / nchunk);
-      const double c = fp64 ? (double)per * (zrun + 0.7) * (wx * wy + 0.5 * (wx + wy) + 24.0)
-                            : (double)per * (zrun + 2.0) * (wx * wy + (wx + wy) + (wx == 64 ? 200.0 : 240.0));
-      if (best.units == 0 || c < cost) {
-        cost = c;
-        best = {q, ntx, nty, (int)nchunk, units};
-      }
+      offer((double)per * ((double)((nz + nchunk - 1) / nchunk) + fill), (int)nchunk, units);
     }
+    // a share of `per` planes touches at most (per - 2) / nz + 2 tiles
+    const long long per = (tiles * nz + G - 1) / G;
+    if (fp64) offer((double)per + 1.5 * (double)(per > 1 ? (per - 2) / nz + 2 : 1), 0, tiles * nz);
   }
   return best;
 }

@@ -39,7 +39,9 @@ def setup(les_mod, shape, precision, walls, max_blocks=0):
     (32, (33, 31, 9), 0),      # partial tiles of the square shape
     (32, (100, 7, 40), 0),     # runs of unequal length
     (32, (70, 50, 3), 1),      # one block walks every tile
-    (64, (130, 33, 24), 0)])   # three tiles along x, of unequal width
+    (64, (130, 33, 24), 0),    # three tiles along x, of unequal width
+    (64, (130, 50, 24), 3),    # equal shares of 80 planes: four tiles of 32 x 32 or five
+    (64, (64, 50, 37), 13)])   # shares of 23 planes: one tile or two, of 32 x 16
 def test_streaming_cg_matches_oracle(les_mod, precision, shape, max_blocks, walls):
     """Tolerances as for the other CG kernels: the solve's own 1e-11 (FP64) or
     1e-6 (FP32) times the condition of these grids, a few hundred at most."""
