@@ -239,7 +239,7 @@ class Clocks:
 # the source files whose change invalidates a kernel's DRAM-traffic record
 TRAFFIC_SOURCES = {
     "cg_wave": ("les_cg_wave.cu", "les_gridsync.cuh", "les_common.cuh"),
-    "cg_regs": ("les_cg_regs.cu", "les_gridsync.cuh", "les_common.cuh"),
+    "cg_regs": ("les_cg_regs.cu", "les_chip.cuh", "les_gridsync.cuh", "les_common.cuh"),
     "scalar": ("les_predict_col.cu", "les_common.cuh"),
     "momentum": ("les_predict_col.cu", "les_common.cuh"),
     "rhs": ("les_stencil_col.cu",),
