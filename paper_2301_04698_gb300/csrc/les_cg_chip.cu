@@ -23,7 +23,7 @@
 // r.r, r.q and q.q per iteration (alpha, and beta from |r - alpha q|^2
 // expanded in the four; les_chip.cuh).  With XS = false the faces' q are tagged words;
 // with more faces these cost more than they save (150 x 140 x 70 FP32: 13 us per
-// iteration instead of 9.3), and counters order them.
+// iteration instead of 9.3 at the time), and counters order them.
 //
 // What bounds it: the latency of the grid sum (2.1 us of an iteration on the
 // smallest grids) and, in FP64, the
@@ -39,11 +39,11 @@
 // bricks fit):
 //   FP64  32^3 9.9 -> 4.7, 256 x 4 x 32 10.1 -> 4.7, 64 x 64 x 48 16.9 -> 9.3,
 //         50 x 47 x 33 28.3 -> 6.8, 77 x 130 x 50 66.8 -> 16.4, 96^3 77 -> 26.5
-//   FP32  32^3 4.2 -> 2.1, 64^3 5.0 -> 2.9, 96^3 7.3 -> 5.0, 160 x 160 x 48
-//         8.4 -> 6.0, 100 x 76 x 61 23.6 -> 3.85, 150 x 140 x 70 36.7 -> 9.3
+//   FP32  32^3 4.2 -> 2.1, 64^3 5.0 -> 2.8, 96^3 7.3 -> 4.7, 160 x 160 x 48
+//         8.4 -> 5.6, 100 x 76 x 61 23.6 -> 3.7, 150 x 140 x 70 36.7 -> 8.2
 // FP32 grids 128 nodes wide keep les_cg_regs.cu, whose four-node lanes read
-// x neighbours by shuffles: 128 x 64 x 64 2.8 there, 4.1 here; 128 x 128 x 96
-// 5.0 and 8.4.
+// x neighbours by shuffles: 128 x 64 x 64 2.8 there, 64 x 128 x 64 3.3 here; 128 x
+// 128 x 96 4.5, 96 x 128 x 128 7.2.
 #include <algorithm>
 #include <string>
 
@@ -166,15 +166,36 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
   constexpr bool kScaled = sizeof(T) == 8;
   const T c0 = T(2) * (cx + cy + cz);
   const T ax = cx / c0, ay = cy / c0, az = cz / c0, mc0 = T(-1) / c0;
-  auto stencil = [&](int j) -> T {
+  auto stencil = [&](int j, bool inner) -> T {  // inner: plane j + 1 is surely of the run
     const T* pj = P + pown + j * SZ;
     const T d = j > 0 ? p[j > 0 ? j - 1 : 0] : pj[ozm];
-    const T u = (j + 1 < ZP && j + 1 < nzp) ? p[j + 1 < ZP ? j + 1 : ZP - 1] : pj[ozp];
+    const T u = (j + 1 < ZP && (inner || j + 1 < nzp)) ? p[j + 1 < ZP ? j + 1 : ZP - 1] : pj[ozp];
     if constexpr (kScaled) {
       return fma(-az, d + u, fma(-ay, pj[oym] + pj[oyp], fma(-ax, pj[oxm] + pj[oxp], p[j])));
     } else {
       const T c2 = T(2) * p[j];
       return (pj[oxm] + pj[oxp] - c2) * cx + (pj[oym] + pj[oyp] - c2) * cy + (d + u - c2) * cz;
+    }
+  };
+
+  // body(plane, its upper neighbour is surely of the run) up this thread's run.  The
+  // plane counts are instantiated in steps of KT, so a run lacks KT planes at most; a
+  // warp whose runs all have the others has no test between those, and their chains
+  // overlap (FP32: 96^3 5.0 -> 4.7 us per iteration, 150 x 140 x 70 9.4 -> 8.2; FP64
+  // waits for its arithmetic, not for chains, and loses 2 % by the longer code).
+  constexpr int KT = XS ? 4 : 2, ZF = sizeof(T) == 4 && ZP > KT ? ZP - KT : 0;
+  const bool full = __all_sync(0xffffffffu, nzp >= ZF);
+  auto each_plane = [&](auto&& body) {
+    if (ZF > 0 && full) {
+#pragma unroll
+      for (int j = 0; j < ZF; ++j) body(j, j + 1 < ZF);
+#pragma unroll
+      for (int j = ZF; j < ZP; ++j)
+        if (j < nzp) body(j, false);
+    } else {
+#pragma unroll
+      for (int j = 0; j < ZP; ++j)
+        if (j < nzp) body(j, false);
     }
   };
 
@@ -261,7 +282,7 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
     for (int j = 0; j < ZP; ++j)
       if (j < nzp) {
         const T bm = r[j] - mean;
-        r[j] = kScaled ? fma(c0, stencil(j), bm) : bm - stencil(j);
+        r[j] = kScaled ? fma(c0, stencil(j, false), bm) : bm - stencil(j, false);
         if (is_face(j)) __stcg(f.rg + gown + j * gpl, r[j]);
         a2[0].add(r[j] * r[j]);
         a2[1].add(bm * bm);
@@ -333,18 +354,16 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
       asm volatile("" : "+r"(pown), "+r"(gown));
       T* qw = (iter & 1) ? f.qg1 : f.qg0;  // this iteration's q faces
       T d0 = T(0), d2 = T(0), d3 = T(0);   // p.q, r.q, q.q
-#pragma unroll
-      for (int j = 0; j < ZP; ++j)
-        if (j < nzp) {
-          q[j] = stencil(j);
-          if (is_face(j)) {
-            if constexpr (XS) __stcg(qw + gown + j * gpl, q[j]);
-            else tagged_store(word(iter & 1, gown + j * gpl), q[j], iter);
-          }
-          d0 += p[j] * q[j];
-          d2 += r[j] * q[j];
-          d3 += q[j] * q[j];
+      each_plane([&](int j, bool inner) {
+        q[j] = stencil(j, inner);
+        if (is_face(j)) {
+          if constexpr (XS) __stcg(qw + gown + j * gpl, q[j]);
+          else tagged_store(word(iter & 1, gown + j * gpl), q[j], iter);
         }
+        d0 += p[j] * q[j];
+        d2 += r[j] * q[j];
+        d3 += q[j] * q[j];
+      });
       Tagged<T> gq[NG];  // the q of the ghosts
       Acc tot[4];        // the totals, in warp 0
       constexpr int WORDS = sizeof(T) == 8 && ZP < 10 ? 5 : 3;
@@ -407,16 +426,14 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
       tb = sc.tb;
       tx = sc.tx;
       rr_own = T(0);
-#pragma unroll
-      for (int j = 0; j < ZP; ++j)
-        if (j < nzp) {
-          if (!kDefer || warp == 0) set_x(j, get_x(j) + tx * p[j]);
-          else po[kDefer ? j : 0] = p[j];
-          r[j] -= ta * q[j];
-          rr_own += r[j] * r[j];
-          p[j] = r[j] + tb * p[j];
-          P[pown + j * SZ] = p[j];
-        }
+      each_plane([&](int j, bool) {
+        if (!kDefer || warp == 0) set_x(j, get_x(j) + tx * p[j]);
+        else po[kDefer ? j : 0] = p[j];
+        r[j] -= ta * q[j];
+        rr_own += r[j] * r[j];
+        p[j] = r[j] + tb * p[j];
+        P[pown + j * SZ] = p[j];
+      });
       if constexpr (XS) {
         for (int id = tid; id < ngh; id += nthr) {
           const int at = GT[id].x;

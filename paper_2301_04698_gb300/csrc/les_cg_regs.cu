@@ -35,8 +35,9 @@
 // The arithmetic takes two nodes per instruction (packed FP32).
 //
 // What bounds it: the grid sum (2.1 us of an iteration) and shared memory.  Measured
-// (GB300, us per iteration): 128 x 64 x 32 2.4, 128 x 64 x 64 2.8, 128 x 128 x 96 5.0;
-// with a sum whose partials were released and then read 3.0, 3.35, 5.1.
+// (GB300, us per iteration): 128 x 64 x 32 2.4, 128 x 64 x 64 2.7, 128 x 128 x 96 4.5;
+// with a sum whose partials were released and then read, scalar arithmetic and a test
+// at every plane 3.0, 3.35, 5.1.
 #include <algorithm>
 #include <string>
 
@@ -161,6 +162,19 @@ __global__ void __launch_bounds__(kRegMaxWarps * 32, 1) k_cg_regs(RegArgs f) {
     };
     return join2(pair(lo2(c), float2{w0 + c.y, c.x + c.z}, lo2(s), lo2(nn), lo2(d), lo2(u)),
                  pair(hi2(c), float2{c.y + c.w, c.z + e3}, hi2(s), hi2(nn), hi2(d), hi2(u)));
+  };
+
+  // body(plane) up this thread's run; a full run has no test between its planes, whose
+  // chains can overlap (128 x 128 x 96: 5.0 -> 4.5 us per iteration)
+  auto each_plane = [&](auto&& body) {
+    if (nzp == ZP) {
+#pragma unroll
+      for (int j = 0; j < ZP; ++j) body(j);
+    } else {
+#pragma unroll
+      for (int j = 0; j < ZP; ++j)
+        if (j < nzp) body(j);
+    }
   };
 
   GridSync gs{f.bar, f.partials, f.spin_cycles, f.expected, 0u};
@@ -290,15 +304,13 @@ __global__ void __launch_bounds__(kRegMaxWarps * 32, 1) k_cg_regs(RegArgs f) {
       asm volatile("" : "+r"(pown), "+r"(xown), "+r"(gown));
       float* qw = (iter & 1) ? f.qg1 : f.qg0;  // this iteration's q faces
       float2 d0{0.f, 0.f}, d2{0.f, 0.f}, d3{0.f, 0.f};  // p.q, r.q, q.q
-#pragma unroll
-      for (int j = 0; j < ZP; ++j)
-        if (j < nzp) {
-          q[j] = stencil(j);
-          if (is_face(j)) stg4(qw + gown + j * gpl, q[j]);
-          dot4(d0, p[j], q[j]);
-          dot4(d2, r[j], q[j]);
-          dot4(d3, q[j], q[j]);
-        }
+      each_plane([&](int j) {
+        q[j] = stencil(j);
+        if (is_face(j)) stg4(qw + gown + j * gpl, q[j]);
+        dot4(d0, p[j], q[j]);
+        dot4(d2, r[j], q[j]);
+        dot4(d3, q[j], q[j]);
+      });
       chip_sum<kFoldWarps<F2>, 3>(
           f, iter, d0.x + d0.y, rr_own, d2.x + d2.y, d3.x + d3.y, shv, part, tot, s_fail,
           [&] {  // the last iteration's x += alpha p of this warp's rows, deferred from its update
@@ -341,16 +353,14 @@ __global__ void __launch_bounds__(kRegMaxWarps * 32, 1) k_cg_regs(RegArgs f) {
       ta = sc.ta;
       tb = sc.tb;
       float2 rr_new{0.f, 0.f};
-#pragma unroll
-      for (int j = 0; j < ZP; ++j)
-        if (j < nzp) {
-          if (warp == 0) sts4(X + xown + j * xpl, fma4(ta, p[j], lds4(X + xown + j * xpl)));
-          else sts4(PO + xown + j * xpl, p[j]);
-          r[j] = fma4(-ta, q[j], r[j]);
-          dot4(rr_new, r[j], r[j]);
-          p[j] = fma4(tb, p[j], r[j]);
-          sts4(P + pown + j * SZ, p[j]);
-        }
+      if (warp == 0) each_plane([&](int j) { sts4(X + xown + j * xpl, fma4(ta, p[j], lds4(X + xown + j * xpl))); });
+      else each_plane([&](int j) { sts4(PO + xown + j * xpl, p[j]); });
+      each_plane([&](int j) {
+        r[j] = fma4(-ta, q[j], r[j]);
+        dot4(rr_new, r[j], r[j]);
+        p[j] = fma4(tb, p[j], r[j]);
+        sts4(P + pown + j * SZ, p[j]);
+      });
       for (int row = warp; row < nr; row += nwarp) {
         int y, z;
         ghost_row(row, y, z);

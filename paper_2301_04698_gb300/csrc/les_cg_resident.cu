@@ -599,7 +599,7 @@ int poisson_solve_resident(const SolverArgs<T>& a, const FusedCfg& fc, const T* 
   if (!(a.op == LES_OP_COMPACT && a.solver == LES_SOLVER_CG && a.g.nz >= 2 && a.bar && a.r && a.p0 && a.p1))
     return LES_OK;
   // The vectors in registers: FP32 grids 128 nodes wide in les_cg_regs.cu
-  // (2.8 against 4.1 us per iteration on 128 x 64 x 64), every other grid in
+  // (2.8 us per iteration on 128 x 64 x 64, against 3.3 on 64 x 128 x 64), every other grid in
   // les_cg_chip.cu, up to 24 FP32 or 12 FP64 nodes per thread of one block per
   // SM, and above that, in FP32 up to 64 planes of 32 x 16 columns per SM, in
   // les_cg_brick.cu.  What is left for the kernel here are FP64 grids of whole
