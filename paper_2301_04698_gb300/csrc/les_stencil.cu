@@ -195,28 +195,53 @@ __global__ void __launch_bounds__(32 * RZ) k_radiation(Grid<T> g, Phys<T> ph, co
 
 // ---- a7: correction (Sec. 2.4) ----------------------------------------------
 // u^{k+1} = u^ - dt G(psi), p^{k+1} = p^k + rho0 psi, psi = alpha0 dp
-template <typename T>
+// for the grids that the column march (les_stencil_col.cu) does not fit.  Bound by
+// latency on small grids and by bytes (nine fields) on large ones: a thread issues the
+// loads of KZ planes of its column together, one plane where four would leave SMs
+// without a block.  Measured per launch (before: eight planes one after the other,
+// every neighbour wrapped for itself): 192 x 192 x 128 FP32 94.7 -> 39.5 us, 100 x 76 x
+// 61 FP32 20.0 -> 12.4, 32^3 FP64 23.3 -> 7.9.
+template <typename T, int KZ>
 __global__ void __launch_bounds__(NTHREADS)
-    k_correct(Grid<T> g, Phys<T> ph, const T* __restrict__ ou, const T* __restrict__ ov,
+    k_correct(Grid<T> g, Phys<T> ph, long long nt, const T* __restrict__ ou, const T* __restrict__ ov,
               const T* __restrict__ ow, const T* __restrict__ psi, T* __restrict__ u,
               T* __restrict__ v, T* __restrict__ w, T* __restrict__ p) {
-  const T* hat[3] = {ou, ov, ow};
-  T* vel[3] = {u, v, w};
-  for (long long t = blockIdx.x; t < g.ntiles; t += gridDim.x) {
-    int i, j, k0, k1;
-    tile_origin(g, t, i, j, k0, k1);
+  const T hx = T(0.5) * g.ih(0), hy = T(0.5) * g.ih(1), hz = T(0.5) * g.ih(2);
+  const size_t plane = (size_t)g.nx * g.ny;
+  for (long long t = blockIdx.x; t < nt; t += gridDim.x) {
+    const long long r = t / g.ntx;
+    const int i = (int)(t - r * g.ntx) * TX + threadIdx.x, j = (int)(r % g.nty) * TY + threadIdx.y;
+    const int k0 = (int)(r / g.nty) * KZ;
     if (i >= g.nx || j >= g.ny) continue;
-    for (int k = k0; k < k1; ++k) {
-      const size_t m = g.lin(i, j, k);
+    const size_t row = (size_t)j * g.nx, c = row + i;
+    const size_t xm = row + (i == 0 ? g.nx - 1 : i - 1), xp = row + (i == g.nx - 1 ? 0 : i + 1);
+    const size_t ym = j == 0 ? c + plane - g.nx : c - g.nx, yp = j == g.ny - 1 ? i : c + g.nx;
+    T pz[KZ + 2], px[KZ][2], py[KZ][2], hat[KZ][3], pp[KZ];  // psi at c on k0 - 1 .. k0 + KZ, ...
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const int ci = c == 0, cj = c == 1, ck = c == 2;
-        const T gr = (g.at(psi, i + ci, j + cj, k + ck, G_EVEN) - g.at(psi, i - ci, j - cj, k - ck, G_EVEN)) *
-                     (T(0.5) * g.ih(c));
-        vel[c][m] = hat[c][m] - ph.dt * gr;
-      }
-      p[m] += ph.rho0[k] * psi[m];
+    for (int q = 0; q < KZ + 2; ++q) {
+      int k = k0 + q - 1;  // planes beyond the one above the grid: any, unused
+      if (g.walls) k = k < 0 ? 0 : min(k, g.nz - 1);
+      else k = k < 0 ? g.nz - 1 : (k >= g.nz ? (k - g.nz) % g.nz : k);
+      pz[q] = __ldg(psi + k * plane + c);
     }
+#pragma unroll
+    for (int q = 0; q < KZ; ++q)
+      if (k0 + q < g.nz) {
+        const size_t b = (size_t)(k0 + q) * plane;
+        px[q][0] = __ldg(psi + b + xm), px[q][1] = __ldg(psi + b + xp);
+        py[q][0] = __ldg(psi + b + ym), py[q][1] = __ldg(psi + b + yp);
+        hat[q][0] = __ldg(ou + b + c), hat[q][1] = __ldg(ov + b + c), hat[q][2] = __ldg(ow + b + c);
+        pp[q] = p[b + c];
+      }
+#pragma unroll
+    for (int q = 0; q < KZ; ++q)
+      if (k0 + q < g.nz) {
+        const size_t m = (size_t)(k0 + q) * plane + c;
+        u[m] = hat[q][0] - ph.dt * ((px[q][1] - px[q][0]) * hx);
+        v[m] = hat[q][1] - ph.dt * ((py[q][1] - py[q][0]) * hy);
+        w[m] = hat[q][2] - ph.dt * ((pz[q + 2] - pz[q]) * hz);
+        p[m] = pp[q] + ph.rho0[k0 + q] * pz[q + 1];
+      }
   }
 }
 
@@ -501,7 +526,11 @@ template <typename T>
 cudaError_t launch_correct(const StageArgs<T>& a, const T* ou, const T* ov, const T* ow, const T* psi, T* u,
                            T* v, T* w, T* p) {
   ProfScope ps(a.prof, KI_CORRECT, a.st);
-  k_correct<T><<<a.lc.grid, a.lc.block, 0, a.st>>>(a.g, a.ph, ou, ov, ow, psi, u, v, w, p);
+  const long long cols = (long long)a.g.ntx * a.g.nty, n4 = cols * ((a.g.nz + 3) / 4), n1 = cols * a.g.nz;
+  constexpr long long kFew = 4 * 152;  // blocks that give every SM a few
+  auto grid = [](long long n) { return dim3((unsigned)std::min<long long>(n, 1 << 30)); };
+  if (n4 >= kFew) k_correct<T, 4><<<grid(n4), a.lc.block, 0, a.st>>>(a.g, a.ph, n4, ou, ov, ow, psi, u, v, w, p);
+  else k_correct<T, 1><<<grid(n1), a.lc.block, 0, a.st>>>(a.g, a.ph, n1, ou, ov, ow, psi, u, v, w, p);
   return cudaGetLastError();
 }
 
