@@ -149,7 +149,8 @@ __device__ __forceinline__ void chip_fold(Acc (&part)[32], Acc (&tot)[4]) {
 // that finds the tag has the value, and neither side orders it against anything
 // else.  A writer that released a flag would wait for its stores to reach L2, and a
 // reader that had seen it would read the value by another trip.  The tags are NaN
-// patterns, which no finite value left in the same memory can look like.
+// patterns, which no finite FP32 value left in the same memory can look like; as the
+// upper half of an FP64 one they are beyond 1e305, whose square stops the solve first.
 __device__ __forceinline__ unsigned chip_tag(int iter) { return 0xff800001u + ((unsigned)iter & 0x3fffffu); }
 // FP32: 8 bytes; FP64: 16, each half of the value with the tag.  A compensated pair
 // takes 8, its tag the last bit of lo (2^-48 of the value): the two values that share a
