@@ -199,11 +199,13 @@ __device__ __forceinline__ void tagged_store(char* at, double v, int iter) {
                "l"(tag | (unsigned)__double2hiint(v))
                : "memory");
 }
-// a word that no reader takes for that of iteration 0 or 1
+// a word that no reader takes for that of iteration 0 or 1.  Of an FP64 one both
+// halves: a vector access is whole only per 8 bytes, and a half left with the tag of an
+// earlier solve's iteration 0 or 1 would pass with the other half's new value.
 template <typename V>
 __device__ __forceinline__ void tagged_clear(char* at) {
-  if constexpr (std::is_same<V, F2>::value) tagged_store8(at, 0u, 1u);
-  else asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(at), "l"(0ull) : "memory");
+  tagged_store8(at, 0u, std::is_same<V, F2>::value ? 1u : 0u);
+  if constexpr (Tagged<V>::BYTES == 16) tagged_store8(at + 8, 0u, 0u);
 }
 
 // The words of a sum's partials: [2 slots][gridDim.x][4 values].  A block's four lie
