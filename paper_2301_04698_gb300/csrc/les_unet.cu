@@ -417,6 +417,12 @@ struct WgradArgs {
   long long ntiles;
 };
 constexpr int kWgWarps = 9;  // one per (dz, dy)
+// Tiles whose products the accumulators take before they are added to the share's
+// partials: 16 x 256 voxels, 256 MMAs in a chain, whatever the grid and the batch.  The
+// error of a chain grows with its length: the gradient of one sample at 64^3 repeated 16
+// and 64 times is off by 1.5e-4 and 6.8e-4 of a layer's norm with chains as long as the
+// shares (162 and 649 tiles), by 1e-5 at most with these.
+constexpr int kWgFold = 16;
 
 template <int CO>
 constexpr size_t wgrad_smem() {
@@ -483,6 +489,45 @@ __global__ void __launch_bounds__(32 * kWgWarps) k_wgrad(WgradArgs a) {
   const unsigned oa = 16u * (unsigned)(G::IN + ((lane & 7) + ((lane >> 4) & 1) * 8) * GS + ((lane >> 3) & 1));
   const unsigned ob = 16u * (unsigned)(dz * G::PZ + (dy + ((lane >> 3) & 1)) * G::P + (lane & 7) * G::S + (lane >> 4));
   const bool bias = blockIdx.x == 0 && warp == 4;
+  // the accumulators into the share's partials (added from the second time on)
+  bool more = false;
+  int held = 0;  // tiles in the accumulators
+  auto fold = [&] {
+    unsigned share = blockIdx.y;
+    asm volatile("" : "+r"(share));  // addresses formed here, not held through the loop
+    const int cout = 16 * CO;
+    float* base = a.part + (size_t)share * 27 * cout * a.cin + 16 * blockIdx.x;
+#pragma unroll
+    for (int t = 0; t < 3; ++t)
+#pragma unroll
+      for (int o = 0; o < CO; ++o)
+#pragma unroll
+        for (int f = 0; f < 2; ++f)
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            float* q = base + ((size_t)(warp * 3 + t) * cout + o * 16 + gid + 8 * h) * a.cin + f * 8 + tig * 2;
+            float2 v = make_float2(acc[t][o][f][2 * h], acc[t][o][f][2 * h + 1]);
+            if (more) {
+              const float2 u = *reinterpret_cast<const float2*>(q);
+              v.x += u.x;
+              v.y += u.y;
+            }
+            *reinterpret_cast<float2*>(q) = v;
+            acc[t][o][f][2 * h] = acc[t][o][f][2 * h + 1] = 0.f;
+          }
+    if (bias && tig == 0)
+#pragma unroll
+      for (int o = 0; o < CO; ++o)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          float* q = a.bpart + (size_t)share * cout + o * 16 + gid + 8 * h;
+          *q = ab[o][2 * h] + (more ? *q : 0.f);
+        }
+#pragma unroll
+    for (int o = 0; o < CO; ++o) ab[o][0] = ab[o][1] = ab[o][2] = ab[o][3] = 0.f;
+    more = true;
+    held = 0;
+  };
   int buf = 0;
   long long tile = blockIdx.y;
   table(tile, 0);
@@ -520,27 +565,9 @@ __global__ void __launch_bounds__(32 * kWgWarps) k_wgrad(WgradArgs a) {
 #pragma unroll
         for (int o = 0; o < CO; ++o) mma_bf16(ab[o], A[o], 0x3F803F80u, 0x3F803F80u);
     }
+    if (++held == kWgFold || tile + gridDim.y >= a.ntiles) fold();
     __syncthreads();  // the buffer is free for the tile after the next
   }
-  const int cout = 16 * CO;
-  float* base = a.part + (size_t)blockIdx.y * 27 * cout * a.cin + 16 * blockIdx.x;
-#pragma unroll
-  for (int t = 0; t < 3; ++t)
-#pragma unroll
-    for (int o = 0; o < CO; ++o)
-#pragma unroll
-      for (int f = 0; f < 2; ++f)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          float* q = base + ((size_t)(warp * 3 + t) * cout + o * 16 + gid + 8 * h) * a.cin + f * 8 + tig * 2;
-          *reinterpret_cast<float2*>(q) = make_float2(acc[t][o][f][2 * h], acc[t][o][f][2 * h + 1]);
-        }
-  if (bias && tig == 0)
-#pragma unroll
-    for (int o = 0; o < CO; ++o) {
-      a.bpart[(size_t)blockIdx.y * cout + o * 16 + gid] = ab[o][0];
-      a.bpart[(size_t)blockIdx.y * cout + o * 16 + gid + 8] = ab[o][2];
-    }
 }
 
 // The partials of every layer, summed over their shares in order, into the
@@ -602,18 +629,23 @@ __global__ void __launch_bounds__(256) k_head_back(const bf16* gy, const bf16* h
   const int half = threadIdx.x & 1;
   const Chunk w = unpack8(__ldg(reinterpret_cast<const uint4*>(hw + 8 * half)));
   float acc[9] = {};
-  for (long long i = (blockIdx.x * 256LL + threadIdx.x) >> 1; i < nvox; i += gridDim.x * 128LL) {
-    const float g = __bfloat162float(gy[i]);
-    const uint4 pu = __ldg(reinterpret_cast<const uint4*>(post + i * 16 + 8 * half));
-    const Chunk p = unpack8(pu);
-    Chunk c;
+  for (long long i = (blockIdx.x * 256LL + threadIdx.x) >> 1; i < nvox;) {
+    float run[9] = {};  // sums of 256 voxels, so that no chain of additions grows with the grid
+    for (int n = 0; n < 256 && i < nvox; ++n, i += gridDim.x * 128LL) {
+      const float g = __bfloat162float(gy[i]);
+      const uint4 pu = __ldg(reinterpret_cast<const uint4*>(post + i * 16 + 8 * half));
+      const Chunk p = unpack8(pu);
+      Chunk c;
 #pragma unroll
-    for (int q = 0; q < 8; ++q) {
-      c.v[q] = g * w.v[q];
-      acc[q] += g * p.v[q];
+      for (int q = 0; q < 8; ++q) {
+        c.v[q] = g * w.v[q];
+        run[q] += g * p.v[q];
+      }
+      run[8] += g;
+      *reinterpret_cast<uint4*>(s + i * 16 + 8 * half) = act_back(pu, pack8(c));
     }
-    acc[8] += g;
-    *reinterpret_cast<uint4*>(s + i * 16 + 8 * half) = act_back(pu, pack8(c));
+#pragma unroll
+    for (int q = 0; q < 9; ++q) acc[q] += run[q];
   }
 #pragma unroll
   for (int q = 0; q < 9; ++q)
