@@ -138,15 +138,8 @@ __global__ void __launch_bounds__(BX* BY, 1) k_cg_brick(ChipArgs<float> f) {
       if (keep) GR[id] = v;
     });
   };
-  // FP32 sums of a column in runs of eight planes
-  struct Run {
-    float s = 0.f, run = 0.f;
-    __device__ __forceinline__ void add(int j, float v) {
-      run += v;
-      if ((j & 7) == 7) s += run, run = 0.f;
-    }
-    __device__ __forceinline__ float total(bool own) const { return own ? s + run : 0.f; }
-  };
+  // the sum of a thread's column, of those that are the brick's
+  auto total = [&](const ChipRun<float, ZP>& s) { return own ? s.total() : F2{0.f, 0.f}; };
 
   GridSync gs{f.bar, f.partials, f.spin_cycles, f.expected, 0u};
   __shared__ struct {
@@ -154,28 +147,27 @@ __global__ void __launch_bounds__(BX* BY, 1) k_cg_brick(ChipArgs<float> f) {
     int status, restart;
     double bb, rel;  // |b - mean|^2 and the relative residual of x0
   } sc;
-  __shared__ float shv[4][kChipWarps];
+  __shared__ F2 shv[4][kChipWarps];
   __shared__ F2 part[32];
   F2 tot[4];  // in warp 0
   __shared__ int s_fail;
   double rr = 0.0, bb = 0.0, rel = 0.0;  // meaningful in thread 0
   int status = 0;  // 0 running, 1 converged, 2 maxit, 3 breakdown, 4 zero rhs, 5 timeout
-  float rr_own = 0.f;  // this thread's share of r.r for the next sum
+  F2 rr_own{0.f, 0.f};  // this thread's share of r.r for the next sum
 
   chip_sum_clear<F2>(f.spread);  // no tag of an earlier solve: cleared here, for everyone after the first sum
   if (tid == 0) s_fail = 0;
 
   // mean of b (b held in r)
   {
-    Run s;
+    ChipRun<float, ZP> s;
     planes([&](int j, int g) {
       if (own) r[j] = __ldcg(f.b + g);
       s.add(j, r[j]);
     });
-    Dot<float> a1[1];
-    a1[0].s = s.total(own);
+    F2 v[1] = {total(s)};
     double t[1];
-    const bool ok = grid_dot_t0<1>(a1, gs, t);
+    const bool ok = grid_sum_t0<1>(v, gs, t);
     if (tid == 0) {
       sc.status = ok ? 0 : 5;
       sc.mean = (float)(t[0] / (double)f.n);
@@ -191,7 +183,7 @@ __global__ void __launch_bounds__(BX* BY, 1) k_cg_brick(ChipArgs<float> f) {
     });
     fill_ghosts(f.x, false);
     __syncthreads();
-    Run s0, s1;
+    ChipRun<float, ZP> s0, s1;
     march([&](int j, int g, float, float q) {
       const float bm = r[j] - mean;
       r[j] = bm - q;
@@ -199,12 +191,10 @@ __global__ void __launch_bounds__(BX* BY, 1) k_cg_brick(ChipArgs<float> f) {
       s0.add(j, r[j] * r[j]);
       s1.add(j, bm * bm);
     });
-    rr_own = s0.total(own);
-    Dot<float> a2[2];
-    a2[0].s = rr_own;
-    a2[1].s = s1.total(own);
+    rr_own = total(s0);
+    F2 v[2] = {rr_own, total(s1)};
     double s2[2];
-    const bool ok = grid_dot_t0<2>(a2, gs, s2);
+    const bool ok = grid_sum_t0<2>(v, gs, s2);
     if (tid == 0) {
       // the plain solver judges a learned first guess: if it leaves a larger
       // residual than x0 = 0, restart from zero (r = b - mean b, r.r = |b|^2)
@@ -216,7 +206,7 @@ __global__ void __launch_bounds__(BX* BY, 1) k_cg_brick(ChipArgs<float> f) {
     __syncthreads();
     status = sc.status;
     if (!status && sc.restart) {
-      Run s;
+      ChipRun<float, ZP> s;
       planes([&](int j, int g) {
         if (!own) return;
         __stcg(f.x + g, 0.f);
@@ -224,7 +214,7 @@ __global__ void __launch_bounds__(BX* BY, 1) k_cg_brick(ChipArgs<float> f) {
         s.add(j, r[j] * r[j]);
         if (is_face(j)) __stcg(f.rg + g, r[j]);
       });
-      rr_own = s.total(own);
+      rr_own = total(s);
       Dot<float> none[1];
       double t[1];
       const bool ok2 = grid_dot_t0<1>(none, gs, t);  // a grid barrier: the new faces are visible
@@ -261,7 +251,7 @@ __global__ void __launch_bounds__(BX* BY, 1) k_cg_brick(ChipArgs<float> f) {
     __syncthreads();
     for (;;) {
       float* qw = (iter & 1) ? f.qg1 : f.qg0;  // this iteration's q faces
-      Run d0, d2, d3;                          // p.q, r.q, q.q
+      ChipRun<float, ZP> d0, d2, d3;           // p.q, r.q, q.q
       march([&](int j, int g, float pv, float q) {
         // three planes of four by a predicated store, whose arithmetic can overlap;
         // a branch at the fourth keeps the compiler from spreading all of them
@@ -273,7 +263,7 @@ __global__ void __launch_bounds__(BX* BY, 1) k_cg_brick(ChipArgs<float> f) {
         d3.add(j, q * q);
       });
       chip_sum<GhostWarps::value, 3>(
-          f, iter, d0.total(own), rr_own, d2.total(own), d3.total(own), shv, part, tot, s_fail, ChipNothing{},
+          f, iter, total(d0), rr_own, total(d2), total(d3), shv, part, tot, s_fail, ChipNothing{},
           [&] {
             each_ghost(GhostWarps{}, [&](int id, float*, int g) { cp_async(GQ + id, qw + g); });
             cp_commit();
@@ -302,12 +292,12 @@ __global__ void __launch_bounds__(BX* BY, 1) k_cg_brick(ChipArgs<float> f) {
       }
       const float ta = sc.ta, tb = sc.tb;
       // r -= alpha q, with q from p as it was
-      Run s;
+      ChipRun<float, ZP> s;
       march([&](int j, int, float, float q) {
         r[j] -= ta * q;
         s.add(j, r[j] * r[j]);
       });
-      rr_own = s.total(own);
+      rr_own = total(s);
       cp_wait<0>();
       __syncthreads();  // every reader of p is done, and the copies of the ghosts' q have landed
       // x += alpha p, p = r + beta p; the loads of eight planes of x together
@@ -343,15 +333,14 @@ __global__ void __launch_bounds__(BX* BY, 1) k_cg_brick(ChipArgs<float> f) {
 
   // zero-mean gauge (or zero for a zero right side); x held in r
   if (status != 5) {
-    Run s;
+    ChipRun<float, ZP> s;
     planes([&](int j, int g) {
       if (own) r[j] = __ldcg(f.x + g);
       s.add(j, r[j]);
     });
-    Dot<float> ax[1];
-    ax[0].s = s.total(own);
+    F2 v[1] = {total(s)};
     double t[1];
-    const bool ok = grid_dot_t0<1>(ax, gs, t);
+    const bool ok = grid_sum_t0<1>(v, gs, t);
     if (tid == 0) {
       if (!ok) status = 5;
       sc.mean = (float)(t[0] / (double)f.n);

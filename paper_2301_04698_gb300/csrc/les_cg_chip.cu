@@ -225,12 +225,12 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
     int status, restart;
     double bb, rel;  // |b - mean|^2 and the relative residual of x0
   } sc;
-  __shared__ T shv[4][kChipWarps];
+  __shared__ Acc shv[4][kChipWarps];
   __shared__ Acc part[32];
   __shared__ int s_fail;
   double rr = 0.0, bb = 0.0, rel = 0.0;  // meaningful in thread 0
   int status = 0;  // 0 running, 1 converged, 2 maxit, 3 breakdown, 4 zero rhs, 5 timeout
-  T rr_own = T(0);  // this thread's share of r.r for the next sum
+  Acc rr_own{};  // this thread's share of r.r for the next sum
 
   // XS = false: a node's tagged word among the published faces of q
   constexpr int W = Tagged<T>::BYTES;
@@ -249,15 +249,16 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
 
   // mean of b (b held in r)
   {
-    Dot<T> a1[1];
+    ChipRun<T, ZP> a1;
 #pragma unroll
     for (int j = 0; j < ZP; ++j)
       if (j < nzp) {
         r[j] = __ldcg(f.b + gown + j * gpl);
-        a1[0].add(r[j]);
+        a1.add(j, r[j]);
       }
+    Acc v[1] = {a1.total()};
     double t[1];
-    const bool ok = grid_dot_t0<1>(a1, gs, t);
+    const bool ok = grid_sum_t0<1>(v, gs, t);
     if (tid == 0) {
       sc.status = ok ? 0 : 5;
       sc.mean = (T)(t[0] / (double)f.n);
@@ -277,19 +278,20 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
       }
     fill_ghosts(f.x, false);
     __syncthreads();
-    Dot<T> a2[2];
+    ChipRun<T, ZP> a2[2];
 #pragma unroll
     for (int j = 0; j < ZP; ++j)
       if (j < nzp) {
         const T bm = r[j] - mean;
         r[j] = kScaled ? fma(c0, stencil(j, false), bm) : bm - stencil(j, false);
         if (is_face(j)) __stcg(f.rg + gown + j * gpl, r[j]);
-        a2[0].add(r[j] * r[j]);
-        a2[1].add(bm * bm);
+        a2[0].add(j, r[j] * r[j]);
+        a2[1].add(j, bm * bm);
       }
-    rr_own = a2[0].s;
+    rr_own = a2[0].total();
+    Acc v[2] = {rr_own, a2[1].total()};
     double s2[2];
-    const bool ok = grid_dot_t0<2>(a2, gs, s2);
+    const bool ok = grid_sum_t0<2>(v, gs, s2);
     if (tid == 0) {
       // the plain solver judges a learned first guess: if it leaves a larger
       // residual than x0 = 0, restart from zero (r = b - mean b, r.r = |b|^2)
@@ -301,15 +303,16 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
     __syncthreads();
     status = sc.status;
     if (!status && sc.restart) {
-      rr_own = T(0);
+      ChipRun<T, ZP> s;
 #pragma unroll
       for (int j = 0; j < ZP; ++j)
         if (j < nzp) {
           set_x(j, T(0));
           r[j] = __ldcg(f.b + gown + j * gpl) - mean;
-          rr_own += r[j] * r[j];
+          s.add(j, r[j] * r[j]);
           if (is_face(j)) __stcg(f.rg + gown + j * gpl, r[j]);
         }
+      rr_own = s.total();
       Dot<T> none[1];
       double t[1];
       const bool ok2 = grid_dot_t0<1>(none, gs, t);  // a grid barrier: the new faces are visible
@@ -353,16 +356,16 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
       // of the loop they would take the registers of the vectors
       asm volatile("" : "+r"(pown), "+r"(gown));
       T* qw = (iter & 1) ? f.qg1 : f.qg0;  // this iteration's q faces
-      T d0 = T(0), d2 = T(0), d3 = T(0);   // p.q, r.q, q.q
+      ChipRun<T, ZP> d0, d2, d3;           // p.q, r.q, q.q
       each_plane([&](int j, bool inner) {
         q[j] = stencil(j, inner);
         if (is_face(j)) {
           if constexpr (XS) __stcg(qw + gown + j * gpl, q[j]);
           else tagged_store(word(iter & 1, gown + j * gpl), q[j], iter);
         }
-        d0 += p[j] * q[j];
-        d2 += r[j] * q[j];
-        d3 += q[j] * q[j];
+        d0.add(j, p[j] * q[j]);
+        d2.add(j, r[j] * q[j]);
+        d3.add(j, q[j] * q[j]);
       });
       Tagged<T> gq[NG];  // the q of the ghosts
       Acc tot[4];        // the totals, in warp 0
@@ -377,7 +380,7 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
       };
       if constexpr (XS) {
         chip_sum<1, WORDS>(
-            f, iter, d0, rr_own, d2, d3, shv, part, tot, s_fail, deferred,
+            f, iter, d0.total(), rr_own, d2.total(), d3.total(), shv, part, tot, s_fail, deferred,
             [&] {
               const int t0 = 32 * chip_ghost_warp<1>();
               for (int id = tid - t0; id < ngh; id += nthr - t0) cp_async(GQ + id, qw + GT[id].y);
@@ -389,7 +392,7 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
 #pragma unroll
         for (int g = 0; g < NG; ++g) miss |= gsm[g] >= 0 ? 1u << g : 0u;
         chip_sum<-1, WORDS>(
-            f, iter, d0, rr_own, d2, d3, shv, part, tot, s_fail, deferred,
+            f, iter, d0.total(), rr_own, d2.total(), d3.total(), shv, part, tot, s_fail, deferred,
             [&] {
 #pragma unroll
               for (int g = 0; g < NG; ++g)
@@ -425,15 +428,16 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
       ta = sc.ta;
       tb = sc.tb;
       tx = sc.tx;
-      rr_own = T(0);
+      ChipRun<T, ZP> s;
       each_plane([&](int j, bool) {
         if (!kDefer || warp == 0) set_x(j, get_x(j) + tx * p[j]);
         else po[kDefer ? j : 0] = p[j];
         r[j] -= ta * q[j];
-        rr_own += r[j] * r[j];
+        s.add(j, r[j] * r[j]);
         p[j] = r[j] + tb * p[j];
         P[pown + j * SZ] = p[j];
       });
+      rr_own = s.total();
       if constexpr (XS) {
         for (int id = tid; id < ngh; id += nthr) {
           const int at = GT[id].x;
@@ -458,12 +462,13 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
 
   // zero-mean gauge (or zero for a zero right side), written back to x
   if (status != 5) {
-    Dot<T> ax[1];
+    ChipRun<T, ZP> s;
 #pragma unroll
     for (int j = 0; j < ZP; ++j)
-      if (j < nzp) ax[0].add(get_x(j));
+      if (j < nzp) s.add(j, get_x(j));
+    Acc v[1] = {s.total()};
     double t[1];
-    const bool ok = grid_dot_t0<1>(ax, gs, t);
+    const bool ok = grid_sum_t0<1>(v, gs, t);
     if (tid == 0) {
       if (!ok) status = 5;
       sc.mean = (T)(t[0] / (double)f.n);

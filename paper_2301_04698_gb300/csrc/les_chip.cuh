@@ -66,7 +66,10 @@ __device__ __forceinline__ void chip_part(int n, int parts, int i, int& first, i
 }
 __device__ __forceinline__ int chip_wrap(int i, int n) { return i < 0 ? i + n : (i >= n ? i - n : i); }
 __device__ __forceinline__ F2 acc_of(float v) { return F2{v, 0.f}; }
+__device__ __forceinline__ F2 acc_of(F2 v) { return v; }
 __device__ __forceinline__ double acc_of(double v) { return v; }
+__device__ __forceinline__ float acc_add(float a, float b) { return a + b; }
+__device__ __forceinline__ float acc_xor(float a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
 __device__ __forceinline__ F2 acc_xor(F2 a, int o) {
   return F2{__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
 }
@@ -96,21 +99,47 @@ __device__ __forceinline__ bool chip_scalars(const double (&t)[4], double& ta, d
   return true;
 }
 
+// A thread's sum over the planes 0 .. ZP - 1 of its run, in order: FP32 within 16
+// planes, compensated across, as in the streaming kernels.
+template <typename T, int ZP>
+struct ChipRun;
+template <int ZP>
+struct ChipRun<float, ZP> {
+  F2 s{0.f, 0.f};
+  float run = 0.f;
+  __device__ __forceinline__ void add(int j, float v) {
+    if (j > 0 && j % 16 == 0) {
+      f2_acc(s, run);
+      run = 0.f;
+    }
+    run += v;
+  }
+  __device__ __forceinline__ F2 total() const {
+    F2 t = s;
+    if (ZP > 16) f2_acc(t, run);
+    else t.hi = run;
+    return t;
+  }
+};
+template <int ZP>
+struct ChipRun<double, ZP> {
+  double s = 0.0;
+  __device__ __forceinline__ void add(int, double v) { s += v; }
+  __device__ __forceinline__ double total() const { return s; }
+};
+
 // a warp's four values by a transposing butterfly (six additions instead of twenty)
-template <typename T>
-__device__ __forceinline__ void chip_butterfly(T d0, T d1, T d2, T d3, T (&shv)[4][kChipWarps]) {
+template <typename D>
+__device__ __forceinline__ void chip_butterfly(D d0, D d1, D d2, D d3, D (&shv)[4][kChipWarps]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   // after the butterfly lanes 8k .. 8k + 7 hold the warp's value k
   const bool up = lane & 16, odd = lane & 8;
-  T a0 = up ? d2 : d0, a1 = up ? d3 : d1;        // kept
-  const T s0 = up ? d0 : d2, s1 = up ? d1 : d3;  // given to lane ^ 16
-  a0 += __shfl_xor_sync(0xffffffffu, s0, 16);
-  a1 += __shfl_xor_sync(0xffffffffu, s1, 16);
-  T v = odd ? a1 : a0;
-  v += __shfl_xor_sync(0xffffffffu, odd ? a0 : a1, 8);
-  v += __shfl_xor_sync(0xffffffffu, v, 4);
-  v += __shfl_xor_sync(0xffffffffu, v, 2);
-  v += __shfl_xor_sync(0xffffffffu, v, 1);
+  const D s0 = up ? d0 : d2, s1 = up ? d1 : d3;  // given to lane ^ 16
+  const D a0 = acc_add(up ? d2 : d0, acc_xor(s0, 16)), a1 = acc_add(up ? d3 : d1, acc_xor(s1, 16));
+  D v = acc_add(odd ? a1 : a0, acc_xor(odd ? a0 : a1, 8));
+  v = acc_add(v, acc_xor(v, 4));
+  v = acc_add(v, acc_xor(v, 2));
+  v = acc_add(v, acc_xor(v, 1));
   if ((lane & 7) == 0) shv[lane >> 3][warp] = v;
 }
 
@@ -229,14 +258,14 @@ __device__ __forceinline__ int chip_ghost_warp() {
 }
 
 // The grid-wide sum of p.q, r.r, r.q and q.q at iteration `iter`: each warp's four
-// values by a transposing butterfly; warp 0 combines the warps' (FP32 ones as
-// compensated pairs) and posts the block's; the first kFoldWarps warps read the words
-// of a part of the blocks each, until all have come, and fold them in a fixed order,
-// so every block obtains the same totals in tot (in // so every block obtains the same totals in tot (in warp 0); Words of a lane's loads
-// are in flight together (3 of 8 warps or 5 of 4 read 160 blocks or more in one turn;
-// fewer cost another trip, more registers).  meanwhile() runs in every
-// warp but warp 0: before its wait, or after it where the warp folds or acquires and
-// the neighbours' words are counted.
+// values by a transposing butterfly (D: the threads' sums, FP64, compensated FP32 pairs,
+// or plain FP32); warp 0 combines the warps' (FP32 ones as compensated pairs) and posts
+// the block's; the first kFoldWarps warps read the words of a part of the blocks each,
+// until all have come, and fold them in a fixed order, so every block obtains the same
+// totals in tot (in warp 0).  Words of a lane's loads are in flight together (3 of 8
+// warps or 5 of 4 read 160 blocks or more in one turn; fewer cost another trip, more
+// registers).  meanwhile() runs in every warp but warp 0: before its wait, or after it
+// where the warp folds or acquires and the neighbours' words are counted.
 //   What a block awaits of its neighbours comes in one of two ways.  As tagged words
 // (W0 < 0): when the sum has come, issue() starts the loads of what this thread awaits,
 // check() takes what has come and tells whether that was all, and both are called
@@ -251,8 +280,8 @@ __device__ __forceinline__ int chip_ghost_warp() {
 struct ChipNothing {
   __device__ __forceinline__ bool operator()() const { return true; }
 };
-template <int W0, int Words, typename Args, typename T, typename Acc, typename Meanwhile, typename Issue, typename Check>
-__device__ __forceinline__ void chip_sum(const Args& f, int iter, T d0, T d1, T d2, T d3, T (&shv)[4][kChipWarps],
+template <int W0, int Words, typename Args, typename D, typename Acc, typename Meanwhile, typename Issue, typename Check>
+__device__ __forceinline__ void chip_sum(const Args& f, int iter, D d0, D d1, D d2, D d3, D (&shv)[4][kChipWarps],
                                          Acc (&part)[32], Acc (&tot)[4], volatile int& fail, Meanwhile&& meanwhile,
                                          Issue&& issue, Check&& check) {
   const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5, nwarp = nthr >> 5;
@@ -269,7 +298,7 @@ __device__ __forceinline__ void chip_sum(const Args& f, int iter, T d0, T d1, T 
   if (warp == 0) {
     // lanes 8k .. 8k + 7: value k of the block
     const int k = lane >> 3, c = lane & 7;
-    Acc a = acc_of(T(0));
+    Acc a{};
     for (int w = c; w < nwarp; w += 8) a = acc_add(a, acc_of(shv[k][w]));
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) a = acc_add(a, acc_xor(a, o));
@@ -292,7 +321,7 @@ __device__ __forceinline__ void chip_sum(const Args& f, int iter, T d0, T d1, T 
   };
   if (warp < FW) {
     for (int id = warp; id < FW; id += nwarp) {  // eight blocks at a time, a lane per value
-      Acc t = acc_of(T(0));
+      Acc t{};
       for (unsigned base = (unsigned)id * 8 + (lane >> 2); base - (lane >> 2) < G; base += 8 * FW * U) {
         const char* at = slot + ((size_t)base * 4 + (lane & 3)) * W;
         Tagged<Acc> w[U];
@@ -309,7 +338,7 @@ __device__ __forceinline__ void chip_sum(const Args& f, int iter, T d0, T d1, T 
           if (__all_sync(0xffffffffu, miss == 0u && f.missing == 0u) || over(spins)) break;
         }
 #pragma unroll
-        for (int u = 0; u < U; ++u) t = acc_add(t, base + 8 * FW * u < G ? tagged_value(w[u]) : acc_of(T(0)));
+        for (int u = 0; u < U; ++u) t = acc_add(t, base + 8 * FW * u < G ? tagged_value(w[u]) : Acc{});
       }
       if (!Counted && id + nwarp >= FW) {
         if (nwarp > FW) asm volatile("bar.arrive 1, %0;" ::"r"(nthr) : "memory");
