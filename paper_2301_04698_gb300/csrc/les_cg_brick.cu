@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(BX* BY, 1) k_cg_brick(ChipArgs<float> f) {
     ChipRun<float, ZP> s0, s1;
     march([&](int j, int g, float, float q) {
       const float bm = r[j] - mean;
-      r[j] = bm - q;
+      r[j] = bm - f.sc * q;
       if (is_face(j)) __stcg(f.rg + g, r[j]);
       s0.add(j, r[j] * r[j]);
       s1.add(j, bm * bm);
@@ -300,10 +300,16 @@ __global__ void __launch_bounds__(BX* BY, 1) k_cg_brick(ChipArgs<float> f) {
       rr_own = total(s);
       cp_wait<0>();
       __syncthreads();  // every reader of p is done, and the copies of the ghosts' q have landed
+      each_ghost(AllWarps{}, [&](int id, float* at, int) {
+        const float rv = GR[id] - ta * GQ[id];
+        GR[id] = rv;
+        *at = rv + tb * *at;
+      });
       // x += alpha p, p = r + beta p; the loads of eight planes of x together
       if (own) {
         int g = g0;
         asm volatile("" : "+r"(g));
+        const float tx = ta * f.isc;  // alpha of x
 #pragma unroll
         for (int b = 0; b < ZP; b += 8) {
           float xv[8];
@@ -314,17 +320,12 @@ __global__ void __launch_bounds__(BX* BY, 1) k_cg_brick(ChipArgs<float> f) {
           for (int c = 0; c < 8; ++c)
             if (b < ZP - 8 || b + c < bz) {
               const float pv = C[SZ * (b + c)];
-              __stcg(f.x + g + c * gpl, xv[c] + ta * pv);
+              __stcg(f.x + g + c * gpl, xv[c] + tx * pv);
               C[SZ * (b + c)] = r[b + c] + tb * pv;
             }
           g += 8 * gpl;
         }
       }
-      each_ghost(AllWarps{}, [&](int id, float* at, int) {
-        const float rv = GR[id] - ta * GQ[id];
-        GR[id] = rv;
-        *at = rv + tb * *at;
-      });
       iter += 1;
       __syncthreads();
     }

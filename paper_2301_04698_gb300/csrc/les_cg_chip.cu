@@ -45,6 +45,7 @@
 // x neighbours by shuffles: 128 x 64 x 64 2.8 there, 64 x 128 x 64 3.3 here; 128 x
 // 128 x 96 4.5, 96 x 128 x 128 7.2.
 #include <algorithm>
+#include <cmath>
 #include <string>
 
 #include "les_chip.cuh"
@@ -283,7 +284,7 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
     for (int j = 0; j < ZP; ++j)
       if (j < nzp) {
         const T bm = r[j] - mean;
-        r[j] = kScaled ? fma(c0, stencil(j, false), bm) : bm - stencil(j, false);
+        r[j] = kScaled ? fma(c0, stencil(j, false), bm) : bm - f.sc * stencil(j, false);
         if (is_face(j)) __stcg(f.rg + gown + j * gpl, r[j]);
         a2[0].add(j, r[j] * r[j]);
         a2[1].add(j, bm * bm);
@@ -405,21 +406,24 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
               return miss == 0u;
             });
       }
-      if (tid == 0) {  // the status, alpha and beta
-        int st = 0;
-        if (s_fail) {
-          st = 5;
-        } else {
-          rr_last = tot[1];
-          T al = T(0), be = T(0);
-          if (acc_le(tot[1], rr_stop)) st = 1;
-          else if (iter >= f.maxit) st = 2;
-          else if (!chip_scalars(tot, al, be)) st = 3;
-          sc.ta = al;
-          sc.tb = be;
-          sc.tx = kScaled ? al * mc0 : al;
+      if (warp == 0) {  // the status, alpha and beta
+        T al = T(0), be = T(0);
+        const bool good = chip_scalars(tot, al, be);
+        if (tid == 0) {
+          int st = 0;
+          if (s_fail) {
+            st = 5;
+          } else {
+            rr_last = tot[1];
+            if (acc_le(tot[1], rr_stop)) st = 1;
+            else if (iter >= f.maxit) st = 2;
+            else if (!good) st = 3;
+            sc.ta = al;
+            sc.tb = be;
+            sc.tx = kScaled ? al * mc0 : al * f.isc;
+          }
+          sc.status = st;
         }
-        sc.status = st;
       }
       if constexpr (XS) cp_wait<0>();
       __syncthreads();
@@ -631,9 +635,13 @@ int poisson_solve_chip(const SolverArgs<T>& a, const FusedCfg& fc, const T* b, T
   f.ny = a.g.ny;
   f.nz = a.g.nz;
   f.walls = a.g.walls;
-  f.cx = a.g.idx * a.g.idx;
-  f.cy = a.g.idy * a.g.idy;
-  f.cz = a.g.idz * a.g.idz;
+  f.sc = sizeof(T) == 4 ? (T)std::ldexp(1.0, std::ilogb(2.0 * ((double)a.g.idx * a.g.idx + (double)a.g.idy * a.g.idy +
+                                                              (double)a.g.idz * a.g.idz)))
+                        : T(1);
+  f.isc = T(1) / f.sc;
+  f.cx = a.g.idx * a.g.idx * f.isc;
+  f.cy = a.g.idy * a.g.idy * f.isc;
+  f.cz = a.g.idz * a.g.idz * f.isc;
   f.px = pl.px;
   f.py = pl.py;
   f.pz = pl.pz;

@@ -19,7 +19,10 @@ constexpr int kChipGhosts = 4;      // ghost nodes per thread in registers
 template <typename T>
 struct ChipArgs {
   int nx, ny, nz, walls;
-  T cx, cy, cz;        // 1/dx^2, 1/dy^2, 1/dz^2
+  // 1/dx^2, 1/dy^2, 1/dz^2; FP32: times 2^-k, so that q is of the size of p and the four
+  // sums of the size of r.r, whatever the spacings (exact, but for what would leave the range)
+  T cx, cy, cz;
+  T sc, isc;           // 2^k, 2^-k (FP64: 1)
   int px, py, pz, zs;  // bricks along x, y, z; runs of planes per brick
   int smem_p, smem_g;  // shared memory of P and (XS) of one ghost array, in elements (even)
   long long n;
@@ -89,13 +92,17 @@ __device__ __forceinline__ bool chip_scalars(const F2 (&t)[4], float& ta, float&
   tb = fmaf(alpha * alpha, q2, fmaf(-2.f * alpha, rq, r2)) / r2;  // |r - alpha q|^2 / r.r
   return true;
 }
+// FP64: called by the whole of warp 0, for both quotients take one division, a lane each.
+// (One of 1 / (r.r p.q) for both would leave the range of FP64 where r.r is beyond
+// 1e154 or below 1e-154.)
 __device__ __forceinline__ bool chip_scalars(const double (&t)[4], double& ta, double& tb) {
   const double pq = t[0], r2 = t[1], rq = t[2], q2 = t[3];
+  const bool odd = threadIdx.x & 1;
+  const double quo = (odd ? 1.0 : r2) / (odd ? r2 : pq);
+  const double alpha = __shfl_sync(0xffffffffu, quo, 0), ir2 = __shfl_sync(0xffffffffu, quo, 1);
   if (!(pq != 0.0) || !isfinite(pq) || !isfinite(r2)) return false;
-  const double inv = 1.0 / (r2 * pq);  // one FP64 division for both
-  const double alpha = r2 * r2 * inv;
   ta = alpha;
-  tb = fma(alpha * alpha, q2, fma(-2.0 * alpha, rq, r2)) * (pq * inv);
+  tb = fma(alpha, fma(alpha, q2, -2.0 * rq), r2) * ir2;
   return true;
 }
 
