@@ -82,6 +82,17 @@ __device__ __forceinline__ float4 ldg4(const float* p) { return __ldcg(reinterpr
 __device__ __forceinline__ void stg4(float* p, float4 v) { __stcg(reinterpret_cast<float4*>(p), v); }
 
 
+// alpha and beta from the totals, in FP32 from their high parts; false on a zero or
+// non-finite p.q or r.r
+__device__ __forceinline__ bool reg_scalars(const F2 (&t)[4], float& ta, float& tb) {
+  const float pq = t[0].hi, r2 = t[1].hi, rq = t[2].hi, q2 = t[3].hi;
+  if (!(pq != 0.f) || !isfinite(pq) || !isfinite(r2)) return false;
+  const float alpha = r2 / pq;
+  ta = alpha;
+  tb = fmaf(alpha * alpha, q2, fmaf(-2.f * alpha, rq, r2)) / r2;  // |r - alpha q|^2 / r.r
+  return true;
+}
+
 template <int ZP>
 __global__ void __launch_bounds__(kRegMaxWarps * 32, 1) k_cg_regs(RegArgs f) {
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -340,7 +351,7 @@ __global__ void __launch_bounds__(kRegMaxWarps * 32, 1) k_cg_regs(RegArgs f) {
           rr_last = tot[1];
           if (acc_le(tot[1], rr_stop)) st = 1;
           else if (iter >= f.maxit) st = 2;
-          else if (!chip_scalars(tot, al, be)) st = 3;
+          else if (!reg_scalars(tot, al, be)) st = 3;
         }
         sc.ta = al;
         sc.tb = be;

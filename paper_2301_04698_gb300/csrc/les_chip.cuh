@@ -82,14 +82,33 @@ __device__ __forceinline__ F2 acc_from_lane(F2 a, int l) {
 }
 __device__ __forceinline__ double acc_from_lane(double a, int l) { return __shfl_sync(0xffffffffu, a, l); }
 
-// alpha and beta from the totals; false on a zero or non-finite p.q or r.r.
-// An FP32 solve takes them in FP32 from the high parts of the totals.
+// alpha and beta from the totals; false on a zero or non-finite p.q or r.r.  beta is
+// |r - alpha q|^2 / r.r, expanded in the totals: where next to nothing is left of r the
+// expansion may come out below zero, and is taken for none.
+// FP32: from the totals as pairs, each product and addition with its rounding error, and
+// rounded once (from FP64 totals in FP64 they would take thread 0 about a microsecond).
+// (a quotient from an approximate reciprocal ib of b and its remainder)
+__device__ __forceinline__ float rcp_approx(float x) {
+  float y;
+  asm("rcp.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float f2_quotient(F2 a, F2 b, float ib) {
+  const float q = a.hi * ib;
+  return q + (fmaf(-q, b.hi, a.hi) + fmaf(-q, b.lo, a.lo)) * ib;
+}
 __device__ __forceinline__ bool chip_scalars(const F2 (&t)[4], float& ta, float& tb) {
-  const float pq = t[0].hi, r2 = t[1].hi, rq = t[2].hi, q2 = t[3].hi;
-  if (!(pq != 0.f) || !isfinite(pq) || !isfinite(r2)) return false;
-  const float alpha = r2 / pq;
-  ta = alpha;
-  tb = fmaf(alpha * alpha, q2, fmaf(-2.f * alpha, rq, r2)) / r2;  // |r - alpha q|^2 / r.r
+  const F2 pq = t[0], r2 = t[1], rq = t[2], q2 = t[3];
+  if (!(pq.hi != 0.f) || !isfinite(pq.hi) || !isfinite(r2.hi)) return false;
+  const float ir = rcp_approx(r2.hi);
+  ta = f2_quotient(r2, pq, rcp_approx(pq.hi));
+  const float m = -2.f * ta, a2 = ta * ta, u = m * rq.hi, v = a2 * q2.hi;
+  F2 n = r2;
+  f2_acc(n, u);
+  f2_acc(n, v);
+  n.lo += (fmaf(m, rq.hi, -u) + m * rq.lo) + (fmaf(a2, q2.hi, -v) + a2 * q2.lo) + fmaf(ta, ta, -a2) * q2.hi;
+  tb = f2_quotient(n, r2, ir);
+  tb = tb < 0.f ? 0.f : tb;
   return true;
 }
 // FP64: called by the whole of warp 0, for both quotients take one division, a lane each.
@@ -102,7 +121,8 @@ __device__ __forceinline__ bool chip_scalars(const double (&t)[4], double& ta, d
   const double alpha = __shfl_sync(0xffffffffu, quo, 0), ir2 = __shfl_sync(0xffffffffu, quo, 1);
   if (!(pq != 0.0) || !isfinite(pq) || !isfinite(r2)) return false;
   ta = alpha;
-  tb = fma(alpha, fma(alpha, q2, -2.0 * rq), r2) * ir2;
+  const double beta = fma(alpha, fma(alpha, q2, -2.0 * rq), r2) * ir2;
+  tb = beta < 0.0 ? 0.0 : beta;
   return true;
 }
 

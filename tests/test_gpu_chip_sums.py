@@ -62,3 +62,17 @@ def test_residual_norm_of_spikes_in_a_faint_field(shape, planes, seed):
     r1 = r0 + laplacian(r0) / 8
     assert np.array_equal(r1, r1.astype(np.float32))
     assert abs(res / np.sqrt((r1 * r1).sum() / (r0 * r0).sum()) - 1) < 1e-9
+
+
+@pytest.mark.parametrize("shape", [(64, 64, 64), (100, 76, 61), (150, 140, 70), (150, 130, 110)])
+def test_alpha_is_rounded_once(shape):
+    """alpha = r.r / p.q from the totals' full precision: within half an ulp of its value
+    in FP64, and what the sums themselves are off (random over the threads, 1e-9 of a
+    total; allowed: a twentieth of an ulp).  From the high parts alone it is up to one and
+    a half."""
+    nx, ny, nz = shape
+    for seed in range(8):
+        b = inputs.uniform(300 + seed, 0, nx * ny * nz, -1, 1).reshape(nz, ny, nx).astype(np.float32)
+        alpha, res, r0 = first_step(shape, b)
+        exact = (r0 * r0).sum() / (r0 * laplacian(r0)).sum()
+        assert abs(alpha - exact) <= 0.55 * np.spacing(np.abs(np.float32(exact))), seed
