@@ -64,6 +64,7 @@ __global__ void __launch_bounds__(kStreamThreads, 2) k_cg_stream(StreamArgs<T> f
   __shared__ struct {
     T ta, tb, mean;
     int status, restart;
+    int e;  // the size of the sums (binary exponent): that of |b - mean|^2
   } sc;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int plane = f.nx * f.ny;
@@ -155,6 +156,7 @@ __global__ void __launch_bounds__(kStreamThreads, 2) k_cg_stream(StreamArgs<T> f
     }
     sc.status = status;
     sc.ta = sc.tb = T(0);
+    sc.e = (__double2hiint(bb) >> 20 & 0x7ff) - 1023;
   }
   __syncthreads();
   status = sc.status;
@@ -167,7 +169,7 @@ __global__ void __launch_bounds__(kStreamThreads, 2) k_cg_stream(StreamArgs<T> f
     const T tb = sc.tb;
     const T* po = f.p[(iter + 1) & 1];
     T* pw = f.p[iter & 1];
-    StreamSum<T> s[1];
+    StreamSum<T> s;
     StreamTurns<Shares> turns(f.nunits);
     int tile, k0, kn;
     while (turns.next(f.nchunk, f.nz, tile, k0, kn)) {
@@ -234,10 +236,10 @@ __global__ void __launch_bounds__(kStreamThreads, 2) k_cg_stream(StreamArgs<T> f
             if (go[m] >= 0) {
               __stcg(f.q + base - plane + go[m], qv);
               __stcg(pw + base - plane + go[m], pc[m]);
-              s[0].add(pc[m] * qv);
+              s.add(pc[m] * qv);
             }
           }
-          s[0].tick();
+          s.tick();
         }
         if (!inside) break;
         __syncthreads();  // plane k is in sm (the other buffer's readers passed the barrier before)
@@ -256,10 +258,9 @@ __global__ void __launch_bounds__(kStreamThreads, 2) k_cg_stream(StreamArgs<T> f
         }
       }
     }
-    double t[1];
-    bool ok = stream_sum<1>(s, gs, t);
+    double pq, rr_new;
+    bool ok = stream_sum_scaled(s, sc.e, gs, pq);
     if (tid == 0) {
-      const double pq = t[0];
       if (!ok) status = 5;
       else if (pq == 0.0 || !isfinite(pq)) status = 3;
       else sc.ta = (T)(rr / pq);
@@ -273,7 +274,7 @@ __global__ void __launch_bounds__(kStreamThreads, 2) k_cg_stream(StreamArgs<T> f
     ta = kScaled ? -tq / c0 : tq;
     pend = true;
     // B: r -= alpha q, r.r
-    StreamSum<T> sb[1];
+    StreamSum<T> sb;
     {
       constexpr int V = StreamVec<T>::N, U = 4;
       const long long nv = f.n / V;
@@ -291,30 +292,31 @@ __global__ void __launch_bounds__(kStreamThreads, 2) k_cg_stream(StreamArgs<T> f
 #pragma unroll
             for (int e = 0; e < V; ++e) {
               ra[j].v[e] -= tq * qa[j].v[e];
-              sb[0].add(ra[j].v[e] * ra[j].v[e]);
+              sb.add(ra[j].v[e] * ra[j].v[e]);
             }
-            sb[0].tick();
+            sb.tick();
             svst(f.r + (v0 + j * gstride) * V, ra[j]);
           }
       }
       for (long long m = nv * V + gtid; m < f.n; m += gstride) {
         const T v = __ldcg(f.r + m) - tq * __ldcg(f.q + m);
-        sb[0].add(v * v);
+        sb.add(v * v);
+        sb.tick();
         __stcg(f.r + m, v);
       }
     }
-    ok = stream_sum<1>(sb, gs, t);
+    ok = stream_sum_scaled(sb, sc.e, gs, rr_new);
     iter += 1;
     if (tid == 0) {
       if (!ok) {
         status = 5;
       } else {
-        rel = sqrt(t[0] / bb);
-        sc.tb = (T)(t[0] / rr);
-        rr = t[0];
+        rel = sqrt(rr_new / bb);
+        sc.tb = (T)(rr_new / rr);
+        rr = rr_new;
         if (rel <= f.tol) status = 1;
         else if (iter >= f.maxit) status = 2;
-        else if (!isfinite(t[0])) status = 3;
+        else if (!isfinite(rr_new)) status = 3;
       }
       sc.status = status;
     }

@@ -50,3 +50,10 @@ def test_on_chip_cg(les_mod, precision, shape):
         check(les_mod, shape, 64, (-300, 300), 1.0, 1e-8, 2000)
     else:
         check(les_mod, shape, 32, (-30, 43), 1 / 64, 1e-5, 2000)
+
+
+@pytest.mark.parametrize("shape", [(128, 24, 40), (70, 33, 40)])
+def test_streaming_cg(les_mod, shape):
+    """Whole tiles, and ragged ones.  Squares of 2^57 fit FP32, their sum over the grid
+    does not."""
+    check(les_mod, shape, 32, (-20, 57), 35.0, 1e-3, 2000, tuning=dict(cg_resident=1, cg_variant=0))
