@@ -9,11 +9,19 @@
 // complete when the plane above arrives.  A grid-wide sum per sweep gives the
 // residual norm of the x it read; x is double-buffered.
 //
+// The norm decides when the solver stops, for residuals of any size that FP32 holds, so
+// no square is rounded to FP32 or leaves its range: the first sweep of an FP32 solve
+// squares and adds in FP64, the later ones in FP32 with each square's and addition's
+// rounding error kept, of residuals scaled by a power of two to the size of the last
+// sweep's.
+//
 // What bounds it: per sweep three fields (x and b in, x out) and the grid sum
 // (about 3 us).  Measured on 256 x 256 x 64 in FP32 (the fields lie in L2): a
 // launch per sweep, with every neighbour through L1 and a division per node, 70
-// us; here 15.
+// us; here 15.  Of a solve's 108 us beside its sweeps 39 are FP64 arithmetic (the right
+// side's norm, the first sweep).
 #include <algorithm>
+#include <cmath>
 #include <string>
 #include <type_traits>
 
@@ -30,6 +38,7 @@ struct JacobiArgs {
   T wd, wd_wall;         // omega / diag(L_c), inside and on a plane next to a wall
   int ntx, nty, nchunk;  // tiles along x and y, runs of planes per tile
   long long n, nunits;
+  int en;                // binary exponent of n
   const T* b;
   T* x[2];               // x_s in x[s & 1]; x[0] the caller's
   double* partials;
@@ -47,6 +56,7 @@ __global__ void __launch_bounds__(kStreamThreads, 2) k_jacobi_stream(JacobiArgs<
   __shared__ T sm[2][SN];
   __shared__ struct {
     T mean;
+    int e;  // FP32: the residuals' size (binary exponent) at the last sweep
     int status;
   } sc;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -58,15 +68,20 @@ __global__ void __launch_bounds__(kStreamThreads, 2) k_jacobi_stream(JacobiArgs<
   double bb = 0.0, rel = 0.0;  // meaningful in thread 0
   int status = 0;  // 0 running, 1 converged, 2 maxit, 3 non-finite, 4 zero rhs, 5 timeout
 
-  // this thread's sums over the nodes of v
+  // sums over the nodes: of FP64 terms in FP64, of FP32 ones with the additions' rounding
+  // errors kept
   auto sum_of = [&](auto&& term) {
-    StreamSum<T> s[1];
-    for (long long m = gtid; m < f.n; m += gstride) {
-      s[0].add(term(m));
-      s[0].tick();
+    double v[1] = {0.0}, t[1];
+    if constexpr (std::is_same<decltype(term(gtid)), float>::value) {
+      F2 a{0.f, 0.f};
+#pragma unroll 4
+      for (long long m = gtid; m < f.n; m += gstride) f2_acc(a, term(m));
+      v[0] = f2_value(a);
+    } else {
+#pragma unroll 4
+      for (long long m = gtid; m < f.n; m += gstride) v[0] += term(m);
     }
-    double t[1];
-    const bool ok = stream_sum<1>(s, gs, t);
+    const bool ok = grid_sum_t0<1>(v, gs, t);
     if (tid == 0 && !ok) status = 5;
     return t[0];
   };
@@ -82,7 +97,7 @@ __global__ void __launch_bounds__(kStreamThreads, 2) k_jacobi_stream(JacobiArgs<
   const T mean = sc.mean;
   if (!status) {
     const double t = sum_of([&](long long m) {
-      const T v = __ldcg(f.b + m) - mean;
+      const double v = (double)(__ldcg(f.b + m) - mean);
       return v * v;
     });
     if (tid == 0) {
@@ -95,10 +110,23 @@ __global__ void __launch_bounds__(kStreamThreads, 2) k_jacobi_stream(JacobiArgs<
   }
 
   int sweep = 0;
-  while (!status) {
+  // the sweep's sum of squares, FP64 or compensated, into t (thread 0)
+  auto relax = [&](auto exact, double (&t)[1]) -> bool {
+    constexpr bool EXACT = decltype(exact)::value;
     const T* xin = f.x[sweep & 1];
     T* xout = f.x[(sweep + 1) & 1];
-    StreamSum<T> s[1];
+    const float scale = EXACT ? 1.f : __int_as_float((127 - sc.e) << 23);
+    double sd[1] = {0.0};
+    F2 sf[1] = {F2{0.f, 0.f}};
+    auto square = [&](T r) {
+      if constexpr (EXACT) {
+        sd[0] += (double)r * (double)r;
+      } else {
+        const float v = r * scale, p = v * v;
+        f2_acc(sf[0], p);
+        sf[0].lo += fmaf(v, v, -p);
+      }
+    };
     for (long long u = blockIdx.x; u < f.nunits; u += gridDim.x) {
       const int tile = (int)(u / f.nchunk), chunk = (int)(u - (long long)tile * f.nchunk);
       int x0, y0, w, h, k0, kn;
@@ -157,9 +185,8 @@ __global__ void __launch_bounds__(kStreamThreads, 2) k_jacobi_stream(JacobiArgs<
               if (FULL || go[m] >= 0) {
                 const T r = bc[m] - (part[m] + (pd[m] + pv[m] - T(2) * pc[m]) * cz);
                 __stcg(xout + base + go[m], pc[m] + wd * r);
-                s[0].add(r * r);
+                square(r);
               }
-            s[0].tick();
           }
           if (!inside) break;
           __syncthreads();  // plane k is in sm (the other buffer's readers passed the barrier before)
@@ -177,8 +204,19 @@ __global__ void __launch_bounds__(kStreamThreads, 2) k_jacobi_stream(JacobiArgs<
       if (w == S::WX && h == S::WY) march(std::true_type{});
       else march(std::false_type{});
     }
+    if constexpr (EXACT) {
+      return grid_sum_t0<1>(sd, gs, t);
+    } else {
+      const bool ok = grid_sum_t0<1>(sf, gs, t);
+      if (tid == 0) t[0] *= pow2(2 * sc.e);
+      return ok;
+    }
+  };
+  while (!status) {
     double t[1];
-    const bool ok = stream_sum<1>(s, gs, t);
+    bool ok;
+    if constexpr (sizeof(T) == 8) ok = relax(std::true_type{}, t);
+    else ok = sweep == 0 ? relax(std::true_type{}, t) : relax(std::false_type{}, t);
     if (tid == 0) {
       if (!ok) {
         status = 5;
@@ -188,6 +226,7 @@ __global__ void __launch_bounds__(kStreamThreads, 2) k_jacobi_stream(JacobiArgs<
         if (!isfinite(t[0])) status = 3;
         else if (rel <= f.tol) status = 1;
         else if (sweep >= f.maxit) status = 2;
+        else sc.e = max(-126, min(126, ((__double2hiint(t[0]) >> 20 & 0x7ff) - 1023 - f.en) >> 1));
       }
       sc.status = status;
     }
@@ -271,6 +310,7 @@ int poisson_solve_jacobi(const SolverArgs<T>& a, const FusedCfg& fc, const T* b,
   f.nchunk = pl.nchunk;
   f.nunits = pl.units;
   f.n = (long long)f.nx * f.ny * f.nz;
+  f.en = std::ilogb((double)f.n);
   f.b = b;
   f.x[0] = x;
   f.x[1] = a.p0;

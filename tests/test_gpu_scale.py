@@ -57,3 +57,9 @@ def test_streaming_cg(les_mod, shape):
     """Whole tiles, and ragged ones.  Squares of 2^57 fit FP32, their sum over the grid
     does not."""
     check(les_mod, shape, 32, (-20, 57), 35.0, 1e-3, 2000, tuning=dict(cg_resident=1, cg_variant=0))
+
+
+@pytest.mark.parametrize("precision,shape", [(32, (65, 33, 20)), (32, (128, 40, 20)), (64, (33, 31, 9))])
+def test_jacobi(les_mod, precision, shape):
+    e = 80 if precision == 32 else 250
+    check(les_mod, shape, precision, (-e, e), 1.0, 1e-30, 20, solver="jacobi")
