@@ -247,8 +247,10 @@ __global__ void __launch_bounds__(C::NT, sizeof(T) == 4 ? 512 / C::NT : 1) k_cg_
   // complete on it; bit s of phase is the parity this thread waits for next
   __shared__ __align__(8) uint64_t bars[D];
   __shared__ decltype(WaveSum<T>().acc()) sums[4][NT];
+  __shared__ long long limit;  // of a wait for copies; -1: one has run out
   unsigned phase = 0;
   if (threadIdx.x == 0) {
+    limit = f.spin_cycles;
     for (int q = 0; q < D; ++q) mbar_init(&bars[q], 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -578,14 +580,16 @@ __global__ void __launch_bounds__(C::NT, sizeof(T) == 4 ? 512 / C::NT : 1) k_cg_
       auto fetch = [&](int sl, int kk) {
         if (tid == NT - 64 || tid == NT - 32) copy(tid == NT - 32, sl, kk);
       };
-      // wait (bounded) for the copies in a ring slot; a wait that runs out raises
-      // the grid's fail flag, so every grid sum of the launch fails
+      // wait (bounded) for the copies in a ring slot.  When one runs out, the block's
+      // later ones do at once, and its sums are not numbers, so that the pass ends as a
+      // timeout in every block.
       auto landed = [&](int sl) {
         if (!mbar_try_wait(&bars[sl], (phase >> sl) & 1u)) {
           const long long t0 = clock64();
           while (!mbar_try_wait(&bars[sl], (phase >> sl) & 1u)) {
-            if (clock64() - t0 > f.spin_cycles) {
+            if (clock64() - t0 > *(volatile long long*)&limit) {
               atomicExch(&f.bar->fail.v, 1u);
+              *(volatile long long*)&limit = -1;
               break;
             }
           }
@@ -720,6 +724,7 @@ __global__ void __launch_bounds__(C::NT, sizeof(T) == 4 ? 512 / C::NT : 1) k_cg_
     WaveSum<T> s[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) s[q] = WaveSum<T>{sums[q][tid]};
+    if (*(volatile long long*)&limit < 0) s[0].add((T)NAN);
     double t[4];
     const bool ok = wave_sum_t0<4>(s, gs, t);
     iter += 1;
@@ -729,7 +734,8 @@ __global__ void __launch_bounds__(C::NT, sizeof(T) == 4 ? 512 / C::NT : 1) k_cg_
       } else {
         const double rr_new = t[0];
         rel = sqrt(rr_new / bb);
-        if (rel <= f.tol) status = 1;
+        if (isnan(rr_new) && ld_volatile(&f.bar->fail.v) != 0u) status = 5;
+        else if (rel <= f.tol) status = 1;
         else if (iter >= f.maxit) status = 2;
         else if (!isfinite(rr_new)) status = 3;
         else {
@@ -784,6 +790,11 @@ __global__ void __launch_bounds__(C::NT, sizeof(T) == 4 ? 512 / C::NT : 1) k_cg_
         for (int q = 0; q < VC; ++q) xq.e[q] = status == 4 ? T(0) : xq.e[q] - mx;
         stch(f.x + (size_t)c * VC, xq);
       }
+    }
+  }
+  if (limit < 0) {  // copies that are still in flight may land before the block ends
+    const long long t0 = clock64();
+    while (clock64() - t0 < f.spin_cycles) {
     }
   }
   if (blockIdx.x == 0 && tid == 0) {
