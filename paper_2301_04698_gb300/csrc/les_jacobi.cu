@@ -342,6 +342,9 @@ int poisson_solve_jacobi(const SolverArgs<T>& a, const FusedCfg& fc, const T* b,
   const SolverCtl& c = *a.ctl_host;
   if (iters) *iters = c.iter;
   if (rel) *rel = c.rel;
+  // the means of b and x and |b|^2: 3, the gauge: x in and out; per pass over the grid,
+  // one more than the sweeps counted, x and b in, x out: 3
+  if (a.prof) a.prof->bytes[KI_JACOBI] += (5.0 + 3.0 * (c.iter + 1)) * (double)f.n * sizeof(T);
   switch (c.done) {
     case 1:
     case 4: return LES_OK;
