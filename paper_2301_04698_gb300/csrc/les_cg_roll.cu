@@ -535,10 +535,8 @@ int poisson_solve_roll(const SolverArgs<T>& a, const FusedCfg& fc, const T* b, T
   const SolverCtl& c = *a.ctl_host;
   if (iters) *iters = c.iter;
   if (rel) *rel = c.rel;
-  // algorithmic traffic of the solve (kCgIterFields per iteration; this
-  // kernel streams 6: r, p_old, x in; p, r, x out; plus one set-up sweep
-  // for alpha_0)
-  if (a.prof) a.prof->bytes[KI_CG_ROLL] += (kCgSetupFields + 1.0 + kCgIterFields * c.iter) * (double)f.n * sizeof(T);
+  // algorithmic traffic of the solve, with one set-up sweep for alpha_0
+  if (a.prof) a.prof->bytes[KI_CG_ROLL] += (kCgSetupFields + 1.0 + kCgOnePassFields * c.iter) * (double)f.n * sizeof(T);
   switch (c.done) {
     case 1:
     case 4: return LES_OK;

@@ -450,8 +450,8 @@ int poisson_solve_stream(const SolverArgs<T>& a, const FusedCfg& fc, const T* b,
   const SolverCtl& c = *a.ctl_host;
   if (iters) *iters = c.iter;
   if (rel) *rel = c.rel;
-  // algorithmic traffic of the solve, as for every CG kernel (this one streams
-  // 9 fields per iteration: A r, p, x in, p, q, x out; B r, q in, r out)
+  // algorithmic traffic of the solve (this kernel streams 9 fields per iteration: A r,
+  // p, x in, p, q, x out; B r, q in, r out)
   if (a.prof) a.prof->bytes[KI_CG_FUSED] += (kCgSetupFields + kCgIterFields * c.iter) * (double)f.n * sizeof(T);
   switch (c.done) {
     case 1:

@@ -953,11 +953,9 @@ int solve_wave(const SolverArgs<T>& a, const FusedCfg& fc, const T* b, T* x, dou
   const SolverCtl& c = *a.ctl_host;
   if (iters) *iters = c.iter;
   if (rel) *rel = c.rel;
-  // algorithmic traffic of the solve (kCgIterFields per iteration; this
-  // kernel streams 5 per iteration, x being read and written every other one,
-  // plus a third of r_i and p_{i-1} again for the halo, and one set-up sweep
-  // for alpha_0)
-  if (a.prof) a.prof->bytes[KI_CG_WAVE] += (kCgSetupFields + 1.0 + kCgIterFields * c.iter) * (double)f.n * sizeof(T);
+  // algorithmic traffic of the solve, with one set-up sweep for alpha_0 (the kernel
+  // also reads a third of r_i and p_{i-1} again for the halo)
+  if (a.prof) a.prof->bytes[KI_CG_WAVE] += (kCgSetupFields + 1.0 + kCgWaveFields * c.iter) * (double)f.n * sizeof(T);
   switch (c.done) {
     case 1:
     case 4: return LES_OK;

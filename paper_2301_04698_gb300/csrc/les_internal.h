@@ -48,13 +48,16 @@ struct Phys {
 };
 
 // Device-side solver control block (lives in the workspace).
-// Algorithmic traffic of a CG solve in fields per node, the same for every
-// CG kernel whatever it moves: the set-up (mean of b: 1; r = b - L_c x0:
-// b, x in, r out: 3; the gauge: x twice in, x out: 3) and, per iteration,
-// the matvec with its dot product (p in, q out: 2) and the update (x, p, r,
-// q in; x, r out: 6).  A kernel's DRAM traffic is measured separately.
+// Algorithmic traffic of a CG solve in fields per node: the set-up (mean of b:
+// 1; r = b - L_c x0: b, x in, r out: 3; the gauge: x twice in, x out: 3) and,
+// per iteration, the matvec with its dot product (p in, q out: 2) and the update
+// (x, p, r, q in; x, r out: 6), whatever a kernel moves beyond that.  The kernels
+// that form all of it in one pass need less: r, p and x in and out, x in every other
+// pass in les_cg_wave.cu.  A kernel's DRAM traffic is measured separately.
 constexpr double kCgSetupFields = 7.0;
 constexpr double kCgIterFields = 8.0;
+constexpr double kCgOnePassFields = 6.0;
+constexpr double kCgWaveFields = 5.0;
 
 struct SolverCtl {
   double sum;       // result of the last mean reduction

@@ -29,3 +29,11 @@ def booked(shape, tuning, sweeps, precision=32, **kw):
 def test_jacobi_books_its_sweeps(sweeps):
     """Set-up and gauge 5 fields, each pass over the grid 3."""
     assert booked((40, 33, 9), {}, sweeps, solver="jacobi") == ("jacobi", 5 + 3 * (sweeps + 1))
+
+
+@pytest.mark.parametrize("variant,name,shape,setup,per", [(4, "cg_wave", (128, 64, 32), 8, 5), (3, "cg_roll", (40, 33, 9), 8, 6),
+                                                          (0, "cg_fused", (40, 33, 9), 7, 8), (2, "cg_fused", (128, 64, 32), 7, 8)])
+def test_streaming_cg_books_what_its_algorithm_needs(variant, name, shape, setup, per):
+    """8 fields per iteration, fewer where one pass forms all of it: a rate above that of
+    memory would not be one."""
+    assert booked(shape, dict(cg_resident=1, cg_variant=variant), 10) == (name, setup + per * 10)
