@@ -38,12 +38,14 @@
 // shared-memory kernel, or the one-pass streaming kernel where no whole
 // bricks fit):
 //   FP64  32^3 9.9 -> 4.7, 256 x 4 x 32 10.1 -> 4.7, 64 x 64 x 48 16.9 -> 9.3,
-//         50 x 47 x 33 28.3 -> 6.8, 77 x 130 x 50 66.8 -> 16.4, 96^3 77 -> 26.5
-//   FP32  32^3 4.2 -> 2.1, 64^3 5.0 -> 2.8, 96^3 7.3 -> 4.7, 160 x 160 x 48
-//         8.4 -> 5.6, 100 x 76 x 61 23.6 -> 3.7, 150 x 140 x 70 36.7 -> 8.2
+//         50 x 47 x 33 28.3 -> 6.9, 77 x 130 x 50 66.8 -> 16.5, 96^3 77 -> 27
+//   FP32  32^3 4.2 -> 2.1, 64^3 5.0 -> 2.8, 96^3 7.3 -> 4.8, 160 x 160 x 48
+//         8.4 -> 5.8, 100 x 76 x 61 23.6 -> 3.8, 150 x 140 x 70 36.7 -> 8.6
+// (in FP32 1 to 4 % of it for sums that are compensated from the threads on, and
+// scalars from the whole totals).
 // FP32 grids 128 nodes wide keep les_cg_regs.cu, whose four-node lanes read
-// x neighbours by shuffles: 128 x 64 x 64 2.8 there, 64 x 128 x 64 3.3 here; 128 x
-// 128 x 96 4.5, 96 x 128 x 128 7.2.
+// x neighbours by shuffles: 128 x 64 x 64 2.7 there, 64 x 128 x 64 3.4 here; 128 x
+// 128 x 96 4.5, 96 x 128 x 128 7.5.
 #include <algorithm>
 #include <cmath>
 #include <string>
@@ -182,8 +184,9 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
   // body(plane, its upper neighbour is surely of the run) up this thread's run.  The
   // plane counts are instantiated in steps of KT, so a run lacks KT planes at most; a
   // warp whose runs all have the others has no test between those, and their chains
-  // overlap (FP32: 96^3 5.0 -> 4.7 us per iteration, 150 x 140 x 70 9.4 -> 8.2; FP64
-  // waits for its arithmetic, not for chains, and loses 2 % by the longer code).
+  // overlap (FP32: 96^3 5.0 -> 4.7 us per iteration, 150 x 140 x 70 9.4 -> 8.2 as the
+  // sums were then; FP64 waits for its arithmetic, not for chains, and loses 2 % by the
+  // longer code).
   constexpr int KT = XS ? 4 : 2, ZF = sizeof(T) == 4 && ZP > KT ? ZP - KT : 0;
   const bool full = __all_sync(0xffffffffu, nzp >= ZF);
   auto each_plane = [&](auto&& body) {
@@ -233,7 +236,9 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
   int status = 0;  // 0 running, 1 converged, 2 maxit, 3 breakdown, 4 zero rhs, 5 timeout
   Acc rr_own{};  // this thread's share of r.r for the next sum
 
-  // XS = false: a node's tagged word among the published faces of q
+  // XS = false: a node's tagged word among the published faces of q (with an odd number
+  // of nodes the last one ends in the padding of its array, whose size is a multiple of
+  // 256 bytes)
   constexpr int W = Tagged<T>::BYTES;
   const int half = (int)(f.n / 2);
   auto word = [&](int s, int g) { return (g < half ? f.qt[0][s] : f.qt[1][s] - (size_t)half * W) + (size_t)g * W; };

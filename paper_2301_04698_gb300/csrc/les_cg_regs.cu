@@ -490,9 +490,9 @@ const void* regs_kernel(int zp) {
 int poisson_solve_regs(const SolverArgs<float>& a, const FusedCfg& fc, const float* b, float* x, double tol,
                        int maxit, int* iters, double* rel, std::string* err, bool* used) {
   *used = false;
-  // a guarded first guess (judged against x0 = 0) is left to the
-  // shared-memory kernel: the learned guess that asks for it needs a cubic
-  // grid, and no 128^3 grid fits on chip
+  // a guarded first guess (judged against x0 = 0) is left to the kernels of
+  // les_cg_chip.cu and les_cg_brick.cu: the learned guess that asks for it needs a
+  // cubic grid, and 128^3 is too large for the registers here
   if (!(a.op == LES_OP_COMPACT && a.solver == LES_SOLVER_CG && a.g.nx == kRegNx && a.g.nz >= 2 && !a.guard &&
         a.bar && a.r && a.p0 && a.p1))
     return LES_OK;

@@ -599,11 +599,12 @@ int poisson_solve_resident(const SolverArgs<T>& a, const FusedCfg& fc, const T* 
   if (!(a.op == LES_OP_COMPACT && a.solver == LES_SOLVER_CG && a.g.nz >= 2 && a.bar && a.r && a.p0 && a.p1))
     return LES_OK;
   // The vectors in registers: FP32 grids 128 nodes wide in les_cg_regs.cu
-  // (2.8 us per iteration on 128 x 64 x 64, against 3.3 on 64 x 128 x 64), every other grid in
+  // (2.7 us per iteration on 128 x 64 x 64, against 3.4 on 64 x 128 x 64), every other grid in
   // les_cg_chip.cu, up to 24 FP32 or 12 FP64 nodes per thread of one block per
   // SM, and above that, in FP32 up to 64 planes of 32 x 16 columns per SM, in
-  // les_cg_brick.cu.  What is left for the kernel here are FP64 grids of whole
-  // bricks between that and the shared memory of all SMs, and cg_resident = 2.
+  // les_cg_brick.cu.  What is left for the kernel here by default are a few shapes of
+  // whole bricks that their plans do not hold and its own does (FP64 96 x 168 x 52, flat
+  // FP32 ones such as 352 x 216 x 20), and cg_resident = 2.
   if constexpr (sizeof(T) == 4) {
     if (fc.resident == 0) {
       const int rc = poisson_solve_regs(a, fc, b, x, tol, maxit, iters, rel, err, used);

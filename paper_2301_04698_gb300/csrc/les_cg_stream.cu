@@ -24,7 +24,7 @@
 // is at hand, which takes a field off phase B; the one-pass kernels' second
 // stencil and two more sums, which save bytes, would cost nine operations.
 // FP32 keeps the second differences formed before scaling.
-// Measured (GB300, FP64, us per iteration): 256 x 256 x 128 186, 512 x 512 x 128 679;
+// Measured (GB300, FP64, us per iteration): 256 x 256 x 128 187, 512 x 512 x 128 680;
 // with runs dealt in turns, before the planes were shared out equally, 192 and 719.
 #include <algorithm>
 #include <string>

@@ -369,16 +369,17 @@ int poisson_solve(const SolverArgs<T>& a, const T* b, T* x, double tol, int maxi
     const int rc = poisson_solve_resident<T>(a, *a.fused, b, x, tol, maxit, iters, rel, err, &used);
     if (used || rc != LES_OK) return rc;
   }
-  // FP32 grids of whole columns: the one-pass kernel streams 6 fields per
-  // iteration against 9 (512 x 512 x 64: 117 us against 175)
+  // FP32 grids of whole columns: the one-pass kernel streams 5 fields per iteration
+  // (512 x 512 x 64: 86 us; 196 with the tile-aligned two-phase kernel, which streams
+  // 10, 256 with the one-pass kernel for any grid)
   if (a.bar && cg_c && (var == 4 || (var == 0 && sizeof(T) == 4)) && wave_cg_eligible(a.g.nx, a.g.ny, a.g.nz))
     return poisson_solve_wave<T>(a, *a.fused, b, x, tol, maxit, iters, rel, err);
   if (a.bar && cg_c && (var == 3 || var == 4)) return poisson_solve_roll<T>(a, *a.fused, b, x, tol, maxit, iters, rel, err);
   // every other grid: two phases, in FP64 because arithmetic bounds it (256 x
-  // 256 x 128: 198 us per iteration, 333 with the tile-aligned two-phase kernel,
-  // 612 and 629 with the one-pass kernels), in FP32 because tiles of any width
-  // keep its lanes full (1000 x 1000 x 100: 804 us against 1505 one-pass, 640 x
-  // 500 x 100: 281 against 403 tile-aligned)
+  // 256 x 128: 187 us per iteration, 329 with the tile-aligned two-phase kernel,
+  // 492 and 625 with the one-pass kernels), in FP32 because tiles of any width
+  // keep its lanes full (1000 x 1000 x 100: 720 us against 1463 one-pass, 640 x
+  // 500 x 100: 253 against 410 tile-aligned)
   if (a.bar && cg_c && var == 0) return poisson_solve_stream<T>(a, *a.fused, b, x, tol, maxit, iters, rel, err);
   if (a.bar && tiled && var == 2) return poisson_solve_fused<T>(a, *a.fused, b, x, tol, maxit, iters, rel, err);
   if (a.bar && a.fused && a.solver == LES_SOLVER_JACOBI)
