@@ -144,6 +144,7 @@ __global__ void __launch_bounds__(BX* BY, 1) k_cg_brick(ChipArgs<float> f) {
   GridSync gs{f.bar, f.partials, f.spin_cycles, f.expected, 0u};
   __shared__ struct {
     float mean, ta, tb;
+    float scale, xs;  // of r, p and q; alpha of x over that of r
     int status, restart;
     double bb, rel;  // |b - mean|^2 and the relative residual of x0
   } sc;
@@ -158,35 +159,42 @@ __global__ void __launch_bounds__(BX* BY, 1) k_cg_brick(ChipArgs<float> f) {
   chip_sum_clear<F2>(f.spread);  // no tag of an earlier solve: cleared here, for everyone after the first sum
   if (tid == 0) s_fail = 0;
 
-  // mean of b (b held in r)
+  // mean of b (b held in r, x0 in P); |b|_1 and |x0|_1
   {
-    ChipRun<float, ZP> s;
+    ChipRun<float, ZP> s, sb, sx;
     planes([&](int j, int g) {
-      if (own) r[j] = __ldcg(f.b + g);
+      float xv = 0.f;
+      if (own) {
+        r[j] = __ldcg(f.b + g);
+        xv = __ldcg(f.x + g);
+        C[SZ * j] = xv;
+      }
       s.add(j, r[j]);
+      sb.add(j, fabsf(r[j]));
+      sx.add(j, fabsf(xv));
     });
-    F2 v[1] = {total(s)};
-    double t[1];
-    const bool ok = grid_sum_t0<1>(v, gs, t);
+    F2 v[3] = {total(s), total(sb), total(sx)};
+    double t[3];
+    const bool ok = grid_sum_t0<3>(v, gs, t);
     if (tid == 0) {
       sc.status = ok ? 0 : 5;
       sc.mean = (float)(t[0] / (double)f.n);
+      sc.scale = chip_scale(t[1], t[2], 2.f * (cx + cy + cz) * f.sc, (double)f.n);
+      sc.xs = f.isc / sc.scale;
     }
     __syncthreads();
     status = sc.status;
   }
   const float mean = sc.mean;
-  // x0 with its ghosts in P; r = (b - mean) - L_c x0, published
+  // x0 with its ghosts in P; r = (b - mean) - L_c x0, scaled, published
   if (!status) {
-    planes([&](int j, int g) {
-      if (own) C[SZ * j] = __ldcg(f.x + g);
-    });
     fill_ghosts(f.x, false);
     __syncthreads();
     ChipRun<float, ZP> s0, s1;
     march([&](int j, int g, float, float q) {
-      const float bm = r[j] - mean;
-      r[j] = bm - f.sc * q;
+      float bm = r[j] - mean;
+      r[j] = (bm - f.sc * q) * sc.scale;
+      bm *= sc.scale;
       if (is_face(j)) __stcg(f.rg + g, r[j]);
       s0.add(j, r[j] * r[j]);
       s1.add(j, bm * bm);
@@ -210,7 +218,7 @@ __global__ void __launch_bounds__(BX* BY, 1) k_cg_brick(ChipArgs<float> f) {
       planes([&](int j, int g) {
         if (!own) return;
         __stcg(f.x + g, 0.f);
-        r[j] = __ldcg(f.b + g) - mean;
+        r[j] = (__ldcg(f.b + g) - mean) * sc.scale;
         s.add(j, r[j] * r[j]);
         if (is_face(j)) __stcg(f.rg + g, r[j]);
       });
@@ -309,7 +317,7 @@ __global__ void __launch_bounds__(BX* BY, 1) k_cg_brick(ChipArgs<float> f) {
       if (own) {
         int g = g0;
         asm volatile("" : "+r"(g));
-        const float tx = ta * f.isc;  // alpha of x
+        const float tx = ta * sc.xs;  // alpha of x
 #pragma unroll
         for (int b = 0; b < ZP; b += 8) {
           float xv[8];
@@ -344,6 +352,7 @@ __global__ void __launch_bounds__(BX* BY, 1) k_cg_brick(ChipArgs<float> f) {
     const bool ok = grid_sum_t0<1>(v, gs, t);
     if (tid == 0) {
       if (!ok) status = 5;
+      else if (status < 3 && !isfinite(t[0])) status = 3;  // x has left the range
       sc.mean = (float)(t[0] / (double)f.n);
       sc.status = status;
     }

@@ -226,6 +226,7 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
   GridSync gs{f.bar, f.partials, f.spin_cycles, f.expected, 0u};
   __shared__ struct {
     T mean, ta, tb, tx;  // alpha and beta of r and p, alpha of x
+    T scale, xs;         // of r, p and q (FP64: 1); alpha of x over that of r
     int status, restart;
     double bb, rel;  // |b - mean|^2 and the relative residual of x0
   } sc;
@@ -253,32 +254,42 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
   }
   if (tid == 0) s_fail = 0;
 
-  // mean of b (b held in r)
+  // mean of b (b held in r, x0 in p), FP32: |b|_1 and |x0|_1
   {
-    ChipRun<T, ZP> a1;
+    constexpr int NV = kScaled ? 1 : 3;
+    ChipRun<T, ZP> a[NV];
 #pragma unroll
     for (int j = 0; j < ZP; ++j)
       if (j < nzp) {
         r[j] = __ldcg(f.b + gown + j * gpl);
-        a1.add(j, r[j]);
+        p[j] = __ldcg(f.x + gown + j * gpl);
+        a[0].add(j, r[j]);
+        if constexpr (!kScaled) {
+          a[1].add(j, fabsf(r[j]));
+          a[2].add(j, fabsf(p[j]));
+        }
       }
-    Acc v[1] = {a1.total()};
-    double t[1];
-    const bool ok = grid_sum_t0<1>(v, gs, t);
+    Acc v[NV];
+#pragma unroll
+    for (int k = 0; k < NV; ++k) v[k] = a[k].total();
+    double t[NV];
+    const bool ok = grid_sum_t0<NV>(v, gs, t);
     if (tid == 0) {
       sc.status = ok ? 0 : 5;
       sc.mean = (T)(t[0] / (double)f.n);
+      if constexpr (kScaled) sc.scale = T(1);
+      else sc.scale = chip_scale(t[1], t[2], c0 * f.sc, (double)f.n);
+      sc.xs = kScaled ? mc0 : f.isc / sc.scale;
     }
     __syncthreads();
     status = sc.status;
   }
   const T mean = sc.mean;
-  // x0 with its ghosts in p and the copy; r = (b - mean) - L_c x0, published
+  // x0 with its ghosts in p and the copy; r = (b - mean) - L_c x0, scaled, published
   if (!status) {
 #pragma unroll
     for (int j = 0; j < ZP; ++j)
       if (j < nzp) {
-        p[j] = __ldcg(f.x + gown + j * gpl);
         set_x(j, p[j]);
         P[pown + j * SZ] = p[j];
       }
@@ -288,8 +299,9 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
 #pragma unroll
     for (int j = 0; j < ZP; ++j)
       if (j < nzp) {
-        const T bm = r[j] - mean;
-        r[j] = kScaled ? fma(c0, stencil(j, false), bm) : bm - f.sc * stencil(j, false);
+        T bm = r[j] - mean;
+        r[j] = kScaled ? fma(c0, stencil(j, false), bm) : (bm - f.sc * stencil(j, false)) * sc.scale;
+        if constexpr (!kScaled) bm *= sc.scale;
         if (is_face(j)) __stcg(f.rg + gown + j * gpl, r[j]);
         a2[0].add(j, r[j] * r[j]);
         a2[1].add(j, bm * bm);
@@ -314,7 +326,7 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
       for (int j = 0; j < ZP; ++j)
         if (j < nzp) {
           set_x(j, T(0));
-          r[j] = __ldcg(f.b + gown + j * gpl) - mean;
+          r[j] = (__ldcg(f.b + gown + j * gpl) - mean) * sc.scale;
           s.add(j, r[j] * r[j]);
           if (is_face(j)) __stcg(f.rg + gown + j * gpl, r[j]);
         }
@@ -425,7 +437,7 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
             else if (!good) st = 3;
             sc.ta = al;
             sc.tb = be;
-            sc.tx = kScaled ? al * mc0 : al * f.isc;
+            sc.tx = al * sc.xs;
           }
           sc.status = st;
         }
@@ -480,6 +492,7 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
     const bool ok = grid_sum_t0<1>(v, gs, t);
     if (tid == 0) {
       if (!ok) status = 5;
+      else if (status < 3 && !isfinite(t[0])) status = 3;  // x has left the range
       sc.mean = (T)(t[0] / (double)f.n);
       sc.status = status;
     }
@@ -640,9 +653,9 @@ int poisson_solve_chip(const SolverArgs<T>& a, const FusedCfg& fc, const T* b, T
   f.ny = a.g.ny;
   f.nz = a.g.nz;
   f.walls = a.g.walls;
-  f.sc = sizeof(T) == 4 ? (T)std::ldexp(1.0, std::ilogb(2.0 * ((double)a.g.idx * a.g.idx + (double)a.g.idy * a.g.idy +
-                                                              (double)a.g.idz * a.g.idz)))
-                        : T(1);
+  // the largest eigenvalue is 2 c0, c0 = 2 (1/dx^2 + 1/dy^2 + 1/dz^2)
+  const double c0 = 2.0 * ((double)a.g.idx * a.g.idx + (double)a.g.idy * a.g.idy + (double)a.g.idz * a.g.idz);
+  f.sc = sizeof(T) == 4 ? (T)std::ldexp(1.0, std::ilogb(c0) + 2) : T(1);
   f.isc = T(1) / f.sc;
   f.cx = a.g.idx * a.g.idx * f.isc;
   f.cy = a.g.idy * a.g.idy * f.isc;

@@ -19,8 +19,8 @@ constexpr int kChipGhosts = 4;      // ghost nodes per thread in registers
 template <typename T>
 struct ChipArgs {
   int nx, ny, nz, walls;
-  // 1/dx^2, 1/dy^2, 1/dz^2; FP32: times 2^-k, so that q is of the size of p and the four
-  // sums of the size of r.r, whatever the spacings (exact, but for what would leave the range)
+  // 1/dx^2, 1/dy^2, 1/dz^2; FP32: times 2^-k, so that no eigenvalue is above one and
+  // none of the four sums above r.r, whatever the spacings (exact)
   T cx, cy, cz;
   T sc, isc;           // 2^k, 2^-k (FP64: 1)
   int px, py, pz, zs;  // bricks along x, y, z; runs of planes per brick
@@ -86,8 +86,8 @@ __device__ __forceinline__ double acc_from_lane(double a, int l) { return __shfl
 // |r - alpha q|^2 / r.r, expanded in the totals: where next to nothing is left of r the
 // expansion may come out below zero, and is taken for none.
 // FP32: from the totals as pairs, each product and addition with its rounding error, and
-// rounded once (from FP64 totals in FP64 they would take thread 0 about a microsecond).
-// (a quotient from an approximate reciprocal ib of b and its remainder)
+// rounded once (from FP64 totals in FP64 they would take thread 0 about a microsecond);
+// a quotient from an approximate reciprocal ib of b and its remainder.
 __device__ __forceinline__ float rcp_approx(float x) {
   float y;
   asm("rcp.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -108,6 +108,10 @@ __device__ __forceinline__ bool chip_scalars(const F2 (&t)[4], float& ta, float&
   f2_acc(n, v);
   n.lo += (fmaf(m, rq.hi, -u) + m * rq.lo) + (fmaf(a2, q2.hi, -v) + a2 * q2.lo) + fmaf(ta, ta, -a2) * q2.hi;
   tb = f2_quotient(n, r2, ir);
+  if (!(isfinite(ta) && isfinite(tb))) {  // nothing left of r but subnormal squares
+    ta = r2.hi / pq.hi;
+    tb = fmaf(ta * ta, q2.hi, fmaf(-2.f * ta, rq.hi, r2.hi)) / r2.hi;
+  }
   tb = tb < 0.f ? 0.f : tb;
   return true;
 }
@@ -154,6 +158,15 @@ struct ChipRun<double, ZP> {
   __device__ __forceinline__ void add(int, double v) { s += v; }
   __device__ __forceinline__ double total() const { return s; }
 };
+
+// FP32: the power of two that brings the right side and L_c x0 to the size of one, from
+// |b|_1 and |x0|_1 (c0: L_c's centre coefficient), so that the solve's sums of squares
+// stay in range.  It changes no rounding.
+__device__ __forceinline__ float chip_scale(double b1, double x1, float c0, double n) {
+  const double m = fmax(b1, x1 * (double)c0) / n;
+  const int e = (__double2hiint(m) >> 20 & 0x7ff) - 1023;
+  return m == 0.0 ? 1.f : __int_as_float((127 - max(-126, min(126, e))) << 23);
+}
 
 // a warp's four values by a transposing butterfly (six additions instead of twenty)
 template <typename D>

@@ -44,12 +44,31 @@ def check(les_mod, shape, precision, exponents, spacing, tol, maxit, tuning=None
 @pytest.mark.parametrize("precision,shape", [(64, (24, 24, 24)), (64, (50, 47, 33)), (64, (77, 60, 50)),
                                              (32, (50, 47, 33)), (32, (100, 76, 61)), (32, (150, 130, 110))])
 def test_on_chip_cg(les_mod, precision, shape):
-    """FP64: r.r p.q would leave the range from 2^256 on.  FP32 at a spacing of 1 / 64: q.q
-    would, whose terms are those of r.r times (12 x 64^2)^2 at most, from 2^43 on."""
+    """FP64: r.r p.q would leave the range from 2^256 on.  FP32: r.r would from 2^64 on,
+    its terms from 2^-63 down; at a spacing of 1 / 64 q.q would from 2^43 on, whose terms
+    are those of r.r times (12 x 64^2)^2 at most."""
     if precision == 64:
         check(les_mod, shape, 64, (-300, 300), 1.0, 1e-8, 2000)
     else:
         check(les_mod, shape, 32, (-30, 43), 1 / 64, 1e-5, 2000)
+        check(les_mod, shape, 32, (-75, 80), 1.0, 1e-5, 2000)
+
+
+def test_first_guess_far_larger_than_the_right_side(les_mod):
+    """A first guess of 1e3 for a right side of 1e-17, its residual 1e21 times that: the
+    FP32 squares of neither may leave their range."""
+    case = inputs.Case(name="guess", nx=50, ny=47, nz=33, dx=1.0, dy=1.0, dz=1.0, walls=True, precision=32,
+                       init="zero", physics=())
+    sim = les_mod.Simulation(case)
+    b = torch.from_numpy(inputs.uniform(92, 0, case.n, -1, 1).reshape(case.shape)).to("cuda", torch.float32)
+    x0 = torch.from_numpy(inputs.uniform(93, 0, case.n, -1, 1).reshape(case.shape)).to("cuda", torch.float32) * 1e3
+    got = []
+    for e in (0, -57):
+        x = x0.clone()
+        rc, it, res = sim.poisson_solve(b * 2.0 ** e * 1e-17 ** (e == 0), x, 1e-30, 30, allow_not_converged=True)
+        got.append((rc, it, torch.isfinite(x).all().item()))
+    assert got == [(les_mod.LES_ERR_NOT_CONVERGED, 30, True)] * 2
+    sim.close()
 
 
 @pytest.mark.parametrize("shape", [(128, 24, 40), (70, 33, 40)])
@@ -63,3 +82,18 @@ def test_streaming_cg(les_mod, shape):
 def test_jacobi(les_mod, precision, shape):
     e = 80 if precision == 32 else 250
     check(les_mod, shape, precision, (-e, e), 1.0, 1e-30, 20, solver="jacobi")
+
+
+@pytest.mark.parametrize("shape", [(50, 47, 33), (150, 130, 110)])
+def test_solution_beyond_fp32_is_reported(les_mod, shape):
+    """A right side of 1e34 at a spacing of 100 has a solution past 1e38: non-finite, not
+    a solve that went well."""
+    nx, ny, nz = shape
+    case = inputs.Case(name="over", nx=nx, ny=ny, nz=nz, dx=100.0, dy=100.0, dz=100.0, walls=True, precision=32,
+                       init="zero", physics=())
+    sim = les_mod.Simulation(case)
+    b = torch.from_numpy(inputs.uniform(94, 0, case.n, -1, 1).reshape(case.shape)).to("cuda", torch.float32) * 1e34
+    with pytest.raises(les_mod.LesError) as e:
+        sim.poisson_solve(b, torch.zeros_like(b), 1e-4, 2000)
+    assert e.value.status == les_mod.LES_ERR_NONFINITE
+    sim.close()
