@@ -346,6 +346,7 @@ __global__ void __launch_bounds__(kChipThreads, 1) k_cg_chip(ChipArgs<T> f) {
         rel = sqrt(rr / bb);
         if (rel <= f.tol) status = 1;
         else if (f.maxit <= 0) status = 2;
+        else if (!isfinite(bb)) status = 3;  // (r.r <= tol^2 |b|^2 would hold)
       }
     }
     sc.status = status;

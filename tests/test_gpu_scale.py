@@ -97,3 +97,20 @@ def test_solution_beyond_fp32_is_reported(les_mod, shape):
         sim.poisson_solve(b, torch.zeros_like(b), 1e-4, 2000)
     assert e.value.status == les_mod.LES_ERR_NONFINITE
     sim.close()
+
+
+@pytest.mark.parametrize("shape,tuning", [((24, 24, 24), {}), ((50, 47, 33), {}), ((77, 60, 50), {}),
+                                          ((64, 32, 32), dict(cg_resident=2))])
+def test_norm_beyond_fp64_is_a_breakdown(les_mod, shape, tuning):
+    """|b|^2 of a right side of 1e200 is infinite, and so is the bound of r.r: no solve
+    that went well."""
+    nx, ny, nz = shape
+    case = inputs.Case(name="inf", nx=nx, ny=ny, nz=nz, dx=1.0, dy=1.0, dz=1.0, walls=True, precision=64,
+                       init="zero", physics=())
+    sim = les_mod.Simulation(case)
+    sim.set_tuning(**tuning)
+    b = torch.from_numpy(inputs.uniform(95, 0, case.n, -1, 1).reshape(case.shape)).cuda() * 1e200
+    with pytest.raises(les_mod.LesError) as e:
+        sim.poisson_solve(b, torch.zeros_like(b), 1e-8, 100)
+    assert e.value.status == les_mod.LES_ERR_NONFINITE
+    sim.close()
