@@ -12,9 +12,9 @@
 // What bounds it: instruction issue (about 75 per node and iteration) and shared
 // memory, 12 accesses per node and iteration (five neighbours twice, p read and
 // written).  Measured (GB300, us per iteration; before: the streaming kernels,
-// which take 27 to 36 bytes per node through L2): 192 x 192 x 128 38.2 -> 19.2,
-// 160 x 160 x 128 30.6 -> 12.8, 256 x 256 x 64 39.0 -> 18.5, 150 x 130 x 110 23.3 ->
-// 12.3 (18.6, 13.0, 17.8 and 12.6 with its scalars in plain FP32 and the ghosts after x).  Bricks of any extents, with their strides and column offsets in registers,
+// which take 27 to 36 bytes per node through L2): 192 x 192 x 128 38.2 -> 19.3,
+// 160 x 160 x 128 30.6 -> 12.8, 256 x 256 x 64 39.0 -> 18.6, 150 x 130 x 110 23.3 ->
+// 12.6 (18.3, 12.7, 17.5 and 12.1 with warps summed and scalars formed in plain FP32).  Bricks of any extents, with their strides and column offsets in registers,
 // spilled r and took 53 us on the first of these.
 #include <algorithm>
 #include <string>

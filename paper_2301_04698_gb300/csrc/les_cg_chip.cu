@@ -40,8 +40,8 @@
 //   FP64  32^3 9.9 -> 4.7, 256 x 4 x 32 10.1 -> 4.7, 64 x 64 x 48 16.9 -> 9.3,
 //         50 x 47 x 33 28.3 -> 6.9, 77 x 130 x 50 66.8 -> 16.5, 96^3 77 -> 27
 //   FP32  32^3 4.2 -> 2.1, 64^3 5.0 -> 2.8, 96^3 7.3 -> 4.8, 160 x 160 x 48
-//         8.4 -> 5.8, 100 x 76 x 61 23.6 -> 3.8, 150 x 140 x 70 36.7 -> 8.6
-// (in FP32 1 to 4 % of it for sums that are compensated from the threads on, and
+//         8.4 -> 5.8, 100 x 76 x 61 23.6 -> 3.8, 150 x 140 x 70 36.7 -> 8.7
+// (in FP32 3 to 6 % of it for sums that are compensated from the threads on, and
 // scalars from the whole totals).
 // FP32 grids 128 nodes wide keep les_cg_regs.cu, whose four-node lanes read
 // x neighbours by shuffles: 128 x 64 x 64 2.7 there, 64 x 128 x 64 3.4 here; 128 x
